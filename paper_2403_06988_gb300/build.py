@@ -1,6 +1,6 @@
 """Builds libdomino.so in-tree with nvcc for sm_103a (GB300).
 
-Three translation units (host.cpp: C ABI and loaders; kernels.cu and trie.cu:
+Three translation units (host.cpp: C ABI and loaders; kernels.cu and rows.cu:
 kernels) are compiled in parallel and linked into paper_2403_06988_gb300/libdomino.so.
 Objects go to paper_2403_06988_gb300/_build/.
 
@@ -24,7 +24,7 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libdomino.so")
 LIB_DEBUG = os.path.join(PKG, "libdomino_debug.so")
-SOURCES = ["host.cpp", "kernels.cu", "trie.cu"]
+SOURCES = ["host.cpp", "kernels.cu", "rows.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

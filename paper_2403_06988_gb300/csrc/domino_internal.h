@@ -73,51 +73,67 @@ struct StepView {
 };
 
 // Prefix tree of the vocabulary's byte-class strings (the subterminal tree of
-// Sec. 3.3, Alg. 2, over byte classes): a prefix shared by many tokens takes
-// its transitions once per row, and a subtree whose prefix dies is never
-// entered.  Nodes are numbered in preorder (children by class), so a subtree
-// is the contiguous range [n, skip) and the tokens of a subtree are a
-// contiguous range of `dtok`: the tokens that end at n first, then those of
-// its children's subtrees.
+// Sec. 3.3, Alg. 2, over byte classes) as domino_get_prefix_tree exports it.
+// Nodes are numbered in preorder (children by class), so a subtree is the
+// contiguous range [n, skip) and the tokens of a subtree are a contiguous
+// range of the token list: the tokens that end at n first, then those of its
+// children's subtrees.
 //   node[2n]     = {skip | cls << 24, tok_lo, n_end, tok_hi}
 //   node[2n + 1] = {sub_lo, sub_hi, 0, 0}
 // cls: the class on the edge into n; [tok_lo, tok_lo + n_end): tokens ending
 // at n; [tok_lo, tok_hi): tokens of the subtree; sub: the classes on the edges
-// below n (K <= 64, for the self-loop skip).
+// below n (K <= 64).
 // Upper nodes: the root and every node whose subtree has more than kTrieTile
 // nodes or more than kTrieBranch branching levels (an ancestor of an upper
-// node is upper).  Units: the subtrees hanging off upper nodes.  Inside a
-// unit, a node with one child and no token is walked together with its child:
-// the walk's records are such runs (up to 255 nodes).  The units are cut into
-// per-CTA batches that fit in shared memory; for a block of rows a CTA
-// computes each row's configuration at the upper nodes its units hang off
-// ("slots"), then each (unit, row live at its slot) pair is walked by one
-// thread, depth first over the unit's records, with a stack of at most
-// kTrieBranch entries (tree_tile_kernel).  The tokens that end at an upper
-// node are set by the one batch that lists that node as an emitting slot.
+// node is upper).  Units: the subtrees hanging off upper nodes.
 constexpr int kTrieTile = 64;
 constexpr int kTrieBranch = 8;
-constexpr int kTrieInterleave = 2;      // places of the tree a CTA's units are drawn from
-constexpr int kTrieMaxSlots = 48;             // slots per batch
 constexpr int32_t kTrieMaxNodes = (1 << 24) - 1;
 
-struct TrieView {
-    const uint4* node;        // the walk's records, two each: {end record, first node, nodes, first token},
-                              //   {tokens ending at the last node, classes below it (64 bits), 0}
-    const uint8_t* ncls;      // [n_nodes]: each node's class (the records' classes, in order)
-    const int32_t* dtok;      // original ids in preorder
-    const uint4* upper;       // [n_upper]: {node, path offset, path length, 0}
-    const uint8_t* upath;     // classes of the upper nodes' paths from the root
-    const uint4* batch;       // [n_batches][2]: {first unit, end unit, first range, end range},
-                              //                 {first slot, end slot, staged nodes, staged tokens}
-    const uint4* range;       // two each: {first record, end record, first token, end token},
-                              //   {first node, end node, 0, 0}; staged one after the other
-    const uint4* slot;        // {upper index, first token ending at its node, tokens it sets (0: none), 0}
-    const uint2* unit;        // {root's staged index, slot index within the batch}
-    const int32_t* cta_batch; // [grid + 1]: CTA c takes batches [cta_batch[c], cta_batch[c + 1])
-    int32_t n_nodes, n_upper, grid, n_batches;
-    int32_t max_nodes, max_cls, max_toks, max_units, max_slots, max_path;   // the largest batch (records, nodes, ...)
+// The trees row_kernel walks (rows.cu).  The first (root: node 0) holds the
+// class strings of all tokens (but EOS and empty ones).  The others belong to
+// the loop sets: a loop set is the classes that keep some state L (with no
+// stack action).  A row in L allows every token made of these classes only
+// (loopbits) and stays where it is over the longest such prefix of any other
+// token, so the set's tree holds the other tokens' remainders after that
+// prefix.
+// Nodes are numbered breadth first per tree: a node's children are
+// consecutive, in class order.  Tokens are listed in preorder, so a subtree's
+// are consecutive, the node's own first.
+//   node[2n]     = {children's classes (64 bits; K > 64: their number, 0),
+//                   first child | tokens ending here (255: or more) << 24,
+//                   the subtree's first token}
+//   node[2n + 1] = {subtree's tokens [x, y) in dtok, classes below (64 bits)}
+// State records (K <= 64), srec_stride bytes each: {live classes, classes
+// that keep the state} (64 bits each), then the live classes' entries.  Bit
+// 63 of the second (K <= 63 where there are loop sets): the state has a loop
+// set.  For masks the states are those of the automaton with equivalent
+// states merged (start: the state a row begins in).
+// Inside any tree, a node entered in L with loop set S: its subtree's tokens
+// p of dtok that stay inside S from the node on are those with keeps[S][p] <=
+// the node's depth; the edges below it that leave S are the entries
+// xrange[S][node] of exits (preorder) whose nearest exit above (0: none) is
+// no deeper than the node.
+struct RowTree {
+    const uint4* node;
+    const uint8_t* ncls;        // [n_nodes] class on the edge into each node
+    const int32_t* dtok;
+    const uint4* srec;
+    const uint16_t* ret;        // pop targets, [triples][4]
+    const uint2* start;         // [Q]: {the record's state, its loop set or ~0}; nullptr: the state itself, no loop sets
+    const uint32_t* loop_of;    // per record its loop set or ~0
+    const uint32_t* loopbits;   // [loop sets][W]
+    const uint8_t* keeps;       // [loop sets][n_dtok]: position after the last class outside the set (at most 255)
+    const uint2* xrange;        // [loop sets][n_nodes]: {first exit below | depth << 24 (255: or more), end exit}
+    const uint2* exits;         // {node, its class | depth of the nearest exit above (at most 255) << 8}
+    int32_t srec_stride, n_nodes, n_dtok, n_loops;
+    int32_t reserve;            // pool entries a depth-first walk of any node can add
+    int32_t max_kids;           // most children of any node (at least 1)
+    int32_t loop_root[4];
 };
+constexpr int kRowLoopSets = 4;           // loop sets with a tree of their own
+constexpr int kRowMaxSlices = 8;          // CTAs per row (one cluster)
+constexpr int kRowSliceWords = 16384;     // mask words a CTA can hold
 
 struct LaunchEnv {
     int num_sms;
@@ -146,19 +162,18 @@ cudaError_t launch_fused_combine(const StepView& v, bool stack, int mode, const 
                                  int32_t n_windows, int32_t* argmax, float* lse, const int32_t* states,
                                  const uint64_t* stacks, int32_t* states_out, uint64_t* stacks_out, cudaStream_t st);
 
-// The mask step over the prefix tree: tree_clear_kernel (one warp per row:
-// clears the row's mask and next states, sets EOS), then tree_tile_kernel
-// (the units, from shared memory).  states / stacks / batch / row_is_state /
-// mask / next / row_ids / row_count as launch_step_mask.  mode: where the tile
-// kernel reads transitions.
-int trie_tile_smem_bytes(const StepView& v, const TrieView& tv, bool stack, int table_bytes);
-// row_next (the precompute: row_is_state, next states written, no row list):
-// tv.n_batches device words through which the CTAs share out the batches' row
-// blocks (nullptr: each CTA walks every row of its own batches).
-cudaError_t launch_trie_step(const StepView& v, const TrieView& tv, const LaunchEnv& env, bool stack, int mode,
-                             const int32_t* states, const uint64_t* stacks, int32_t batch, bool row_is_state,
-                             uint32_t* mask, int32_t* next, cudaStream_t st, const int32_t* row_ids = nullptr,
-                             const int32_t* row_count = nullptr, int32_t* row_next = nullptr);
+// The mask step with one CTA (or a cluster of them) per row; arguments as
+// launch_step_mask.  Any K, V <= kRowMaxSlices * kRowSliceWords * 32, and a
+// tree whose row_smem_bytes fit.
+cudaError_t launch_row_step(const StepView& v, const RowTree& t, const LaunchEnv& env, bool stack,
+                            const int32_t* states, const uint64_t* stacks, int32_t batch, bool row_is_state,
+                            uint32_t* mask, int32_t* next, cudaStream_t st, const int32_t* row_ids = nullptr,
+                            const int32_t* row_count = nullptr);
+// The host's side of the walk's pool bound (RowTree::reserve): a node with
+// `kids` children, the deepest of which need `below`; and the shared memory a
+// CTA needs.
+int32_t row_reserve(int32_t kids, int32_t below);
+int row_smem_bytes(int32_t n_words, int32_t reserve, bool stack, bool loops);
 
 // Log-probabilities only (bf16 logits, rows on 16-byte boundaries), given the
 // rows' lse: logprobs[b][t] = logit - lse[b] for allowed t, -inf else.

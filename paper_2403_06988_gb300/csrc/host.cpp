@@ -59,28 +59,19 @@ struct domino_ctx {
     DevBuf d_dense, d_sparse, d_accept, d_self, d_tok_cls;
     DevBuf d_err, d_partials, d_counters, d_lse_tmp, d_fpart;
     bool arena_ready = false;
-    // prefix tree of the class strings and its per-CTA batches (see TrieView)
-    DevBuf d_tnode, d_tncls, d_tdtok, d_tupper, d_tupath, d_tbatch, d_trange, d_tslot, d_tunit, d_tcta;
-    DevBuf d_trow;                   // the precompute's row counter per batch
-    std::vector<uint4> t_node;       // host copies (domino_get_prefix_tree)
-    std::vector<uint4> t_cnode;      // the walk's records (chains of nodes), two per record
-    std::vector<uint32_t> t_hc;      // [n_nodes + 1]: records before each node
-    std::vector<uint8_t> t_ncls;     // each node's class
+    // prefix tree of the class strings (domino_get_prefix_tree)
+    std::vector<uint4> t_node;
     std::vector<int32_t> t_dtok;
     std::vector<uint4> t_upper;      // {node, path offset, path length, 0}
     std::vector<uint8_t> t_upath;
     std::vector<uint2> t_unit;       // {root node, parent upper index}
-    // per-CTA batches (see TrieView)
-    std::vector<uint4> t_batch;      // two per batch
-    std::vector<uint4> t_range;      // {first node, end node, first token, end token}
-    std::vector<uint4> t_slot;
-    std::vector<uint2> t_bunit;      // {root node, slot within the batch}
-    std::vector<int32_t> t_cta;      // [grid + 1] first batch of each CTA
-    int32_t t_nodes = 0, t_grid = 0;
-    int32_t t_max_nodes = 0, t_max_cls = 0, t_max_toks = 0, t_max_units = 0, t_max_slots = 0, t_max_path = 0;
-    int t_mode = kDenseGlobal;       // where the tile kernel reads transitions
-    bool trie_built = false;         // host arrays valid
-    bool trie_ready = false;         // device copies valid
+    int32_t t_nodes = 0;
+    bool trie_built = false;
+    // the trees row_kernel walks (see RowTree)
+    DevBuf d_rnode, d_rncls, d_rdtok, d_srec, d_srec_next, d_rret, d_rstart, d_loop_of, d_loopbits, d_keeps, d_xrange,
+        d_exits;
+    RowTree rows{}, rows_next{};     // for masks; for next states
+    bool rows_ready = false;
     // which walk the mask step takes: -1 chosen from the automaton (see
     // use_tree), 1 the prefix tree, 0 every token on its own (DOMINO_WALK=tree
     // or =token in the environment when the handle is created)
@@ -181,18 +172,16 @@ void clear_host_graphs(domino_ctx* h) {
     h->t_wall_ms[0] = h->t_wall_ms[1] = 0.0;   // the paths are timed afresh
 }
 
-// The prefix tree of the tokens' class strings (TrieView), built from the
+// The prefix tree of the tokens' class strings, built from the
 // tokens sorted by class string: a token shares with its predecessor the
 // nodes of their longest common prefix and opens new nodes for the rest, so
 // nodes come out in preorder.  EOS and empty tokens are not in the tree (the
 // kernel sets EOS from the row's acceptance; other empty tokens are never
-// allowed).  Host arrays only; build_trie uploads them.
+// allowed).  Host arrays only (domino_get_prefix_tree; build_rows lays out
+// the trees the kernel walks).
 void build_trie_host(domino_ctx* h) {
-    h->trie_built = h->trie_ready = false;
+    h->trie_built = false;
     h->t_node.clear();
-    h->t_cnode.clear();
-    h->t_hc.clear();
-    h->t_ncls.clear();
     h->t_dtok.clear();
     h->t_upper.clear();
     h->t_upath.clear();
@@ -296,41 +285,6 @@ void build_trie_host(domino_ctx* h) {
         node[2 * (size_t)n] = make_uint4(skip[n] | ((uint32_t)ncls[n] << 24), tok_lo[n], n_end[n], tok_hi[n]);
         node[2 * (size_t)n + 1] = make_uint4((uint32_t)sub[n], (uint32_t)(sub[n] >> 32), 0u, 0u);
     }
-    // Chains: inside a unit, a node with one child and no token ending at it
-    // is walked together with that child.  The walk's records are the chains'
-    // first nodes (heads); a record covers `len` nodes (at most 255), its
-    // classes are those nodes' classes, and its tokens and classes-below are
-    // those of its last node.  Upper nodes stay records of their own.
-    std::vector<uint32_t> nchild(N, 0);
-    for (uint32_t n = 1; n < N; n++) nchild[parent[n]]++;
-    std::vector<uint8_t> head(N, 1);
-    std::vector<uint32_t> clen(N, 1);   // a head's chain length
-    for (const uint2& u : unit) {
-        uint32_t cur = u.x;
-        for (uint32_t n = u.x + 1; n < skip[u.x]; n++) {
-            const uint32_t pp = parent[n];
-            if (nchild[pp] == 1 && n_end[pp] == 0 && pp + 1 == n && clen[cur] < 255 &&
-                cur + clen[cur] == n) {
-                head[n] = 0;
-                clen[cur]++;
-            } else {
-                cur = n;
-            }
-        }
-    }
-    std::vector<uint32_t> hc((size_t)N + 1, 0);   // heads before each node
-    for (uint32_t n = 0; n < N; n++) hc[n + 1] = hc[n] + head[n];
-    std::vector<uint4> cnode((size_t)hc[N] * 2);
-    for (uint32_t n = 0; n < N; n++) {
-        if (!head[n]) continue;
-        const uint32_t b = n + clen[n] - 1;   // the chain's last node
-        const size_t c = hc[n];
-        cnode[2 * c] = make_uint4(hc[skip[n]], n, clen[n], tok_lo[n]);
-        cnode[2 * c + 1] = make_uint4(n_end[b], (uint32_t)sub[b], (uint32_t)(sub[b] >> 32), 0u);
-    }
-    h->t_cnode.swap(cnode);
-    h->t_hc.swap(hc);
-    h->t_ncls.swap(ncls);
     h->t_node.swap(node);
     h->t_dtok.swap(dtok);
     h->t_upper.swap(upper);
@@ -340,279 +294,389 @@ void build_trie_host(domino_ctx* h) {
     h->trie_built = true;
 }
 
-// Cuts the units into per-CTA batches that fit in the tile kernel's shared
-// memory next to the transition table, for a grid of one CTA per SM.  Units
-// are weighed by their estimated walk cost, cut in preorder into kTrieInterleave
-// chunks per CTA of equal weight, and CTA c takes chunks c, c + grid, ...; a
-// batch holds some of one CTA's units (staged as node, record and token ranges
-// one after the other, costliest units first), the upper nodes they hang off
-// (slots), and the upper nodes whose tokens it sets (emitting slots: each upper
-// node with tokens is set by the batch of the first unit after it in preorder).
-// Chooses the table placement: in shared memory when that leaves room for
-// batches, else through L1/L2.  false: some unit alone does not fit (the
-// per-token walk is used).
-bool cut_batches(domino_ctx* h) {
-    const int smem = h->env.max_smem_optin > 0 ? h->env.max_smem_optin : 232448;
-    const int grid = h->env.num_sms > 0 ? h->env.num_sms : 1;
-    StepView v = make_view(h);
-    const bool self = !h->self_mask.empty();
-    const std::vector<uint2>& unit = h->t_unit;
-    const std::vector<uint4>& node = h->t_node;
-    const std::vector<uint4>& upper = h->t_upper;
-    auto skip_of = [&](uint32_t n) { return node[2 * (size_t)n].x & 0xFFFFFFu; };
-    // fixed shared memory with an empty batch, per table placement
-    TrieView tv0{};
-    const int fixed = trie_tile_smem_bytes(v, tv0, h->stack, 0) + 1024;
-    constexpr int kMinBatch = 24 * 1024;
-    int mode = kDenseGlobal;
-    int64_t table = 0;
-    const int modes[2] = {kDenseSmem, h->sp_words == 2 ? kSparse32Smem : kSparse64Smem};
-    for (int m : modes) {
-        if (m != kDenseSmem && h->sp_nnz == 0) continue;
-        const int64_t t = table_smem_bytes(v, h->stack, m);
-        if ((int64_t)smem - fixed - t >= kMinBatch) {
-            mode = m;
-            table = t;
-            break;
+// The host side of RowTree while it is built.
+struct RowStr {
+    const uint8_t* p;   // a token's (remaining) classes
+    uint32_t len;
+    int32_t token;
+};
+bool row_str_less(const RowStr& a, const RowStr& b) {
+    const int c = std::memcmp(a.p, b.p, std::min(a.len, b.len));
+    if (c != 0) return c < 0;
+    if (a.len != b.len) return a.len < b.len;
+    return a.token < b.token;
+}
+struct RowBuild {
+    bool wide = false;
+    std::vector<uint64_t> sets;   // the loop sets
+    std::vector<uint4> node;
+    std::vector<uint8_t> ncls;
+    std::vector<int32_t> dtok;
+    std::vector<std::vector<uint8_t>> keeps;   // per loop set
+    std::vector<std::vector<uint2>> xrange, exits;
+    int32_t reserve = 0, max_kids = 1;
+};
+
+// Appends the tree over `strs` (sorted).  Returns its root, or -1 when the
+// node or exit numbers run out of their 24 bits.
+int64_t add_row_tree(RowBuild& rb, const std::vector<RowStr>& strs) {
+    const int64_t root = (int64_t)(rb.node.size() / 2);
+    // preorder: the subtree ends and token ranges (as build_trie_host)
+    std::vector<uint32_t> skip, lo, own, hi, path;
+    std::vector<uint8_t> cls, depth;
+    auto open_node = [&](uint8_t c) {
+        depth.push_back((uint8_t)std::min<size_t>(path.size(), 255));
+        path.push_back((uint32_t)skip.size());
+        skip.push_back(0);
+        lo.push_back((uint32_t)rb.dtok.size());
+        own.push_back(0);
+        hi.push_back(0);
+        cls.push_back(c);
+    };
+    auto close_node = [&]() {
+        const uint32_t n = path.back();
+        path.pop_back();
+        skip[n] = (uint32_t)skip.size();
+        hi[n] = (uint32_t)rb.dtok.size();
+    };
+    open_node(0);
+    const RowStr* prev = nullptr;
+    for (const RowStr& s : strs) {
+        uint32_t l = 0;
+        while (prev && l < std::min(s.len, prev->len) && prev->p[l] == s.p[l]) l++;
+        while (path.size() > (size_t)l + 1) close_node();
+        for (uint32_t d = l; d < s.len; d++) open_node(s.p[d]);
+        if ((int64_t)skip.size() + root > (int64_t)kTrieMaxNodes) return -1;
+        own[path.back()]++;
+        rb.dtok.push_back(s.token);
+        for (size_t i = 0; i < rb.sets.size(); i++) {
+            uint32_t k = s.len;
+            while (k > 0 && ((rb.sets[i] >> s.p[k - 1]) & 1ull)) k--;
+            rb.keeps[i].push_back((uint8_t)std::min<uint32_t>(k, 255));
         }
+        prev = &s;
     }
-    // A unit costs about the transitions its walk takes, which depend on the
-    // rows.  For a DFA they are counted here by walking the tree from up to
-    // 1024 states spread evenly over the automaton (the visits inside each
-    // unit); the CTAs' shares are balanced on those counts plus the units'
-    // node counts.  Pushdown automata are balanced on node counts.
-    std::vector<int64_t> unit_nodes(unit.size());
-    for (size_t u = 0; u < unit.size(); u++) unit_nodes[u] = skip_of(unit[u].x) - unit[u].x;
-    if (!h->stack && !h->t16.empty() && h->Q > 1 && !unit.empty()) {
-        const int32_t Q = h->Q, K = h->K;
-        const uint32_t N = skip_of(0);
-        std::vector<int32_t> unit_of(N, -1);
-        for (size_t u = 0; u < unit.size(); u++)
-            for (uint32_t n = unit[u].x; n < skip_of(unit[u].x); n++) unit_of[n] = (int32_t)u;
-        std::vector<int64_t> visits(unit.size(), 0);
-        struct Frame {
-            uint32_t next, end, s;
-        };
-        std::vector<Frame> stk;
-        const int32_t stride = std::max<int32_t>(1, (Q - 1) / 1024);
-        for (int32_t q = 1; q < Q; q += stride) {
-            uint32_t n = 1, end = N, s = (uint32_t)q;
-            stk.clear();
-            for (;;) {
-                if (n >= end) {
-                    if (stk.empty()) break;
-                    const Frame f = stk.back();
-                    stk.pop_back();
-                    n = f.next, end = f.end, s = f.s;
-                    continue;
-                }
-                const uint32_t x = node[2 * (size_t)n].x, sk = x & 0xFFFFFFu;
-                const uint32_t s2 = h->t16[(size_t)s * K + (x >> 24)];
-                if (unit_of[n] >= 0) visits[(size_t)unit_of[n]]++;
-                if (s2 != 0 && sk > n + 1) {
-                    stk.push_back({sk, end, s});
-                    n = n + 1, end = sk, s = s2;
-                } else {
-                    n = sk;
-                }
-            }
+    while (!path.empty()) close_node();
+    const uint32_t N = (uint32_t)skip.size();
+    std::vector<uint64_t> sub(N, 0);
+    std::vector<int32_t> need(N, 0);
+    for (uint32_t n = N; n-- > 0;) {
+        int32_t kids = 0, below = 0;
+        for (uint32_t c = n + 1; c < skip[n]; c = skip[c]) {
+            kids++;
+            below = std::max(below, need[c]);
+            if (!rb.wide) sub[n] |= (1ull << cls[c]) | sub[c];
         }
-        for (size_t u = 0; u < unit.size(); u++) unit_nodes[u] += visits[u];
+        need[n] = std::min<int32_t>(1 << 20, row_reserve(kids, below));
+        rb.max_kids = std::max(rb.max_kids, kids);
     }
-    int64_t total = 0;
-    for (size_t u = 0; u < unit.size(); u++) total += unit_nodes[u];
-    const int per_rec = 16 + (self ? 8 : 0);   // a staged walk record (and its classes below)
-    const std::vector<uint32_t>& hc = h->t_hc;
-    if (unit.empty()) return false;
-    // the upper nodes whose tokens a unit's batch sets: those with tokens
-    // between the previous unit's root and its own (trailing ones: the last)
-    std::vector<std::vector<uint32_t>> emit_at(unit.size());
-    {
-        size_t ui = 0;
-        for (size_t u = 0; u < upper.size(); u++) {
-            if (node[2 * (size_t)upper[u].x].z == 0) continue;
-            while (ui < unit.size() && unit[ui].x < upper[u].x) ui++;
-            emit_at[std::min(ui, unit.size() - 1)].push_back((uint32_t)u);
+    rb.reserve = std::max(rb.reserve, need[0]);
+    // breadth first: order[i] is the preorder number of node root + i
+    std::vector<uint32_t> order(1, 0), at(N, 0);
+    order.reserve(N);
+    rb.node.resize((size_t)(root + N) * 2);
+    rb.ncls.resize((size_t)(root + N));
+    for (size_t i = 0; i < order.size(); i++) {
+        const uint32_t n = order[i];
+        const uint32_t first = (uint32_t)(root + (int64_t)order.size());
+        uint64_t kids = 0;
+        for (uint32_t c = n + 1; c < skip[n]; c = skip[c]) {
+            order.push_back(c);
+            kids = rb.wide ? kids + 1 : kids | (1ull << cls[c]);
         }
+        at[n] = (uint32_t)(root + (int64_t)i);
+        rb.ncls[(size_t)root + i] = cls[n];
+        const uint32_t first_tok = lo[n] < hi[n] ? (uint32_t)rb.dtok[lo[n]] : 0u;
+        rb.node[2 * ((size_t)root + i)] = make_uint4((uint32_t)kids, (uint32_t)(kids >> 32),
+                                                     first | (std::min<uint32_t>(own[n], 255u) << 24), first_tok);
+        rb.node[2 * ((size_t)root + i) + 1] =
+            make_uint4(lo[n], hi[n], (uint32_t)sub[n], (uint32_t)(sub[n] >> 32));
     }
-    // The units in preorder are cut into grid x kTrieInterleave chunks of
-    // equal cost; CTA c takes chunks c, c + grid, ...  The rows live at a
-    // unit vary from one batch of rows to the next, and nearby units share
-    // their upper nodes, so a CTA's share drawn from several places of the
-    // tree varies less than one run of it.
-    const int nchunk = grid * kTrieInterleave;
-    std::vector<size_t> cbeg((size_t)nchunk + 1, unit.size());
-    {
-        int64_t done = 0;
-        size_t u = 0;
-        for (int j = 0; j < nchunk; j++) {
-            cbeg[(size_t)j] = u;
-            const int64_t goal = total * (j + 1) / nchunk;
-            while (u < unit.size() && (done < goal || j == nchunk - 1)) done += unit_nodes[u++];
+    // the edges that leave each loop set, in preorder
+    for (size_t i = 0; i < rb.sets.size(); i++) {
+        std::vector<uint2>& ex = rb.exits[i];
+        std::vector<uint2>& xr = rb.xrange[i];
+        xr.resize((size_t)(root + N));
+        std::vector<uint32_t> first(N + 1, 0);   // exits before each preorder number
+        std::vector<uint8_t> above(N, 0);        // depth of the nearest exit on the path to the node, itself included
+        for (uint32_t n = 0; n < N; n++) {
+            first[n] = (uint32_t)ex.size();
+            const bool out = n != 0 && !((rb.sets[i] >> cls[n]) & 1ull);
+            if (out) ex.push_back(make_uint2(at[n], (uint32_t)cls[n] | ((uint32_t)above[n] << 8)));
+            if (out) above[n] = depth[n];
+            for (uint32_t c = n + 1; c < skip[n]; c = skip[c]) above[c] = above[n];
         }
+        first[N] = (uint32_t)ex.size();
+        if (ex.size() >= (size_t)(1u << 24)) return -1;
+        for (uint32_t n = 0; n < N; n++)
+            xr[at[n]] = make_uint2(first[n + 1] | ((uint32_t)depth[n] << 24), first[skip[n]]);
     }
-    for (int64_t budget = (int64_t)smem - fixed - table; budget >= 4096; budget = budget * 9 / 10) {
-        std::vector<uint4> batch, slot, range;
-        std::vector<uint2> bunit;
-        std::vector<int64_t> bweight;   // the estimated cost of each bunit entry
-        std::vector<int32_t> cta((size_t)grid + 1, 0);
-        int32_t mx_nodes = 0, mx_cls = 0, mx_toks = 0, mx_units = 0, mx_slots = 0, mx_path = 0;
-        bool ok = true;
-        for (int c = 0; c < grid && ok; c++) {
-            cta[(size_t)c] = (int32_t)(batch.size() / 2);
-            std::vector<std::pair<size_t, size_t>> runs;   // this CTA's unit runs, in preorder
-            for (int k = 0; k < kTrieInterleave; k++) {
-                const size_t j = (size_t)c + (size_t)k * grid;
-                if (cbeg[j] < cbeg[j + 1]) runs.emplace_back(cbeg[j], cbeg[j + 1]);
-            }
-            size_t ri = 0, u = runs.empty() ? 0 : runs[0].first;
-            while (ri < runs.size() && ok) {
-                // one batch: units of this CTA's runs from u on, staged as node
-                // and token ranges one after the other
-                const size_t slot0 = slot.size(), unit0 = bunit.size(), range0 = range.size();
-                std::vector<std::pair<uint32_t, uint32_t>> slots;   // (upper index, slot)
-                auto slot_of = [&](uint32_t ui, bool emit) -> int {
-                    const uint32_t n = upper[ui].x;
-                    for (auto& p : slots)
-                        if (p.first == ui) {
-                            if (emit) slot[slot0 + p.second].z = node[2 * (size_t)n].z;
-                            return (int)p.second;
-                        }
-                    if ((int)slots.size() >= kTrieMaxSlots) return -1;
-                    slot.push_back(make_uint4(ui, node[2 * (size_t)n].y, emit ? node[2 * (size_t)n].z : 0u, 0u));
-                    slots.emplace_back(ui, (uint32_t)slots.size());
-                    mx_path = std::max<int32_t>(mx_path, (int32_t)upper[ui].z);
-                    return (int)slots.size() - 1;
-                };
-                int64_t recs_b = 0, cls_b = 0, toks_b = 0;   // staged by the closed ranges
-                bool open = false;
-                uint32_t rn0 = 0, rn1 = 0, rt0 = 0, rt1 = 0;   // the open range (nodes, tokens)
-                auto close_range = [&]() {
-                    if (!open) return;
-                    range.push_back(make_uint4(hc[rn0], hc[rn1], rt0, rt1));
-                    range.push_back(make_uint4(rn0, rn1, 0u, 0u));
-                    recs_b += hc[rn1] - hc[rn0];
-                    cls_b += rn1 - rn0;
-                    toks_b += rt1 - rt0;
-                    open = false;
-                };
-                size_t added = 0;
-                while (ri < runs.size()) {
-                    if (u >= runs[ri].second) {   // the run is done: its range closes
-                        close_range();
-                        if (++ri < runs.size()) u = runs[ri].first;
-                        continue;
-                    }
-                    const size_t keep_slots = slot.size();
-                    const auto keep_list = slots;
-                    std::vector<uint32_t> keep_z;
-                    for (size_t k = slot0; k < slot.size(); k++) keep_z.push_back(slot[k].z);
-                    bool fit = true;
-                    for (uint32_t e : emit_at[u])
-                        if (fit) fit = slot_of(e, true) >= 0;
-                    const int sl = fit ? slot_of(unit[u].y, false) : -1;
-                    fit = sl >= 0;
-                    const uint32_t n0 = open ? rn0 : unit[u].x, t0 = open ? rt0 : node[2 * (size_t)unit[u].x].y;
-                    const uint32_t n1 = skip_of(unit[u].x), t1 = node[2 * (size_t)unit[u].x].w;
-                    const int64_t recs_all = recs_b + (hc[n1] - hc[n0]), cls_all = cls_b + (n1 - n0);
-                    const int64_t toks_all = toks_b + (t1 - t0);
-                    if (fit)
-                        fit = recs_all <= 0xFFFF && toks_all <= 0xFFFF &&
-                              recs_all * per_rec + ((cls_all + 15) & ~15) + toks_all * 4 +
-                                      (int64_t)(bunit.size() - unit0 + 1) * 4 + (int64_t)slots.size() * (16 + 64) <=
-                                  budget;
-                    if (!fit) {   // undo this unit's slots; the batch ends before it
-                        slot.resize(keep_slots);
-                        slots = keep_list;
-                        for (size_t k = slot0; k < slot.size(); k++) slot[k].z = keep_z[k - slot0];
-                        if (added == 0) ok = false;   // a unit alone does not fit
-                        break;
-                    }
-                    bunit.push_back(make_uint2((uint32_t)(recs_b + (hc[unit[u].x] - hc[n0])), (uint32_t)sl));
-                    bweight.push_back(unit_nodes[u]);
-                    if (!open) {
-                        rn0 = n0;
-                        rt0 = t0;
-                        open = true;
-                    }
-                    rn1 = n1;
-                    rt1 = t1;
-                    added++;
-                    u++;
-                }
-                if (!ok) break;
-                close_range();
-                {   // the costliest units first: the warps' last claims are short ones
-                    std::vector<size_t> ord(bunit.size() - unit0);
-                    for (size_t k = 0; k < ord.size(); k++) ord[k] = unit0 + k;
-                    std::stable_sort(ord.begin(), ord.end(),
-                                     [&](size_t x, size_t y) { return bweight[x] > bweight[y]; });
-                    std::vector<uint2> su;
-                    std::vector<int64_t> sw;
-                    for (size_t k : ord) {
-                        su.push_back(bunit[k]);
-                        sw.push_back(bweight[k]);
-                    }
-                    std::copy(su.begin(), su.end(), bunit.begin() + (ptrdiff_t)unit0);
-                    std::copy(sw.begin(), sw.end(), bweight.begin() + (ptrdiff_t)unit0);
-                }
-                batch.push_back(make_uint4((uint32_t)unit0, (uint32_t)bunit.size(), (uint32_t)(range0 / 2),
-                                           (uint32_t)(range.size() / 2)));
-                batch.push_back(make_uint4((uint32_t)slot0, (uint32_t)slot.size(), (uint32_t)recs_b,
-                                           (uint32_t)toks_b));
-                mx_nodes = std::max<int32_t>(mx_nodes, (int32_t)recs_b);
-                mx_cls = std::max<int32_t>(mx_cls, (int32_t)cls_b);
-                mx_toks = std::max<int32_t>(mx_toks, (int32_t)toks_b);
-                mx_units = std::max<int32_t>(mx_units, (int32_t)(bunit.size() - unit0));
-                mx_slots = std::max<int32_t>(mx_slots, (int32_t)(slot.size() - slot0));
-            }
-        }
-        if (!ok) continue;
-        cta[(size_t)grid] = (int32_t)(batch.size() / 2);
-        TrieView tv{};
-        tv.max_nodes = mx_nodes;
-        tv.max_cls = mx_cls;
-        tv.max_toks = mx_toks;
-        tv.max_units = mx_units;
-        tv.max_slots = mx_slots;
-        tv.max_path = mx_path;
-        if (trie_tile_smem_bytes(v, tv, h->stack, (int)table) > smem) continue;   // the maxima together: cut tighter
-        h->t_batch.swap(batch);
-        h->t_range.swap(range);
-        h->t_slot.swap(slot);
-        h->t_bunit.swap(bunit);
-        h->t_cta.swap(cta);
-        h->t_grid = grid;
-        h->t_max_nodes = mx_nodes;
-        h->t_max_cls = mx_cls;
-        h->t_max_toks = mx_toks;
-        h->t_max_units = mx_units;
-        h->t_max_slots = mx_slots;
-        h->t_max_path = mx_path;
-        h->t_mode = mode;
-        return true;
-    }
-    return false;
+    return root;
 }
 
-// The prefix tree and its batches on the device.
-int build_trie(domino_ctx* h) {
-    build_trie_host(h);
-    if (!h->trie_built || !cut_batches(h)) return DOMINO_OK;
+// A transition entry with its target states renamed: push and plain entries
+// hold the target, a pop's triple is renamed state by state.
+struct RowEntries {
+    std::vector<uint32_t> e;      // [states][K]
+    std::vector<uint16_t> ret;    // pop targets, four per triple
+    int32_t Q = 0;
+};
+
+// The states of the loaded automaton that allow the same tokens whatever the
+// stack, merged: `id` names each state's class (0: the dead state).  Two
+// states of a class have entries of the same kind and symbol whose targets
+// are in the same classes (acceptance only matters to EOS, which is decided
+// from the row's own state).  Partition refinement; without a fixed point
+// after kMergeRounds rounds (long chains) nothing is merged.
+RowEntries merge_states(const domino_ctx* h, std::vector<int32_t>& id) {
+    constexpr int kMergeRounds = 64;
+    const int32_t Q = h->Q, K = h->K;
+    auto entry = [&](int64_t q, int k) -> uint32_t {
+        return h->stack ? h->t32[(size_t)(q * K + k)] : h->t16[(size_t)(q * K + k)];
+    };
+    // an entry's identity under the current classes
+    auto seen = [&](const std::vector<int32_t>& c, uint32_t e) -> uint64_t {
+        if (!h->stack) return (uint64_t)c[(size_t)e];
+        const uint32_t kind = (e >> kKindShift) & 3u;
+        const uint64_t head = ((uint64_t)kind << 1 | ((e >> kSymShift) & 1u)) << 48;
+        if (kind != 2) return head | (uint64_t)c[(size_t)(e & 0xFFFFu)];
+        const uint16_t* r = h->ret.data() + (size_t)(e >> kRetShift) * 4;
+        return head | (uint64_t)c[r[0]] << 32 | (uint64_t)c[r[1]] << 16 | (uint64_t)c[r[2]];
+    };
+    id.assign((size_t)Q, 1);
+    id[0] = 0;
+    int32_t n = Q > 1 ? 2 : 1;
+    bool fixed = Q <= 1;
+    for (int round = 0; round < kMergeRounds && !fixed; round++) {
+        std::vector<int32_t> next((size_t)Q, 0);
+        std::unordered_map<uint64_t, int32_t> at;
+        int32_t m = 1;
+        for (int64_t q = 1; q < Q; q++) {
+            uint64_t hash = 1469598103934665603ull ^ (uint64_t)id[(size_t)q];
+            for (int k = 0; k < K; k++) {
+                hash = (hash ^ seen(id, entry(q, k))) * 0x9E3779B97F4A7C15ull;
+                hash ^= hash >> 29;
+            }
+            const auto r = at.emplace(hash, m);
+            if (r.second) m++;
+            next[(size_t)q] = r.first->second;
+        }
+        fixed = m == n;
+        n = m;
+        id.swap(next);
+    }
+    std::vector<int64_t> first((size_t)n, -1);
+    for (int64_t q = 0; q < Q; q++)
+        if (first[(size_t)id[(size_t)q]] < 0) first[(size_t)id[(size_t)q]] = q;
+    for (int64_t q = 1; q < Q && fixed; q++) {   // exact, whatever the hashes did
+        const int64_t f = first[(size_t)id[(size_t)q]];
+        for (int k = 0; k < K && fixed; k++) fixed = seen(id, entry(q, k)) == seen(id, entry(f, k));
+    }
+    if (!fixed) {
+        std::iota(id.begin(), id.end(), 0);
+        first.resize((size_t)Q);
+        std::iota(first.begin(), first.end(), 0);
+        n = Q;
+    }
+    RowEntries r;
+    r.Q = n;
+    r.ret = h->ret;
+    for (size_t i = 0; i < r.ret.size(); i++)
+        if (i % 4 != 3) r.ret[i] = (uint16_t)id[r.ret[i]];
+    r.e.resize((size_t)n * (size_t)K);
+    for (int32_t c = 0; c < n; c++)
+        for (int k = 0; k < K; k++) {
+            const uint32_t e = entry(first[(size_t)c], k);
+            const bool pop = h->stack && ((e >> kKindShift) & 3u) == 2u;
+            r.e[(size_t)c * K + k] = pop ? e : (e & ~0xFFFFu) | (uint32_t)id[(size_t)(e & 0xFFFFu)];
+        }
+    return r;
+}
+
+// Per state its live classes and the classes that keep it, then its live
+// entries, padded to whole 32-byte sectors (RowTree).  flag[q]: the state has
+// a loop set.
+std::vector<uint8_t> state_records(const RowEntries& r, int K, bool stack, const std::vector<uint32_t>& loop,
+                                   int32_t* stride_out) {
+    const size_t esz = stack ? 4 : 2;
+    size_t most = 0;
+    for (int64_t q = 0; q < r.Q; q++) {
+        size_t n = 0;
+        for (int k = 0; k < K; k++) n += r.e[(size_t)(q * K + k)] != 0;
+        most = std::max(most, n);
+    }
+    const size_t stride = (16 + most * esz + 31) / 32 * 32;
+    std::vector<uint8_t> out((size_t)r.Q * stride, 0);
+    for (int64_t q = 0; q < r.Q; q++) {
+        uint8_t* p = out.data() + (size_t)q * stride;
+        uint64_t live = 0, self = 0;
+        size_t n = 0;
+        for (int k = 0; k < K; k++) {
+            const uint32_t e = r.e[(size_t)(q * K + k)];
+            if (!e) continue;
+            live |= 1ull << k;
+            if (e == (uint32_t)q) self |= 1ull << k;   // next state q, no push or pop
+            const uint16_t e16 = (uint16_t)e;
+            std::memcpy(p + 16 + n * esz, stack ? (const void*)&e : (const void*)&e16, esz);
+            n++;
+        }
+        if (!loop.empty() && loop[(size_t)q] != 0xFFFFFFFFu) self |= 1ull << 63;
+        std::memcpy(p, &live, 8);
+        std::memcpy(p + 8, &self, 8);
+    }
+    *stride_out = (int32_t)stride;
+    return out;
+}
+
+// The trees, state records and loop sets of RowTree.  rows_ready stays false
+// (the per-token walk is used) when the vocabulary or its tree is too large.
+int build_rows(domino_ctx* h) {
+    h->rows_ready = false;
+    if (!h->trie_built || h->W > kRowMaxSlices * kRowSliceWords) return DOMINO_OK;
+    const int smem = h->env.max_smem_optin > 0 ? h->env.max_smem_optin : 232448;
+    const bool wide = h->K > 64;
+    const int32_t Q = h->Q, K = h->K;
+    std::vector<uint8_t> cls(h->tok_bytes.size());
+    for (size_t i = 0; i < cls.size(); i++) cls[i] = h->byte_class[h->tok_bytes[i]];
+    std::vector<RowStr> strs;
+    strs.reserve(h->t_dtok.size());
+    for (int32_t t : h->t_dtok)   // sorted by class string already
+        strs.push_back({cls.data() + h->tok_off[t], (uint32_t)(h->tok_off[t + 1] - h->tok_off[t]), t});
+    std::vector<int32_t> id;
+    RowEntries merged;
+    std::vector<uint64_t> sets, self;   // the loop sets; per merged state the classes that keep it
+    if (!wide) {
+        merged = merge_states(h, id);
+        self.assign((size_t)merged.Q, 0);
+        for (int64_t q = 1; q < merged.Q; q++)
+            for (int k = 0; k < K; k++)
+                if (merged.e[(size_t)(q * K + k)] == (uint32_t)q) self[(size_t)q] |= 1ull << k;
+    }
+    // the loop sets worth a tree: at least a quarter of the classes (the rule
+    // of self_mask), those of most states first
+    if (!wide && K <= 63 && h->walk_pref != 1) {
+        std::vector<std::pair<uint64_t, int32_t>> all;   // (set, states)
+        std::unordered_map<uint64_t, size_t> at;
+        for (int32_t q = 1; q < Q; q++) {
+            const uint64_t m = self[(size_t)id[(size_t)q]];
+            if (4 * __builtin_popcountll(m) < K) continue;
+            const auto r = at.emplace(m, all.size());
+            if (r.second) all.emplace_back(m, 0);
+            all[r.first->second].second++;
+        }
+        std::stable_sort(all.begin(), all.end(), [](const auto& a, const auto& b) { return a.second > b.second; });
+        for (size_t i = 0; i < all.size() && i < (size_t)kRowLoopSets; i++) sets.push_back(all[i].first);
+    }
+    RowBuild rb;
+    std::vector<int64_t> roots;
+    std::vector<uint32_t> loopbits;
+    for (bool ok = false; !ok;) {   // once more without loop sets when they make the trees too large
+        rb = RowBuild();
+        rb.wide = wide;
+        rb.sets = sets;
+        rb.keeps.resize(sets.size());
+        rb.xrange.resize(sets.size());
+        rb.exits.resize(sets.size());
+        roots.clear();
+        loopbits.clear();
+        ok = add_row_tree(rb, strs) == 0;
+        for (size_t i = 0; ok && i < sets.size(); i++) {
+            std::vector<uint32_t> bits((size_t)h->W, 0);
+            std::vector<RowStr> rest;
+            for (const RowStr& s : strs) {
+                uint32_t l = 0;
+                while (l < s.len && ((sets[i] >> s.p[l]) & 1ull)) l++;
+                if (l == s.len) bits[(size_t)(s.token >> 5)] |= 1u << (s.token & 31);
+                else rest.push_back({s.p + l, s.len - l, s.token});
+            }
+            std::sort(rest.begin(), rest.end(), row_str_less);
+            roots.push_back(add_row_tree(rb, rest));
+            ok = roots.back() >= 0;
+            loopbits.insert(loopbits.end(), bits.begin(), bits.end());
+        }
+        size_t n_exits = 0;
+        for (auto& e : rb.exits) n_exits += e.size();
+        ok = ok && n_exits < (size_t)(1u << 24) &&
+             row_smem_bytes(h->W, rb.reserve, h->stack, !sets.empty()) <= smem - 1024;
+        if (!ok && sets.empty()) return DOMINO_OK;
+        if (!ok) sets.clear();
+    }
+    const size_t n_sets = sets.size();
+    std::vector<uint8_t> keeps;
+    std::vector<uint2> xrange, exits;
+    for (size_t i = 0; i < n_sets; i++) {
+        const uint32_t base = (uint32_t)exits.size();
+        keeps.insert(keeps.end(), rb.keeps[i].begin(), rb.keeps[i].end());
+        for (uint2 x : rb.xrange[i]) xrange.push_back(make_uint2(x.x + base, x.y + base));
+        exits.insert(exits.end(), rb.exits[i].begin(), rb.exits[i].end());
+    }
+    std::vector<uint32_t> loop_of;   // per merged state its loop set
+    std::vector<uint2> start;        // per state {merged state, its loop set}
+    std::vector<uint8_t> srec, srec_next;
+    int32_t stride = 0, stride_next = 0;
+    const bool same = wide || merged.Q == Q;   // nothing was merged: one set of records
+    if (!wide) {
+        loop_of.assign((size_t)merged.Q, 0xFFFFFFFFu);
+        for (int32_t q = 1; q < merged.Q; q++) {
+            const auto it = std::find(sets.begin(), sets.end(), self[(size_t)q]);
+            if (it != sets.end()) loop_of[(size_t)q] = (uint32_t)(it - sets.begin());
+        }
+        srec = state_records(merged, K, h->stack, loop_of, &stride);
+        if (!same || n_sets) {
+            for (int32_t q = 0; q < Q; q++)
+                start.push_back(make_uint2((uint32_t)id[(size_t)q], loop_of[(size_t)id[(size_t)q]]));
+            // next states: the automaton's own, without loop sets
+            RowEntries own;
+            own.Q = Q;
+            own.e.resize((size_t)Q * (size_t)K);
+            for (size_t i = 0; i < own.e.size(); i++) own.e[i] = h->stack ? h->t32[i] : h->t16[i];
+            srec_next = state_records(own, K, h->stack, {}, &stride_next);
+        }
+    }
     int rc;
-    auto up = [&](DevBuf& b, const void* p, size_t n) { return dev_upload(b, p, std::max<size_t>(16, n)); };
-    if ((rc = up(h->d_tnode, h->t_cnode.data(), h->t_cnode.size() * sizeof(uint4)))) return rc;
-    if ((rc = up(h->d_tncls, h->t_ncls.data(), h->t_ncls.size()))) return rc;
-    if ((rc = up(h->d_tdtok, h->t_dtok.data(), h->t_dtok.size() * 4))) return rc;
-    if ((rc = up(h->d_tupper, h->t_upper.data(), h->t_upper.size() * sizeof(uint4)))) return rc;
-    if ((rc = up(h->d_tupath, h->t_upath.data(), h->t_upath.size()))) return rc;
-    if ((rc = up(h->d_tbatch, h->t_batch.data(), h->t_batch.size() * sizeof(uint4)))) return rc;
-    if ((rc = up(h->d_trange, h->t_range.data(), h->t_range.size() * sizeof(uint4)))) return rc;
-    if ((rc = up(h->d_tslot, h->t_slot.data(), h->t_slot.size() * sizeof(uint4)))) return rc;
-    if ((rc = up(h->d_tunit, h->t_bunit.data(), h->t_bunit.size() * sizeof(uint2)))) return rc;
-    if ((rc = up(h->d_tcta, h->t_cta.data(), h->t_cta.size() * 4))) return rc;
-    if ((rc = dev_reserve(h->d_trow, std::max<size_t>(1, h->t_batch.size() / 2) * 4))) return rc;
-    h->trie_ready = true;
+    auto up = [&](DevBuf& b, const void* p, size_t n) { return dev_upload(b, n ? p : nullptr, std::max<size_t>(16, n)); };
+    if ((rc = up(h->d_rnode, rb.node.data(), rb.node.size() * sizeof(uint4)))) return rc;
+    if ((rc = up(h->d_rncls, rb.ncls.data(), rb.ncls.size()))) return rc;
+    if ((rc = up(h->d_rdtok, rb.dtok.data(), rb.dtok.size() * 4))) return rc;
+    if ((rc = up(h->d_srec, srec.data(), srec.size()))) return rc;
+    if ((rc = up(h->d_srec_next, srec_next.data(), srec_next.size()))) return rc;
+    if ((rc = up(h->d_rret, merged.ret.data(), merged.ret.size() * 2))) return rc;
+    if ((rc = up(h->d_rstart, start.data(), start.size() * sizeof(uint2)))) return rc;
+    if ((rc = up(h->d_loop_of, loop_of.data(), loop_of.size() * 4))) return rc;
+    if ((rc = up(h->d_loopbits, loopbits.data(), loopbits.size() * 4))) return rc;
+    if ((rc = up(h->d_keeps, keeps.data(), keeps.size()))) return rc;
+    if ((rc = up(h->d_xrange, xrange.data(), xrange.size() * sizeof(uint2)))) return rc;
+    if ((rc = up(h->d_exits, exits.data(), exits.size() * sizeof(uint2)))) return rc;
+    const StepView v = make_view(h);
+    RowTree t{};
+    t.node = (const uint4*)h->d_rnode.p;
+    t.ncls = (const uint8_t*)h->d_rncls.p;
+    t.dtok = (const int32_t*)h->d_rdtok.p;
+    t.srec = (const uint4*)h->d_srec.p;
+    t.ret = wide ? v.ret : (const uint16_t*)h->d_rret.p;
+    t.start = start.empty() ? nullptr : (const uint2*)h->d_rstart.p;
+    t.loop_of = (const uint32_t*)h->d_loop_of.p;
+    t.loopbits = (const uint32_t*)h->d_loopbits.p;
+    t.keeps = (const uint8_t*)h->d_keeps.p;
+    t.xrange = (const uint2*)h->d_xrange.p;
+    t.exits = (const uint2*)h->d_exits.p;
+    t.srec_stride = stride;
+    t.n_nodes = (int32_t)(rb.node.size() / 2);
+    t.n_dtok = (int32_t)rb.dtok.size();
+    t.n_loops = (int32_t)n_sets;
+    t.reserve = rb.reserve;
+    t.max_kids = rb.max_kids;
+    for (size_t i = 0; i < n_sets; i++) t.loop_root[i] = (int32_t)roots[i];
+    h->rows = t;
+    if (!start.empty()) {
+        t.srec = (const uint4*)h->d_srec_next.p;
+        t.srec_stride = stride_next;
+        t.ret = v.ret;
+        t.start = nullptr;
+        t.n_loops = 0;
+    }
+    h->rows_next = t;
+    h->rows_ready = true;
     return DOMINO_OK;
 }
 
@@ -699,7 +763,8 @@ int build_arena(domino_ctx* h) {
     }
     if ((rc = dev_upload(h->d_eos_slot, eos_slot.data(), eos_slot.size() * 2))) return rc;
     h->n_windows = nw;
-    if ((rc = build_trie(h))) return rc;
+    build_trie_host(h);
+    if ((rc = build_rows(h))) return rc;
     h->arena_ready = true;
     return DOMINO_OK;
 }
@@ -749,40 +814,25 @@ int choose_mode(const domino_ctx* h, const StepView& v, bool next) {
     return kDenseGlobal;
 }
 
-TrieView make_trie_view(const domino_ctx* h) {
-    TrieView tv{};
-    tv.node = (const uint4*)h->d_tnode.p;
-    tv.ncls = (const uint8_t*)h->d_tncls.p;
-    tv.dtok = (const int32_t*)h->d_tdtok.p;
-    tv.upper = (const uint4*)h->d_tupper.p;
-    tv.upath = (const uint8_t*)h->d_tupath.p;
-    tv.batch = (const uint4*)h->d_tbatch.p;
-    tv.range = (const uint4*)h->d_trange.p;
-    tv.slot = (const uint4*)h->d_tslot.p;
-    tv.unit = (const uint2*)h->d_tunit.p;
-    tv.cta_batch = (const int32_t*)h->d_tcta.p;
-    tv.n_nodes = h->t_nodes;
-    tv.n_upper = (int32_t)h->t_upper.size();
-    tv.grid = h->t_grid;
-    tv.n_batches = (int32_t)(h->t_batch.size() / 2);
-    tv.max_nodes = h->t_max_nodes;
-    tv.max_cls = h->t_max_cls;
-    tv.max_toks = h->t_max_toks;
-    tv.max_units = h->t_max_units;
-    tv.max_slots = h->t_max_slots;
-    tv.max_path = h->t_max_path;
-    return tv;
+// One tree for all rows: no state loops on many classes (or DOMINO_WALK=tree).
+bool use_tree(const domino_ctx* h) {
+    if (!h->rows_ready || h->walk_pref == 0) return false;
+    return h->walk_pref == 1 || h->self_mask.empty();
 }
 
-// The tree shares each prefix's transitions among the tokens below it and
-// drops a subtree as soon as its prefix dies, so it wins when most prefixes
-// die early (sparse masks).  States that loop on many classes (strings,
-// numbers, whitespace: the self-loop mask) keep long prefixes alive and make
-// rows dense; there the per-token walk, which skips a whole token whose later
-// classes all loop on the state, is faster.
-bool use_tree(const domino_ctx* h) {
-    if (!h->trie_ready || h->walk_pref == 0) return false;
-    return h->walk_pref == 1 || h->self_mask.empty();
+// Whether row_kernel takes a mask step.  Its time is the latency of the walk's
+// rounds (8 to 40 us) and hardly grows until every SM has rows; the per-token
+// walk's grows with the (row, token) pairs.  Without loop sets the row kernel
+// wins from one row on (GB300, 5000 states, V = 128256, batch 16: 14.0
+// against 17.9 us).  With them the lines cross near 2^21 pairs: 200 states,
+// V = 32000, batch 32 (2^20): 7.9 against 5.3 us; JSON, V = 50001, batch 24
+// (2^20.2): 18.6 against 16.2 us; V = 152064, batch 128 (2^24): 36.5 against
+// 74.4 us; 200 states, V = 64000, batch 500: 12.9 against 24.3 us.
+// Next states of such automata are the per-token walk's (the loop sets hold
+// masks only).
+bool use_rows(const domino_ctx* h, int64_t batch, bool next) {
+    if (use_tree(h)) return true;
+    return h->rows_ready && h->walk_pref != 0 && !next && batch * h->V >= ((int64_t)1 << 21);
 }
 
 int ready_for_compute(domino_ctx* h) {
@@ -877,8 +927,8 @@ int domino_destroy(domino_t h) {
         DevBuf* all[] = {&h->d_head, &h->d_info, &h->d_tail_off, &h->d_tail, &h->d_pos_of, &h->d_cls_start,
                          &h->d_eos_slot, &h->d_dense, &h->d_sparse, &h->d_accept, &h->d_self, &h->d_tok_cls, &h->d_err, &h->d_fpart, &h->d_partials,
                          &h->d_counters, &h->d_lse_tmp, &h->s_logits, &h->s_mask, &h->s_io,
-                         &h->o_prop, &h->o_rows, &h->o_count, &h->d_tnode, &h->d_tdtok, &h->d_tupper, &h->d_tupath, &h->d_tbatch, &h->d_tslot,
-                         &h->d_tunit, &h->d_tcta, &h->d_trange, &h->d_tncls, &h->d_trow};
+                         &h->o_prop, &h->o_rows, &h->o_count, &h->d_rnode, &h->d_rncls, &h->d_rdtok, &h->d_srec, &h->d_srec_next, &h->d_rret,
+                         &h->d_rstart, &h->d_loop_of, &h->d_loopbits, &h->d_keeps, &h->d_xrange, &h->d_exits};
         for (auto* b : all) dev_free(*b);
         for (cudaEvent_t& e : h->ev_chunk)
             if (e) cudaEventDestroy(e);
@@ -1168,7 +1218,7 @@ int domino_get_info(domino_t h, domino_info* out) {
     }
     out->device_bytes = dev_bytes(h);
     out->walk_tree = use_tree(h) ? 1 : 0;
-    out->tree_units = h->trie_ready ? (int32_t)h->t_bunit.size() : 0;
+    out->tree_units = h->rows_ready ? (int32_t)h->t_unit.size() : 0;
     return DOMINO_OK;
 }
 
@@ -1215,9 +1265,9 @@ int domino_step_mask(domino_t h, const int32_t* states_dev, const uint64_t* stac
     if (batch == 0) return DOMINO_OK;
     DeviceGuard g(h->device);
     StepView v = make_view(h);
-    if (use_tree(h)) {
-        return cuda_status(launch_trie_step(v, make_trie_view(h), h->env, h->stack, h->t_mode, states_dev, stacks_dev,
-                                            batch, false, mask_dev, next_dev, (cudaStream_t)stream));
+    if (use_rows(h, batch, next_dev != nullptr)) {
+        return cuda_status(launch_row_step(v, next_dev ? h->rows_next : h->rows, h->env, h->stack, states_dev,
+                                           stacks_dev, batch, false, mask_dev, next_dev, (cudaStream_t)stream));
     }
     const int mode = choose_mode(h, v, next_dev != nullptr);
     return cuda_status(launch_step_mask(v, h->env, h->stack, mode, states_dev, stacks_dev, batch, false, mask_dev,
@@ -1232,10 +1282,9 @@ int domino_precompute_table(domino_t h, int32_t* next_dev, uint32_t* mask_dev, v
     if (h->stack) return DOMINO_E_UNSUPPORTED;
     DeviceGuard g(h->device);
     StepView v = make_view(h);
-    if (use_tree(h)) {
-        return cuda_status(launch_trie_step(v, make_trie_view(h), h->env, false, h->t_mode, nullptr, nullptr, h->Q,
-                                            true, mask_dev, next_dev, (cudaStream_t)stream, nullptr, nullptr,
-                                            (int32_t*)h->d_trow.p));
+    if (use_rows(h, h->Q, next_dev != nullptr)) {
+        return cuda_status(launch_row_step(v, next_dev ? h->rows_next : h->rows, h->env, false, nullptr, nullptr, h->Q, true, mask_dev,
+                                           next_dev, (cudaStream_t)stream));
     }
     const int mode = choose_mode(h, v, next_dev != nullptr);
     return cuda_status(launch_step_mask(v, h->env, false, mode, nullptr, nullptr, h->Q, true, mask_dev, next_dev,

@@ -1,0 +1,707 @@
+// rows.cu -- C.mask() with one CTA per row (sm_103a).
+//
+// The mask of a row is the set of tokens whose class string can be walked
+// from the row's configuration without reaching the dead state (Alg. 1's
+// mask at lookahead k = infinity, Sec. 3.5; EOS iff the state accepts with an
+// empty stack).  row_kernel expands, for one row, only the live part of the
+// prefix tree of the class strings (the subterminal tree of Sec. 3.3 / Alg. 2
+// over byte classes): the children of a live node that stay alive are the
+// intersection of the node's child classes with its state's live classes, so
+// a prefix that dies is never visited at all.
+//
+// Work is a pool of (node, state[, stack]) items in shared memory.  In a
+// round every thread takes one item from the pool's top, reads the node's and
+// the state's 32-byte record together (both L2-resident, one round trip),
+// leaves the node's tokens to be set and adds the live children.  The mask is
+// built in shared memory and written once; with next states the row is filled
+// first and the allowed tokens' states are stored over it.
+//
+// What bounds it: latency.  A round is one L2 round trip (about 650 cycles)
+// plus about 1100 cycles of dependent shared-memory, shuffle and barrier
+// steps, whatever its width; a row of the 5000-state random DFA over 128256
+// tokens takes 8 to 11 rounds for its 1000 live nodes.  One CTA per row keeps
+// these rounds free of any grid-wide step, and neither the tree nor the
+// transition table is staged.  Measured (GB300, that workload, back to back):
+// batch 256 16.1 us (35.8 us for the walk it replaced, whose CTAs each staged
+// a share of the tree and walked every row in it), batch 1000 52.5 us (94.1),
+// batch 16 14.0 us (17.0); the 20000-state table 2.67 ms (3.25 ms).
+//
+// States that loop on most classes (string bodies) allow nearly every token.
+// For the widest such loop sets the host keeps the tokens that stay inside
+// the set as a bitmap, copied into the row's mask, and a second tree over the
+// other tokens' remainders after their longest prefix inside the set, so that
+// such a row costs a copy and a short walk.  A subtree entered in such a state
+// is a filtered range of its tokens plus the edges that leave the set (see
+// RowTree).
+//
+// Batches with fewer rows than SMs give each row a cluster of CTAs that share
+// out the row's mask words; each walks the row itself (the walk is latency,
+// not work) and keeps the tokens of its words.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <climits>
+#include <cstdint>
+#include <mutex>
+
+#include "domino_internal.h"
+#include "walk_common.cuh"
+
+namespace domino {
+namespace {
+
+constexpr int kRowThreads = 512;
+constexpr int kRowWarps = kRowThreads / 32;
+constexpr int kRowPool = 2048;        // items a round may leave in the pool (see run())
+constexpr int kRowMargin = 256;
+constexpr int kRowFan = 8;            // threads per item while there are few
+constexpr int kRowSmall = 512;        // ranges of 2 to kRowSmallTokens tokens left to the whole CTA
+constexpr int kRowSmallTokens = 64;
+constexpr int kRowBig = 128;          // longer ranges
+constexpr int kRowExits = 512;        // loop subtrees whose exits are still to be walked
+constexpr int kRowLoopMin = 16;       // fewest tokens of a subtree taken as a loop subtree
+constexpr int kRowMaxDevices = 64;
+static_assert(kRowBig <= kRowThreads && kRowExits <= kRowThreads, "one entry per thread in the prefix sums");
+
+enum RowOut : int {
+    kRowMask = 0,    // the mask
+    kRowNext = 1,    // the mask (optional) and the next states
+};
+
+// How child and live classes are held: a 32-bit mask (K <= 32), a 64-bit
+// mask (K <= 64), or, for more classes, child classes listed one byte each
+// and transitions read from the dense table.
+enum RowClasses : int { kRow32 = 0, kRow64 = 1, kRowWide = 2 };
+
+struct RowArgs {
+    const int32_t* states;
+    const uint64_t* stacks;
+    int32_t batch;          // rows (the cap of a row list)
+    int32_t row_is_state;
+    int32_t slices;         // CTAs per row (a cluster)
+    int32_t slice_words;    // mask words per CTA (a multiple of 4)
+    uint32_t* mask;
+    int32_t* next;
+};
+
+// Shared-memory layout (byte offsets).  The mask slice has a zero word on
+// either side.
+struct RowLayout {
+    int mask, items, bits, small, big, exits, pre, total;
+};
+
+__host__ __device__ inline int row_pool_cap(int reserve) { return kRowPool + reserve; }
+
+__host__ __device__ inline RowLayout row_layout(int slice_words, int reserve, bool stack, bool loops) {
+    RowLayout L{};
+    int o = 16;
+    L.mask = o;   o += align16(slice_words * 4) + 16;
+    L.items = o;  o += align16(2 * row_pool_cap(reserve) * 8);
+    L.bits = o;   o += stack ? align16(2 * row_pool_cap(reserve) * 4) : 0;
+    L.small = o;  o += kRowSmall * 8;
+    L.big = o;    o += kRowBig * 16;
+    L.exits = o;  o += loops ? kRowExits * 16 : 0;
+    L.pre = o;    o += align16((kRowThreads + 1) * 4);
+    L.total = align16(o);
+    return L;
+}
+
+struct RowShared {
+    int4 st[3];      // by round: {items added, the first place that did not fit, lists half full, 0}
+    int back;        // items put back
+    int nsmall, nbig, nexit;
+    int wsum[kRowWarps];
+};
+
+__device__ __forceinline__ int warp_scan_incl(int x, int lane) {
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, off);
+        if (lane >= off) x += y;
+    }
+    return x;
+}
+
+__device__ __forceinline__ int popc(uint32_t m) { return __popc(m); }
+__device__ __forceinline__ int popc(unsigned long long m) { return __popcll(m); }
+
+// the entry k of the prefix sums pre[0..n] (pre[0] = 0) with pre[k] <= f < pre[k + 1]
+__device__ __forceinline__ int find_range(const int* pre, int n, int f) {
+    int lo = 0, hi = n;
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (pre[mid] <= f) lo = mid;
+        else hi = mid;
+    }
+    return lo;
+}
+
+// One row's walk.
+template <bool STACK, int CLS, int OUT>
+struct RowWalk {
+    static constexpr bool WIDE = CLS == kRowWide;
+    using Mask = typename std::conditional<CLS == kRow32, uint32_t, unsigned long long>::type;
+
+    const StepView& v;
+    const RowTree& t;
+    uint32_t* s_mask;
+    uint2* s_item;       // {node, state | depth << 16}
+    uint32_t* s_bits;    // the items' stack symbols
+    uint2* s_small;      // {first token, state | tokens << 16}
+    uint4* s_big;        // {first token, tokens, state, least depth | (loop set + 1) << 8, or 0}
+    uint4* s_exit;       // {first exit | depth << 24, exits, state | stack depth << 16, stack symbols}
+    int* s_pre;
+    RowShared& sh;
+    int32_t* nrow;       // the row's next states
+    int tok0, ntok;      // this CTA's token ids
+    int tid, lane, warp;
+
+    struct Item {
+        uint32_t node, s, depth, bits;   // s == 0: none
+    };
+
+    // Tokens allowed with state s: n of the preorder list from lo on, the
+    // first of which is `first`.
+    struct Tokens {
+        uint32_t lo, n, first, s;
+    };
+    // An item's expansion: its live children and its tokens.
+    struct Node {
+        Mask m, live, kids;   // live children, the state's live classes, the node's child classes
+        uint32_t first_child;
+        int c;                // WIDE: children
+        Tokens em;
+    };
+
+    __device__ __forceinline__ void emit(int tk, uint32_t s) const {
+        const int x = tk - tok0;
+        if ((unsigned)x >= (unsigned)ntok) return;
+        atomicOr(&s_mask[x >> 5], 1u << (x & 31));
+        if constexpr (OUT == kRowNext) {
+            if (nrow) nrow[tk] = (int32_t)s;
+        }
+    }
+
+    // a node's tokens: one is set here, a range is left to the whole CTA (a
+    // thread would wait for its token ids)
+    __device__ __forceinline__ void emit(const Tokens& x, int4* st) const {
+        if (x.n == 1u) emit((int)x.first, x.s);
+        if (x.n > 1u) {
+            const bool small = x.n <= (uint32_t)kRowSmallTokens;
+            const int i = atomicAdd(small ? &sh.nsmall : &sh.nbig, 1);
+            if (i >= (small ? kRowSmall : kRowBig) / 2) st->z = 1;
+            if (small && i < kRowSmall) {
+                s_small[i] = make_uint2(x.lo, x.s | (x.n << 16));
+            } else if (!small && i < kRowBig) {
+                s_big[i] = make_uint4(x.lo, x.n, x.s, 0u);
+            } else {
+#pragma unroll 1
+                for (uint32_t j = 0; j < x.n; ++j) emit(__ldg(t.dtok + x.lo + j), x.s);
+            }
+        }
+    }
+
+    // the entry of a class in state s, given its rank among the state's live classes
+    __device__ __forceinline__ uint32_t target(uint32_t s, int rank) const {
+        const unsigned char* r = reinterpret_cast<const unsigned char*>(t.srec) + (size_t)s * t.srec_stride + 16;
+        if constexpr (STACK) return __ldg(reinterpret_cast<const uint32_t*>(r) + rank);
+        else return __ldg(reinterpret_cast<const uint16_t*>(r) + rank);
+    }
+    __device__ __forceinline__ uint4 state_header(uint32_t s) const {
+        return __ldg(reinterpret_cast<const uint4*>(reinterpret_cast<const unsigned char*>(t.srec) +
+                                                    (size_t)s * t.srec_stride));
+    }
+    __device__ __forceinline__ uint32_t dense(uint32_t s, uint32_t c) const {
+        if constexpr (STACK) return __ldg(v.t32 + (size_t)s * v.K + c);
+        else return __ldg(v.t16 + (size_t)s * v.K + c);
+    }
+    __device__ __forceinline__ static Mask mask_of(uint32_t lo, uint32_t hi) {
+        if constexpr (CLS == kRow32) return lo;
+        else return ((unsigned long long)hi << 32) | lo;
+    }
+
+    // entry e taken with the stack (depth, bits): the child item (s == 0 when refused)
+    __device__ __forceinline__ Item step(uint32_t child, uint32_t e, uint32_t depth, uint32_t bits) const {
+        Item it{child, e, depth, bits};
+        if constexpr (STACK) it.s = pda_apply(e, it.bits, it.depth, (uint32_t)v.max_depth, t.ret);
+        return it;
+    }
+
+    __device__ __forceinline__ void put(int slot, const Item& it) const {
+        s_item[slot] = make_uint2(it.node, it.s | (it.depth << 16));
+        if constexpr (STACK) s_bits[slot] = it.bits;
+    }
+    __device__ __forceinline__ Item get(int slot) const {
+        const uint2 x = s_item[slot];
+        return Item{x.x, x.y & 0xFFFFu, x.y >> 16, STACK ? s_bits[slot] : 0u};
+    }
+
+    // The item's node record and state record, read together.  lead: this
+    // thread answers for the item (and may add it to the loop subtrees).
+    // before: the tokens of the thread's last item, set meanwhile.
+    __device__ __forceinline__ Node read(const Item& it, bool lead, const Tokens& before, int4* st) const {
+        Node x{};
+        uint4 A = make_uint4(0u, 0u, 0u, 0u), B = A, h = A;
+        if (it.s != 0u) {
+#ifdef DOMINO_DEBUG
+            if (it.node >= (uint32_t)t.n_nodes || it.s >= (uint32_t)v.Q) atomicOr(v.err, DOMINO_DEVERR_INTERNAL);
+#endif
+            A = __ldg(t.node + 2 * (size_t)it.node);
+            B = __ldg(t.node + 2 * (size_t)it.node + 1);
+            if constexpr (!WIDE) h = state_header(it.s);
+        }
+        emit(before, st);   // while the records are on their way
+        if (it.s == 0u) return x;
+        x.first_child = A.z & 0xFFFFFFu;
+        x.em.lo = B.x;
+        x.em.first = A.w;
+        x.em.s = it.s;
+        x.em.n = A.z >> 24;   // the tokens that end here
+        if constexpr (WIDE) {
+            x.c = (int)A.x;   // refused children become dead items
+            if (x.c == 0) x.em.n = B.y - B.x;
+            else if (x.em.n == 255u) x.em.n = __ldg(&t.node[2 * (size_t)x.first_child + 1].x) - B.x;
+        } else {
+            x.live = mask_of(h.x, h.y);
+            x.kids = mask_of(A.x, A.y);
+            const Mask keep = mask_of(h.z, CLS == kRow32 ? 0u : h.w & 0x7FFFFFFFu);
+            if ((mask_of(B.z, B.w) & ~keep) == 0) {
+                x.em.n = B.y - B.x;   // every class below keeps the state: the subtree is allowed with it
+            } else {
+                x.m = x.kids & x.live;
+                if (x.em.n == 255u) x.em.n = __ldg(&t.node[2 * (size_t)x.first_child + 1].x) - B.x;
+                if ((h.w >> 31) && lead && B.y - B.x > (uint32_t)kRowLoopMin && (x.kids & keep) != 0 &&
+                    loop_subtree(it, B.x + x.em.n, B.y))
+                    x.m = 0;
+            }
+        }
+        return x;
+    }
+
+    // Expands the pool's n items until none are left.  In a round every
+    // thread takes one item from the pool's top (kRowFan threads share one
+    // while there are few) and adds its live children: to the pool's other
+    // half when the round takes all items, else in their place.
+    //
+    // Neither half can overflow kRowPool + t.reserve items.  A warp whose
+    // children would pass kRowPool - kRowThreads - kRowMargin puts its items
+    // back instead.  When that goes for all of a round's items, or when the
+    // pool is nearly full, a round takes only as many items as could all have
+    // t.max_kids children and stay within kRowPool, or else a single one:
+    // then the pool is walked depth first, strictly from its top, and the
+    // item's subtree adds at most t.reserve (the host's bound over the tree).
+    __device__ __forceinline__ void run(int n, int cap) const {
+        bool stuck = false;   // no item of the last round was expanded
+        int half = 0;   // where the items lie
+        Tokens before{0u, 0u, 0u, 0u};
+        for (int r = 0;; r = r == 2 ? 0 : r + 1) {
+            int4* st = &sh.st[r];
+            if (n == 0) {
+                n = spawn_exits();   // the same for every thread of the CTA
+                if (n == 0) break;
+                half = 0;
+            }
+            const bool careful = stuck || n > kRowPool - kRowMargin;
+            int take = min(n, kRowThreads);
+            if (careful) take = max(1, min(take, (kRowPool - n) / t.max_kids));
+            const int base = n - take;
+            const bool fan = take * kRowFan <= kRowThreads;
+            const int i = fan ? tid / kRowFan : tid;
+            const bool lead = !fan || (tid & (kRowFan - 1)) == 0;
+            Item it{0u, 0u, 0u, 0u};
+            if (i < take) it = get(half + base + i);
+            if (tid == 0) {
+                sh.st[r == 2 ? 0 : r + 1] = make_int4(0, INT_MAX, 0, 0);   // read by all two rounds ago
+                sh.back = 0;
+            }
+            if (base > 0) __syncthreads();   // the items are read before others take their place
+            else half ^= cap;
+            bool failed = false;
+            if ((fan ? (tid & ~31) / kRowFan : tid & ~31) < take) {   // warps with an item
+                Node x = read(it, lead, before, st);
+                // this thread's share of the children
+                int c;
+                Mask m = 0;
+                if constexpr (WIDE) {
+                    const int q = fan ? tid & (kRowFan - 1) : 0, step = fan ? kRowFan : 1;
+                    c = x.c > q ? (x.c - q + step - 1) / step : 0;
+                } else {
+                    m = x.m;
+                    if (fan) {
+                        if (t.n_loops > 0) m = shfl_lead(m);   // the lead may have taken the subtree whole
+                        constexpr int kWidth = (int)sizeof(Mask) * 8 / kRowFan;   // classes per thread
+                        m &= (((Mask)1 << kWidth) - 1) << (kWidth * (tid & (kRowFan - 1)));
+                    }
+                    c = popc(m);
+                }
+                // places for the children, warp by warp
+                const unsigned some = __ballot_sync(0xffffffffu, c > 0);
+                if (some) {
+                    int at, tot;
+                    if (!__any_sync(0xffffffffu, c > 1)) {
+                        at = __popc(some & ((1u << lane) - 1u));
+                        tot = __popc(some);
+                    } else {
+                        const int incl = warp_scan_incl(c, lane);
+                        at = incl - c;
+                        tot = __shfl_sync(0xffffffffu, incl, 31);
+                    }
+                    int first = 0;
+                    if (lane == 0) first = base + atomicAdd(&st->x, tot);
+                    first = __shfl_sync(0xffffffffu, first, 0);
+                    at += half + first;
+                    if (first + tot > kRowPool - kRowThreads - kRowMargin && !careful) {
+                        failed = true;
+                        x.em.n = 0u;
+                        if (lane == 0) atomicMin(&st->y, first);
+                    } else if constexpr (WIDE) {
+                        for (int k = fan ? tid & (kRowFan - 1) : 0; c > 0; k += fan ? kRowFan : 1, --c) {
+                            const uint32_t child = x.first_child + (uint32_t)k;
+                            put(at++, step(child, dense(it.s, __ldg(t.ncls + child)), it.depth, it.bits));
+                        }
+                    } else {
+                        for (; m; m &= m - 1) {
+                            const Mask below = (m & (~m + 1)) - 1;
+                            put(at++, step(x.first_child + (uint32_t)popc(x.kids & below),
+                                           target(it.s, popc(x.live & below)), it.depth, it.bits));
+                        }
+                    }
+                }
+                before = x.em;
+                if (!lead) before.n = 0u;
+            }
+            __syncthreads();   // the next round's items are in place
+            const int4 q = *st;
+            stuck = false;
+            n = base + q.x;
+            if (q.y != INT_MAX) {   // some did not fit
+                if (failed) {
+                    const unsigned b = __ballot_sync(0xffffffffu, lead && it.s != 0u);
+                    int first = 0;
+                    if (lane == 0) first = atomicAdd(&sh.back, __popc(b));
+                    first = __shfl_sync(0xffffffffu, first, 0);
+                    if (lead && it.s != 0u) put(half + q.y + first + __popc(b & ((1u << lane) - 1u)), it);
+                }
+                __syncthreads();
+                n = q.y + *reinterpret_cast<volatile int*>(&sh.back);
+                stuck = q.y == base;   // none did
+                __syncthreads();
+            }
+            if (q.z) ranges();
+        }
+        emit(before, &sh.st[0]);
+    }
+
+    __device__ __forceinline__ uint32_t shfl_lead(uint32_t m) const {
+        return __shfl_sync(0xffffffffu, m, lane & ~(kRowFan - 1));
+    }
+    __device__ __forceinline__ unsigned long long shfl_lead(unsigned long long m) const {
+        return ((unsigned long long)shfl_lead((uint32_t)(m >> 32)) << 32) | shfl_lead((uint32_t)m);
+    }
+
+    // A node entered in a looping state (RowTree).  The tokens [lo, hi) below
+    // it whose remainder stays inside the loop set are a filtered range, the
+    // others are reached through the edges that first leave the set; both are
+    // left to the whole CTA.  false: not taken.
+    __device__ __forceinline__ bool loop_subtree(const Item& it, uint32_t lo, uint32_t hi) const {
+        const uint32_t set = __ldg(t.loop_of + it.s);
+        const uint2 x = __ldg(t.xrange + (size_t)set * t.n_nodes + it.node);   // {first exit below | depth << 24, end}
+        const uint32_t d = x.x >> 24, n_exit = x.y - (x.x & 0xFFFFFFu);
+        if (d == 255u) return false;   // deeper than a byte holds
+        const int i = atomicAdd(&sh.nbig, 1);
+        if (i >= kRowBig) return false;
+        s_big[i] = make_uint4(lo, 0u, it.s, d | ((set + 1u) << 8));
+        if (n_exit) {
+            const int j = atomicAdd(&sh.nexit, 1);
+            if (j >= kRowExits) return false;   // (an empty range stays behind)
+            s_exit[j] = make_uint4(x.x, n_exit, it.s | (it.depth << 16), it.bits);
+        }
+        s_big[i].y = hi - lo;
+        return true;
+    }
+
+    // Exclusive prefix sums of x over threads 0..n-1 into s_pre[0..n]; the total.
+    __device__ __forceinline__ int prefix(int n, int x) const {
+        int incl = warp_scan_incl(tid < n ? x : 0, lane);
+        if (lane == 31) sh.wsum[warp] = incl;
+        __syncthreads();
+        for (int k = 0; k < warp; ++k) incl += sh.wsum[k];
+        if (tid < n) s_pre[tid + 1] = incl;
+        if (tid == 0) s_pre[0] = 0;
+        __syncthreads();
+        return s_pre[n];
+    }
+
+    // The loop subtrees' exits become the pool's items, in its first half
+    // (the pool is empty before).  Returns their number, 0 when none are left.
+    __device__ __forceinline__ int spawn_exits() const {
+        if (t.n_loops == 0) return 0;
+        for (;;) {
+            const int nx = min(*reinterpret_cast<volatile int*>(&sh.nexit), kRowExits);
+            if (nx == 0) return 0;
+            if (tid == 0) sh.back = 0;
+            const int total = prefix(nx, tid < nx ? (int)s_exit[tid].y : 0);
+            // as many as fit this time, the last entries first (the list is a
+            // stack); an entry taken in part is cut back
+            const int f0 = max(0, total - kRowPool);
+            for (int b = f0 + warp * 32; b < total; b += kRowThreads) {
+                const int f = b + lane;
+                Item x{0u, 0u, 0u, 0u};
+                if (f < total) {
+                    const int k = find_range(s_pre, nx, f);
+                    const uint4 e = s_exit[k];
+                    const uint2 q = __ldg(t.exits + (e.x & 0xFFFFFFu) + (uint32_t)(f - s_pre[k]));
+                    if ((q.y >> 8) <= e.x >> 24) {   // no edge before it leaves the set
+                        const uint32_t s = e.z & 0xFFFFu;
+                        const uint4 h = state_header(s);
+                        const Mask live = mask_of(h.x, h.y), bit = (Mask)1 << (q.y & 0xFFu);
+                        if (live & bit) x = step(q.x, target(s, popc(live & (bit - 1))), e.z >> 16, e.w);
+                    }
+                }
+                const unsigned ok = __ballot_sync(0xffffffffu, x.s != 0u);
+                int first = 0;
+                if (lane == 0 && ok) first = atomicAdd(&sh.back, __popc(ok));
+                first = __shfl_sync(0xffffffffu, first, 0);
+                if (x.s != 0u) put(first + __popc(ok & ((1u << lane) - 1u)), x);
+            }
+            __syncthreads();   // the items are in place, the list has been read
+            if (tid == 0) {
+                int left = 0;
+                if (f0 > 0) {
+                    left = find_range(s_pre, nx, f0);
+                    const int part = f0 - s_pre[left];
+                    if (part > 0) {
+                        s_exit[left].y = (uint32_t)part;
+                        left++;
+                    }
+                }
+                sh.nexit = left;
+            }
+            const int n = *reinterpret_cast<volatile int*>(&sh.back);
+            __syncthreads();
+            if (n > 0) return n;
+        }
+    }
+
+    // Sets the token ranges left by the rounds and empties their lists.
+    // Every thread calls it, after a barrier that follows the last round.
+    __device__ __forceinline__ void ranges() const {
+        const int ns = min(*reinterpret_cast<volatile int*>(&sh.nsmall), kRowSmall);
+        const int nb = min(*reinterpret_cast<volatile int*>(&sh.nbig), kRowBig);
+        // short ones: four threads each
+        for (int i = tid / 4; i < ns; i += kRowThreads / 4) {
+            const uint2 x = s_small[i];
+            const uint32_t n = x.y >> 16, s = x.y & 0xFFFFu;
+            for (uint32_t j = tid & 3; j < n; j += 32) {
+                int tk[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) tk[q] = j + 4 * q < n ? __ldg(t.dtok + x.x + j + 4 * q) : -1;
+#pragma unroll
+                for (int q = 0; q < 8; ++q)
+                    if (tk[q] >= 0) emit(tk[q], s);
+            }
+        }
+        if (nb > 0) {   // long ones: the CTA over all of them
+            const int total = prefix(nb, tid < nb ? (int)s_big[tid].y : 0);
+            constexpr int kUnroll = 8;
+            for (int f0 = tid; f0 < total; f0 += kUnroll * kRowThreads) {
+                int tk[kUnroll];
+                uint32_t st[kUnroll];
+                int k = find_range(s_pre, nb, f0);
+#pragma unroll
+                for (int q = 0; q < kUnroll; ++q) {
+                    const int f = f0 + q * kRowThreads;
+                    tk[q] = -1;
+                    st[q] = 0u;
+                    if (f < total) {
+                        while (f >= s_pre[k + 1]) ++k;
+                        const uint4 b = s_big[k];
+                        const uint32_t i = b.x + (uint32_t)(f - s_pre[k]);
+                        tk[q] = __ldg(t.dtok + i);
+                        if (b.w != 0u && __ldg(t.keeps + (size_t)((b.w >> 8) - 1u) * t.n_dtok + i) > (b.w & 0xFFu))
+                            tk[q] = -1;
+                        st[q] = b.z;
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < kUnroll; ++q)
+                    if (tk[q] >= 0) emit(tk[q], st[q]);
+            }
+        }
+        __syncthreads();   // the lists have been read
+        if (tid == 0) sh.nsmall = sh.nbig = 0;
+        __syncthreads();
+    }
+};
+
+template <bool STACK, int CLS, int OUT>
+__global__ void __launch_bounds__(kRowThreads, 2)
+    row_kernel(const __grid_constant__ StepView v, const __grid_constant__ RowTree t,
+               const __grid_constant__ RowArgs a, const RowList list) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ RowShared sh;
+    const RowLayout L = row_layout(a.slice_words, t.reserve, STACK, t.n_loops > 0);
+    uint32_t* s_mask = reinterpret_cast<uint32_t*>(smem + L.mask);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int row = blockIdx.x / a.slices, slice = blockIdx.x - row * a.slices;
+    const int w0 = slice * a.slice_words, nw = max(0, min(a.slice_words, v.W - w0));
+    const int tok0 = w0 * 32, ntok = max(0, min(nw * 32, v.V - tok0));
+    for (int j = tid; j < a.slice_words / 4; j += kRowThreads)
+        reinterpret_cast<uint4*>(s_mask)[j] = make_uint4(0u, 0u, 0u, 0u);
+    if (tid == 0) {
+        sh.nsmall = sh.nbig = sh.nexit = 0;
+        sh.st[0] = make_int4(0, INT_MAX, 0, 0);
+    }
+    pdl_wait();
+    pdl_trigger();
+    if (row >= list.rows(a.batch)) return;   // the whole cluster
+    // the row's configuration (invalid ones set the error word, once per row)
+    uint4 rc;
+    if (a.row_is_state) {
+        const uint32_t q = (uint32_t)row;
+        rc = make_uint4(q, 0u, 0u, 1u | (((__ldg(v.accept_bits + (q >> 5)) >> (q & 31u)) & 1u) ? 2u : 0u));
+    } else {
+        rc = read_row(v, a.states, a.stacks, list.row(row), tid == 0 && slice == 0);
+    }
+    // the state the walk starts from, and its loop set
+    uint32_t s0 = (rc.w & 1u) ? rc.x : 0u, root = 0u;
+    if (t.start) {
+        const uint2 w = __ldg(t.start + s0);
+        s0 = w.x;
+        if (w.y != 0xFFFFFFFFu) {   // the tokens that stay inside the set, then the walk of the others
+            const uint32_t* loop = t.loopbits + (size_t)w.y * v.W + w0;
+            __syncthreads();   // the mask has been cleared
+            for (int j = tid; j < nw; j += kRowThreads) s_mask[j] = __ldg(loop + j);
+            root = (uint32_t)t.loop_root[w.y];
+        }
+    }
+    int32_t* nrow = nullptr;
+    if constexpr (OUT == kRowNext) {
+        // the row's next states are 0 before the walk stores its tokens'
+        nrow = a.next ? a.next + (size_t)row * v.V : nullptr;
+        if (nrow) {
+            if ((v.V & 3) == 0 && (reinterpret_cast<uintptr_t>(a.next) & 15) == 0) {
+                int4* dst = reinterpret_cast<int4*>(nrow + tok0);
+                for (int j = tid; j < ntok / 4; j += kRowThreads) dst[j] = make_int4(0, 0, 0, 0);
+            } else {
+                for (int j = tid; j < ntok; j += kRowThreads) nrow[tok0 + j] = 0;
+            }
+        }
+    }
+    const RowWalk<STACK, CLS, OUT> wk{v, t, s_mask, reinterpret_cast<uint2*>(smem + L.items),
+                                      reinterpret_cast<uint32_t*>(smem + L.bits),
+                                      reinterpret_cast<uint2*>(smem + L.small), reinterpret_cast<uint4*>(smem + L.big),
+                                      reinterpret_cast<uint4*>(smem + L.exits), reinterpret_cast<int*>(smem + L.pre), sh,
+                                      nrow, tok0, ntok, tid, lane, warp};
+    if (tid == 0) wk.put(0, {root, s0, rc.z, rc.y});
+    __syncthreads();   // the mask (and the next states) are filled
+    wk.run(s0 != 0u ? 1 : 0, row_pool_cap(t.reserve));
+    __syncthreads();
+    wk.ranges();
+    if (tid == 0 && (rc.w & 2u) && v.eos_id >= 0) wk.emit(v.eos_id, rc.x);   // EOS keeps the state
+    __syncthreads();
+    if (a.mask) {
+        uint32_t* mrow = a.mask + (size_t)row * v.W + w0;
+        if ((v.W & 3) == 0 && (reinterpret_cast<uintptr_t>(a.mask) & 15) == 0) {
+            for (int j = tid; j < nw / 4; j += kRowThreads)
+                reinterpret_cast<uint4*>(mrow)[j] = reinterpret_cast<const uint4*>(s_mask)[j];
+        } else {
+            for (int j = tid; j < nw; j += kRowThreads) mrow[j] = s_mask[j];
+        }
+    }
+}
+
+template <typename... KArgs, typename... Args>
+cudaError_t launch_rows(void (*kern)(KArgs...), int grid, int cluster, int smem, cudaStream_t st, Args&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(kRowThreads);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)cluster;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
+}
+
+// Raises a kernel's dynamic shared-memory limit on the current device once
+// per size (one array of configured sizes per kernel instance).
+template <typename K>
+cudaError_t rows_allow_smem(K kern, int bytes, int* configured, std::mutex& mu) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (bytes <= 48 * 1024) return cudaSuccess;
+    std::lock_guard<std::mutex> lk(mu);
+    if (dev < kRowMaxDevices && configured[dev] >= bytes) return cudaSuccess;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess && dev < kRowMaxDevices) configured[dev] = bytes;
+    return e;
+}
+
+template <bool STACK, int CLS, int OUT>
+cudaError_t launch_row_t(const StepView& v, const RowTree& t, const LaunchEnv& env, RowArgs a, const RowList& list,
+                         cudaStream_t st) {
+    // CTAs per row: enough to give every SM one, and enough for the row's
+    // words to fit
+    int s = 1;
+    while (s < kRowMaxSlices && ((int64_t)a.batch * s * 2 <= env.num_sms || (v.W + s - 1) / s > kRowSliceWords)) s *= 2;
+    a.slices = s;
+    a.slice_words = ((v.W + s - 1) / s + 3) / 4 * 4;
+    const RowLayout L = row_layout(a.slice_words, t.reserve, STACK, t.n_loops > 0);
+    if (L.total > env.max_smem_optin) return cudaErrorInvalidConfiguration;
+    auto kern = row_kernel<STACK, CLS, OUT>;
+    static int configured[kRowMaxDevices] = {0};
+    static std::mutex mu;
+    cudaError_t e = rows_allow_smem(kern, L.total, configured, mu);
+    if (e != cudaSuccess) return e;
+    return launch_rows(kern, a.batch * s, s, L.total, st, v, t, a, list);
+}
+
+template <bool STACK, int CLS>
+cudaError_t launch_row_o(const StepView& v, const RowTree& t, const LaunchEnv& env, const RowArgs& a,
+                         const RowList& list, cudaStream_t st) {
+    return a.next ? launch_row_t<STACK, CLS, kRowNext>(v, t, env, a, list, st)
+                  : launch_row_t<STACK, CLS, kRowMask>(v, t, env, a, list, st);
+}
+
+}  // namespace
+
+cudaError_t launch_row_step(const StepView& v, const RowTree& t, const LaunchEnv& env, bool stack,
+                            const int32_t* states, const uint64_t* stacks, int32_t batch, bool row_is_state,
+                            uint32_t* mask, int32_t* next, cudaStream_t st, const int32_t* row_ids,
+                            const int32_t* row_count) {
+    if (batch <= 0) return cudaSuccess;
+    RowArgs a{};
+    a.states = states;
+    a.stacks = stacks;
+    a.batch = batch;
+    a.row_is_state = row_is_state ? 1 : 0;
+    a.mask = mask;
+    a.next = next;
+    const RowList list{row_ids, row_count, 0};
+    if (v.K <= 32)
+        return stack ? launch_row_o<true, kRow32>(v, t, env, a, list, st)
+                     : launch_row_o<false, kRow32>(v, t, env, a, list, st);
+    if (v.K <= 64)
+        return stack ? launch_row_o<true, kRow64>(v, t, env, a, list, st)
+                     : launch_row_o<false, kRow64>(v, t, env, a, list, st);
+    return stack ? launch_row_o<true, kRowWide>(v, t, env, a, list, st)
+                 : launch_row_o<false, kRowWide>(v, t, env, a, list, st);
+}
+
+// The pool entries that walking a node alone, depth first, can add: its
+// children replace it, then the deepest of them is walked.
+int32_t row_reserve(int32_t kids, int32_t below) { return std::max(0, kids - 1) + below; }
+
+int row_smem_bytes(int32_t n_words, int32_t reserve, bool stack, bool loops) {
+    return row_layout(std::min(n_words, kRowSliceWords) + 4, reserve, stack, loops).total;
+}
+
+}  // namespace domino

@@ -1,5 +1,5 @@
 // walk_common.cuh -- device helpers shared by the kernels of kernels.cu and
-// trie.cu: launches with programmatic dependent launch, the online (max,
+// rows.cu: launches with programmatic dependent launch, the online (max,
 // lowest-index argmax, sum of exp) fold, the transition table lookups of the
 // four table modes, the bracket-stack step, the row configuration decode and
 // the update of one row (Alg. 1's update).
