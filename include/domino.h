@@ -31,8 +31,8 @@
  *  - A handle is not thread-safe; calls on one handle must be serialised by
  *    the caller, and their kernels must not overlap on the GPU either (issue
  *    them on one stream, or order the streams with events): the handle's
- *    scratch (the logits pass's partials and tickets, the fused decode's
- *    partials, the host-buffer step's staging) is shared by its calls.
+ *    scratch (the fused decode's partials, opportunistic masking's row list,
+ *    the host-buffer step's staging) is shared by its calls.
  *    Different handles are independent.
  */
 #ifndef DOMINO_H
@@ -200,7 +200,7 @@ int domino_step_mask(domino_t h, const int32_t* states_dev, const uint64_t* stac
  *   DOMINO_DTYPE_BF16), row_stride_elems >= V apart; mask_dev [batch][W];
  *   argmax_dev int32 [batch] (required); lse_dev float [batch] or NULL;
  *   logprobs_dev float [batch][V] or NULL.
- * Logits must be finite.  Uses scratch memory owned by the handle. */
+ * Logits must be finite. */
 int domino_mask_logits(domino_t h, const void* logits_dev, int32_t dtype, int32_t batch,
                        int64_t row_stride_elems, const uint32_t* mask_dev, int32_t* argmax_dev, float* lse_dev,
                        float* logprobs_dev, void* stream);
@@ -229,12 +229,15 @@ int domino_advance(domino_t h, const int32_t* states_dev, const uint64_t* stacks
  *   states_out int32 [batch] or NULL (no update), stacks_out uint64 [batch]
  *   (required with states_out when stacks_dev is given): the configurations
  *   after the decoded token; they may alias states_dev / stacks_dev.
- * The fused form needs bf16 rows on 16-byte boundaries; other inputs run the
- * two kernels one after the other.  Results equal domino_step_mask followed
- * by domino_mask_logits.  The first call with a larger batch allocates
- * scratch and synchronises `stream`; if `stream` is being captured into a
- * CUDA graph at that point, the call returns DOMINO_E_INVALID_ARG and
- * launches nothing (make one uncaptured call at the largest batch first). */
+ * One kernel walks, decodes and advances each row where the prefix-tree walk
+ * is chosen or the batch is large; smaller batches fold the decode into the
+ * per-token walk (bf16 rows on 16-byte boundaries) or run the kernels one
+ * after the other.  Results equal domino_step_mask followed by
+ * domino_mask_logits.  The folded per-token walk's first call with a larger
+ * batch allocates scratch and synchronises `stream`; if `stream` is being
+ * captured into a CUDA graph at that point, the call returns
+ * DOMINO_E_INVALID_ARG and launches nothing (make one uncaptured call at the
+ * largest batch first). */
 int domino_step_decode(domino_t h, const int32_t* states_dev, const uint64_t* stacks_dev, int32_t batch,
                        const void* logits_dev, int32_t dtype, int64_t row_stride_elems, uint32_t* mask_dev,
                        int32_t* argmax_dev, float* lse_dev, float* logprobs_dev, int32_t* states_out,
@@ -251,7 +254,7 @@ int domino_step_decode(domino_t h, const int32_t* states_dev, const uint64_t* st
  * fp32 operations (ln by the atanh series), so draws are reproducible bit for
  * bit by an independent implementation.  A caller passes a new offset per
  * decode step.  temperature must be finite and > 0.  Same logits and mask
- * layout as domino_mask_logits; uses the handle's scratch memory. */
+ * layout as domino_mask_logits. */
 int domino_mask_sample(domino_t h, const void* logits_dev, int32_t dtype, int32_t batch, int64_t row_stride_elems,
                        const uint32_t* mask_dev, float temperature, uint64_t seed, uint64_t offset,
                        int32_t* tokens_dev, void* stream);
@@ -322,7 +325,7 @@ int domino_spec_accept(domino_t h, const int32_t* proposals_dev, const int32_t* 
  * table written by domino_precompute_table for this handle's automaton and
  * vocabulary.  A state outside [0, Q) reads as an empty row (argmax -1) and
  * sets DOMINO_DEVERR_BAD_STATE.  Pushdown automata: DOMINO_E_UNSUPPORTED
- * (their masks depend on the stack).  Uses the handle's scratch memory. */
+ * (their masks depend on the stack). */
 int domino_mask_logits_table(domino_t h, const void* logits_dev, int32_t dtype, int32_t batch,
                              int64_t row_stride_elems, const uint32_t* table_mask_dev, const int32_t* states_dev,
                              int32_t* argmax_dev, float* lse_dev, float* logprobs_dev, void* stream);
@@ -364,17 +367,10 @@ int domino_decode_step_host(domino_t h, const void* logits_host, int32_t dtype, 
  *   Same arguments and results as domino_mask_logits, with the vocabulary size
  *   n_tokens passed directly; batch <= 512 (larger batches return
  *   DOMINO_E_INVALID_ARG: split them into calls of at most 512 rows).
- *   Scratch: a fixed 516 KiB array inside libdomino.so (per-row partials,
- *   tickets, temporary lse); every GPU that loads the library holds it until
- *   the process exits.  Nothing is allocated by this call: no cudaMalloc,
- *   cudaFree or allocating library routine.
- *   The first call on a device looks up the array's device address with that
- *   device current (the calling thread's current device); make that first
- *   call before any stream capture.
- *   All calls share the one array and each call clears the tickets it uses;
- *   calls that overlap on the GPU (other streams or host threads without
- *   ordering between them) race on it and corrupt each other's results, so
- *   order them, e.g. on one stream. */
+ *   Nothing is allocated by this call: no cudaMalloc, cudaFree or allocating
+ *   library routine, and no scratch in device memory.  The first call on a
+ *   device queries it, with that device current (the calling thread's current
+ *   device); make that first call before any stream capture. */
 int domino_mask_logits_noalloc(const void* logits_dev, int32_t dtype, int32_t batch, int32_t n_tokens,
                                int64_t row_stride_elems, const uint32_t* mask_dev, int32_t* argmax_dev,
                                float* lse_dev, float* logprobs_dev, void* stream);

@@ -1,7 +1,7 @@
 """Builds libdomino.so in-tree with nvcc for sm_103a (GB300).
 
-Three translation units (host.cpp: C ABI and loaders; kernels.cu and rows.cu:
-kernels) are compiled in parallel and linked into paper_2403_06988_gb300/libdomino.so.
+Four translation units (host.cpp: C ABI and loaders; kernels.cu, rows.cu and
+logits.cu: kernels) are compiled in parallel and linked into paper_2403_06988_gb300/libdomino.so.
 Objects go to paper_2403_06988_gb300/_build/.
 
 build(debug=True) makes libdomino_debug.so instead (objects in _build_debug/),
@@ -24,7 +24,7 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libdomino.so")
 LIB_DEBUG = os.path.join(PKG, "libdomino_debug.so")
-SOURCES = ["host.cpp", "kernels.cu", "rows.cu"]
+SOURCES = ["host.cpp", "kernels.cu", "rows.cu", "logits.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -38,6 +38,7 @@ def nvcc() -> str:
 def _inputs():
     files = [os.path.join(CSRC, f) for f in SOURCES]
     files += [os.path.join(CSRC, "domino_internal.h"), os.path.join(CSRC, "walk_common.cuh"),
+              os.path.join(CSRC, "decode.cuh"),
               os.path.join(INCLUDE, "domino.h")]
     return files
 

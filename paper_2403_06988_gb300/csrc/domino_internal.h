@@ -24,8 +24,6 @@ constexpr int kWalkChains = 4;                 // rows walked together by one la
 constexpr int kHeadBytes = 16;                 // class ids per 16-byte head block
 constexpr int kInlineBytes = 32;               // class ids stored inline per token (two head blocks)
 constexpr int kLogitThreads = 256;
-constexpr int kMaxLogitRows = 4096;            // rows per mask_logits pass (scratch size)
-constexpr int kMaxSegments = 64;               // CTAs sharing one row in mask_logits
 constexpr int kAdvanceThreads = 128;
 
 // slot info word: bits 0..9 original id within the window, bit 10 valid,
@@ -167,8 +165,14 @@ cudaError_t launch_fused_combine(const StepView& v, bool stack, int mode, const 
 // tree whose row_smem_bytes fit.
 cudaError_t launch_row_step(const StepView& v, const RowTree& t, const LaunchEnv& env, bool stack,
                             const int32_t* states, const uint64_t* stacks, int32_t batch, bool row_is_state,
-                            uint32_t* mask, int32_t* next, cudaStream_t st, const int32_t* row_ids = nullptr,
-                            const int32_t* row_count = nullptr);
+                            uint32_t* mask, int32_t* next, cudaStream_t st);
+// The mask step, the masked greedy decode and (with states_out) the update in
+// one kernel; logits in device or mapped host memory, any dtype and alignment;
+// outputs may alias states / stacks.
+cudaError_t launch_row_decode(const StepView& v, const RowTree& t, const LaunchEnv& env, bool stack,
+                              const int32_t* states, const uint64_t* stacks, int32_t batch, const void* logits,
+                              int dtype, int64_t row_stride, uint32_t* mask, int32_t* argmax, float* lse,
+                              float* logprobs, int32_t* states_out, uint64_t* stacks_out, cudaStream_t st);
 // The host's side of the walk's pool bound (RowTree::reserve): a node with
 // `kids` children, the deepest of which need `below`; and the shared memory a
 // CTA needs.
@@ -180,7 +184,7 @@ int row_smem_bytes(int32_t n_words, int32_t reserve, bool stack, bool loops);
 cudaError_t launch_logprobs_bf16(const LaunchEnv& env, const void* logits, int32_t batch, int64_t row_stride,
                                  int32_t V, const uint32_t* mask, const float* lse, float* logprobs, cudaStream_t st);
 
-// Sampling decode: Gumbel-max with Philox4x32-10 uniforms (kernels.cu).
+// Sampling decode: Gumbel-max with Philox4x32-10 uniforms (decode.cuh).
 struct SampleArgs {
     uint32_t key0, key1;     // the 64-bit seed
     uint32_t off0, off1;     // the 64-bit offset (counter words 2 and 3)
@@ -194,21 +198,16 @@ struct SampleArgs {
 // token allowed.  row_ids / row_count (device): only rows row_ids[i] for
 // i < *row_count are processed, their masks being the compact rows i of
 // `mask`; argmax and lse are indexed by batch row; no logprobs.
-// raises the logits kernels' shared-memory limit on the current device; called
-// once per handle and device, outside any stream capture
-cudaError_t prepare_logits_kernels();
 cudaError_t launch_mask_logits(const LaunchEnv& env, const void* logits, int dtype, int32_t batch,
                                int64_t row_stride, int32_t V, const uint32_t* mask, int32_t* argmax, float* lse,
-                               float* logprobs, float4* partials, uint32_t* counters, float* lse_tmp,
-                               cudaStream_t st, const int32_t* row_state = nullptr, int32_t Q = 0,
+                               float* logprobs, cudaStream_t st, const int32_t* row_state = nullptr, int32_t Q = 0,
                                uint32_t* err = nullptr, const SampleArgs* sample = nullptr,
                                const int32_t* row_ids = nullptr, const int32_t* row_count = nullptr);
 
 // Fills the sampling arguments (1/T in fp32, seed and offset words).
 cudaError_t launch_mask_sample(const LaunchEnv& env, const void* logits, int dtype, int32_t batch,
                                int64_t row_stride, int32_t V, const uint32_t* mask, float temperature,
-                               uint64_t seed, uint64_t offset, int32_t* tokens, float4* partials,
-                               uint32_t* counters, cudaStream_t st);
+                               uint64_t seed, uint64_t offset, int32_t* tokens, cudaStream_t st);
 
 // `mode` names the table image the step kernel reads (it is L2-resident after a step).
 cudaError_t launch_advance(const StepView& v, bool stack, int mode, const int32_t* states, const uint64_t* stacks,

@@ -57,7 +57,7 @@ struct domino_ctx {
     // ---- device copies
     DevBuf d_head, d_info, d_tail_off, d_tail, d_pos_of, d_cls_start, d_eos_slot;
     DevBuf d_dense, d_sparse, d_accept, d_self, d_tok_cls;
-    DevBuf d_err, d_partials, d_counters, d_lse_tmp, d_fpart;
+    DevBuf d_err, d_fpart;
     bool arena_ready = false;
     // prefix tree of the class strings (domino_get_prefix_tree)
     std::vector<uint4> t_node;
@@ -135,8 +135,7 @@ void dev_free(DevBuf& b) {
 
 int64_t dev_bytes(const domino_ctx* h) {
     const DevBuf* all[] = {&h->d_head, &h->d_info, &h->d_tail_off, &h->d_tail, &h->d_pos_of, &h->d_cls_start,
-                           &h->d_eos_slot, &h->d_dense, &h->d_sparse, &h->d_accept, &h->d_self, &h->d_tok_cls, &h->d_err, &h->d_fpart, &h->d_partials,
-                           &h->d_counters, &h->d_lse_tmp, &h->s_logits, &h->s_mask, &h->s_io,
+                           &h->d_eos_slot, &h->d_dense, &h->d_sparse, &h->d_accept, &h->d_self, &h->d_tok_cls, &h->d_err, &h->d_fpart, &h->s_logits, &h->s_mask, &h->s_io,
                            &h->o_prop, &h->o_rows, &h->o_count};
     int64_t n = 0;
     for (auto* b : all) n += (int64_t)b->n;
@@ -835,6 +834,20 @@ bool use_rows(const domino_ctx* h, int64_t batch, bool next) {
     return h->rows_ready && h->walk_pref != 0 && !next && batch * h->V >= ((int64_t)1 << 21);
 }
 
+// Whether the whole decode step is row_kernel's (one launch).  With loop sets
+// the lines cross near 3 * 2^20 (row, token) pairs against the per-token walk
+// with the decode folded in (two launches; bf16 rows on 16-byte boundaries):
+// 200 states, V = 32000, batch 32: 13.4 against 8.8 us, batch 100: 12.6
+// against 11.8 us (with log-probabilities 15.1 against 16.3 us); JSON, V =
+// 50001, batch 64: 28.8 against 33.7 us; V = 152064, batch 8: 18.6 against
+// 15.0 us, batch 128: 54.6 against 86.1 us, batch 512: 102 against 304 us; and
+// near 2^20 against the three kernels one after the other (V = 50001, batch
+// 24: 26.8 against 27.9 us and two launches more).
+bool decode_rows(const domino_ctx* h, int64_t batch, bool fusable) {
+    return use_tree(h) || (h->rows_ready && h->walk_pref != 0 &&
+                           batch * h->V >= (fusable ? (int64_t)3 << 20 : (int64_t)1 << 20));
+}
+
 int ready_for_compute(domino_ctx* h) {
     if (!h) return DOMINO_E_INVALID_ARG;
     if (is_host_only(h)) return DOMINO_E_NO_DEVICE;
@@ -900,13 +913,8 @@ int domino_create(domino_t* out, int32_t cuda_device) {
         }
         cudaDeviceGetAttribute(&h->env.num_sms, cudaDevAttrMultiProcessorCount, h->device);
         cudaDeviceGetAttribute(&h->env.max_smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
-        int rc = prepare_logits_kernels() == cudaSuccess ? DOMINO_OK : DOMINO_E_CUDA;
-        if (!rc) rc = dev_reserve(h->d_err, 16);
-        if (!rc) rc = dev_reserve(h->d_partials, sizeof(float4) * (size_t)kMaxLogitRows * kMaxSegments);
-        if (!rc) rc = dev_reserve(h->d_counters, sizeof(uint32_t) * (size_t)kMaxLogitRows);
-        if (!rc) rc = dev_reserve(h->d_lse_tmp, sizeof(float) * (size_t)kMaxLogitRows);
-        if (!rc && (cudaMemset(h->d_err.p, 0, 16) != cudaSuccess ||
-                    cudaMemset(h->d_counters.p, 0, sizeof(uint32_t) * (size_t)kMaxLogitRows) != cudaSuccess)) {
+        int rc = dev_reserve(h->d_err, 16);
+        if (!rc && cudaMemset(h->d_err.p, 0, 16) != cudaSuccess) {
             cudaGetLastError();
             rc = DOMINO_E_CUDA;
         }
@@ -925,8 +933,7 @@ int domino_destroy(domino_t h) {
         DeviceGuard g(h->device);
         cudaDeviceSynchronize();
         DevBuf* all[] = {&h->d_head, &h->d_info, &h->d_tail_off, &h->d_tail, &h->d_pos_of, &h->d_cls_start,
-                         &h->d_eos_slot, &h->d_dense, &h->d_sparse, &h->d_accept, &h->d_self, &h->d_tok_cls, &h->d_err, &h->d_fpart, &h->d_partials,
-                         &h->d_counters, &h->d_lse_tmp, &h->s_logits, &h->s_mask, &h->s_io,
+                         &h->d_eos_slot, &h->d_dense, &h->d_sparse, &h->d_accept, &h->d_self, &h->d_tok_cls, &h->d_err, &h->d_fpart, &h->s_logits, &h->s_mask, &h->s_io,
                          &h->o_prop, &h->o_rows, &h->o_count, &h->d_rnode, &h->d_rncls, &h->d_rdtok, &h->d_srec, &h->d_srec_next, &h->d_rret,
                          &h->d_rstart, &h->d_loop_of, &h->d_loopbits, &h->d_keeps, &h->d_xrange, &h->d_exits};
         for (auto* b : all) dev_free(*b);
@@ -1304,9 +1311,7 @@ int domino_mask_logits(domino_t h, const void* logits_dev, int32_t dtype, int32_
     if (!logits_dev || !mask_dev || !argmax_dev) return DOMINO_E_INVALID_ARG;
     DeviceGuard g(h->device);
     return cuda_status(launch_mask_logits(h->env, logits_dev, dtype, batch, row_stride_elems, h->V, mask_dev,
-                                          argmax_dev, lse_dev, logprobs_dev, (float4*)h->d_partials.p,
-                                          (uint32_t*)h->d_counters.p, (float*)h->d_lse_tmp.p,
-                                          (cudaStream_t)stream));
+                                          argmax_dev, lse_dev, logprobs_dev, (cudaStream_t)stream));
 }
 
 int domino_advance(domino_t h, const int32_t* states_dev, const uint64_t* stacks_dev, const int32_t* tokens_dev,
@@ -1339,18 +1344,21 @@ int domino_step_decode(domino_t h, const int32_t* states_dev, const uint64_t* st
         return DOMINO_E_INVALID_ARG;
     DeviceGuard g(h->device);
     cudaStream_t st = (cudaStream_t)stream;
+    // the decode can ride on the per-token walk
+    const bool fusable = dtype == DOMINO_DTYPE_BF16 && reinterpret_cast<uintptr_t>(logits_dev) % 16 == 0 &&
+                         ((size_t)row_stride_elems * 2) % 16 == 0 &&
+                         (int64_t)batch * h->n_windows < (int64_t)INT32_MAX;   // partial slots are int
+    if (decode_rows(h, batch, fusable)) {   // the whole step in one kernel
+        StepView v = make_view(h);
+        return cuda_status(launch_row_decode(v, h->rows, h->env, h->stack, states_dev, stacks_dev, batch, logits_dev,
+                                             dtype, row_stride_elems, mask_dev, argmax_dev, lse_dev, logprobs_dev,
+                                             states_out, states_out && stacks_dev ? stacks_out : nullptr, st));
+    }
     // logits in device memory are pulled into L2 a tile ahead of their fold;
     // host-resident logits are read only where the mask allows a token
     cudaPointerAttributes pa{};
     const bool on_device = cudaPointerGetAttributes(&pa, logits_dev) == cudaSuccess && pa.type == cudaMemoryTypeDevice;
     if (!on_device) cudaGetLastError();
-    // the fold rides on the per-token walk; where the prefix-tree walk is the
-    // faster mask step and the logits sit in device memory, the tree walk, the
-    // logits pass and the update run one after the other instead
-    const bool fusable = dtype == DOMINO_DTYPE_BF16 && reinterpret_cast<uintptr_t>(logits_dev) % 16 == 0 &&
-                         ((size_t)row_stride_elems * 2) % 16 == 0 &&
-                         (int64_t)batch * h->n_windows < (int64_t)INT32_MAX &&   // partial slots are int
-                         !(on_device && use_tree(h));
     if (!fusable) {   // the kernels one after the other
         if ((rc = domino_step_mask(h, states_dev, stacks_dev, batch, mask_dev, nullptr, stream))) return rc;
         if ((rc = domino_mask_logits(h, logits_dev, dtype, batch, row_stride_elems, mask_dev, argmax_dev, lse_dev,
@@ -1401,8 +1409,7 @@ int domino_mask_sample(domino_t h, const void* logits_dev, int32_t dtype, int32_
     if (!logits_dev || !mask_dev || !tokens_dev) return DOMINO_E_INVALID_ARG;
     DeviceGuard g(h->device);
     return cuda_status(launch_mask_sample(h->env, logits_dev, dtype, batch, row_stride_elems, h->V, mask_dev,
-                                          temperature, seed, offset, tokens_dev, (float4*)h->d_partials.p,
-                                          (uint32_t*)h->d_counters.p, (cudaStream_t)stream));
+                                          temperature, seed, offset, tokens_dev, (cudaStream_t)stream));
 }
 
 int domino_opportunistic_step(domino_t h, const void* logits_dev, int32_t dtype, int32_t batch,
@@ -1433,7 +1440,7 @@ int domino_opportunistic_step(domino_t h, const void* logits_dev, int32_t dtype,
     // 1. the unmasked argmax (every token allowed)
     if (e == cudaSuccess)
         e = launch_mask_logits(h->env, logits_dev, dtype, batch, row_stride_elems, h->V, nullptr, prop, nullptr,
-                               nullptr, (float4*)h->d_partials.p, (uint32_t*)h->d_counters.p, nullptr, st);
+                               nullptr, st);
     // 2. one walk per row: keep the proposal or list the row for the fallback
     if (e == cudaSuccess)
         e = launch_propose_check(v, h->stack, mode, states_dev, stacks_dev, prop, batch, tokens_dev, rows, count, st);
@@ -1443,8 +1450,7 @@ int domino_opportunistic_step(domino_t h, const void* logits_dev, int32_t dtype,
                              nullptr, st, rows, count);
     if (e == cudaSuccess)
         e = launch_mask_logits(h->env, logits_dev, dtype, batch, row_stride_elems, h->V, mask_scratch_dev,
-                               tokens_dev, nullptr, nullptr, (float4*)h->d_partials.p, (uint32_t*)h->d_counters.p,
-                               nullptr, st, nullptr, 0, nullptr, nullptr, rows, count);
+                               tokens_dev, nullptr, nullptr, st, nullptr, 0, nullptr, nullptr, rows, count);
     return cuda_status(e);
 }
 
@@ -1513,9 +1519,7 @@ int domino_mask_logits_table(domino_t h, const void* logits_dev, int32_t dtype, 
     if (!logits_dev || !table_mask_dev || !states_dev || !argmax_dev) return DOMINO_E_INVALID_ARG;
     DeviceGuard g(h->device);
     return cuda_status(launch_mask_logits(h->env, logits_dev, dtype, batch, row_stride_elems, h->V, table_mask_dev,
-                                          argmax_dev, lse_dev, logprobs_dev, (float4*)h->d_partials.p,
-                                          (uint32_t*)h->d_counters.p, (float*)h->d_lse_tmp.p, (cudaStream_t)stream,
-                                          states_dev, h->Q, (uint32_t*)h->d_err.p));
+                                          argmax_dev, lse_dev, logprobs_dev, (cudaStream_t)stream, states_dev, h->Q, (uint32_t*)h->d_err.p));
 }
 
 int domino_advance_table(domino_t h, const int32_t* table_next_dev, const int32_t* states_dev,

@@ -18,16 +18,6 @@
 //                   (Alg. 2's traversal, precomputed offline, Sec. 3.5), and,
 //                   over a device-side row list, masks only the rows that
 //                   opportunistic masking rejected.
-//  logits_reduce    Alg. 1's v' = m (.) v and decode: a balanced flat split of
-//                   the batch x mask words over one-warp CTAs; the 16-byte
-//                   logit vectors that hold an allowed token are staged with
-//                   cp.async (the others are never read); a lane folds its
-//                   word into a masked max / lowest-index argmax / sum of
-//                   exp, or a Gumbel-max draw (sampling); per-row segments are
-//                   combined by the last CTA to finish (atomic ticket, no
-//                   spinning).  Rows may come from a precomputed mask table
-//                   (table-driven step) or a device-side row list.
-//  logprobs         the second pass for log-probabilities.
 //  advance          C.update(o): the chosen token's walk (or one read of the
 //                   precomputed next-state table).
 //  propose_check,   opportunistic masking's one-walk check, and count-based
@@ -600,661 +590,6 @@ __global__ void __launch_bounds__(kStepThreads, 1)
 }
 
 // ---------------------------------------------------------------------------
-// masked argmax / log-sum-exp
-// ---------------------------------------------------------------------------
-template <bool BF16>
-__device__ __forceinline__ float logit_at(const void* row, int t) {
-    if constexpr (BF16) {
-        const unsigned short u = __ldg(reinterpret_cast<const unsigned short*>(row) + t);
-        return __uint_as_float((uint32_t)u << 16);
-    } else {
-        return __ldg(reinterpret_cast<const float*>(row) + t);
-    }
-}
-
-
-// cp.async: 16 bytes global -> shared without a register round trip
-__device__ __forceinline__ void cp_async16(void* smem_dst, const void* gmem_src) {
-    const unsigned dst = (unsigned)__cvta_generic_to_shared(smem_dst);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(gmem_src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
-
-constexpr int kReduceThreads = 32;            // one warp per CTA: no block barriers
-
-// ---- sampling: Gumbel-max over the allowed logits --------------------------
-// Philox4x32-10 (Salmon, Moraes, Dror and Shaw, SC'11): ten rounds of two
-// 32x32 -> 64-bit products on the counter, the key advanced by the Weyl
-// constants between rounds.
-__device__ __forceinline__ uint4 philox10(uint4 c, uint32_t k0, uint32_t k1) {
-#pragma unroll
-    for (int i = 0; i < 10; ++i) {
-        const uint32_t lo0 = 0xD2511F53u * c.x, hi0 = __umulhi(0xD2511F53u, c.x);
-        const uint32_t lo1 = 0xCD9E8D57u * c.z, hi1 = __umulhi(0xCD9E8D57u, c.z);
-        c = make_uint4(hi1 ^ c.y ^ k0, lo1, hi0 ^ c.w ^ k1, lo0);
-        k0 += 0x9E3779B9u;
-        k1 += 0xBB67AE85u;
-    }
-    return c;
-}
-
-// ln(x) for a positive normal float: x = 2^e m, m in [sqrt(1/2), sqrt(2)),
-// ln x = e ln 2 + 2 atanh(z), z = (m - 1) / (m + 1), with atanh's odd power
-// series up to z^11.  Every operation is an explicitly rounded fp32 intrinsic
-// (no contraction), so the value is reproducible bit for bit.
-__device__ __forceinline__ float ln_rn(float x) {
-    const uint32_t bits = __float_as_uint(x);
-    int e = (int)((bits >> 23) & 0xFFu) - 127;
-    float m = __uint_as_float((bits & 0x7FFFFFu) | 0x3F800000u);
-    if (m > 0x1.6a09e6p+0f) {
-        m = __fmul_rn(m, 0.5f);
-        e += 1;
-    }
-    const float z = __fdiv_rn(__fsub_rn(m, 1.0f), __fadd_rn(m, 1.0f));
-    const float z2 = __fmul_rn(z, z);
-    float p = 0x1.745d18p-4f;
-    p = __fmaf_rn(p, z2, 0x1.c71c72p-4f);
-    p = __fmaf_rn(p, z2, 0x1.24924ap-3f);
-    p = __fmaf_rn(p, z2, 0x1.99999ap-3f);
-    p = __fmaf_rn(p, z2, 0x1.555556p-2f);
-    p = __fmaf_rn(p, z2, 1.0f);
-    const float r = __fmul_rn(__fadd_rn(z, z), p);
-    const float ef = __int2float_rn(e);
-    return __fmaf_rn(ef, 0x1.62e43p-1f, __fmaf_rn(ef, -0x1.05c61p-29f, r));
-}
-
-// Gumbel variate of token t of row r: g_t = -ln(-ln(u_t)), u_t = (2k + 1) / 2^24,
-// k = (word t % 4 of Philox on (t / 4, r, offset)) >> 9.  `blk` / `rnd` cache
-// the last Philox block.
-__device__ __forceinline__ float gumbel(const SampleArgs& a, int r, int t, int& blk, uint4& rnd) {
-    if ((t >> 2) != blk) {
-        blk = t >> 2;
-        rnd = philox10(make_uint4((uint32_t)blk, (uint32_t)r, a.off0, a.off1), a.key0, a.key1);
-    }
-    const uint32_t w = (t & 2) ? ((t & 1) ? rnd.w : rnd.z) : ((t & 1) ? rnd.y : rnd.x);
-    const float u = __fmul_rn(__uint2float_rn(2u * (w >> 9) + 1u), 0x1p-24f);
-    return -ln_rn(-ln_rn(u));
-}
-
-// Every g_t is below this: u_t <= 1 - 2^-24 gives -ln(u_t) >= 5.96e-8 and
-// g_t <= 16.64.  A token with x / T + kGumbelMax below the best score so far
-// cannot win (rounding is monotonic), so its variate is never drawn.
-constexpr float kGumbelMax = 17.0f;
-
-// Where row r's mask words are: row r of `base` ([batch][W]), or, for the
-// table-driven step, row states[r] of a precomputed [Q][W] state table.  An
-// out-of-range state reads as an all-zero row (nothing allowed) and sets the
-// error word.
-struct MaskRows {
-    const uint32_t* base;       // nullptr (and no row_state): every token allowed
-    const int32_t* row_state;   // nullptr: base is [batch][W]
-    int32_t Q;
-    uint32_t* err;
-    __device__ __forceinline__ bool all() const { return base == nullptr; }
-    __device__ __forceinline__ const uint32_t* row(int r, int W, bool report) const {
-        if (all()) return nullptr;
-        if (!row_state) return base + (size_t)r * W;
-        const int32_t q = __ldg(row_state + r);
-        if (q < 0 || q >= Q) {
-            if (report) atomicOr(err, DOMINO_DEVERR_BAD_STATE);
-            return nullptr;
-        }
-        return base + (size_t)q * W;
-    }
-    // word j of a row given by row(); all-allowed rows read as all ones
-    __device__ __forceinline__ uint32_t word(const uint32_t* mrow, int j) const {
-        return all() ? 0xFFFFFFFFu : (mrow ? __ldg(mrow + j) : 0u);
-    }
-};
-
-constexpr int kStageDepth = 3;                // 32-word batches in flight per warp
-
-// Units are mask words (32 tokens); row r holds W units.  Each CTA takes a
-// contiguous range of the batch x W units; the CTAs sharing a row leave
-// (max, argmax, sum) partials and the last one to finish combines them.
-// STAGE (bf16 rows on 16-byte boundaries): a warp takes 32 consecutive words
-// of its row at a time; the 16-byte logit vectors that hold an allowed token
-// are copied, fully coalesced, into the warp's three-deep staging area
-// with cp.async (masks are read four batches ahead, logits two), and each lane
-// then folds its own word's allowed logits.  Otherwise each allowed logit is
-// read on its own.
-// What a row's allowed logits are folded into.
-enum Fold : int {
-    kFoldLse = 0,      // max, lowest-index argmax and sum of exp (log-sum-exp)
-    kFoldMax = 1,      // max and lowest-index argmax only (no lse requested)
-    kFoldSample = 2,   // Gumbel-max draw
-};
-
-template <bool BF16, bool STAGE, int FOLD>
-__global__ void __launch_bounds__(kReduceThreads)
-    logits_reduce_kernel(const void* __restrict__ logits, int64_t stride, const MaskRows mask, int V,
-                         int W, int B, long long per_cta, float4* __restrict__ partials,
-                         uint32_t* __restrict__ counters, int32_t* __restrict__ argmax, float* __restrict__ lse,
-                         const SampleArgs sa, int row0, const RowList list) {
-    // [buffer][word][16-byte vector]
-    __shared__ __align__(16) uint4 stage[STAGE ? kStageDepth * 32 * 4 : 1];
-    pdl_wait();
-    pdl_trigger();
-    const long long N = (long long)list.rows(B) * W;
-    const int lane = threadIdx.x;
-    long long u = (long long)blockIdx.x * per_cta;
-    const long long u_end = min(N, u + per_cta);
-    while (u < u_end) {
-        const int r = (int)(u / W);
-        const long long row_end = (long long)(r + 1) * W;
-        const long long seg_end = min(u_end, row_end);
-        const int j0 = (int)(u - (long long)r * W), j1 = (int)(seg_end - (long long)r * W);
-        const uint32_t* mrow = mask.row(r, W, lane == 0 && j0 == 0);
-        const int orow = list.row(r);   // the batch row: logits, outputs and the sampling counter
-        const char* lrow = reinterpret_cast<const char*>(logits) + (size_t)orow * stride * (BF16 ? 2 : 4);
-        float m = -INFINITY, mL = -INFINITY, s = 0.0f;
-        int idx = INT_MAX;
-        int blk = -1;                       // Philox block cached by gumbel_score
-        uint4 rnd = make_uint4(0u, 0u, 0u, 0u);
-        // one allowed logit x of token t (t increasing within a lane)
-        auto fold = [&](float x, int t) {
-            if constexpr (FOLD == kFoldSample) {
-                const float sx = __fmul_rn(x, sa.inv_t);
-                if (__fadd_rn(sx, kGumbelMax) < m) return;
-                const float sc = __fadd_rn(sx, gumbel(sa, row0 + orow, t, blk, rnd));
-                if (sc > m) {
-                    m = sc;
-                    idx = t;
-                }
-            } else if constexpr (FOLD == kFoldMax) {
-                if (x > m) {
-                    m = x;
-                    idx = t;
-                }
-            } else {
-                acc_add(m, mL, idx, s, x, t);
-            }
-        };
-        if constexpr (STAGE) {
-            const int nb = (j1 - j0 + 31) / 32;   // batches of 32 words
-            const int full_words = V / 32;       // words whose 64 bytes of logits lie inside the row
-            auto mask_of = [&](int b) -> uint32_t {
-                const int j = j0 + 32 * b + lane;
-                return (b < nb && j < j1) ? mask.word(mrow, j) : 0u;
-            };
-            auto issue = [&](int b, uint32_t mw) {
-                if (b < nb) {
-                    const char* base = lrow + (size_t)(j0 + 32 * b) * 64;
-                    uint4* dst = stage + (b % kStageDepth) * 128;
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const int q = 32 * k + lane, wi = q >> 2, sub = q & 3;
-                        const uint32_t mq = __shfl_sync(0xffffffffu, mw, wi);
-                        if (((mq >> (8 * sub)) & 0xFFu) && j0 + 32 * b + wi < full_words)
-                            cp_async16(dst + q, base + (size_t)q * 16);
-                    }
-                }
-                cp_async_commit();
-            };
-            uint32_t mw[kStageDepth + 1];
-#pragma unroll
-            for (int k = 0; k <= kStageDepth; ++k) mw[k] = mask_of(k);
-#pragma unroll
-            for (int k = 0; k < kStageDepth - 1; ++k) issue(k, mw[k]);
-            for (int b = 0; b < nb; ++b) {
-                issue(b + kStageDepth - 1, mw[kStageDepth - 1]);
-                const uint32_t mw_far = mask_of(b + kStageDepth + 1);
-                cp_async_wait<kStageDepth - 1>();   // batch b has landed
-                __syncwarp();
-                const int j = j0 + 32 * b + lane;
-                uint32_t word = mw[0];
-                if (word) {
-                    const int t0 = j * 32;
-                    if (FOLD != kFoldSample && j < full_words && __popc(word) > 12) {
-                        // a dense word: the word's maximum first (every token compared in
-                        // order, no bit scan), then, for the log-sum-exp, one rescale and
-                        // the sum of the word's terms
-                        const uint4* sv = stage + (b % kStageDepth) * 128 + lane * 4;
-                        uint32_t qs[16];
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            const uint4 q = ((word >> (8 * k)) & 0xFFu) ? sv[k] : make_uint4(0u, 0u, 0u, 0u);
-                            qs[4 * k] = q.x;
-                            qs[4 * k + 1] = q.y;
-                            qs[4 * k + 2] = q.z;
-                            qs[4 * k + 3] = q.w;
-                        }
-                        float wm = -INFINITY;
-                        int wi = 0;
-#pragma unroll
-                        for (int e = 0; e < 32; ++e) {
-                            const float x = (e & 1) ? bf16_hi(qs[e >> 1]) : bf16_lo(qs[e >> 1]);
-                            if (((word >> e) & 1u) && x > wm) {
-                                wm = x;
-                                wi = e;
-                            }
-                        }
-                        if constexpr (FOLD == kFoldMax) {
-                            if (wm > m) {
-                                m = wm;
-                                idx = t0 + wi;
-                            }
-                        } else {
-                            if (wm > m) {   // earlier words hold lower ids: equal maxima keep idx
-                                const float wL = wm * kLog2e;
-                                s = s == 0.0f ? 0.0f : s * ex2(mL - wL);
-                                m = wm;
-                                mL = wL;
-                                idx = t0 + wi;
-                            }
-                            float acc = 0.0f;
-#pragma unroll
-                            for (int e = 0; e < 32; ++e) {
-                                const float x = (e & 1) ? bf16_hi(qs[e >> 1]) : bf16_lo(qs[e >> 1]);
-                                acc += ((word >> e) & 1u) ? ex2(fmaf(x, kLog2e, -mL)) : 0.0f;
-                            }
-                            s += acc;
-                        }
-                    } else if (j < full_words) {
-                        const unsigned short* st =
-                            reinterpret_cast<const unsigned short*>(stage + (b % kStageDepth) * 128 + lane * 4);
-                        while (word) {
-                            const int e = __ffs(word) - 1;
-                            word &= word - 1;
-                            fold(__uint_as_float((uint32_t)st[e] << 16), t0 + e);
-                        }
-                    } else {   // the row's partial last word
-                        while (word) {
-                            const int e = __ffs(word) - 1;
-                            word &= word - 1;
-                            if (t0 + e < V) fold(logit_at<BF16>(lrow, t0 + e), t0 + e);
-                        }
-                    }
-                }
-                __syncwarp();   // this buffer is refilled by the next issue
-#pragma unroll
-                for (int k = 0; k < kStageDepth; ++k) mw[k] = mw[k + 1];
-                mw[kStageDepth] = mw_far;
-            }
-            cp_async_wait<0>();
-        } else {
-            for (int j = j0 + lane; j < j1; j += 32) {
-                uint32_t word = mask.word(mrow, j);
-                const int t0 = j * 32;
-                while (word) {
-                    const int e = __ffs(word) - 1;
-                    word &= word - 1;
-                    if (t0 + e < V) fold(logit_at<BF16>(lrow, t0 + e), t0 + e);
-                }
-            }
-        }
-        warp_merge(m, idx, s);
-        const long long first = ((long long)r * W) / per_cta;
-        const long long last = (row_end - 1) / per_cta;
-        const int nseg = (int)(last - first + 1);
-        bool is_last = false;
-        if (lane == 0) {
-            if (nseg == 1) {
-                argmax[orow] = m == -INFINITY ? -1 : idx;
-                if (lse) lse[orow] = m == -INFINITY ? -INFINITY : m + logf(s);
-            } else {
-                partials[(size_t)r * kMaxSegments + (blockIdx.x - first)] =
-                    make_float4(m, __int_as_float(idx), s, 0.f);
-                __threadfence();
-                is_last = atomicAdd(counters + r, 1u) == (unsigned)(nseg - 1);
-            }
-        }
-        if (__shfl_sync(0xffffffffu, is_last, 0)) {
-            // last CTA of the row: combine its segments
-            __threadfence();
-            m = -INFINITY;
-            s = 0.0f;
-            idx = INT_MAX;
-            for (int k = lane; k < nseg; k += 32) {
-                const float4 p = __ldcg(partials + (size_t)r * kMaxSegments + k);
-                acc_merge(m, idx, s, p.x, __float_as_int(p.y), p.z);
-            }
-            warp_merge(m, idx, s);
-            if (lane == 0) {
-                argmax[orow] = m == -INFINITY ? -1 : idx;
-                if (lse) lse[orow] = m == -INFINITY ? -INFINITY : m + logf(s);
-                counters[r] = 0u;   // ready for the next launch (stream-ordered)
-            }
-        }
-        u = seg_end;
-    }
-}
-
-// ---- the greedy / log-sum-exp pass over bf16 rows: a compacted gather -----
-// One CTA per row, its warps (up to 16) on consecutive segments of the row's
-// mask words, each segment cut into spans of 32 x kGatherSpan words (lane l
-// holds words l*kGatherSpan ... +kGatherSpan-1 of the span).  Each lane finds
-// its words' 16-byte logit vectors that hold an allowed token (a 32-bit map,
-// one bit per vector), a warp scan places the lanes' lists one after the
-// other in token order, and the warp then loads the listed vectors
-// kGatherRound per lane at once (entry k goes to lane k % 32, so each lane
-// still sees its tokens in increasing order) and folds them.  Zero words cost
-// a few instructions, every load of a span is independent, and a span costs
-// one memory latency whatever its density.  The warps' partials are merged in
-// shared memory.  Logit lines are not kept in L1, and in L2 only when a
-// log-prob pass reads them again (evict-last; otherwise evict-first).
-constexpr int kGatherMaxWarps = 16;   // warps per CTA (one row); two CTAs per SM
-constexpr int kGatherSpan = 8;     // mask words per lane per span (8192 tokens)
-constexpr int kGatherWarpSmem = 32 * kGatherSpan * (4 + 4 * 2);   // a span's words and its list
-constexpr int kGatherRound = 4;    // vectors per lane loaded together
-
-__device__ __forceinline__ uint64_t l2_policy(bool keep) {
-    uint64_t p;
-    if (keep)
-        asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;\n" : "=l"(p));
-    else
-        asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;\n" : "=l"(p));
-    return p;
-}
-
-__device__ __forceinline__ uint4 ld_once16(const void* p, uint64_t pol) {
-    uint4 v;
-    asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v4.u32 {%0, %1, %2, %3}, [%4], %5;\n"
-                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-                 : "l"(p), "l"(pol));
-    return v;
-}
-
-// bit b of the result: byte b of x is not zero
-__device__ __forceinline__ uint32_t nonzero_bytes(uint32_t x) {
-    x |= x >> 4;
-    x |= x >> 2;
-    x |= x >> 1;
-    return ((x & 0x01010101u) * 0x10204080u) >> 28;
-}
-
-// element e (0..7) of eight bf16 values
-__device__ __forceinline__ float bf16_of(const uint4& q, int e) {
-    const uint32_t h = (e & 4) ? ((e & 2) ? q.w : q.z) : ((e & 2) ? q.y : q.x);
-    return (e & 1) ? bf16_hi(h) : bf16_lo(h);
-}
-
-// chunk: words per warp, a multiple of kGatherSpan.  A sampling pass draws
-// row r with counter row row0 + (batch row of r).
-template <int FOLD>
-__global__ void __launch_bounds__(kGatherMaxWarps * 32, 2)
-    logits_gather_kernel(const void* __restrict__ logits, int64_t stride, const MaskRows mask, int V, int W, int B,
-                         int chunk, int32_t* __restrict__ argmax, float* __restrict__ lse, const SampleArgs sa,
-                         int row0, int keep_l2, const RowList list) {
-    constexpr int kSpanWords = 32 * kGatherSpan;
-    extern __shared__ __align__(16) unsigned char g_smem[];   // per warp: words, then list
-    __shared__ float4 s_part[kGatherMaxWarps];
-    pdl_wait();
-    pdl_trigger();
-    const int r = blockIdx.x;
-    if (r >= list.rows(B)) return;   // the whole CTA
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    uint32_t* sw = reinterpret_cast<uint32_t*>(g_smem + wid * kGatherWarpSmem);   // a span's mask words
-    uint16_t* lst = reinterpret_cast<uint16_t*>(sw + kSpanWords);                // its vectors, in token order
-    const uint64_t pol = l2_policy(keep_l2 != 0);
-    const int full_vec = V / 8;   // vectors that lie wholly inside the row
-    const int j0 = wid * chunk, j1 = min(W, j0 + chunk);
-    const uint32_t* mrow = mask.row(r, W, threadIdx.x == 0);
-    const int orow = list.row(r);
-    const char* lrow = reinterpret_cast<const char*>(logits) + (size_t)orow * stride * 2;
-    float m = -INFINITY, mL = -INFINITY, s = 0.0f;
-    int idx = INT_MAX;
-    int blk = -1;   // Philox block cached by gumbel()
-    uint4 rnd = make_uint4(0u, 0u, 0u, 0u);
-    // one allowed logit x of token t (t increasing within a lane)
-    auto fold1 = [&](float x, int t) {
-        if constexpr (FOLD == kFoldSample) {
-            const float sx = __fmul_rn(x, sa.inv_t);
-            if (__fadd_rn(sx, kGumbelMax) < m) return;
-            const float sc = __fadd_rn(sx, gumbel(sa, row0 + orow, t, blk, rnd));
-            if (sc > m) {
-                m = sc;
-                idx = t;
-            }
-        } else if constexpr (FOLD == kFoldMax) {
-            if (x > m) {
-                m = x;
-                idx = t;
-            }
-        } else {
-            acc_add(m, mL, idx, s, x, t);
-        }
-    };
-    for (int js = j0; js < j1; js += kSpanWords) {
-        uint32_t w[kGatherSpan];
-        const int jl = js + lane * kGatherSpan;
-        if (mrow && jl + kGatherSpan <= j1 && (reinterpret_cast<uintptr_t>(mrow + jl) & 15) == 0) {
-            const uint4 a = __ldg(reinterpret_cast<const uint4*>(mrow + jl));
-            const uint4 b = __ldg(reinterpret_cast<const uint4*>(mrow + jl) + 1);
-            w[0] = a.x, w[1] = a.y, w[2] = a.z, w[3] = a.w, w[4] = b.x, w[5] = b.y, w[6] = b.z, w[7] = b.w;
-        } else {
-#pragma unroll
-            for (int g = 0; g < kGatherSpan; ++g) w[g] = jl + g < j1 ? mask.word(mrow, jl + g) : 0u;
-        }
-        uint32_t nb = 0;   // bit 4g + b: byte b of word g holds an allowed token
-#pragma unroll
-        for (int g = 0; g < kGatherSpan; ++g) nb |= nonzero_bytes(w[g]) << (4 * g);
-        reinterpret_cast<uint4*>(sw)[2 * lane] = make_uint4(w[0], w[1], w[2], w[3]);
-        reinterpret_cast<uint4*>(sw)[2 * lane + 1] = make_uint4(w[4], w[5], w[6], w[7]);
-        const int c = __popc(nb);
-        int incl = c;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, incl, off);
-            if (lane >= off) incl += y;
-        }
-        const int T = __shfl_sync(0xffffffffu, incl, 31);
-        if (T == 0) continue;   // warp-uniform
-        int pos = incl - c;
-        while (nb) {
-            const int bit = __ffs(nb) - 1;
-            nb &= nb - 1;
-            lst[pos++] = (uint16_t)(lane * 4 * kGatherSpan + bit);
-        }
-        __syncwarp();
-        const int vbase = js * 4;   // the span's first vector in the row
-        // rounds of kGatherRound vectors per lane; the next round's loads are
-        // issued before this round is folded
-        int ent[kGatherRound];
-        uint4 q[kGatherRound];
-        auto load_round = [&](int k0, int(&en)[kGatherRound], uint4(&qq)[kGatherRound]) {
-#pragma unroll
-            for (int i = 0; i < kGatherRound; ++i) {
-                const int k = k0 + i * 32 + lane;
-                en[i] = k < T ? (int)lst[k] : -1;
-                const int vi = vbase + en[i];
-                qq[i] = (en[i] >= 0 && vi < full_vec) ? ld_once16(lrow + (size_t)vi * 16, pol)
-                                                     : make_uint4(0u, 0u, 0u, 0u);
-            }
-        };
-        load_round(0, ent, q);
-        for (int k0 = 0; k0 < T; k0 += 32 * kGatherRound) {
-            int ent_n[kGatherRound];
-            uint4 q_n[kGatherRound];
-            const bool more = k0 + 32 * kGatherRound < T;   // warp-uniform
-            if (more) load_round(k0 + 32 * kGatherRound, ent_n, q_n);
-#pragma unroll
-            for (int i = 0; i < kGatherRound; ++i) {
-                if (ent[i] < 0) continue;
-                const int vi = vbase + ent[i], t0 = vi * 8;
-                uint32_t bm = (sw[ent[i] >> 2] >> (8 * (ent[i] & 3))) & 0xFFu;
-                if (vi >= full_vec) {   // the row's last, partial vector: token by token
-                    while (bm) {
-                        const int e = __ffs(bm) - 1;
-                        bm &= bm - 1;
-                        if (t0 + e >= V) break;
-                        fold1(logit_at<true>(lrow, t0 + e), t0 + e);
-                    }
-                } else if (FOLD == kFoldSample) {
-                    while (bm) {
-                        const int e = __ffs(bm) - 1;
-                        bm &= bm - 1;
-                        fold1(bf16_of(q[i], e), t0 + e);
-                    }
-                } else if (__popc(bm) > 2) {
-                    // a dense vector: its allowed maximum (first on ties), one
-                    // rescale, then its sum, all eight lanes of it predicated;
-                    // earlier vectors hold lower ids, so an equal maximum keeps idx
-                    float xs[8];
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) xs[e] = ((bm >> e) & 1u) ? bf16_of(q[i], e) : -INFINITY;
-                    float vm = xs[0];
-                    int ve = 0;
-#pragma unroll
-                    for (int e = 1; e < 8; ++e)
-                        if (xs[e] > vm) {
-                            vm = xs[e];
-                            ve = e;
-                        }
-                    if constexpr (FOLD == kFoldMax) {
-                        if (vm > m) {
-                            m = vm;
-                            idx = t0 + ve;
-                        }
-                    } else {
-                        if (vm > m) {
-                            const float vL = vm * kLog2e;
-                            s = s == 0.0f ? 0.0f : s * ex2(mL - vL);
-                            m = vm;
-                            mL = vL;
-                            idx = t0 + ve;
-                        }
-                        float acc = 0.0f;
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) acc += ((bm >> e) & 1u) ? ex2(fmaf(xs[e], kLog2e, -mL)) : 0.0f;
-                        s += acc;
-                    }
-                } else {
-                    while (bm) {
-                        const int e = __ffs(bm) - 1;
-                        bm &= bm - 1;
-                        fold1(bf16_of(q[i], e), t0 + e);
-                    }
-                }
-            }
-            if (more) {
-#pragma unroll
-                for (int i = 0; i < kGatherRound; ++i) {
-                    ent[i] = ent_n[i];
-                    q[i] = q_n[i];
-                }
-            }
-        }
-        __syncwarp();   // the span buffers are rewritten by the next span
-    }
-    warp_merge(m, idx, s);
-    if (lane == 0) s_part[wid] = make_float4(m, __int_as_float(idx), s, 0.f);
-    __syncthreads();
-    if (wid == 0) {
-        m = -INFINITY;
-        s = 0.0f;
-        idx = INT_MAX;
-        if (lane < nwarps) {
-            const float4 p = s_part[lane];
-            m = p.x;
-            idx = __float_as_int(p.y);
-            s = p.z;
-        }
-        warp_merge(m, idx, s);
-        if (lane == 0) {
-            argmax[orow] = m == -INFINITY ? -1 : idx;
-            if (lse) lse[orow] = m == -INFINITY ? -INFINITY : m + logf(s);
-        }
-    }
-}
-
-// logprob[t] = logit[t] - lse for allowed t, -inf otherwise.  VEC (bf16 rows on
-// 16-byte boundaries, V % 4 == 0): a thread takes 16 consecutive tokens when
-// V % 16 == 0 (32 bytes of logits read unconditionally, four float4 stores),
-// else 4 (their 8 bytes read only when one is allowed, one float4 store);
-// grid-stride over the batch's groups.  Otherwise one mask word (32 tokens) per
-// thread, one token at a time.
-template <bool BF16, bool VEC>
-__global__ void __launch_bounds__(kLogitThreads)
-    logprobs_kernel(const void* __restrict__ logits, int64_t stride, const MaskRows mask, int V, int W,
-                    int B, const float* __restrict__ lse, float* __restrict__ out, int wide) {
-    pdl_wait();
-    pdl_trigger();
-    if (VEC && BF16 && V % 16 == 0) {
-        // 16 tokens per thread: two 16-byte logit loads and the mask half-word,
-        // all independent, then four float4 stores
-        const int ng = V / 16;
-        const long long N = (long long)B * ng;
-        for (long long u = (long long)blockIdx.x * kLogitThreads + threadIdx.x; u < N;
-             u += (long long)gridDim.x * kLogitThreads) {
-            const int r = (int)(u / ng), g = (int)(u - (long long)r * ng);
-            const uint32_t* mrow = mask.row(r, W, false);
-            const char* lrow = reinterpret_cast<const char*>(logits) + (size_t)r * stride * 2;
-            const uint4* src = reinterpret_cast<const uint4*>(lrow) + 2 * (size_t)g;
-            uint32_t ws[8];
-            if (wide) {   // one 32-byte load (32-byte aligned rows)
-                asm volatile("ld.global.cs.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                             : "=r"(ws[0]), "=r"(ws[1]), "=r"(ws[2]), "=r"(ws[3]), "=r"(ws[4]), "=r"(ws[5]),
-                               "=r"(ws[6]), "=r"(ws[7])
-                             : "l"(src));
-            } else {
-                const uint4 a = __ldcs(src), c = __ldcs(src + 1);
-                ws[0] = a.x; ws[1] = a.y; ws[2] = a.z; ws[3] = a.w;
-                ws[4] = c.x; ws[5] = c.y; ws[6] = c.z; ws[7] = c.w;
-            }
-            const uint32_t bits = (mask.word(mrow, g >> 1) >> (16 * (g & 1))) & 0xFFFFu;
-            const float l = __ldg(lse + r);
-            float o[16];
-#pragma unroll
-            for (int e = 0; e < 16; ++e) {
-                const float x = (e & 1) ? bf16_hi(ws[e >> 1]) : bf16_lo(ws[e >> 1]);
-                o[e] = ((bits >> e) & 1u) ? x - l : -INFINITY;
-            }
-            float* dst = out + (size_t)r * V + 16 * (size_t)g;
-            if (wide) {   // two 32-byte stores
-#pragma unroll
-                for (int h = 0; h < 2; ++h)
-                    asm volatile("st.global.cs.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(dst + 8 * h),
-                                 "f"(o[8 * h]), "f"(o[8 * h + 1]), "f"(o[8 * h + 2]), "f"(o[8 * h + 3]),
-                                 "f"(o[8 * h + 4]), "f"(o[8 * h + 5]), "f"(o[8 * h + 6]), "f"(o[8 * h + 7])
-                                 : "memory");
-            } else {
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    __stcs(reinterpret_cast<float4*>(dst) + q, make_float4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]));
-            }
-        }
-    } else if constexpr (VEC && BF16) {
-        const int nq = V / 4;
-        const long long N = (long long)B * nq;
-        for (long long u = (long long)blockIdx.x * kLogitThreads + threadIdx.x; u < N;
-             u += (long long)gridDim.x * kLogitThreads) {
-            const int r = (int)(u / nq), qd = (int)(u - (long long)r * nq);
-            const uint32_t* mrow = mask.row(r, W, false);
-            const uint32_t nib = (mask.word(mrow, qd >> 3) >> (4 * (qd & 7))) & 0xFu;
-            float4 o = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-            if (nib) {
-                const char* lrow = reinterpret_cast<const char*>(logits) + (size_t)r * stride * 2;
-                const uint2 v = __ldcs(reinterpret_cast<const uint2*>(lrow) + qd);
-                const float l = __ldg(lse + r);
-                if (nib & 1u) o.x = bf16_lo(v.x) - l;
-                if (nib & 2u) o.y = bf16_hi(v.x) - l;
-                if (nib & 4u) o.z = bf16_lo(v.y) - l;
-                if (nib & 8u) o.w = bf16_hi(v.y) - l;
-            }
-            __stcs(reinterpret_cast<float4*>(out + (size_t)r * V) + qd, o);
-        }
-    } else {
-        const long long N = (long long)B * W;
-        for (long long u = (long long)blockIdx.x * kLogitThreads + threadIdx.x; u < N;
-             u += (long long)gridDim.x * kLogitThreads) {
-            const int r = (int)(u / W), j = (int)(u - (long long)r * W);
-            const uint32_t* mrow = mask.row(r, W, false);
-            const uint32_t word = mask.word(mrow, j);
-            const char* lrow = reinterpret_cast<const char*>(logits) + (size_t)r * stride * (BF16 ? 2 : 4);
-            float* orow = out + (size_t)r * V + (size_t)j * 32;
-            const float l = __ldg(lse + r);
-            for (int e = 0; e < 32 && j * 32 + e < V; ++e)
-                orow[e] = ((word >> e) & 1u) ? logit_at<BF16>(lrow, j * 32 + e) - l : -INFINITY;
-        }
-    }
-}
-
-// ---------------------------------------------------------------------------
 // advance
 // ---------------------------------------------------------------------------
 template <bool STACK, int MODE>
@@ -1588,140 +923,6 @@ cudaError_t launch_step_s(const StepView& v, const LaunchEnv& env, int mode, con
     }
 }
 
-// Resident CTAs per SM of one kernel, cached per (kernel, device).
-int occupancy(const void* kern, int threads) {
-    struct Entry {
-        const void* fn;
-        int dev, n;
-    };
-    static Entry cache[64];
-    static int used = 0;
-    static std::mutex mu;   // handles on different host threads share the cache
-    int dev = 0;
-    cudaGetDevice(&dev);
-    {
-        std::lock_guard<std::mutex> lk(mu);
-        for (int i = 0; i < used; i++)
-            if (cache[i].fn == kern && cache[i].dev == dev) return cache[i].n;
-    }
-    int n = 1;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, threads, 0) != cudaSuccess || n < 1) {
-        cudaGetLastError();
-        n = 1;
-    }
-    std::lock_guard<std::mutex> lk(mu);
-    if (used < 64) cache[used++] = Entry{kern, dev, n};
-    return n;
-}
-
-// the gather kernels' dynamic shared memory passes the default 48 KB at 16
-// warps: the limit is raised once per device and fold
-template <int FOLD>
-cudaError_t gather_smem_ready() {
-    static bool configured[kMaxDevices] = {false};   // one array per fold
-    static std::mutex mu;
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return cudaGetLastError();
-    if (dev >= kMaxDevices) dev = kMaxDevices - 1;
-    std::lock_guard<std::mutex> lk(mu);
-    if (!configured[dev]) {
-        cudaError_t e = cudaFuncSetAttribute(logits_gather_kernel<FOLD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             kGatherMaxWarps * kGatherWarpSmem);
-        if (e != cudaSuccess) return e;
-        configured[dev] = true;
-    }
-    return cudaSuccess;
-}
-
-}  // namespace
-
-cudaError_t prepare_logits_kernels() {
-    cudaError_t e = gather_smem_ready<kFoldLse>();
-    if (e == cudaSuccess) e = gather_smem_ready<kFoldMax>();
-    if (e == cudaSuccess) e = gather_smem_ready<kFoldSample>();
-    return e;
-}
-
-namespace {
-
-template <bool BF16, bool STAGE>
-cudaError_t launch_logits_t(const LaunchEnv& env, const void* logits, int32_t batch, int64_t stride, int32_t V,
-                            const MaskRows& mask, int32_t* argmax, float* lse, float* logprobs, float4* partials,
-                            uint32_t* counters, float* lse_tmp, bool out_vec, const SampleArgs* sample,
-                            const RowList& list, cudaStream_t st) {
-    const int W = (V + 31) / 32;
-    const size_t esz = BF16 ? 2 : 4;
-    const SampleArgs sa = sample ? *sample : SampleArgs{0u, 0u, 0u, 0u, 1.0f};
-    auto reduce = sample ? logits_reduce_kernel<BF16, STAGE, kFoldSample>
-                         : (lse || logprobs) ? logits_reduce_kernel<BF16, STAGE, kFoldLse>
-                                             : logits_reduce_kernel<BF16, STAGE, kFoldMax>;
-    for (int32_t r0 = 0; r0 < batch; r0 += kMaxLogitRows) {
-        const int rows = min(kMaxLogitRows, batch - r0);
-        // a row list addresses batch rows itself: logits and outputs stay unshifted
-        const size_t shift = list.ids ? 0 : (size_t)r0;
-        const void* lg = reinterpret_cast<const char*>(logits) + shift * stride * esz;
-        MaskRows mk = mask;
-        if (mk.row_state) mk.row_state += r0;
-        else if (mk.base) mk.base += (size_t)r0 * W;
-        RowList lst = list;
-        lst.base = r0;
-        float* lse_rows = lse ? lse + shift : (logprobs ? lse_tmp : nullptr);
-        const long long N = (long long)rows * W;
-        // at least 4 batches of 32 words per warp; a pass too small to fill the
-        // GPU that way gives each warp fewer (down to one batch) instead
-        const int slots = env.num_sms * occupancy((const void*)reduce, kReduceThreads);
-        int grid = (int)std::min<long long>((long long)slots, (N + 127) / 128);
-        if (grid < slots) grid = (int)std::min<long long>((long long)slots, (N + 31) / 32);
-        grid = max(grid, 1);
-        long long per_cta = (N + grid - 1) / grid;
-        per_cta = std::max<long long>(per_cta, ((long long)W + kMaxSegments - 3) / (kMaxSegments - 2));
-        grid = (int)((N + per_cta - 1) / per_cta);
-        cudaError_t e0;
-        // the gather takes one CTA per row: used when the rows alone fill the
-        // SMs (with fewer rows the flat split over rows x words keeps more
-        // warps busy)
-        if (BF16 && STAGE && rows > env.num_sms) {
-            auto gather = sample ? logits_gather_kernel<kFoldSample>
-                                 : (lse || logprobs) ? logits_gather_kernel<kFoldLse> : logits_gather_kernel<kFoldMax>;
-            // a warp per span of the row, at most kGatherMaxWarps (two CTAs per
-            // SM); a warp's words rounded up to whole lanes
-            const int nwarps =
-                std::max(1, std::min(kGatherMaxWarps, (W + 32 * kGatherSpan - 1) / (32 * kGatherSpan)));
-            int chunk = (W + nwarps - 1) / nwarps;
-            chunk = (chunk + kGatherSpan - 1) / kGatherSpan * kGatherSpan;
-            const int smem = nwarps * kGatherWarpSmem;
-            if (cudaError_t e = sample ? gather_smem_ready<kFoldSample>()
-                                       : (lse || logprobs) ? gather_smem_ready<kFoldLse>() : gather_smem_ready<kFoldMax>();
-                e != cudaSuccess)
-                return e;
-            e0 = launch_pdl(gather, dim3((unsigned)rows), dim3(nwarps * 32), (size_t)smem, st, lg, stride, mk, V, W,
-                            rows, chunk, argmax + shift, lse_rows, sa, (int)shift, logprobs ? 1 : 0, lst);
-        } else {
-            // a sampling pass draws row r of this chunk with counter row r0 + r
-            e0 = launch_pdl(reduce, dim3(grid), dim3(kReduceThreads), 0, st, lg, stride, mk, V, W, rows, per_cta,
-                            partials, counters, argmax + shift, lse_rows, sa, (int)shift, lst);
-        }
-        if (e0 != cudaSuccess) return e0;
-        if (logprobs) {
-            const long long n_items = (out_vec && STAGE) ? (long long)rows * (V % 16 == 0 ? V / 16 : V / 4) : N;
-            int g2 = env.num_sms * occupancy((const void*)logprobs_kernel<BF16, true>, kLogitThreads);
-            g2 = (int)std::max<long long>(1, std::min<long long>((long long)g2,
-                                                                 (n_items + kLogitThreads - 1) / kLogitThreads));
-            // 32-byte vector loads and stores where rows start on 32-byte boundaries
-            float* lp = logprobs + (size_t)r0 * V;
-            const int wide = (reinterpret_cast<uintptr_t>(lg) % 32 == 0) && ((size_t)stride * esz) % 32 == 0 &&
-                             (reinterpret_cast<uintptr_t>(lp) % 32 == 0) && V % 16 == 0;
-            cudaError_t e1 = (out_vec && STAGE)
-                                 ? launch_pdl(logprobs_kernel<BF16, true>, dim3(g2), dim3(kLogitThreads), 0, st, lg,
-                                              stride, mk, V, W, rows, (const float*)lse_rows, lp, wide)
-                                 : launch_pdl(logprobs_kernel<BF16, false>, dim3(g2), dim3(kLogitThreads), 0, st, lg,
-                                              stride, mk, V, W, rows, (const float*)lse_rows, lp, 0);
-            if (e1 != cudaSuccess) return e1;
-        }
-    }
-    return cudaSuccess;
-}
-
 }  // namespace
 
 int64_t table_smem_bytes(const StepView& v, bool stack, int mode) {
@@ -1810,60 +1011,6 @@ cudaError_t launch_fused_combine(const StepView& v, bool stack, int mode, const 
                           batch, n_windows, argmax, lse, adv);
     if (stack) return launch_combine_adv<true>(v, mode, part, batch, n_windows, argmax, lse, adv, grid, st);
     return launch_combine_adv<false>(v, mode, part, batch, n_windows, argmax, lse, adv, grid, st);
-}
-
-cudaError_t launch_logprobs_bf16(const LaunchEnv& env, const void* logits, int32_t batch, int64_t row_stride,
-                                 int32_t V, const uint32_t* mask, const float* lse, float* logprobs, cudaStream_t st) {
-    const int W = (V + 31) / 32;
-    const bool out_vec = (reinterpret_cast<uintptr_t>(logprobs) % 16 == 0) && (V % 4 == 0);
-    for (int32_t r0 = 0; r0 < batch; r0 += kMaxLogitRows) {
-        const int rows = min(kMaxLogitRows, batch - r0);
-        const void* lg = reinterpret_cast<const char*>(logits) + (size_t)r0 * row_stride * 2;
-        const MaskRows mk{mask + (size_t)r0 * W, nullptr, 0, nullptr};
-        const long long n_items = out_vec ? (long long)rows * (V % 16 == 0 ? V / 16 : V / 4) : (long long)rows * W;
-        int g = env.num_sms * occupancy((const void*)logprobs_kernel<true, true>, kLogitThreads);
-        g = (int)std::max<long long>(1, std::min<long long>((long long)g, (n_items + kLogitThreads - 1) / kLogitThreads));
-        float* lp = logprobs + (size_t)r0 * V;
-        const int wide = (reinterpret_cast<uintptr_t>(lg) % 32 == 0) && ((size_t)row_stride * 2) % 32 == 0 &&
-                         (reinterpret_cast<uintptr_t>(lp) % 32 == 0) && V % 16 == 0;
-        cudaError_t e = out_vec ? launch_pdl(logprobs_kernel<true, true>, dim3(g), dim3(kLogitThreads), 0, st, lg,
-                                             row_stride, mk, V, W, rows, lse + r0, lp, wide)
-                                : launch_pdl(logprobs_kernel<true, false>, dim3(g), dim3(kLogitThreads), 0, st, lg,
-                                             row_stride, mk, V, W, rows, lse + r0, lp, 0);
-        if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
-}
-
-cudaError_t launch_mask_logits(const LaunchEnv& env, const void* logits, int dtype, int32_t batch,
-                               int64_t row_stride, int32_t V, const uint32_t* mask, int32_t* argmax, float* lse,
-                               float* logprobs, float4* partials, uint32_t* counters, float* lse_tmp,
-                               cudaStream_t st, const int32_t* row_state, int32_t Q, uint32_t* err,
-                               const SampleArgs* sample, const int32_t* row_ids, const int32_t* row_count) {
-    const MaskRows mr{mask, row_state, Q, err};
-    const RowList list{row_ids, row_count, 0};
-    const bool bf16 = dtype == DOMINO_DTYPE_BF16;
-    const bool out_vec = logprobs && (reinterpret_cast<uintptr_t>(logprobs) % 16 == 0) && (V % 4 == 0);
-    if (bf16) {
-        const bool stage = (reinterpret_cast<uintptr_t>(logits) % 16 == 0) && ((size_t)row_stride * 2) % 16 == 0;
-        if (stage)
-            return launch_logits_t<true, true>(env, logits, batch, row_stride, V, mr, argmax, lse, logprobs,
-                                               partials, counters, lse_tmp, out_vec, sample, list, st);
-        return launch_logits_t<true, false>(env, logits, batch, row_stride, V, mr, argmax, lse, logprobs, partials,
-                                            counters, lse_tmp, out_vec, sample, list, st);
-    }
-    return launch_logits_t<false, false>(env, logits, batch, row_stride, V, mr, argmax, lse, logprobs, partials,
-                                         counters, lse_tmp, out_vec, sample, list, st);
-}
-
-cudaError_t launch_mask_sample(const LaunchEnv& env, const void* logits, int dtype, int32_t batch,
-                               int64_t row_stride, int32_t V, const uint32_t* mask, float temperature,
-                               uint64_t seed, uint64_t offset, int32_t* tokens, float4* partials,
-                               uint32_t* counters, cudaStream_t st) {
-    const SampleArgs sa{(uint32_t)seed, (uint32_t)(seed >> 32), (uint32_t)offset, (uint32_t)(offset >> 32),
-                        1.0f / temperature};   // one correctly rounded fp32 division
-    return launch_mask_logits(env, logits, dtype, batch, row_stride, V, mask, tokens, nullptr, nullptr, partials,
-                              counters, nullptr, st, nullptr, 0, nullptr, &sa);
 }
 
 // The table image of `mode` staged in shared memory (the step kernel's image:
@@ -1995,90 +1142,3 @@ cudaError_t launch_spec_accept(const int32_t* proposals, const int32_t* n_prop, 
 
 }  // namespace domino
 
-// ---------------------------------------------------------------------------
-// domino_mask_logits_noalloc: the masked argmax / log-sum-exp for callers that
-// cannot allocate device memory.  Its scratch (per-row partials, tickets and a
-// temporary lse) is the fixed array below, part of this library's image, so
-// every GPU that loads the library holds it until the process exits.
-// ---------------------------------------------------------------------------
-namespace {
-
-constexpr int kNoAllocMaxRows = 512;
-constexpr int kNoAllocMaxDevices = 64;
-constexpr size_t kNoAllocPartialsBytes = sizeof(float4) * (size_t)kNoAllocMaxRows * domino::kMaxSegments;
-constexpr size_t kNoAllocCountersBytes = sizeof(uint32_t) * (size_t)kNoAllocMaxRows;
-constexpr size_t kNoAllocScratchBytes = kNoAllocPartialsBytes + kNoAllocCountersBytes + sizeof(float) * kNoAllocMaxRows;
-
-static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];   // 516 KiB
-
-struct NoAllocDevice {
-    bool ready;
-    unsigned char* scratch;   // device address of g_noalloc_scratch on this device
-    int num_sms;
-};
-NoAllocDevice g_noalloc_dev[kNoAllocMaxDevices];
-std::mutex g_noalloc_mu;
-
-// Once per device, with that device current: the array's device address.
-int noalloc_setup(int dev, NoAllocDevice* out) {
-    std::lock_guard<std::mutex> lock(g_noalloc_mu);
-    NoAllocDevice& d = g_noalloc_dev[dev];
-    if (!d.ready) {
-        void* p = nullptr;
-        if (cudaGetSymbolAddress(&p, g_noalloc_scratch) != cudaSuccess || p == nullptr) {
-            cudaGetLastError();
-            return DOMINO_E_CUDA;
-        }
-        int sms = 0;
-        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) {
-            cudaGetLastError();
-            return DOMINO_E_CUDA;
-        }
-        if (domino::prepare_logits_kernels() != cudaSuccess) {
-            cudaGetLastError();
-            return DOMINO_E_CUDA;
-        }
-        d.scratch = static_cast<unsigned char*>(p);
-        d.num_sms = sms;
-        d.ready = true;
-    }
-    *out = d;
-    return DOMINO_OK;
-}
-
-}  // namespace
-
-extern "C" int domino_mask_logits_noalloc(const void* logits_dev, int32_t dtype, int32_t batch, int32_t n_tokens,
-                                          int64_t row_stride_elems, const uint32_t* mask_dev, int32_t* argmax_dev,
-                                          float* lse_dev, float* logprobs_dev, void* stream) {
-    if (dtype != DOMINO_DTYPE_F32 && dtype != DOMINO_DTYPE_BF16) return DOMINO_E_INVALID_ARG;
-    if (batch < 0 || batch > kNoAllocMaxRows || n_tokens < 1 || n_tokens > (1 << 24) || row_stride_elems < n_tokens)
-        return DOMINO_E_INVALID_ARG;
-    if (batch == 0) return DOMINO_OK;
-    if (!logits_dev || !mask_dev || !argmax_dev) return DOMINO_E_INVALID_ARG;
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) {
-        cudaGetLastError();
-        return DOMINO_E_CUDA;
-    }
-    if (dev < 0 || dev >= kNoAllocMaxDevices) return DOMINO_E_UNSUPPORTED;
-    NoAllocDevice d{};
-    int rc = noalloc_setup(dev, &d);
-    if (rc != DOMINO_OK) return rc;
-    float4* partials = reinterpret_cast<float4*>(d.scratch);
-    uint32_t* counters = reinterpret_cast<uint32_t*>(d.scratch + kNoAllocPartialsBytes);
-    float* lse_tmp = reinterpret_cast<float*>(d.scratch + kNoAllocPartialsBytes + kNoAllocCountersBytes);
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    // the tickets must start at zero; the array keeps whatever the last call left
-    cudaError_t e = cudaMemsetAsync(counters, 0, sizeof(uint32_t) * (size_t)batch, st);
-    if (e == cudaSuccess) {
-        domino::LaunchEnv env{d.num_sms, 0};
-        e = domino::launch_mask_logits(env, logits_dev, dtype, batch, row_stride_elems, n_tokens, mask_dev,
-                                       argmax_dev, lse_dev, logprobs_dev, partials, counters, lse_tmp, st);
-    }
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        return DOMINO_E_CUDA;
-    }
-    return DOMINO_OK;
-}

@@ -1,0 +1,198 @@
+"""The decode of one row by a CTA or a cluster of CTAs (decode.cuh) against
+the oracle: bf16 and fp32 rows at every alignment, vocabularies around the
+vector, word and segment sizes, 1 to 8 CTAs per row, sparse and dense masks,
+masks with bits past V, rows with nothing allowed, ties, infinite logits; the
+Gumbel-max draw over the same rows; and the mask step with the decode and the
+update folded in, over unaligned rows.  Tokens bit-exact.
+
+Tolerance of lse and log-probabilities: a lane's sequential fp32 sum of at most
+1024 terms errs by at most 1024 * 2^-24 = 6.1e-5 relative, a term's exponent
+(below 64 in log2) by 64 * 2^-24 * ln 2 = 2.7e-6 and ex2 by 2^-22, so
+ln(sum) errs by less than 6.5e-5, and its rounding below 32 by 2^-19 = 2e-6:
+1e-4 in all.  Output buffers start as 0xAB bytes (tests/poison.py)."""
+import functools
+import os
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+from paper_2403_06988_gb300 import Domino, synth  # noqa: E402
+from paper_2403_06988_gb300 import _binding as B  # noqa: E402
+import poison  # noqa: E402
+from poison import assert_exact, assert_no_poison  # noqa: E402
+
+NT = os.cpu_count() or 1
+TOL = 1e-4
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2403_06988_gb300 import build
+    build.build()
+
+
+@functools.lru_cache(maxsize=2)
+def handle(V):
+    toks = [b"%d" % i for i in range(V - 1)] + [b""]
+    d = Domino(0)
+    d.load_vocab(synth.Vocab.from_tokens(toks, eos_id=V - 1))
+    return d
+
+
+def rows(dt, batch, V, offset, pad, seed, sigma=3.0):
+    """(the oracle's contiguous [batch][V] logits, device buffer, address of row 0, row stride): rows of V + pad
+    elements, the first one `offset` elements past an allocation."""
+    rng = np.random.default_rng(seed)
+    x = (rng.standard_normal((batch, V + pad)) * sigma).astype(np.float32)
+    x = x if dt == B.DTYPE_F32 else synth.f32_to_bf16_bits(x)
+    buf = np.zeros(offset + batch * (V + pad), x.dtype)
+    buf[offset:] = x.reshape(-1)
+    t = torch.from_numpy(buf.view(np.int16) if dt == B.DTYPE_BF16 else buf).cuda()
+    return np.ascontiguousarray(x[:, :V]), t, t.data_ptr() + offset * x.dtype.itemsize, V + pad
+
+
+def masks(batch, V, share, seed):
+    rng = np.random.default_rng([seed, 1])
+    W = (V + 31) // 32
+    bits = rng.random((batch, W * 32)) < share * (0.2 + 1.6 * rng.random((batch, 1)))
+    if batch > 2:
+        bits[1] = False
+    return np.packbits(bits.reshape(batch, W, 32), axis=2, bitorder="little").view(np.uint32).reshape(batch, W)
+
+
+def check(x, m, V, arg, lse, lp):
+    import oracle
+    clean = m.copy()
+    if V % 32:
+        clean[:, -1] &= (1 << (V % 32)) - 1
+    a_o, l_o, p_o = oracle.mask_logits(x, clean, n_tokens=V, want_logprobs=lp is not None, n_threads=NT)
+    assert_exact(arg, np.asarray(a_o, np.int32), "argmax")
+    for name, got, want in (("lse", lse, l_o), ("log-probs", lp, p_o)):
+        if got is None:
+            continue
+        assert_no_poison(got, name)
+        g = got.cpu().numpy()
+        fin = np.isfinite(want)
+        assert (np.isfinite(g) == fin).all(), name
+        assert np.abs(g[fin].astype(np.float64) - want[fin]).max(initial=0) < TOL, name
+
+
+@pytest.mark.parametrize("dt", [B.DTYPE_BF16, B.DTYPE_F32])
+@pytest.mark.parametrize("V,batch,offset,pad", [(1, 1, 0, 0), (7, 3, 1, 0), (33, 5, 3, 0), (1000, 1, 0, 0),
+                                                (4099, 2, 5, 0), (8191, 24, 7, 0), (50001, 3, 2, 6), (32000, 64, 0, 0),
+                                                (32001, 80, 0, 0), (131105, 9, 0, 7), (140000, 160, 1, 0),
+                                                (300007, 2, 4, 1)])
+@pytest.mark.parametrize("share", [0.003, 0.6])
+def test_rows_of_any_alignment(dt, V, batch, offset, pad, share):
+    import oracle
+    x, t, ptr, stride = rows(dt, batch, V, offset, pad, V + batch)
+    m = masks(batch, V, share, V)
+    d = handle(V)
+    mt = torch.from_numpy(m.view(np.int32)).cuda()
+    for want_lp in (False, True):
+        arg, lse = poison.empty(batch, torch.int32), poison.empty(batch, torch.float32)
+        lp = poison.empty((batch, V), torch.float32) if want_lp else None
+        B.domino_mask_logits(d.h, ptr, dt, batch, stride, mt, arg, lse, lp)
+        check(x, m, V, arg, lse, lp)
+    arg = poison.empty(batch, torch.int32)
+    B.domino_mask_logits(d.h, ptr, dt, batch, stride, mt, arg)
+    check(x, m, V, arg, None, None)
+    tok = poison.empty(batch, torch.int32)
+    B.domino_mask_sample(d.h, ptr, dt, batch, stride, mt, 0.7, 11, 5, tok)
+    clean = m.copy()
+    if V % 32:
+        clean[:, -1] &= (1 << (V % 32)) - 1
+    assert_exact(tok, np.asarray(oracle.mask_sample(x, clean, 0.7, 11, 5), np.int32), "drawn token")
+    del t
+
+
+@pytest.mark.parametrize("temperature", [1e-3, 0.05, 40.0])
+def test_draws_at_extreme_temperatures(temperature):
+    """Scores of up to about 1e4: the rounding of the bound on a variate must not drop the winner."""
+    import oracle
+    V, batch = 5003, 6
+    x, t, ptr, stride = rows(B.DTYPE_F32, batch, V, 0, 0, 3, sigma=10.0)
+    m = masks(batch, V, 0.7, 3)
+    m[:, -1] &= (1 << (V % 32)) - 1
+    tok = poison.empty(batch, torch.int32)
+    B.domino_mask_sample(handle(V).h, ptr, B.DTYPE_F32, batch, stride, torch.from_numpy(m.view(np.int32)).cuda(),
+                         temperature, 2, 9, tok)
+    assert_exact(tok, np.asarray(oracle.mask_sample(x, m, temperature, 2, 9), np.int32), "drawn token")
+    del t
+
+
+@pytest.mark.parametrize("dt", [B.DTYPE_BF16, B.DTYPE_F32])
+def test_infinite_logits(dt):
+    """-inf logits never win and add nothing; a row of only -inf allowed logits decodes as nothing allowed; +inf wins."""
+    V, batch = 2001, 4
+    x, _, _, _ = rows(dt, batch, V, 0, 0, 21)
+    f = x if dt == B.DTYPE_F32 else synth.bf16_bits_to_f32(x)
+    f = f.copy()
+    m = masks(batch, V, 0.5, 4)
+    m[1] = m[0]
+    m[:, -1] &= (1 << (V % 32)) - 1
+    bits = np.unpackbits(m.view(np.uint8), bitorder="little").reshape(batch, -1)[:, :V].astype(bool)
+    f[0, ::3] = -np.inf
+    f[1] = -np.inf
+    f[2, 900] = np.inf
+    bits[2, 900] = True
+    m[2, 900 // 32] |= np.uint32(1 << (900 % 32))
+    raw = f if dt == B.DTYPE_F32 else synth.f32_to_bf16_bits(f)
+    t = torch.from_numpy(raw.view(np.int16) if dt == B.DTYPE_BF16 else raw).cuda()
+    arg, lse = poison.empty(batch, torch.int32), poison.empty(batch, torch.float32)
+    B.domino_mask_logits(handle(V).h, t.data_ptr(), dt, batch, V, torch.from_numpy(m.view(np.int32)).cuda(), arg, lse)
+    for b in range(batch):
+        v = np.where(bits[b], f[b].astype(np.float64), -np.inf)
+        if b == 1:
+            assert arg[b] == -1 and lse[b] == -np.inf
+        elif b == 2:
+            assert arg[b] == 900 and lse[b] == np.inf
+        else:
+            assert arg[b] == int(np.argmax(v))
+            assert abs(float(lse[b]) - np.logaddexp.reduce(v[np.isfinite(v)])) < TOL
+
+
+@pytest.mark.parametrize("dt,offset,pad", [(B.DTYPE_BF16, 0, 5), (B.DTYPE_BF16, 3, 0), (B.DTYPE_F32, 0, 0),
+                                           (B.DTYPE_F32, 1, 2)])
+@pytest.mark.parametrize("grammar,batch", [("json", 60), ("json", 170), ("sparse", 5), ("sparse", 200)])
+def test_whole_step_in_one_kernel(dt, offset, pad, grammar, batch):
+    import oracle
+    rng = np.random.default_rng(batch)
+    V = 19997
+    v = synth.random_vocab(rng, V, bytes(range(256)), synth.geometric_lengths(4.0, 32), synth._mixed_bytes)
+    if grammar == "json":
+        a, _ = synth.json_pda(rng)
+        cfg = [synth.random_pda_walk(a, rng, int(rng.integers(0, 33))) for _ in range(30)]
+        pick = rng.integers(0, len(cfg), batch)
+        states = np.array([cfg[i][0] for i in pick], np.int32)
+        stacks = np.array([synth.pack_stack(cfg[i][1]) for i in pick], np.uint64)
+    else:
+        a = synth.random_sparse_dfa(rng, 300)
+        states, stacks = rng.integers(0, 300, batch).astype(np.int32), None
+    d = Domino.from_parts(a, v, device=0)
+    P = oracle.Problem.from_parts(a, v)
+    x, t, ptr, stride = rows(dt, batch, V, offset, pad, 5)
+    st = torch.from_numpy(states).cuda()
+    sk = None if stacks is None else torch.from_numpy(stacks.view(np.int64)).cuda()
+    mask = poison.empty((batch, d.info()["n_words"]), torch.int32)
+    arg, lse = poison.empty(batch, torch.int32), poison.empty(batch, torch.float32)
+    lp = poison.empty((batch, V), torch.float32)
+    B.domino_step_decode(d.h, st, sk, batch, ptr, dt, stride, mask, arg, lse, lp, st, sk)
+    m_o, _, bad = P.step_mask(states, stacks, n_threads=NT)
+    assert bad == 0
+    assert_exact(mask, m_o, "mask")
+    check(x, m_o, V, arg, lse, lp)
+    a_o, _, _ = oracle.mask_logits(x, m_o, n_tokens=V, n_threads=NT)
+    s_o, k_o, _ = P.advance(states, stacks, a_o, a.start)
+    assert_exact(st, s_o, "states")
+    if sk is not None:
+        assert_exact(sk, k_o, "stacks")
+    assert d.device_error() == 0
+    d.close()
+    del t
