@@ -123,6 +123,7 @@ struct RowTree {
     const uint32_t* loopbits;   // [loop sets][W]
     const uint8_t* keeps;       // [loop sets][n_dtok]: position after the last class outside the set (at most 255)
     const uint2* xrange;        // [loop sets][n_nodes]: {first exit below | depth << 24 (255: or more), end exit}
+    const uint8_t* trec;        // [V][32]: {token length (255: or more), its first 31 classes}
     const uint2* exits;         // {node, its class | depth of the nearest exit above (at most 255) << 8}
     int32_t srec_stride, n_nodes, n_dtok, n_loops;
     int32_t reserve;            // pool entries a depth-first walk of any node can add
@@ -171,8 +172,8 @@ cudaError_t launch_row_step(const StepView& v, const RowTree& t, const LaunchEnv
 // outputs may alias states / stacks.
 cudaError_t launch_row_decode(const StepView& v, const RowTree& t, const LaunchEnv& env, bool stack,
                               const int32_t* states, const uint64_t* stacks, int32_t batch, const void* logits,
-                              int dtype, int64_t row_stride, uint32_t* mask, int32_t* argmax, float* lse,
-                              float* logprobs, int32_t* states_out, uint64_t* stacks_out, cudaStream_t st);
+                              int dtype, int64_t row_stride, bool on_device, uint32_t* mask, int32_t* argmax,
+                              float* lse, float* logprobs, int32_t* states_out, uint64_t* stacks_out, cudaStream_t st);
 // The host's side of the walk's pool bound (RowTree::reserve): a node with
 // `kids` children, the deepest of which need `below`; and the shared memory a
 // CTA needs.

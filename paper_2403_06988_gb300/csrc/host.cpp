@@ -69,7 +69,7 @@ struct domino_ctx {
     bool trie_built = false;
     // the trees row_kernel walks (see RowTree)
     DevBuf d_rnode, d_rncls, d_rdtok, d_srec, d_srec_next, d_rret, d_rstart, d_loop_of, d_loopbits, d_keeps, d_xrange,
-        d_exits;
+        d_exits, d_trec;
     RowTree rows{}, rows_next{};     // for masks; for next states
     bool rows_ready = false;
     // which walk the mask step takes: -1 chosen from the automaton (see
@@ -646,8 +646,16 @@ int build_rows(domino_ctx* h) {
     if ((rc = up(h->d_keeps, keeps.data(), keeps.size()))) return rc;
     if ((rc = up(h->d_xrange, xrange.data(), xrange.size() * sizeof(uint2)))) return rc;
     if ((rc = up(h->d_exits, exits.data(), exits.size() * sizeof(uint2)))) return rc;
+    std::vector<uint8_t> trec((size_t)h->V * 32, 0);
+    for (int32_t t = 0; t < h->V; t++) {
+        const int64_t len = t == h->eos_id ? 0 : h->tok_off[t + 1] - h->tok_off[t];
+        trec[(size_t)t * 32] = (uint8_t)std::min<int64_t>(len, 255);
+        if (len > 0) std::memcpy(&trec[(size_t)t * 32 + 1], cls.data() + h->tok_off[t], (size_t)std::min<int64_t>(len, 31));
+    }
+    if ((rc = up(h->d_trec, trec.data(), trec.size()))) return rc;
     const StepView v = make_view(h);
     RowTree t{};
+    t.trec = (const uint8_t*)h->d_trec.p;
     t.node = (const uint4*)h->d_rnode.p;
     t.ncls = (const uint8_t*)h->d_rncls.p;
     t.dtok = (const int32_t*)h->d_rdtok.p;
@@ -935,7 +943,8 @@ int domino_destroy(domino_t h) {
         DevBuf* all[] = {&h->d_head, &h->d_info, &h->d_tail_off, &h->d_tail, &h->d_pos_of, &h->d_cls_start,
                          &h->d_eos_slot, &h->d_dense, &h->d_sparse, &h->d_accept, &h->d_self, &h->d_tok_cls, &h->d_err, &h->d_fpart, &h->s_logits, &h->s_mask, &h->s_io,
                          &h->o_prop, &h->o_rows, &h->o_count, &h->d_rnode, &h->d_rncls, &h->d_rdtok, &h->d_srec, &h->d_srec_next, &h->d_rret,
-                         &h->d_rstart, &h->d_loop_of, &h->d_loopbits, &h->d_keeps, &h->d_xrange, &h->d_exits};
+                         &h->d_rstart, &h->d_loop_of, &h->d_loopbits, &h->d_keeps, &h->d_xrange, &h->d_exits,
+                         &h->d_trec};
         for (auto* b : all) dev_free(*b);
         for (cudaEvent_t& e : h->ev_chunk)
             if (e) cudaEventDestroy(e);
@@ -1348,17 +1357,17 @@ int domino_step_decode(domino_t h, const int32_t* states_dev, const uint64_t* st
     const bool fusable = dtype == DOMINO_DTYPE_BF16 && reinterpret_cast<uintptr_t>(logits_dev) % 16 == 0 &&
                          ((size_t)row_stride_elems * 2) % 16 == 0 &&
                          (int64_t)batch * h->n_windows < (int64_t)INT32_MAX;   // partial slots are int
-    if (decode_rows(h, batch, fusable)) {   // the whole step in one kernel
-        StepView v = make_view(h);
-        return cuda_status(launch_row_decode(v, h->rows, h->env, h->stack, states_dev, stacks_dev, batch, logits_dev,
-                                             dtype, row_stride_elems, mask_dev, argmax_dev, lse_dev, logprobs_dev,
-                                             states_out, states_out && stacks_dev ? stacks_out : nullptr, st));
-    }
-    // logits in device memory are pulled into L2 a tile ahead of their fold;
+    // logits in device memory are pulled into L2 ahead of their fold;
     // host-resident logits are read only where the mask allows a token
     cudaPointerAttributes pa{};
     const bool on_device = cudaPointerGetAttributes(&pa, logits_dev) == cudaSuccess && pa.type == cudaMemoryTypeDevice;
     if (!on_device) cudaGetLastError();
+    if (decode_rows(h, batch, fusable)) {   // the whole step in one kernel
+        StepView v = make_view(h);
+        return cuda_status(launch_row_decode(v, h->rows, h->env, h->stack, states_dev, stacks_dev, batch, logits_dev,
+                                             dtype, row_stride_elems, on_device, mask_dev, argmax_dev, lse_dev, logprobs_dev,
+                                             states_out, states_out && stacks_dev ? stacks_out : nullptr, st));
+    }
     if (!fusable) {   // the kernels one after the other
         if ((rc = domino_step_mask(h, states_dev, stacks_dev, batch, mask_dev, nullptr, stream))) return rc;
         if ((rc = domino_mask_logits(h, logits_dev, dtype, batch, row_stride_elems, mask_dev, argmax_dev, lse_dev,
