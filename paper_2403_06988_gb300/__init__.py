@@ -71,12 +71,14 @@ class Domino:
     def step_mask(self, states, stacks=None, want_next: bool = False, out_mask=None, out_next=None,
                   stream=None):
         import torch
-        info = self.info()
         b = states.shape[0]
-        mask = out_mask if out_mask is not None else self._empty((b, info["n_words"]), torch.int32, states.device)
-        nxt = out_next
-        if want_next and nxt is None:
-            nxt = self._empty((b, info["n_tokens"]), torch.int32, states.device)
+        mask, nxt = out_mask, out_next
+        if mask is None or (want_next and nxt is None):
+            V, W = B.sizes(self.h)
+            if mask is None:
+                mask = self._empty((b, W), torch.int32, states.device)
+            if want_next and nxt is None:
+                nxt = self._empty((b, V), torch.int32, states.device)
         B.domino_step_mask(self.h, states, stacks, b, mask, nxt, stream)
         return mask, nxt
 
@@ -91,11 +93,16 @@ class Domino:
             raise TypeError("logits must be float32 or bfloat16")
         if logits.stride(1) != 1:
             raise ValueError("logits rows must be contiguous")
-        mask = out_mask if out_mask is not None else self._empty((b, self.info()["n_words"]), torch.int32,
-                                                                 states.device)
-        argmax = self._empty(b, torch.int32, states.device)
-        lse = self._empty(b, torch.float32, states.device)
-        lp = self._empty((b, self.info()["n_tokens"]), torch.float32, states.device) if want_logprobs else None
+        dev = states.device
+        mask, lp = out_mask, None
+        if mask is None or want_logprobs:
+            V, W = B.sizes(self.h)
+            if mask is None:
+                mask = self._empty((b, W), torch.int32, dev)
+            if want_logprobs:
+                lp = self._empty((b, V), torch.float32, dev)
+        argmax = self._empty(b, torch.int32, dev)
+        lse = self._empty(b, torch.float32, dev)
         B.domino_step_decode(self.h, states, stacks, b, logits.data_ptr(), dtype, logits.stride(0), mask, argmax, lse,
                              lp, states if advance else None, stacks if advance else None, stream)
         return mask, argmax, lse, lp
@@ -113,7 +120,8 @@ class Domino:
                     = None, out=None, stream=None) -> Tuple:
         import torch
         b = logits.shape[0]
-        V = n_tokens if n_tokens is not None else self.info()["n_tokens"]
+        if n_tokens is None and want_logprobs and (out is None or out[2] is None):
+            n_tokens = B.sizes(self.h)[0]
         dtype = DTYPE_BF16 if logits.dtype == torch.bfloat16 else DTYPE_F32
         if dtype == DTYPE_F32 and logits.dtype != torch.float32:
             raise TypeError("logits must be float32 or bfloat16")
@@ -125,7 +133,7 @@ class Domino:
         if want_lse and lse is None:
             lse = self._empty(b, torch.float32, logits.device)
         if want_logprobs and lp is None:
-            lp = self._empty((b, V), torch.float32, logits.device)
+            lp = self._empty((b, n_tokens), torch.float32, logits.device)
         B.domino_mask_logits(self.h, logits.data_ptr(), dtype, b, logits.stride(0), mask, argmax,
                              lse if want_lse else None, lp if want_logprobs else None, stream)
         return argmax, (lse if want_lse else None), (lp if want_logprobs else None)
@@ -156,7 +164,7 @@ class Domino:
         dtype = DTYPE_BF16 if logits.dtype == torch.bfloat16 else DTYPE_F32
         if logits.stride(1) != 1:
             raise ValueError("logits rows must be contiguous")
-        W = self.info()["n_words"]
+        W = B.sizes(self.h)[1]
         scratch = self._empty((b, W), torch.int32, logits.device)
         tokens = self._empty(b, torch.int32, logits.device)
         n_fb = torch.zeros(1, dtype=torch.int32, device=logits.device)
@@ -169,13 +177,12 @@ class Domino:
         """Table-driven mask + decode: row b's mask is table_mask[states[b]] (DFA only)."""
         import torch
         b = logits.shape[0]
-        V = self.info()["n_tokens"]
         dtype = DTYPE_BF16 if logits.dtype == torch.bfloat16 else DTYPE_F32
         if logits.stride(1) != 1:
             raise ValueError("logits rows must be contiguous")
         argmax = self._empty(b, torch.int32, logits.device)
         lse = self._empty(b, torch.float32, logits.device) if want_lse else None
-        lp = self._empty((b, V), torch.float32, logits.device) if want_logprobs else None
+        lp = self._empty((b, B.sizes(self.h)[0]), torch.float32, logits.device) if want_logprobs else None
         B.domino_mask_logits_table(self.h, logits, dtype, b, logits.stride(0), table_mask, states, argmax, lse, lp,
                                    stream)
         return argmax, lse, lp

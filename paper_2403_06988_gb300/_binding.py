@@ -115,22 +115,25 @@ def _ptr(x) -> Optional[int]:
     """Device or host address of a torch tensor / numpy array (None passes NULL)."""
     if x is None:
         return None
-    if isinstance(x, np.ndarray):
-        assert x.flags["C_CONTIGUOUS"]
-        return x.ctypes.data
-    if hasattr(x, "data_ptr"):
-        assert x.is_contiguous()
-        return x.data_ptr()
-    if isinstance(x, int):
-        return x
-    raise TypeError(type(x))
+    try:   # a torch tensor first: a step passes up to nine of them
+        address = x.data_ptr
+    except AttributeError:
+        if isinstance(x, np.ndarray):
+            assert x.flags["C_CONTIGUOUS"]
+            return x.ctypes.data
+        if isinstance(x, int):
+            return x
+        raise TypeError(type(x)) from None
+    assert x.is_contiguous()
+    return address()
 
 
 def _stream(stream) -> Optional[int]:
-    if stream is not None:
-        return stream if isinstance(stream, int) else stream.cuda_stream
-    import torch
-    return torch.cuda.current_stream().cuda_stream
+    if stream is None:
+        import torch
+        # torch.cuda.current_stream().cuda_stream without the Stream object
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return stream if isinstance(stream, int) else stream.cuda_stream
 
 
 def status_string(status: int) -> str:
@@ -186,6 +189,13 @@ def domino_get_info(h: int) -> dict:
     info = Info()
     _check("domino_get_info", lib().domino_get_info(h, ctypes.byref(info)))
     return {name: getattr(info, name) for name, _ in Info._fields_}
+
+
+def sizes(h: int):
+    """(n_tokens, n_words) of the handle's vocabulary, as domino_get_info reports them."""
+    info = Info()
+    _check("domino_get_info", lib().domino_get_info(h, ctypes.byref(info)))
+    return info.n_tokens, info.n_words
 
 
 def domino_get_byte_classes(h: int) -> np.ndarray:
