@@ -225,55 +225,73 @@ struct Decoder {
         return x;
     }
 
-    __device__ __forceinline__ void fold(const Vec& x, uint32_t bits, int t0) {
+    // N vectors, of which vector k's allowed tokens are bits[k] (0: none) and
+    // whose element 0 is token t0[k].  Without branches between the vectors, so
+    // that their latencies overlap.
+    template <int N>
+    __device__ __forceinline__ void fold(const Vec (&x)[N], const uint32_t (&bits)[N], const int (&t0)[N]) {
         if constexpr (FOLD == kFoldSample) {
-            sample(x, bits, t0);
+#pragma unroll
+            for (int k = 0; k < N; ++k) {
+                if (bits[k]) sample(x[k], bits[k], t0[k]);
+                share();
+            }
         } else {
-            // the masked tokens as -inf, the vector's maximum, then its sum
-            uint32_t w[kWords];
-            float2 xs[4];
-            float vm;
-            if constexpr (BF16) {
-                const uint4 k = keep[bits];
-                w[0] = (x.q[0] & k.x) | (0xFF80FF80u & ~k.x), w[1] = (x.q[1] & k.y) | (0xFF80FF80u & ~k.y);
-                w[2] = (x.q[2] & k.z) | (0xFF80FF80u & ~k.z), w[3] = (x.q[3] & k.w) | (0xFF80FF80u & ~k.w);
-                const uint32_t mm = max2_bf16(max2_bf16(w[0], w[1]), max2_bf16(w[2], w[3]));
-                vm = fmaxf(bf16_lo(mm), bf16_hi(mm));
+            // the tokens not allowed as -inf, and the vectors' maxima
+            uint32_t w[N][kWords];
+            float vm[N];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) xs[e] = make_float2(bf16_lo(w[e]), bf16_hi(w[e]));
-            } else {
+            for (int k = 0; k < N; ++k) {
+                if constexpr (BF16) {
+                    const uint4 y = keep[bits[k]];
+                    w[k][0] = (x[k].q[0] & y.x) | (0xFF80FF80u & ~y.x), w[k][1] = (x[k].q[1] & y.y) | (0xFF80FF80u & ~y.y);
+                    w[k][2] = (x[k].q[2] & y.z) | (0xFF80FF80u & ~y.z), w[k][3] = (x[k].q[3] & y.w) | (0xFF80FF80u & ~y.w);
+                    const uint32_t mm = max2_bf16(max2_bf16(w[k][0], w[k][1]), max2_bf16(w[k][2], w[k][3]));
+                    vm[k] = fmaxf(bf16_lo(mm), bf16_hi(mm));
+                } else {
+                    float y[8];
 #pragma unroll
-                for (int e = 0; e < 8; ++e) w[e] = (bits >> e) & 1u ? x.q[e] : 0xFF800000u;
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    xs[e] = make_float2(__uint_as_float(w[2 * e]), __uint_as_float(w[2 * e + 1]));
-                vm = fmaxf(fmaxf(fmaxf(xs[0].x, xs[0].y), fmaxf(xs[1].x, xs[1].y)),
-                           fmaxf(fmaxf(xs[2].x, xs[2].y), fmaxf(xs[3].x, xs[3].y)));
+                    for (int e = 0; e < 8; ++e) {
+                        w[k][e] = (bits[k] >> e) & 1u ? x[k].q[e] : 0xFF800000u;
+                        y[e] = __uint_as_float(w[k][e]);
+                    }
+                    vm[k] = fmaxf(fmaxf(fmaxf(y[0], y[1]), fmaxf(y[2], y[3])), fmaxf(fmaxf(y[4], y[5]), fmaxf(y[6], y[7])));
+                }
             }
             if constexpr (FOLD == kFoldLse) {
-                constexpr float kLag = 16.0f;   // 2^24 at most: no overflow, and nothing lost in relative terms
-                const float vL = vm * kLog2e;
-                if (vL > ref + kLag || m == -INFINITY) {   // rare after the first vector
-                    if (vm != -INFINITY) {
-                        s *= s == 0.0f ? 0.0f : ex2(ref - vL);
-                        ref = vL;
+                constexpr float kLag = 16.0f;   // terms of 2^16 at most: no overflow, and nothing lost in relative terms
+                float most = vm[0];
+#pragma unroll
+                for (int k = 1; k < N; ++k) most = fmaxf(most, vm[k]);
+                const float vL = most * kLog2e;
+                if ((vL > ref + kLag || m == -INFINITY) && most != -INFINITY) {   // rare after the first vectors
+                    s *= s == 0.0f ? 0.0f : ex2(ref - vL);
+                    ref = vL;
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < N; ++k)
+                if (vm[k] > m || (vm[k] == m && t0[k] < idx)) {
+                    m = vm[k];
+                    idx = t0[k];
+#pragma unroll
+                    for (int e = 0; e < kWords; ++e) top[e] = w[k][e];
+                }
+            if constexpr (FOLD == kFoldLse) {
+                float2 acc[N];
+#pragma unroll
+                for (int k = 0; k < N; ++k) {
+                    acc[k] = make_float2(0.0f, 0.0f);
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const float2 z = BF16 ? make_float2(bf16_lo(w[k][e]), bf16_hi(w[k][e]))
+                                              : make_float2(__uint_as_float(w[k][BF16 ? 0 : 2 * e]), __uint_as_float(w[k][BF16 ? 0 : 2 * e + 1]));
+                        const float2 y = fma2(z, kLog2e, -ref);
+                        acc[k] = add2(acc[k], make_float2(ex2(y.x), ex2(y.y)));   // not allowed: 2^-inf = 0
                     }
                 }
-            }
-            if (vm > m || (vm == m && t0 < idx)) {
-                m = vm;
-                idx = t0;
 #pragma unroll
-                for (int k = 0; k < kWords; ++k) top[k] = w[k];
-            }
-            if constexpr (FOLD == kFoldLse) {
-                float2 acc = make_float2(0.0f, 0.0f);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const float2 y = fma2(xs[k], kLog2e, -ref);
-                    acc = add2(acc, make_float2(ex2(y.x), ex2(y.y)));   // not allowed: 2^-inf = 0
-                }
-                s += acc.x + acc.y;
+                for (int k = 0; k < N; ++k) s += acc[k].x + acc[k].y;
             }
         }
     }
@@ -464,7 +482,14 @@ struct Decoder {
                 for (int k = 0; k < kWords; ++k) x.q[k] = 0u;
                 const uint32_t u = __float_as_uint(logit_at<BF16>(lrow, t0 + e));
                 x.q[0] = BF16 ? u >> 16 : u;   // as element 0 of a vector that starts at the token
-                fold(x, 1u, t0 + e);
+                if constexpr (FOLD == kFoldSample) {
+                    sample(x, 1u, t0 + e);   // (fold's sampling form is the whole warp's)
+                } else {
+                    const Vec xs[1] = {x};
+                    const uint32_t one[1] = {1u};
+                    const int at[1] = {t0 + e};
+                    fold<1>(xs, one, at);
+                }
             }
         }
     }
@@ -474,16 +499,16 @@ struct Decoder {
                                                   const int (&b)[kTogether]) {
         Vec x[kTogether];
         uint32_t by[kTogether];
+        int t0[kTogether];
 #pragma unroll
         for (int k = 0; k < kTogether; ++k) {
             by[k] = b[k] >= 0 ? allowed(bytes, b[k]) : 0u;
+            t0[k] = base + 8 * b[k];
+#pragma unroll
+            for (int e = 0; e < kWords; ++e) x[k].q[e] = 0u;
             if (by[k]) x[k] = load(vec, b[k]);
         }
-#pragma unroll
-        for (int k = 0; k < kTogether; ++k) {
-            if (by[k]) fold(x[k], by[k], base + 8 * b[k]);
-            share();
-        }
+        fold<kTogether>(x, by, t0);
     }
 
     // sampling: the warp's best score so far bounds what a lane has to draw

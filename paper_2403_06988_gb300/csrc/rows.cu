@@ -535,13 +535,6 @@ struct RowWalk {
         }
     }
 
-    // token i of the preorder list as part of a range, -1 where the range's filter drops it
-    __device__ __forceinline__ int token(const uint4& range, uint32_t i) const {
-        const int tk = __ldg(t.dtok + i);
-        if (range.w == 0u) return tk;
-        return __ldg(t.keeps + (size_t)((range.w >> 8) - 1u) * t.n_dtok + i) <= (range.w & 0xFFu) ? tk : -1;
-    }
-
     // Sets the token ranges left by the rounds and empties their lists.
     // Every thread calls it, after a barrier that follows the last round.
     __device__ __forceinline__ void ranges() const {
@@ -552,41 +545,50 @@ struct RowWalk {
             const uint4 x = s_range[i];
             for (uint32_t j = tid & 3; j < x.y; j += 32) {
                 int tk[8];
+                uint32_t out[8];   // the filter's byte: greater than the range's depth drops the token
                 const int32_t* p = t.dtok + x.x + j;
+                const uint8_t* k = t.keeps + (x.w ? (size_t)((x.w >> 8) - 1u) * t.n_dtok + x.x + j : 0);
 #pragma unroll
-                for (int q = 0; q < 8; ++q) tk[q] = j + 4 * q < x.y ? __ldg(p + 4 * q) : -1;
-                if (x.w) {
-                    const uint8_t* k = t.keeps + (size_t)((x.w >> 8) - 1u) * t.n_dtok + x.x + j;
-#pragma unroll
-                    for (int q = 0; q < 8; ++q)
-                        if (tk[q] >= 0 && __ldg(k + 4 * q) > (x.w & 0xFFu)) tk[q] = -1;
+                for (int q = 0; q < 8; ++q) {
+                    tk[q] = j + 4 * q < x.y ? __ldg(p + 4 * q) : -1;
+                    out[q] = x.w && j + 4 * q < x.y ? __ldg(k + 4 * q) : 0u;
                 }
 #pragma unroll
                 for (int q = 0; q < 8; ++q)
-                    if (tk[q] >= 0) emit(tk[q], x.z);
+                    if (tk[q] >= 0 && out[q] <= (x.w & 0xFFu)) emit(tk[q], x.z);
             }
         }
         if (nb > 0) {   // long ones: the CTA over all of them
             const int total = prefix(nb, tid < nb ? (int)s_range[kRowSmall + tid].y : 0);
-            constexpr int kUnroll = 8;
-            for (int f0 = tid; f0 < total; f0 += kUnroll * kRowThreads) {
+            // a warp takes 256 tokens in a row: they lie in a few ranges
+            constexpr int kUnroll = STACK ? 8 : 4;   // 8 spill beside a DFA's folded decode: +0.8 us at 128256x256
+            for (int f0 = warp * 32 * kUnroll; f0 < total; f0 += kRowThreads * kUnroll) {
                 int tk[kUnroll];
-                uint32_t st[kUnroll];
+                uint32_t st[kUnroll], out[kUnroll];
+                int k = find_range(s_pre, nb, f0), end = s_pre[k + 1];
+                uint4 b = s_range[kRowSmall + k];
+                uint32_t at = b.x - (uint32_t)s_pre[k];   // the list's index of token f is at + f
 #pragma unroll
                 for (int q = 0; q < kUnroll; ++q) {
-                    const int f = f0 + q * kRowThreads;
+                    const int f = f0 + 32 * q + lane;
                     tk[q] = -1;
-                    st[q] = 0u;
+                    st[q] = out[q] = 0u;
                     if (f < total) {
-                        const int k = find_range(s_pre, nb, f);
-                        const uint4 b = s_range[kRowSmall + k];
-                        tk[q] = token(b, b.x + (uint32_t)(f - s_pre[k]));
-                        st[q] = b.z;
+                        while (f >= end) {
+                            ++k;
+                            b = s_range[kRowSmall + k];
+                            at = b.x - (uint32_t)end;
+                            end = s_pre[k + 1];
+                        }
+                        const uint32_t i = at + (uint32_t)f;
+                        tk[q] = __ldg(t.dtok + i);
+                        st[q] = b.z | (b.w << 16);   // the state and the filter's depth
+                        if (b.w) out[q] = __ldg(t.keeps + (size_t)((b.w >> 8) - 1u) * t.n_dtok + i);
                     }
                 }
 #pragma unroll
                 for (int q = 0; q < kUnroll; ++q)
-                    if (tk[q] >= 0) emit(tk[q], st[q]);
+                    if (tk[q] >= 0 && out[q] <= ((st[q] >> 16) & 0xFFu)) emit(tk[q], st[q] & 0xFFFFu);
             }
         }
         __syncthreads();   // the lists have been read
@@ -597,7 +599,7 @@ struct RowWalk {
 
 // C.update() of a row in configuration rc (read_row) by its token tk, or by
 // -1: as advance_row, with the token's classes in one record.
-template <bool STACK>
+template <bool STACK, int CLS>
 __device__ __forceinline__ void update(const StepView& v, const RowTree& t, const uint4& rc, int32_t tk, int b,
                                        int32_t* states_out, uint64_t* stacks_out) {
     uint32_t s = 0, bits = 0, depth = 0;
@@ -614,13 +616,13 @@ __device__ __forceinline__ void update(const StepView& v, const RowTree& t, cons
             head = reinterpret_cast<const uint8_t*>(v.head + 2 * (size_t)p);
             if (len > kInlineBytes) tail += __ldg(v.tail_off + p);
         }
+        bits = rc.y;
+        depth = rc.z;
         using E = typename std::conditional<STACK, uint32_t, uint16_t>::type;
         Tab<E, kDenseGlobal> tab;
         tab.dense = reinterpret_cast<const E*>(STACK ? (const void*)v.t32 : (const void*)v.t16);
         tab.K = (uint32_t)v.K;
         debug_bounds(tab, v);
-        bits = rc.y;
-        depth = rc.z;
         s = len > 0 ? walk<STACK, 0>(tab, v.ret, (uint32_t)v.max_depth, rc.x, bits, depth, head, len, tail) : 0u;
         if (s == 0) bits = depth = 0;
     }
@@ -730,7 +732,7 @@ __global__ void __launch_bounds__(kRowThreads, 2)
             a.argmax[b] = tk;
             if (a.lse) a.lse[b] = lse;
             // every CTA of the row has read its configuration (the outputs may alias it)
-            if (a.states_out) update<STACK>(v, t, rc, tk, b, a.states_out, a.stacks_out);
+            if (a.states_out) update<STACK, CLS>(v, t, rc, tk, b, a.states_out, a.stacks_out);
         }
         if (a.slices > 1) cluster_wait();
     }
