@@ -299,7 +299,7 @@ struct RowWalk {
             } else {
                 x.m = x.kids & x.live;
                 if (x.em.n == 255u) x.em.n = __ldg(&t.node[2 * (size_t)x.first_child + 1].x) - B.x;
-                if ((h.w >> 31) && lead && B.y - B.x > (uint32_t)kRowLoopMin && (x.kids & keep) != 0 &&
+                if ((h.w >> 31) && t.n_loops > 0 && lead && B.y - B.x > (uint32_t)kRowLoopMin && (x.kids & keep) != 0 &&
                     loop_subtree(it, B.x + x.em.n, B.y, st))
                     x.m = 0;
             }
@@ -745,7 +745,7 @@ cudaError_t rows_allow_smem(K kern, int bytes, int* configured, std::mutex& mu) 
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if (bytes <= 48 * 1024) return cudaSuccess;
+    if (bytes <= 40 * 1024) return cudaSuccess;   // with the static part within the default 48 KiB
     std::lock_guard<std::mutex> lk(mu);
     if (dev < kRowMaxDevices && configured[dev] >= bytes) return cudaSuccess;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
