@@ -142,25 +142,18 @@ __global__ void __launch_bounds__(kDecodeThreads, 2)
     if (a.slices > 1) cluster_wait();
 }
 
-// slices: CTAs per row (no cluster: the rows' log-sum-exp is given)
+// The log-probabilities alone, slice_words mask words per CTA, read in place:
+// a pass of loads per thread and no barrier (staged through shared memory in
+// clusters' slices it took 3.0 us instead of 2.3 at 64000 tokens, batch 24).
 template <bool BF16>
 __global__ void __launch_bounds__(kDecodeThreads, 2)
     logprobs_kernel(const __grid_constant__ LogitsArgs a) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    uint32_t* s_mask = reinterpret_cast<uint32_t*>(smem + 16);
-    const int tid = threadIdx.x, r = blockIdx.x / a.slices, slice = blockIdx.x - r * a.slices;
+    const int r = blockIdx.x / a.slices, w0 = (blockIdx.x - r * a.slices) * a.slice_words;
     pdl_wait();
     pdl_trigger();
-    const int w0 = slice * a.slice_words, w1 = min(a.W, w0 + a.slice_words);
-    const uint32_t* mrow = a.mask.row(r, a.W, false);
-    const float lse = __ldg(a.lse + r);
-    for (int j = w0; j < w1; j += a.segment) {
-        const int n = min(a.segment, w1 - j);
-        if (j > w0) __syncthreads();
-        stage_mask(s_mask, a.mask, mrow, j, n, a.V, tid);
-        write_logprobs<BF16>(reinterpret_cast<const char*>(a.logits) + (size_t)r * (size_t)a.stride * (BF16 ? 2 : 4),
-                             a.V, s_mask, 32 * j, min(32 * n, a.V - 32 * j), lse, a.logprobs + (size_t)r * a.V, tid);
-    }
+    write_logprobs<BF16>(reinterpret_cast<const char*>(a.logits) + (size_t)r * (size_t)a.stride * (BF16 ? 2 : 4), a.V,
+                         a.mask.row(r, a.W, false) + w0, 32 * w0, min(32 * a.slice_words, a.V - 32 * w0),
+                         __ldg(a.lse + r), a.logprobs + (size_t)r * a.V, threadIdx.x);
 }
 
 // Gumbel variate of token t of row r: g_t = -ln(-ln(u_t)), u_t = (2k + 1) / 2^24,
@@ -389,11 +382,18 @@ __global__ void __launch_bounds__(kGatherMaxWarps * 32, 2)
     }
 }
 
-// CTAs per row: doubled while two per SM are not reached and a warp has more
-// than four mask words.
+// CTAs per row: doubled while every SM has at most one and a warp more than 16
+// mask words, or at most two and 128 words.  Two CTAs an SM whose warps have
+// fewer wait for the launch and the cluster's barriers (GB300, batch 100, V =
+// 8000, 1 % allowed: one CTA a row 4.4 us, two 7.1; fp32, batch 32, V = 32000,
+// half allowed: two 7.0, four 6.5, eight 8.4, a draw 12.7 / 10.2 / 12.4; V =
+// 152064, batch 128, 80 %: one 15.2, two 12.9, with log-probabilities 38.2 /
+// 27.7, a draw 97 / 59).
 void cut_rows(LogitsArgs& a, int num_sms) {
     int s = 1;
-    while (s < 8 && (int64_t)a.batch * s * 2 <= 2 * num_sms && a.W > 128 * s) s *= 2;
+    while (s < 8 && ((int64_t)a.batch * s * 2 <= num_sms ? a.W > 256 * s
+                                                         : (int64_t)a.batch * s <= num_sms && a.W > 2048 * s))
+        s *= 2;
     a.slices = s;
     a.slice_words = ((a.W + s - 1) / s + 3) / 4 * 4;
     a.segment = std::min(a.slice_words, kLogitsSegment);
@@ -469,10 +469,10 @@ cudaError_t launch_mask_logits(const LaunchEnv& env, const void* logits, int dty
     // 1000: 22 against 29 us; JSON, V = 152064, batch 512, mostly dense: 45
     // against 38 us).  With fewer rows, or rows off 16-byte boundaries, fp32 or
     // log-probabilities, the cluster kernel: V = 152064, batch 128, 80 %
-    // allowed: 17.0 us (24.6 us for the flat split over one-warp CTAs that it
-    // replaced), with log-probabilities 31.5 us (40.0); batch 24, V = 50001:
-    // 8.1 us (13.6); fp32, V = 32000, batch 64, with log-probabilities: 10.5 us
-    // (28.9); a draw at V = 152064, batch 128, 80 %: 62 us (115).
+    // allowed: 12.9 us (24.6 us for the flat split over one-warp CTAs that it
+    // replaced), with log-probabilities 27.7 us (40.0); batch 24, V = 50001:
+    // 7.1 us (13.6); fp32, V = 32000, batch 64, with log-probabilities: 9.0 us
+    // (28.9); a draw at V = 152064, batch 128, 80 %: 57.9 us (115).
     const bool aligned = reinterpret_cast<uintptr_t>(logits) % 16 == 0 && ((size_t)row_stride * 2) % 16 == 0;
     if (dtype == DOMINO_DTYPE_BF16 && aligned && batch > env.num_sms && !logprobs)
         return sample ? launch_gather<kFoldSample>(a, list, st)
@@ -492,9 +492,9 @@ cudaError_t launch_logprobs_bf16(const LaunchEnv& env, const void* logits, int32
     a.batch = batch;
     a.lse = const_cast<float*>(lse);
     a.logprobs = logprobs;
-    cut_rows(a, env.num_sms);
-    return launch_pdl(logprobs_kernel<true>, dim3((unsigned)batch * (unsigned)a.slices), dim3(kDecodeThreads),
-                      (size_t)(32 + a.segment * 4), st, a);
+    a.slice_words = 128;   // one 8-token vector per thread
+    a.slices = (a.W + a.slice_words - 1) / a.slice_words;
+    return launch_pdl(logprobs_kernel<true>, dim3((unsigned)batch * (unsigned)a.slices), dim3(kDecodeThreads), 0, st, a);
 }
 
 cudaError_t launch_mask_sample(const LaunchEnv& env, const void* logits, int dtype, int32_t batch,
