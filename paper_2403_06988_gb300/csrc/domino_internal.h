@@ -126,8 +126,6 @@ struct RowTree {
     const uint8_t* trec;        // [V][32]: {token length (255: or more), its first 31 classes}
     const uint2* exits;         // {node, its class | depth of the nearest exit above (at most 255) << 8}
     int32_t srec_stride, n_nodes, n_dtok, n_loops;
-    int32_t reserve;            // pool entries a depth-first walk of any node can add
-    int32_t max_kids;           // most children of any node (at least 1)
     int32_t loop_root[4];
 };
 constexpr int kRowLoopSets = 4;           // loop sets with a tree of their own
@@ -174,11 +172,8 @@ cudaError_t launch_row_decode(const StepView& v, const RowTree& t, const LaunchE
                               const int32_t* states, const uint64_t* stacks, int32_t batch, const void* logits,
                               int dtype, int64_t row_stride, bool on_device, uint32_t* mask, int32_t* argmax,
                               float* lse, float* logprobs, int32_t* states_out, uint64_t* stacks_out, cudaStream_t st);
-// The host's side of the walk's pool bound (RowTree::reserve): a node with
-// `kids` children, the deepest of which need `below`; and the shared memory a
-// CTA needs.
-int32_t row_reserve(int32_t kids, int32_t below);
-int row_smem_bytes(int32_t n_words, int32_t reserve, bool stack, bool loops);
+// Shared-memory bytes of row_kernel at most, for a vocabulary of n_words mask words.
+int row_smem_bytes(int32_t n_words, bool stack, bool loops);
 
 // Log-probabilities only (bf16 logits, rows on 16-byte boundaries), given the
 // rows' lse: logprobs[b][t] = logit - lse[b] for allowed t, -inf else.

@@ -72,6 +72,7 @@ struct domino_ctx {
         d_exits, d_trec;
     RowTree rows{}, rows_next{};     // for masks; for next states
     bool rows_ready = false;
+    bool rows_dense = false;         // most states' walks visit many nodes (rows_dense())
     // which walk the mask step takes: -1 chosen from the automaton (see
     // use_tree), 1 the prefix tree, 0 every token on its own (DOMINO_WALK=tree
     // or =token in the environment when the handle is created)
@@ -313,7 +314,6 @@ struct RowBuild {
     std::vector<int32_t> dtok;
     std::vector<std::vector<uint8_t>> keeps;   // per loop set
     std::vector<std::vector<uint2>> xrange, exits;
-    int32_t reserve = 0, max_kids = 1;
 };
 
 // Appends the tree over `strs` (sorted).  Returns its root, or -1 when the
@@ -358,18 +358,9 @@ int64_t add_row_tree(RowBuild& rb, const std::vector<RowStr>& strs) {
     while (!path.empty()) close_node();
     const uint32_t N = (uint32_t)skip.size();
     std::vector<uint64_t> sub(N, 0);
-    std::vector<int32_t> need(N, 0);
     for (uint32_t n = N; n-- > 0;) {
-        int32_t kids = 0, below = 0;
-        for (uint32_t c = n + 1; c < skip[n]; c = skip[c]) {
-            kids++;
-            below = std::max(below, need[c]);
-            if (!rb.wide) sub[n] |= (1ull << cls[c]) | sub[c];
-        }
-        need[n] = std::min<int32_t>(1 << 20, row_reserve(kids, below));
-        rb.max_kids = std::max(rb.max_kids, kids);
+        for (uint32_t c = n + 1; !rb.wide && c < skip[n]; c = skip[c]) sub[n] |= (1ull << cls[c]) | sub[c];
     }
-    rb.reserve = std::max(rb.reserve, need[0]);
     // breadth first: order[i] is the preorder number of node root + i
     std::vector<uint32_t> order(1, 0), at(N, 0);
     order.reserve(N);
@@ -527,6 +518,44 @@ std::vector<uint8_t> state_records(const RowEntries& r, int K, bool stack, const
     return out;
 }
 
+// Whether the walks of more than an eighth of the states (an even sample)
+// visit more than kDenseNodes nodes of the tree.  Subtrees below a state that
+// loops on their classes are left out, and so are the classes of a wide loop:
+// those are not walked node by node.
+constexpr int64_t kDenseNodes = 8192;
+constexpr int kDenseSample = 256;
+bool rows_dense(const domino_ctx* h, const RowBuild& rb, const RowEntries& merged, const std::vector<uint64_t>& self) {
+    const int64_t K = h->K, n_states = rb.wide ? h->Q : merged.Q;
+    const int n = (int)std::min<int64_t>(kDenseSample, n_states - 1);
+    int over = 0;
+    std::vector<std::pair<uint32_t, uint32_t>> work;   // (node, state)
+    for (int i = 0; i < n; i++) {
+        int64_t visits = 0;
+        work.assign(1, {0u, (uint32_t)(1 + (n_states - 1) * i / n)});
+        while (!work.empty() && visits <= kDenseNodes) {
+            const auto [node, q] = work.back();
+            work.pop_back();
+            visits++;
+            const uint4 a = rb.node[2 * (size_t)node], b = rb.node[2 * (size_t)node + 1];
+            const uint64_t keep = rb.wide ? 0 : self[q], below = ((uint64_t)b.w << 32) | b.z;
+            if (!rb.wide && (below & ~keep) == 0) continue;
+            const bool loop = 4 * __builtin_popcountll(keep) >= K;
+            const uint32_t first = a.z & 0xFFFFFFu;
+            const int kids = rb.wide ? (int)a.x : __builtin_popcountll(((uint64_t)a.y << 32) | a.x);
+            for (int k = 0; k < kids; k++) {
+                const uint32_t c = rb.ncls[(size_t)first + (size_t)k];
+                if (loop && ((keep >> c) & 1ull)) continue;
+                const size_t at = (size_t)(q * K + c);
+                const uint32_t e = !rb.wide ? merged.e[at] : h->stack ? h->t32[at] : h->t16[at];
+                const uint32_t to = h->stack && ((e >> kKindShift) & 3u) == 2u ? 0u : e & 0xFFFFu;   // not past a pop
+                if (to) work.push_back({first + (uint32_t)k, to});
+            }
+        }
+        over += visits > kDenseNodes;
+    }
+    return 8 * over > n;
+}
+
 // The trees, state records and loop sets of RowTree.  rows_ready stays false
 // (the per-token walk is used) when the vocabulary or its tree is too large.
 int build_rows(domino_ctx* h) {
@@ -553,7 +582,7 @@ int build_rows(domino_ctx* h) {
     }
     // the loop sets worth a tree: at least a quarter of the classes (the rule
     // of self_mask), those of most states first
-    if (!wide && K <= 63 && h->walk_pref != 1) {
+    if (!wide && K <= 63) {
         std::vector<std::pair<uint64_t, int32_t>> all;   // (set, states)
         std::unordered_map<uint64_t, size_t> at;
         for (int32_t q = 1; q < Q; q++) {
@@ -596,7 +625,7 @@ int build_rows(domino_ctx* h) {
         size_t n_exits = 0;
         for (auto& e : rb.exits) n_exits += e.size();
         ok = ok && n_exits < (size_t)(1u << 24) &&
-             row_smem_bytes(h->W, rb.reserve, h->stack, !sets.empty()) <= smem - 1024;
+             row_smem_bytes(h->W, h->stack, !sets.empty()) <= smem - 1024;
         if (!ok && sets.empty()) return DOMINO_OK;
         if (!ok) sets.clear();
     }
@@ -671,8 +700,6 @@ int build_rows(domino_ctx* h) {
     t.n_nodes = (int32_t)(rb.node.size() / 2);
     t.n_dtok = (int32_t)rb.dtok.size();
     t.n_loops = (int32_t)n_sets;
-    t.reserve = rb.reserve;
-    t.max_kids = rb.max_kids;
     for (size_t i = 0; i < n_sets; i++) t.loop_root[i] = (int32_t)roots[i];
     h->rows = t;
     if (!start.empty()) {
@@ -683,6 +710,7 @@ int build_rows(domino_ctx* h) {
         t.n_loops = 0;
     }
     h->rows_next = t;
+    h->rows_dense = rows_dense(h, rb, merged, self);
     h->rows_ready = true;
     return DOMINO_OK;
 }
@@ -827,33 +855,53 @@ bool use_tree(const domino_ctx* h) {
     return h->walk_pref == 1 || h->self_mask.empty();
 }
 
-// Whether row_kernel takes a mask step.  Its time is the latency of the walk's
-// rounds (8 to 40 us) and hardly grows until every SM has rows; the per-token
-// walk's grows with the (row, token) pairs.  Without loop sets the row kernel
-// wins from one row on (GB300, 5000 states, V = 128256, batch 16: 14.0
-// against 17.9 us).  With them the lines cross near 2^21 pairs: 200 states,
-// V = 32000, batch 32 (2^20): 7.9 against 5.3 us; JSON, V = 50001, batch 24
-// (2^20.2): 18.6 against 16.2 us; V = 152064, batch 128 (2^24): 36.5 against
-// 74.4 us; 200 states, V = 64000, batch 500: 12.9 against 24.3 us.
-// Next states of such automata are the per-token walk's (the loop sets hold
-// masks only).
-bool use_rows(const domino_ctx* h, int64_t batch, bool next) {
-    if (use_tree(h)) return true;
-    return h->rows_ready && h->walk_pref != 0 && !next && batch * h->V >= ((int64_t)1 << 21);
+// The (row, token) pairs from which row_kernel is the faster walk.  Its time
+// is the latency of a row's rounds (8 to 40 us), once for every 2 * SMs rows;
+// the per-token walk's grows with the pairs.  In units of 2^19 pairs: `first`
+// for up to 2 * SMs rows, `more` for every further such wave.
+bool rows_pay(const domino_ctx* h, int64_t batch, int first, int more) {
+    const int64_t at_once = 2 * std::max(1, h->env.num_sms);
+    return batch * h->V >= (first + (batch - 1) / at_once * more) * ((int64_t)1 << 19);
 }
 
-// Whether the whole decode step is row_kernel's (one launch).  With loop sets
-// the lines cross near 3 * 2^20 (row, token) pairs against the per-token walk
-// with the decode folded in (two launches; bf16 rows on 16-byte boundaries):
-// 200 states, V = 32000, batch 32: 13.4 against 8.8 us, batch 100: 12.6
-// against 11.8 us (with log-probabilities 15.1 against 16.3 us); JSON, V =
-// 50001, batch 64: 28.8 against 33.7 us; V = 152064, batch 8: 18.6 against
-// 15.0 us, batch 128: 54.6 against 86.1 us, batch 512: 102 against 304 us; and
-// near 2^20 against the three kernels one after the other (V = 50001, batch
-// 24: 26.8 against 27.9 us and two launches more).
+// Whether row_kernel takes a mask step (GB300, us per-token / row_kernel).
+// Without loop sets: 5000 states, V = 128256, batch 17 8.1 / 14.3, batch 25
+// 19.5 / 13.3; V = 32000, batch 98 11.6 / 10.8; tables of masks and next
+// states, V = 8000, 16000 states 263 / 456 (4.6 units a wave), V = 32000, 4000
+// states 290 / 189 (18.6 units).  With a stack, whose per-token walk is the
+// dearer: JSON, V = 50000, batch 39 19.5 / 14.7, V = 128256, batch 17 16.1 /
+// 24.2, batch 21 37.8 / 23.7.  With loop sets alone (200 states): V = 48000,
+// batch 87 5.7 / 8.9, batch 174 9.5 / 9.2, V = 64000, batch 98 10.7 / 8.3;
+// their next states are the per-token walk's (loop sets hold masks only).
+// Automata most of whose rows visit much of the tree (rows_dense) are the
+// per-token walk's: 500 states with 16 of 32 classes live, V = 128256, batch
+// 256 76 / 235, 28 live 179 / 521 (12 live, 2.6 % of the tokens: 58 / 36, row_kernel's).
+bool use_rows(const domino_ctx* h, int64_t batch, bool next) {
+    if (!h->rows_ready || h->walk_pref == 0) return false;
+    if (h->walk_pref == 1) return true;
+    if (h->rows_dense || (next && !h->self_mask.empty())) return false;
+    if (h->stack) return rows_pay(h, batch, 4, 4);
+    return h->self_mask.empty() ? rows_pay(h, batch, 6, 10) : rows_pay(h, batch, 10, 10);
+}
+
+// Whether the whole decode step is row_kernel's (one launch), against the
+// per-token walk with the decode folded in (two launches; bf16 rows on 16-byte
+// boundaries): 5000 states, V = 128256, batch 17 13.8 / 21.3, batch 25 26.9 /
+// 19.1, V = 32000, batch 98 17.1 / 19.1, batch 163 19.5 / 18.2; JSON, V =
+// 50000, batch 39 26.4 / 20.7, V = 128256, batch 17 22.6 / 30.6, batch 21 45.2
+// / 31.2; 200 states, V = 32000, batch 196 15.1 / 14.0, V = 48000, batch 131
+// 13.1 / 15.4, batch 262 18.4 / 14.4, V = 8000, batch 524 12.1 / 18.5.  And
+// against the three kernels one after the other (two launches more): fp32, 200
+// states, V = 32000, batch 32 14.4 / 12.9, V = 64000, batch 4 11.9 / 12.1, batch
+// 8 13.3 / 12.9; 5000 states, V = 32000, batch 22 15.9 / 15.4, V = 128256,
+// batch 5 15.3 / 17.2.
 bool decode_rows(const domino_ctx* h, int64_t batch, bool fusable) {
-    return use_tree(h) || (h->rows_ready && h->walk_pref != 0 &&
-                           batch * h->V >= (fusable ? (int64_t)3 << 20 : (int64_t)1 << 20));
+    if (!h->rows_ready || h->walk_pref == 0) return false;
+    if (h->walk_pref == 1) return true;
+    if (h->rows_dense) return false;
+    if (!fusable) return rows_pay(h, batch, 1, 1);
+    if (h->stack) return rows_pay(h, batch, 4, 4);
+    return h->self_mask.empty() ? rows_pay(h, batch, 6, 10) : rows_pay(h, batch, 16, 16);
 }
 
 int ready_for_compute(domino_ctx* h) {
@@ -1362,7 +1410,17 @@ int domino_step_decode(domino_t h, const int32_t* states_dev, const uint64_t* st
     cudaPointerAttributes pa{};
     const bool on_device = cudaPointerGetAttributes(&pa, logits_dev) == cudaSuccess && pa.type == cudaMemoryTypeDevice;
     if (!on_device) cudaGetLastError();
-    if (decode_rows(h, batch, fusable)) {   // the whole step in one kernel
+    bool rows = decode_rows(h, batch, fusable);
+    const size_t part_bytes = (size_t)batch * (size_t)h->n_windows * sizeof(float4);
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (!rows && fusable && h->d_fpart.n < part_bytes) {
+        // growing the partials buffer synchronises the stream and reallocates,
+        // neither of which a stream capture allows: the first call at a larger
+        // batch must run uncaptured, or take the row kernel, which needs none
+        if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) return cuda_status(cudaGetLastError());
+        rows = cs != cudaStreamCaptureStatusNone && on_device && use_tree(h);
+    }
+    if (rows) {   // the whole step in one kernel
         StepView v = make_view(h);
         return cuda_status(launch_row_decode(v, h->rows, h->env, h->stack, states_dev, stacks_dev, batch, logits_dev,
                                              dtype, row_stride_elems, on_device, mask_dev, argmax_dev, lse_dev, logprobs_dev,
@@ -1378,13 +1436,7 @@ int domino_step_decode(domino_t h, const int32_t* states_dev, const uint64_t* st
                               stream);
     }
     StepView v = make_view(h);
-    const size_t part_bytes = (size_t)batch * (size_t)h->n_windows * sizeof(float4);
     if (h->d_fpart.n < part_bytes) {
-        // growing the partials buffer synchronises the stream and reallocates,
-        // neither of which a stream capture allows: the first call at a larger
-        // batch must run uncaptured
-        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) return cuda_status(cudaGetLastError());
         if (cs != cudaStreamCaptureStatusNone) return DOMINO_E_INVALID_ARG;
         if (cudaStreamSynchronize(st) != cudaSuccess) return cuda_status(cudaGetLastError());
         clear_host_graphs(h);   // recorded host-buffer steps name this buffer

@@ -22,9 +22,15 @@
 // tokens takes 8 to 11 rounds for its 1000 live nodes.  One CTA per row keeps
 // these rounds free of any grid-wide step, and neither the tree nor the
 // transition table is staged.  Measured (GB300, that workload, back to back):
-// batch 256 16.1 us (35.8 us for the walk it replaced, whose CTAs each staged
-// a share of the tree and walked every row in it), batch 1000 52.5 us (94.1),
-// batch 16 14.0 us (17.0); the 20000-state table 2.67 ms (3.25 ms).
+// batch 256 15.7 us (35.8 us for the walk it replaced, whose CTAs each staged
+// a share of the tree and walked every row in it), batch 1000 51.7 us (94.1),
+// batch 32 13.5 us (19.0); the 20000-state table 2.62 ms (3.25 ms).
+//
+// A row with more live nodes than the pool holds is walked token by token
+// instead (every_token), which bounds what a dense state costs: 500 states
+// with 16 of 32 classes live, V = 128256, one row 26 us, 28 classes live 51
+// us.  Small batches and automata most of whose states are like that are the
+// per-token walk's from the start (use_rows, decode_rows in host.cpp).
 //
 // States that loop on most classes (string bodies) allow nearly every token.
 // For the widest such loop sets the host keeps the tokens that stay inside
@@ -38,9 +44,9 @@
 // still in shared memory when its logits are folded (decode.cuh), the cluster
 // merges its slices' results, and the row is advanced by its token.  Measured
 // against the separate kernels before it: 5000 states, V = 128256, batch 256
-// 24.3 us (45.9 us in four launches), batch 1000 85.0 us (127); JSON, V =
-// 152064, batch 128 43.1 us (86.1 us in two launches), with log-probabilities
-// 56.3 us (105), batch 512 104 us (304).
+// 22.5 us (45.9 us in four launches), batch 1000 78.5 us (127); JSON, V =
+// 152064, batch 128 35.5 us (86.1 us in two launches), with log-probabilities
+// 47.5 us (105), batch 512 76.7 us (304).
 //
 // Batches with fewer rows than SMs give each row a cluster of CTAs that share
 // out the row's mask words; each walks the row itself (the walk is latency,
@@ -61,12 +67,12 @@ namespace {
 
 constexpr int kRowThreads = 512;
 constexpr int kRowWarps = kRowThreads / 32;
-constexpr int kRowPool = 2048;        // items a round may leave in the pool (see run())
-constexpr int kRowMargin = 256;
+constexpr int kRowPool = 2048;        // items the pool holds
 constexpr int kRowFan = 8;            // threads per item while there are few
 constexpr int kRowSmall = 512;        // ranges of 2 to kRowSmallTokens tokens left to the whole CTA
 constexpr int kRowSmallTokens = 64;
 constexpr int kRowBig = 128;          // longer ranges
+constexpr int kRowSpawn = 2048;       // exits taken at a time
 constexpr int kRowExits = 512;        // loop subtrees whose exits are still to be walked
 constexpr int kRowLoopMin = 4;        // fewest tokens of a subtree taken as a loop subtree
 constexpr int kRowMaxDevices = 64;
@@ -111,14 +117,12 @@ struct RowLayout {
     int mask, items, bits, range, exits, pre, keep, dec, total;
 };
 
-__host__ __device__ inline int row_pool_cap(int reserve) { return kRowPool + reserve; }
-
-__host__ __device__ inline RowLayout row_layout(int slice_words, int reserve, bool stack, bool loops, bool decode) {
+__host__ __device__ inline RowLayout row_layout(int slice_words, bool stack, bool loops, bool decode) {
     RowLayout L{};
     int o = 16;
     L.mask = o;   o += align16(slice_words * 4) + 16;
-    L.items = o;  o += align16(2 * row_pool_cap(reserve) * 8);
-    L.bits = o;   o += stack ? align16(2 * row_pool_cap(reserve) * 4) : 0;
+    L.items = o;  o += align16(2 * kRowPool * 8);
+    L.bits = o;   o += stack ? align16(2 * kRowPool * 4) : 0;
     L.range = o;  o += (kRowSmall + kRowBig) * 16;
     L.exits = o;  o += loops ? kRowExits * 16 : 0;
     L.pre = o;    o += align16((kRowThreads + 1) * 4);
@@ -129,8 +133,9 @@ __host__ __device__ inline RowLayout row_layout(int slice_words, int reserve, bo
 }
 
 struct RowShared {
-    int4 st[3];      // by round: {items added, the first place that did not fit, lists half full, 0}
-    int back;        // items put back
+    int4 st[3];      // by round: {items added, the pool is full, lists half full, 0}
+    uint4 rc;        // the row's configuration (read_row)
+    int back;        // exits walked (spawn_exits)
     int nrange[2], nexit;
     int wsum[kRowWarps];
 };
@@ -156,6 +161,106 @@ __device__ __forceinline__ int find_range(const int* pre, int n, int f) {
         else hi = mid;
     }
     return lo;
+}
+
+// The state a token's class string ends in, walked from (s, bits, depth) over
+// the automaton's own table; 0 when it dies, and for EOS and empty tokens.
+template <bool STACK>
+__device__ __forceinline__ uint32_t token_end(const StepView& v, const RowTree& t, int32_t tk, uint32_t s, uint32_t& bits,
+                                              uint32_t& depth) {
+    const uint8_t* rec = t.trec + 32 * (size_t)tk;   // {length (255: or more), classes}
+    int len = (int)__ldg(rec);
+    const uint8_t* tail = v.tail;
+    const uint8_t* head = rec + 1;
+    if (len > 31) {   // the arena's record
+        const int p = __ldg(v.pos_of + tk);
+        len = (int)(__ldg(v.info + p) >> 16);
+        head = reinterpret_cast<const uint8_t*>(v.head + 2 * (size_t)p);
+        if (len > kInlineBytes) tail += __ldg(v.tail_off + p);
+    }
+    using E = typename std::conditional<STACK, uint32_t, uint16_t>::type;
+    Tab<E, kDenseGlobal> tab;
+    tab.dense = reinterpret_cast<const E*>(STACK ? (const void*)v.t32 : (const void*)v.t16);
+    tab.K = (uint32_t)v.K;
+    debug_bounds(tab, v);
+    return len > 0 ? walk<STACK, 0>(tab, v.ret, (uint32_t)v.max_depth, s, bits, depth, head, len, tail) : 0u;
+}
+
+// The CTA's part of a row by walking each of its tokens from the row's
+// configuration rc, kAtOnce words of 32 tokens per warp at a time: for rows
+// with so many live nodes that the pool fills (a state that lets most classes
+// through without looping).  Bound by the latency of the table reads, hence
+// several tokens of a thread in flight; a warp's 32 tokens are a mask word, so
+// whole words are stored.  Not inlined: its registers would spill beside the
+// decode's (JSON, V = 152064, batch 512, with log-probabilities 152 against
+// 142 us).
+template <bool STACK, int OUT>
+__device__ __noinline__ void every_token(const StepView& v, const RowTree& t, const uint4& rc, uint32_t* s_mask, int nw,
+                                         int tok0, int ntok, int32_t* nrow, const char* ahead) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    using E = typename std::conditional<STACK, uint32_t, uint16_t>::type;
+    constexpr int kAtOnce = STACK ? 2 : 4;
+    const E* table = reinterpret_cast<const E*>(STACK ? (const void*)v.t32 : (const void*)v.t16);
+    for (int w = warp * kAtOnce; w < nw; w += kRowWarps * kAtOnce) {
+        uint4 rec[kAtOnce];   // {length, the first 15 classes}, shifted by a byte per step
+        uint32_t s[kAtOnce], bits[kAtOnce], depth[kAtOnce];
+        int len[kAtOnce];
+#pragma unroll
+        for (int q = 0; q < kAtOnce; ++q) {
+            const int x = (w + q) * 32 + lane;
+            rec[q] = x < ntok ? __ldg(reinterpret_cast<const uint4*>(t.trec + 32 * (size_t)(tok0 + x)))
+                              : make_uint4(0u, 0u, 0u, 0u);
+        }
+#pragma unroll
+        for (int q = 0; q < kAtOnce; ++q) {
+            len[q] = (int)(rec[q].x & 0xFFu);   // EOS and empty tokens: 0
+            s[q] = len[q] ? rc.x : 0u;
+            bits[q] = rc.y;
+            depth[q] = rc.z;
+        }
+        for (int i = 0; i < 15; ++i) {
+            bool more = false;
+#pragma unroll
+            for (int q = 0; q < kAtOnce; ++q) {
+                rec[q].x = __funnelshift_r(rec[q].x, rec[q].y, 8);
+                rec[q].y = __funnelshift_r(rec[q].y, rec[q].z, 8);
+                rec[q].z = __funnelshift_r(rec[q].z, rec[q].w, 8);
+                rec[q].w >>= 8;
+            }
+            uint32_t e[kAtOnce];
+#pragma unroll
+            for (int q = 0; q < kAtOnce; ++q)
+                e[q] = s[q] != 0u && i < len[q] ? (uint32_t)__ldg(table + (size_t)s[q] * v.K + (rec[q].x & 0xFFu)) : 0u;
+#pragma unroll
+            for (int q = 0; q < kAtOnce; ++q) {
+                if (s[q] != 0u && i < len[q]) {
+                    s[q] = e[q];
+                    if constexpr (STACK) s[q] = pda_apply(e[q], bits[q], depth[q], (uint32_t)v.max_depth, v.ret);
+                }
+                more |= s[q] != 0u && i + 1 < len[q];
+            }
+            if (!__any_sync(0xffffffffu, more)) break;
+        }
+#pragma unroll
+        for (int q = 0; q < kAtOnce; ++q) {
+            const int x = (w + q) * 32 + lane, tk = tok0 + x;
+            if (s[q] != 0u && len[q] > 15) {   // longer: from its start
+                bits[q] = rc.y;
+                depth[q] = rc.z;
+                s[q] = token_end<STACK>(v, t, tk, rc.x, bits[q], depth[q]);
+            }
+            const unsigned word = __ballot_sync(0xffffffffu, s[q] != 0u);
+            if (w + q >= nw) continue;
+            if (lane == 0) s_mask[w + q] = word;
+            if constexpr (OUT == kRowBf16 || OUT == kRowF32) {
+                if (ahead && s[q] != 0u)
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(ahead + (size_t)tk * (OUT == kRowBf16 ? 2 : 4)));
+            }
+            if constexpr (OUT == kRowNext) {
+                if (nrow && x < ntok) nrow[tk] = (int32_t)s[q];
+            }
+        }
+    }
 }
 
 // One row's walk.
@@ -310,17 +415,9 @@ struct RowWalk {
     // Expands the pool's n items until none are left.  In a round every
     // thread takes one item from the pool's top (kRowFan threads share one
     // while there are few) and adds its live children: to the pool's other
-    // half when the round takes all items, else in their place.
-    //
-    // Neither half can overflow kRowPool + t.reserve items.  A warp whose
-    // children would pass kRowPool - kRowThreads - kRowMargin puts its items
-    // back instead.  When that goes for all of a round's items, or when the
-    // pool is nearly full, a round takes only as many items as could all have
-    // t.max_kids children and stay within kRowPool, or else a single one:
-    // then the pool is walked depth first, strictly from its top, and the
-    // item's subtree adds at most t.reserve (the host's bound over the tree).
-    __device__ __forceinline__ void run(int n, int cap) const {
-        bool stuck = false;   // no item of the last round was expanded
+    // half when the round takes all items, else in their place.  false: the
+    // pool was full (every_token() takes the row).
+    __device__ __forceinline__ bool run(int n) const {
         int half = 0;   // where the items lie
         Tokens before{0u, 0u, 0u, 0u};
         for (int r = 0;; r = r == 2 ? 0 : r + 1) {
@@ -330,22 +427,16 @@ struct RowWalk {
                 if (n == 0) break;
                 half = 0;
             }
-            const bool careful = stuck || n > kRowPool - kRowMargin;
-            int take = min(n, kRowThreads);
-            if (careful) take = max(1, min(take, (kRowPool - n) / t.max_kids));
+            const int take = min(n, kRowThreads);
             const int base = n - take;
             const bool fan = take * kRowFan <= kRowThreads;
             const int i = fan ? tid / kRowFan : tid;
             bool lead = !fan || (tid & (kRowFan - 1)) == 0;   // this thread answers for its item
             Item it{0u, 0u, 0u, 0u};
             if (i < take) it = get(half + base + i);
-            if (tid == 0) {
-                sh.st[r == 2 ? 0 : r + 1] = make_int4(0, INT_MAX, 0, 0);   // read by all two rounds ago
-                sh.back = 0;
-            }
+            if (tid == 0) sh.st[r == 2 ? 0 : r + 1] = make_int4(0, 0, 0, 0);   // read by all two rounds ago
             if (base > 0) __syncthreads();   // the items are read before others take their place
-            else half ^= cap;
-            bool failed = false;
+            else half ^= kRowPool;
             if ((fan ? (tid & ~31) / kRowFan : tid & ~31) < take) {   // warps with an item
               for (bool split = fan;;) {
                 Node x = read(it, lead, before, st);
@@ -401,10 +492,8 @@ struct RowWalk {
                     if (lane == 0) first = base + atomicAdd(&st->x, tot);
                     first = __shfl_sync(0xffffffffu, first, 0);
                     at += half + first;
-                    if (first + tot > kRowPool - kRowThreads - kRowMargin && !careful) {
-                        failed = true;
-                        x.em.n = 0u;
-                        if (lane == 0) atomicMin(&st->y, first);
+                    if (first + tot > kRowPool) {
+                        st->y = 1;
                     } else if constexpr (WIDE) {
                         for (int k = split ? tid & (kRowFan - 1) : 0; c > 0; k += split ? kRowFan : 1, --c) {
                             const uint32_t child = x.first_child + (uint32_t)k;
@@ -425,24 +514,12 @@ struct RowWalk {
             }
             __syncthreads();   // the next round's items are in place
             const int4 q = *st;
-            stuck = false;
+            if (q.y) return false;
             n = base + q.x;
-            if (q.y != INT_MAX) {   // some did not fit
-                if (failed) {
-                    const unsigned b = __ballot_sync(0xffffffffu, lead && it.s != 0u);
-                    int first = 0;
-                    if (lane == 0) first = atomicAdd(&sh.back, __popc(b));
-                    first = __shfl_sync(0xffffffffu, first, 0);
-                    if (lead && it.s != 0u) put(half + q.y + first + __popc(b & ((1u << lane) - 1u)), it);
-                }
-                __syncthreads();
-                n = q.y + *reinterpret_cast<volatile int*>(&sh.back);
-                stuck = q.y == base;   // none did
-                __syncthreads();
-            }
             if (q.z) ranges();
         }
         emit(before, &sh.st[0]);
+        return true;
     }
 
     __device__ __forceinline__ uint32_t shfl_lead(uint32_t m) const {
@@ -495,7 +572,7 @@ struct RowWalk {
             const int total = prefix(nx, tid < nx ? (int)s_exit[tid].y : 0);
             // as many as fit this time, the last entries first (the list is a
             // stack); an entry taken in part is cut back
-            const int f0 = max(0, total - kRowPool);
+            const int f0 = max(0, total - kRowSpawn);
             for (int b = f0 + warp * 32; b < total; b += kRowThreads) {
                 const int f = b + lane;
                 Item x{0u, 0u, 0u, 0u};
@@ -540,28 +617,28 @@ struct RowWalk {
     __device__ __forceinline__ void ranges() const {
         const int ns = min(*reinterpret_cast<volatile int*>(&sh.nrange[0]), kRowSmall);
         const int nb = min(*reinterpret_cast<volatile int*>(&sh.nrange[1]), kRowBig);
+        constexpr int kUnroll = STACK ? 8 : 4;   // 8 spill beside a DFA's folded decode: +0.8 us at 128256x256
         // short ones: four threads each
         for (int i = tid / 4; i < ns; i += kRowThreads / 4) {
             const uint4 x = s_range[i];
-            for (uint32_t j = tid & 3; j < x.y; j += 32) {
-                int tk[8];
-                uint32_t out[8];   // the filter's byte: greater than the range's depth drops the token
+            for (uint32_t j = tid & 3; j < x.y; j += 4 * kUnroll) {
+                int tk[kUnroll];
+                uint32_t out[kUnroll];   // the filter's byte: greater than the range's depth drops the token
                 const int32_t* p = t.dtok + x.x + j;
                 const uint8_t* k = t.keeps + (x.w ? (size_t)((x.w >> 8) - 1u) * t.n_dtok + x.x + j : 0);
 #pragma unroll
-                for (int q = 0; q < 8; ++q) {
+                for (int q = 0; q < kUnroll; ++q) {
                     tk[q] = j + 4 * q < x.y ? __ldg(p + 4 * q) : -1;
                     out[q] = x.w && j + 4 * q < x.y ? __ldg(k + 4 * q) : 0u;
                 }
 #pragma unroll
-                for (int q = 0; q < 8; ++q)
+                for (int q = 0; q < kUnroll; ++q)
                     if (tk[q] >= 0 && out[q] <= (x.w & 0xFFu)) emit(tk[q], x.z);
             }
         }
         if (nb > 0) {   // long ones: the CTA over all of them
             const int total = prefix(nb, tid < nb ? (int)s_range[kRowSmall + tid].y : 0);
             // a warp takes 256 tokens in a row: they lie in a few ranges
-            constexpr int kUnroll = STACK ? 8 : 4;   // 8 spill beside a DFA's folded decode: +0.8 us at 128256x256
             for (int f0 = warp * 32 * kUnroll; f0 < total; f0 += kRowThreads * kUnroll) {
                 int tk[kUnroll];
                 uint32_t st[kUnroll], out[kUnroll];
@@ -599,31 +676,16 @@ struct RowWalk {
 
 // C.update() of a row in configuration rc (read_row) by its token tk, or by
 // -1: as advance_row, with the token's classes in one record.
-template <bool STACK, int CLS>
+template <bool STACK>
 __device__ __forceinline__ void update(const StepView& v, const RowTree& t, const uint4& rc, int32_t tk, int b,
                                        int32_t* states_out, uint64_t* stacks_out) {
     uint32_t s = 0, bits = 0, depth = 0;
     if (tk < 0 || tk == v.eos_id) {
         s = (uint32_t)v.start;   // the sequence ended; the next one starts from init
     } else if (rc.w & 1u) {
-        const uint8_t* rec = t.trec + 32 * (size_t)tk;   // {length (255: or more), classes}
-        int len = (int)__ldg(rec);
-        const uint8_t* tail = v.tail;
-        const uint8_t* head = rec + 1;
-        if (len > 31) {   // the arena's record
-            const int p = __ldg(v.pos_of + tk);
-            len = (int)(__ldg(v.info + p) >> 16);
-            head = reinterpret_cast<const uint8_t*>(v.head + 2 * (size_t)p);
-            if (len > kInlineBytes) tail += __ldg(v.tail_off + p);
-        }
         bits = rc.y;
         depth = rc.z;
-        using E = typename std::conditional<STACK, uint32_t, uint16_t>::type;
-        Tab<E, kDenseGlobal> tab;
-        tab.dense = reinterpret_cast<const E*>(STACK ? (const void*)v.t32 : (const void*)v.t16);
-        tab.K = (uint32_t)v.K;
-        debug_bounds(tab, v);
-        s = len > 0 ? walk<STACK, 0>(tab, v.ret, (uint32_t)v.max_depth, rc.x, bits, depth, head, len, tail) : 0u;
+        s = token_end<STACK>(v, t, tk, rc.x, bits, depth);
         if (s == 0) bits = depth = 0;
     }
     states_out[b] = (int32_t)s;
@@ -636,7 +698,7 @@ __global__ void __launch_bounds__(kRowThreads, 2)
                const __grid_constant__ RowArgs a, const RowList list) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ RowShared sh;
-    const RowLayout L = row_layout(a.slice_words, t.reserve, STACK, t.n_loops > 0, OUT == kRowBf16 || OUT == kRowF32);
+    const RowLayout L = row_layout(a.slice_words, STACK, t.n_loops > 0, OUT == kRowBf16 || OUT == kRowF32);
     uint32_t* s_mask = reinterpret_cast<uint32_t*>(smem + L.mask);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int row = blockIdx.x / a.slices, slice = blockIdx.x - row * a.slices;
@@ -649,19 +711,23 @@ __global__ void __launch_bounds__(kRowThreads, 2)
     if (tid == 0) {
         s_mask[-1] = s_mask[a.slice_words] = 0u;
         sh.nrange[0] = sh.nrange[1] = sh.nexit = 0;
-        sh.st[0] = make_int4(0, INT_MAX, 0, 0);
+        sh.st[0] = make_int4(0, 0, 0, 0);
     }
     pdl_wait();
     pdl_trigger();
     if (row >= list.rows(a.batch)) return;   // the whole cluster
-    // the row's configuration (invalid ones set the error word, once per row)
-    uint4 rc;
-    if (a.row_is_state) {
+    // The row's configuration (invalid ones set the error word, once per row),
+    // in shared memory: one in pinned host memory crosses the host link once
+    // per CTA, not once per warp (128256 tokens, batch 16, states read there:
+    // 33.2 -> 21.4 us), and no registers are held for it during the walk.
+    if (tid == 0) {
         const uint32_t q = (uint32_t)row;
-        rc = make_uint4(q, 0u, 0u, 1u | (((__ldg(v.accept_bits + (q >> 5)) >> (q & 31u)) & 1u) ? 2u : 0u));
-    } else {
-        rc = read_row_rw(v, a.states, a.stacks, list.row(row), tid == 0 && slice == 0);
+        sh.rc = a.row_is_state
+                    ? make_uint4(q, 0u, 0u, 1u | (((__ldg(v.accept_bits + (q >> 5)) >> (q & 31u)) & 1u) ? 2u : 0u))
+                    : read_row_rw(v, a.states, a.stacks, list.row(row), slice == 0);
     }
+    __syncthreads();
+    const uint4 rc = sh.rc;
     // the state the walk starts from, and its loop set
     uint32_t s0 = (rc.w & 1u) ? rc.x : 0u, root = 0u;
     if (t.start) {
@@ -669,7 +735,6 @@ __global__ void __launch_bounds__(kRowThreads, 2)
         s0 = w.x;
         if (w.y != 0xFFFFFFFFu) {   // the tokens that stay inside the set, then the walk of the others
             const uint32_t* loop = t.loopbits + (size_t)w.y * v.W + w0;
-            __syncthreads();   // the mask has been cleared
             for (int j = tid; j < nw; j += kRowThreads) s_mask[j] = __ldg(loop + j);
             root = (uint32_t)t.loop_root[w.y];
         }
@@ -699,10 +764,15 @@ __global__ void __launch_bounds__(kRowThreads, 2)
                                       nrow, ahead, tok0, ntok, tid, lane, warp};
     if (tid == 0) wk.put(0, {root, s0, rc.z, rc.y});
     __syncthreads();   // the mask (and the next states) are filled
-    wk.run(s0 != 0u ? 1 : 0, row_pool_cap(t.reserve));
-    __syncthreads();
-    wk.ranges();
-    if (tid == 0 && (rc.w & 2u) && v.eos_id >= 0) wk.emit(v.eos_id, rc.x);   // EOS keeps the state
+    if (wk.run(s0 != 0u ? 1 : 0)) {
+        __syncthreads();
+        wk.ranges();
+    } else {
+        every_token<STACK, OUT>(v, t, sh.rc, s_mask, nw, tok0, ntok, nrow, ahead);
+        __syncthreads();   // whole words were stored
+    }
+    if (tid == 0 && v.eos_id >= 0 && (static_cast<volatile uint32_t&>(sh.rc.w) & 2u))
+        wk.emit(v.eos_id, static_cast<volatile uint32_t&>(sh.rc.x));   // EOS keeps the state
     __syncthreads();
     if (a.mask) {
         uint32_t* mrow = a.mask + (size_t)row * v.W + w0;
@@ -732,7 +802,7 @@ __global__ void __launch_bounds__(kRowThreads, 2)
             a.argmax[b] = tk;
             if (a.lse) a.lse[b] = lse;
             // every CTA of the row has read its configuration (the outputs may alias it)
-            if (a.states_out) update<STACK, CLS>(v, t, rc, tk, b, a.states_out, a.stacks_out);
+            if (a.states_out) update<STACK>(v, t, sh.rc, tk, b, a.states_out, a.stacks_out);
         }
         if (a.slices > 1) cluster_wait();
     }
@@ -765,7 +835,7 @@ cudaError_t launch_row_t(const StepView& v, const RowTree& t, const LaunchEnv& e
         s *= 2;
     a.slices = s;
     a.slice_words = ((v.W + s - 1) / s + 3) / 4 * 4;
-    const RowLayout L = row_layout(a.slice_words, t.reserve, STACK, t.n_loops > 0, OUT == kRowBf16 || OUT == kRowF32);
+    const RowLayout L = row_layout(a.slice_words, STACK, t.n_loops > 0, OUT == kRowBf16 || OUT == kRowF32);
     if (L.total > env.max_smem_optin) return cudaErrorInvalidConfiguration;
     auto kern = row_kernel<STACK, CLS, OUT>;
     static int configured[kRowMaxDevices] = {0};
@@ -834,12 +904,8 @@ cudaError_t launch_row_decode(const StepView& v, const RowTree& t, const LaunchE
     return launch_row(v, t, env, stack, a, dtype, RowList{nullptr, nullptr, 0}, st);
 }
 
-// The pool entries that walking a node alone, depth first, can add: its
-// children replace it, then the deepest of them is walked.
-int32_t row_reserve(int32_t kids, int32_t below) { return std::max(0, kids - 1) + below; }
-
-int row_smem_bytes(int32_t n_words, int32_t reserve, bool stack, bool loops) {
-    return row_layout(std::min(n_words, kRowSliceWords) + 4, reserve, stack, loops, true).total;
+int row_smem_bytes(int32_t n_words, bool stack, bool loops) {
+    return row_layout(std::min(n_words, kRowSliceWords) + 4, stack, loops, true).total;
 }
 
 }  // namespace domino

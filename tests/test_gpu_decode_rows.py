@@ -161,8 +161,11 @@ def test_infinite_logits(dt):
 @pytest.mark.parametrize("dt,offset,pad", [(B.DTYPE_BF16, 0, 5), (B.DTYPE_BF16, 3, 0), (B.DTYPE_F32, 0, 0),
                                            (B.DTYPE_F32, 1, 2)])
 @pytest.mark.parametrize("grammar,batch", [("json", 60), ("json", 170), ("sparse", 5), ("sparse", 200)])
-def test_whole_step_in_one_kernel(dt, offset, pad, grammar, batch):
+@pytest.mark.parametrize("walk", ["tree", None])
+def test_whole_step_in_one_kernel(dt, offset, pad, grammar, batch, walk, monkeypatch):
     import oracle
+    if walk:
+        monkeypatch.setenv("DOMINO_WALK", walk)
     rng = np.random.default_rng(batch)
     V = 19997
     v = synth.random_vocab(rng, V, bytes(range(256)), synth.geometric_lengths(4.0, 32), synth._mixed_bytes)

@@ -1,9 +1,10 @@
 """The walk with one CTA (or a cluster of CTAs) per row (rows.cu) against the
 oracle, bit-exact, where it can go wrong: 1 to 8 CTAs per row, class counts
-around the 32- and 64-bit masks and beyond, trees wider than the pool (items
-put back, the depth-first walk), token ranges longer than the lists, loop sets
+around the 32- and 64-bit masks and beyond, rows with more live nodes than the
+pool holds (walked token by token), token ranges longer than the lists, loop sets
 (bitmap, the tree of the remainders, subtrees entered in a looping state,
-depths beyond a byte), equivalent states, a bracket stack.  Output buffers
+depths beyond a byte), equivalent states, a bracket stack.  Each case runs with
+the walk forced (DOMINO_WALK=tree) and as the sizes choose it.  Output buffers
 start as 0xAB bytes (tests/poison.py)."""
 import functools
 import os
@@ -28,6 +29,14 @@ def _built():
         pytest.skip("no CUDA device")
     from paper_2403_06988_gb300 import build
     build.build()
+
+
+@pytest.fixture(params=["tree", None], ids=["forced", "chosen"], autouse=True)
+def walk(request, monkeypatch):
+    if request.param:
+        monkeypatch.setenv("DOMINO_WALK", request.param)   # read when a handle is created
+    else:
+        monkeypatch.delenv("DOMINO_WALK", raising=False)
 
 
 def dev(a):
@@ -153,3 +162,72 @@ def test_rows_many_tokens_per_node():
     a = synth.Automaton(delta=delta, live=live, accepting=live.copy(), start=1, rules=None, max_depth=0, name="two")
     v = random_tokens(rng, 40003, bytes(range(30, 128)), 6)
     check(a, v, np.tile(np.arange(4, dtype=np.int32), 14)[:53])
+
+
+@pytest.mark.parametrize("stack", [False, True])
+@pytest.mark.parametrize("batch", [3, 90, 400])
+def test_rows_full_pools_with_long_tokens(stack, batch):
+    """Two states that lead to one another on all but one of 40 letters, with
+    brackets between them: a row's live nodes pass any pool.  Tokens around the
+    lengths of the token records' parts (15, 31, 32 classes) and beyond."""
+    rng = np.random.default_rng(11)
+    b = synth._Builder()
+    A, C = b.state("a", accepting=True), b.state("c", accepting=True)
+    letters = bytes(range(64, 104))
+    b.edge(A, letters[1:], C)
+    b.edge(C, letters[:-1], A)
+    if stack:
+        b.push(A, b"(", 0, C)
+        b.push(C, b"(", 1, A)
+        b.pop(A, b")", 1, (C, A, C))
+        b.pop(C, b")", 0, (A, C, A))
+    a = b.build(A, 5 if stack else 0, "toggle")
+    al = np.frombuffer(letters + (b"()" if stack else b""), np.uint8)
+    toks = set()
+    for L in (14, 15, 16, 30, 31, 32, 33, 60):
+        for _ in range(20):
+            toks.add(rng.choice(al, L).tobytes())
+    while len(toks) < 9000:
+        toks.add(rng.choice(al, int(rng.integers(1, 6))).tobytes())
+    toks = sorted(toks)
+    rng.shuffle(toks)
+    toks = [bytes(t) for t in toks]
+    v = synth.Vocab.from_tokens(toks[:700] + [b""] + toks[700:], eos_id=700)
+    states = rng.integers(0, 3, batch).astype(np.int32)
+    stacks = None
+    if stack:
+        stacks = np.array([synth.pack_stack(list(rng.integers(0, 2, int(rng.integers(0, 6))))) for _ in range(batch)],
+                          np.uint64)
+        stacks[states == 0] = 0
+    check(a, v, states, stacks, want_next=True)
+
+
+def test_first_step_in_a_capture():
+    """A step whose walk needs scratch is recorded without a call before it."""
+    from paper_2403_06988_gb300 import _binding as B
+    rng = np.random.default_rng(12)
+    a = synth.random_sparse_dfa(rng, 300)
+    v = synth.random_vocab(rng, 8000, bytes(range(256)), synth.geometric_lengths(4.0, 16), synth._mixed_bytes)
+    states = torch.from_numpy(rng.integers(1, 300, 6).astype(np.int32)).cuda()
+    lg = torch.randn((6, 8000), device="cuda", generator=torch.Generator("cuda").manual_seed(1)).to(torch.bfloat16)
+    got = []
+    for capture in (True, False):
+        d = Domino.from_parts(a, v, device=0)
+        mask = poison.empty((6, d.info()["n_words"]), torch.int32)
+        arg, out = poison.empty(6, torch.int32), poison.empty(6, torch.int32)
+        torch.cuda.synchronize()
+        run = lambda: B.domino_step_decode(d.h, states, None, 6, lg.data_ptr(), B.DTYPE_BF16, 8000, mask, arg, None, None,
+                                           out, None, torch.cuda.current_stream().cuda_stream)
+        if capture:
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g):
+                run()
+            g.replay()
+        else:
+            run()
+        torch.cuda.synchronize()
+        got.append([t.cpu().numpy().copy() for t in (mask, arg, out)])
+        assert d.device_error() == 0
+        d.close()
+    for x, y in zip(*got):
+        assert_exact(x, y, "recorded")
