@@ -206,6 +206,19 @@ def csrc_digest() -> str:
     return hs.hexdigest()[:16]
 
 
+def takes_rows(info, dev_id, batch, V, decode=False, fusable=True):
+    """Whether the call is row_kernel's (use_rows and decode_rows in host.cpp, for the launch counts)."""
+    import torch
+    sms = torch.cuda.get_device_properties(dev_id).multi_processor_count
+    if not decode:
+        first, more = (4, 4) if info["has_stack"] else (6, 10) if info["walk_tree"] else (10, 10)
+    elif not fusable:
+        first, more = 1, 1
+    else:
+        first, more = (4, 4) if info["has_stack"] else (6, 10) if info["walk_tree"] else (16, 16)
+    return batch * V >= (first + (batch - 1) // (2 * sms) * more) << 19
+
+
 def ncu_traffic(name: str) -> dict:
     """DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from
     the committed ncu summary, per kernel; a kernel whose source changed since
@@ -460,8 +473,7 @@ def run_precompute(args, dist: Dist):
         "e2e": {"value": n * Q * V * Ke / (e2e_ms / 1e3), "unit": UNIT, "h2d_bytes_per_step": 0,
                 "d2h_bytes_per_step": out_bytes, "steps": Ke,
                 "api": "domino_precompute_table + copy of the table to pinned host memory"},
-        # the tree walk: tree_clear_kernel then tree_tile_kernel; else one step_kernel
-        "gpu_launches": K * (2 if info["walk_tree"] else 1),
+        "gpu_launches": K,   # row_kernel or step_kernel
         "clocks": sampler.summary(),
     }
     if dist.rank == 0 and n == 1 and not args.no_cpu_baseline:
@@ -513,14 +525,14 @@ def run_domino(args, dist: Dist):
     p_mask, p_arg, p_lse = mask.data_ptr(), argmax.data_ptr(), lse.data_ptr()
     p_lp = logprobs.data_ptr() if logprobs is not None else None
     p_logits = [t.data_ptr() for t in logits]
-    # one step = one call. With the per-token walk and bf16 logits: the mask
-    # step with the greedy decode folded in, then the per-row merge that also
-    # advances each row. With the prefix-tree walk (two launches: clear, tree
-    # tiles) or fp32 logits: mask step, logits pass, update. Plus the
-    # log-probs pass where the workload asks for them.
-    walk_launches = 2 if info.get("walk_tree") else 1
-    fused = w.logits_dtype == "bf16" and not info.get("walk_tree")
-    launches_per_step = (2 if fused else walk_launches + 2) + (1 if w.want_logprobs else 0)
+    # one step = one call: row_kernel alone; or, for few (row, token) pairs and
+    # bf16 logits, the per-token walk with the greedy decode folded in, then the
+    # per-row merge that also advances each row, plus the log-probs pass where
+    # the workload asks for them; or (fp32) mask step, logits pass, update.
+    rows_decode = takes_rows(info, dev_id, Bsz, V, decode=True, fusable=w.logits_dtype == "bf16")
+    rows_mask = takes_rows(info, dev_id, Bsz, V)
+    fused = not rows_decode and w.logits_dtype == "bf16"
+    launches_per_step = 1 if rows_decode else 2 + (1 if w.want_logprobs else 0) if fused else 3
 
     def step(i, stream_ptr):
         rc = L.domino_step_decode(h, p_states, p_stacks, Bsz, p_logits[i % nbuf], dtype_code, V, p_mask, p_arg, p_lse,
@@ -620,11 +632,11 @@ def run_domino(args, dist: Dist):
             raise RuntimeError("mask_sample failed")
     # the other mask walk, on a second handle: the prefix tree (Alg. 2's
     # subterminal tree over byte classes) and the per-token walk each timed alone
-    walk_kind = "prefix tree" if info.get("walk_tree") else "per token"
-    os.environ["DOMINO_WALK"] = "token" if info.get("walk_tree") else "tree"
+    walk_kind = "prefix tree" if rows_mask else "per token"
+    os.environ["DOMINO_WALK"] = "token" if rows_mask else "tree"
     d_other = Domino.from_parts(a, v, device=dev_id)
     del os.environ["DOMINO_WALK"]
-    other_kind = "prefix tree" if d_other.info().get("walk_tree") else "per token"
+    other_kind = "per token" if rows_mask else "prefix tree"
     h_other = d_other.h
 
     def k_step_other(i, sp):
@@ -845,6 +857,7 @@ def run_domino(args, dist: Dist):
                         "dram_bytes_ncu": traffic.get("step_decode_fused") if fused else None,
                         "note": ("the timed step's mask + decode: the mask step folds the allowed logits of each "
                                  "tile (then a per-row merge; log-probs in one more pass where asked for)") if fused
+                        else "the timed step's mask and decode, one kernel a row" if rows_decode
                         else ("the timed step's mask + decode + update: the mask step, the logits pass, "
                               "then the update, back to back")},
         "advance": {"us": per_kernel["advance"] * 1e3},
@@ -859,7 +872,7 @@ def run_domino(args, dist: Dist):
     sm_clk = float(peaks.get("sm_max_mhz", 2070.0)) * 1e6
     lookup_peak = torch.cuda.get_device_properties(dev_id).multi_processor_count * 32 * sm_clk / 1e9
     kernels["step_mask"]["walk"] = walk_kind
-    kernels["step_mask_" + ("token" if info.get("walk_tree") else "tree")] = {
+    kernels["step_mask_" + ("token" if rows_mask else "tree")] = {
         "us": per_kernel["step_mask_other"] * 1e3, "walk": other_kind,
         "checks_per_s": Bsz * V / (per_kernel["step_mask_other"] * 1e-3)}
     if walk is not None:
@@ -875,9 +888,9 @@ def run_domino(args, dist: Dist):
                     "note": ("walk bound by shared-memory gathers and issue, not HBM; the mask step timed alone "
                              "(in the timed step the same kernel also folds the logits: kernels.step_decode)")
                     if fused else
-                            ("the prefix-tree mask step (clear + tree-tile kernels, one call) timed alone as it runs "
-                             "in the step; units are the lookups the plain per-token definition makes, of which "
-                             "the tree walk makes fewer (shared prefixes walked once)")}
+                            ("the prefix-tree mask step (row_kernel) timed alone; in the timed step the same kernel "
+                             "also folds the logits and advances the rows; units are the lookups the plain per-token "
+                             "definition makes, of which the tree walk makes fewer (shared prefixes walked once)")}
     else:
         roofline = {"kernel": "mask_logits", "bound": "hbm", "achieved": gbs, "peak": hbm_peak, "unit": "GB/s",
                     "frac": gbs / hbm_peak, "traffic": traffic.get("mask_logits"),

@@ -100,9 +100,10 @@ typedef struct {
     int32_t table_in_smem; /* 1 when the transition table is staged in shared memory */
     int32_t device;        /* CUDA ordinal, -1 for a host-only handle */
     int64_t device_bytes;  /* device memory the handle owns */
-    int32_t walk_tree;     /* 1: the mask step walks the vocabulary's prefix tree (domino_get_prefix_tree);
-                              0: it walks every token on its own */
-    int32_t tree_units;    /* subtrees the tree walk deals out (0 without a tree) */
+    int32_t walk_tree;     /* 1: masks and next states may be walked over the vocabulary's prefix tree
+                              (domino_get_prefix_tree); 0: masks of large batches only, next states never.
+                              Small calls walk every token on its own either way */
+    int32_t tree_units;    /* units of that tree (0 without a tree) */
 } domino_info;
 
 /* Creates a handle on CUDA device `cuda_device` (it becomes the current device
