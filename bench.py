@@ -211,11 +211,11 @@ def takes_rows(info, dev_id, batch, V, decode=False, fusable=True):
     import torch
     sms = torch.cuda.get_device_properties(dev_id).multi_processor_count
     if not decode:
-        first, more = (4, 4) if info["has_stack"] else (6, 10) if info["walk_tree"] else (10, 10)
+        first, more = (4, 4) if info["has_stack"] else (6, 5) if info["walk_tree"] else (10, 2)
     elif not fusable:
         first, more = 1, 1
     else:
-        first, more = (4, 4) if info["has_stack"] else (6, 10) if info["walk_tree"] else (16, 16)
+        first, more = (4, 4) if info["has_stack"] else (6, 5) if info["walk_tree"] else (16, 6)
     return batch * V >= (first + (batch - 1) // (2 * sms) * more) << 19
 
 

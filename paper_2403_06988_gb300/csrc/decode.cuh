@@ -24,7 +24,7 @@ enum Fold : int {
     kFoldSample = 2,   // Gumbel-max draw
 };
 
-constexpr int kDecodeThreads = 512;
+constexpr int kDecodeThreads = 512;   // a CTA's, where nothing else is said
 constexpr int kDecodeWarps = kDecodeThreads / 32;
 constexpr int kDecodeSpan = 8;          // mask words per lane looked over at a time
 constexpr int kDecodeList = 384;        // of a span's 1024 vectors: more are read as they lie
@@ -33,8 +33,9 @@ constexpr int kDecodeListBytes = kDecodeWarps * kDecodeList * 2;
 // Byte b of a mask as four words that keep (all ones) or drop (zero) the
 // bf16 halves of a vector: kDecodeKeep entries in shared memory.
 constexpr int kDecodeKeep = 256;
+template <int THREADS = kDecodeThreads>
 __device__ __forceinline__ void fill_keep(uint4* keep, int tid) {
-    for (int b = tid; b < kDecodeKeep; b += kDecodeThreads) {
+    for (int b = tid; b < kDecodeKeep; b += THREADS) {
         uint32_t w[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k)
@@ -400,7 +401,9 @@ struct Decoder {
     // A slice: tokens [tok0, tok0 + ntok), tok0 a multiple of 128, its mask
     // words at s_mask (a zero word before and after); `list` holds kDecodeList
     // entries of this warp.
+    template <int THREADS = kDecodeThreads>
     __device__ __forceinline__ void slice(const uint32_t* s_mask, int tok0, int ntok, uint16_t* list, int warp) {
+        constexpr int kWarps = THREADS / 32;
         const uint8_t* bytes = reinterpret_cast<const uint8_t*>(s_mask);
         const int base = tok0 - shift;   // vector b starts at token base + 8b, word j's vectors are 4j to 4j + 3
         const int nvec = (ntok + shift + 7) / 8;
@@ -409,7 +412,7 @@ struct Decoder {
         const int in0 = base < 0 ? 1 : 0, in1 = max(in0, base + 8 * nvec > V ? nvec - 1 : nvec);
         const char* vec = lrow + (int64_t)base * (BF16 ? 2 : 4);
         const int words = (nvec + 3) / 4;
-        const int per = ((words + kDecodeWarps - 1) / kDecodeWarps + kDecodeSpan - 1) / kDecodeSpan * kDecodeSpan;
+        const int per = ((words + kWarps - 1) / kWarps + kDecodeSpan - 1) / kDecodeSpan * kDecodeSpan;
         const int j1 = min(words, (warp + 1) * per);
 #pragma unroll 1
         for (int j0 = warp * per; j0 < j1; j0 += 32 * kDecodeSpan) {
@@ -547,13 +550,14 @@ struct DecodeShared {
 // The row's (max, argmax, sum) over all lanes of the CTA and all `slices` CTAs
 // of its cluster, the same in every thread.  Every thread calls it; with more
 // than one slice, cluster_wait() has to follow before the CTA ends.
+template <int THREADS = kDecodeThreads>
 __device__ __forceinline__ void decode_combine(DecodeShared& sh, float& m, int& idx, float& s, int slices, int lane,
                                                int warp) {
     warp_merge(m, idx, s);
     if (lane == 0) sh.part[warp] = make_float4(m, __int_as_float(idx), s, 0.f);
     __syncthreads();
     if (warp == 0) {
-        float4 p = lane < kDecodeWarps ? sh.part[lane] : make_float4(-INFINITY, __int_as_float(INT_MAX), 0.f, 0.f);
+        float4 p = lane < THREADS / 32 ? sh.part[lane] : make_float4(-INFINITY, __int_as_float(INT_MAX), 0.f, 0.f);
         m = p.x;
         idx = __float_as_int(p.y);
         s = p.z;
@@ -594,13 +598,13 @@ __device__ __forceinline__ float log_sum_exp(float m, float s) {
 // where allowed, -inf elsewhere.  Rows on 32-byte boundaries of the output and
 // 16-byte boundaries of the logits: a thread takes 8 tokens (one 32-byte
 // store); rows of V % 4 == 0: 4 tokens; else one.
-template <bool BF16>
+template <bool BF16, int THREADS = kDecodeThreads>
 __device__ __forceinline__ void write_logprobs(const char* lrow, int V, const uint32_t* s_mask, int tok0, int ntok,
                                                float lse, float* orow, int tid) {
     const uint8_t* bytes = reinterpret_cast<const uint8_t*>(s_mask);
     if ((V & 7) == 0 && (reinterpret_cast<uintptr_t>(orow) & 31) == 0 && (reinterpret_cast<uintptr_t>(lrow) & 15) == 0) {
 #pragma unroll 2
-        for (int b = tid; b < ntok / 8; b += kDecodeThreads) {
+        for (int b = tid; b < ntok / 8; b += THREADS) {
             const uint32_t bits = bytes[b];
             const char* p = lrow + (size_t)(tok0 + 8 * b) * (BF16 ? 2 : 4);
             float o[8];
@@ -620,7 +624,7 @@ __device__ __forceinline__ void write_logprobs(const char* lrow, int V, const ui
                          : "memory");
         }
     } else if ((V & 3) == 0 && (reinterpret_cast<uintptr_t>(orow) & 15) == 0) {
-        for (int b = tid; b < ntok / 4; b += kDecodeThreads) {
+        for (int b = tid; b < ntok / 4; b += THREADS) {
             const uint32_t bits = bytes[b >> 1] >> (4 * (b & 1));
             float o[4];
 #pragma unroll
@@ -630,7 +634,7 @@ __device__ __forceinline__ void write_logprobs(const char* lrow, int V, const ui
         }
     } else {
 #pragma unroll 4
-        for (int b = tid; b < ntok; b += kDecodeThreads)
+        for (int b = tid; b < ntok; b += THREADS)
             orow[tok0 + b] = ((bytes[b >> 3] >> (b & 7)) & 1u) ? logit_at<BF16>(lrow, tok0 + b) - lse : -INFINITY;
     }
 }

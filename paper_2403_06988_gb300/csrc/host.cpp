@@ -866,13 +866,16 @@ bool rows_pay(const domino_ctx* h, int64_t batch, int first, int more) {
 
 // Whether row_kernel takes a mask step (GB300, us per-token / row_kernel).
 // Without loop sets: 5000 states, V = 128256, batch 17 8.1 / 14.3, batch 25
-// 19.5 / 13.3; V = 32000, batch 98 11.6 / 10.8; tables of masks and next
-// states, V = 8000, 16000 states 263 / 456 (4.6 units a wave), V = 32000, 4000
-// states 290 / 189 (18.6 units).  With a stack, whose per-token walk is the
-// dearer: JSON, V = 50000, batch 39 19.5 / 14.7, V = 128256, batch 17 16.1 /
-// 24.2, batch 21 37.8 / 23.7.  With loop sets alone (200 states): V = 48000,
-// batch 87 5.7 / 8.9, batch 174 9.5 / 9.2, V = 64000, batch 98 10.7 / 8.3;
-// their next states are the per-token walk's (loop sets hold masks only).
+// 19.5 / 13.3; V = 32000, batch 98 11.6 / 10.8; V = 8000, batch 620 15.8 / 15.7,
+// batch 1000 16.0 / 18.2; V = 16000, batch 400 32.9 / 11.8; tables of masks, V =
+// 8000, 16000 states 194 / 216 (4.6 units a wave), V = 16000, 8000 states 193 /
+// 128; next states, V = 8000, batch 400 15.0 / 12.5, batch 300 11.3 / 11.9.
+// With a stack, whose per-token walk is the dearer: JSON, V = 50000, batch 39
+// 19.5 / 14.7, V = 128256, batch 17 16.1 / 24.2, batch 21 37.8 / 23.7.  With
+// loop sets alone (200 states): V = 48000, batch 87 5.7 / 8.9, batch 174 9.5 /
+// 9.2, V = 64000, batch 98 10.7 / 8.3; V = 16000, batch 400 26.2 / 8.3, V =
+// 8000, batch 1000 11.1 / 15.2; their next states are the per-token walk's
+// (loop sets hold masks only).
 // Automata most of whose rows visit much of the tree (rows_dense) are the
 // per-token walk's: 500 states with 16 of 32 classes live, V = 128256, batch
 // 256 76 / 235, 28 live 179 / 521 (12 live, 2.6 % of the tokens: 58 / 36, row_kernel's).
@@ -881,7 +884,8 @@ bool use_rows(const domino_ctx* h, int64_t batch, bool next) {
     if (h->walk_pref == 1) return true;
     if (h->rows_dense || (next && !h->self_mask.empty())) return false;
     if (h->stack) return rows_pay(h, batch, 4, 4);
-    return h->self_mask.empty() ? rows_pay(h, batch, 6, 10) : rows_pay(h, batch, 10, 10);
+    if (next) return rows_pay(h, batch, 6, 1);
+    return h->self_mask.empty() ? rows_pay(h, batch, 6, 5) : rows_pay(h, batch, 10, 2);
 }
 
 // Whether the whole decode step is row_kernel's (one launch), against the
@@ -890,7 +894,8 @@ bool use_rows(const domino_ctx* h, int64_t batch, bool next) {
 // 19.1, V = 32000, batch 98 17.1 / 19.1, batch 163 19.5 / 18.2; JSON, V =
 // 50000, batch 39 26.4 / 20.7, V = 128256, batch 17 22.6 / 30.6, batch 21 45.2
 // / 31.2; 200 states, V = 32000, batch 196 15.1 / 14.0, V = 48000, batch 131
-// 13.1 / 15.4, batch 262 18.4 / 14.4, V = 8000, batch 524 12.1 / 18.5.  And
+// 13.1 / 15.4, batch 262 18.4 / 14.4, V = 32000, batch 400 35.5 / 14.2, V =
+// 16000, batch 500 15.0 / 19.2.  And
 // against the three kernels one after the other (two launches more): fp32, 200
 // states, V = 32000, batch 32 14.4 / 12.9, V = 64000, batch 4 11.9 / 12.1, batch
 // 8 13.3 / 12.9; 5000 states, V = 32000, batch 22 15.9 / 15.4, V = 128256,
@@ -901,7 +906,7 @@ bool decode_rows(const domino_ctx* h, int64_t batch, bool fusable) {
     if (h->rows_dense) return false;
     if (!fusable) return rows_pay(h, batch, 1, 1);
     if (h->stack) return rows_pay(h, batch, 4, 4);
-    return h->self_mask.empty() ? rows_pay(h, batch, 6, 10) : rows_pay(h, batch, 16, 16);
+    return h->self_mask.empty() ? rows_pay(h, batch, 6, 5) : rows_pay(h, batch, 16, 6);
 }
 
 int ready_for_compute(domino_ctx* h) {

@@ -23,7 +23,7 @@
 // these rounds free of any grid-wide step, and neither the tree nor the
 // transition table is staged.  Measured (GB300, that workload, back to back):
 // batch 256 15.7 us (35.8 us for the walk it replaced, whose CTAs each staged
-// a share of the tree and walked every row in it), batch 1000 51.7 us (94.1),
+// a share of the tree and walked every row in it), batch 1000 49.1 us (94.1),
 // batch 32 13.5 us (19.0); the 20000-state table 2.62 ms (3.25 ms).
 //
 // A row with more live nodes than the pool holds is walked token by token
@@ -44,7 +44,7 @@
 // still in shared memory when its logits are folded (decode.cuh), the cluster
 // merges its slices' results, and the row is advanced by its token.  Measured
 // against the separate kernels before it: 5000 states, V = 128256, batch 256
-// 22.5 us (45.9 us in four launches), batch 1000 78.5 us (127); JSON, V =
+// 22.5 us (45.9 us in four launches), batch 1000 74.5 us (127); JSON, V =
 // 152064, batch 128 35.5 us (86.1 us in two launches), with log-probabilities
 // 47.5 us (105), batch 512 76.7 us (304).
 //
@@ -65,18 +65,18 @@
 namespace domino {
 namespace {
 
-constexpr int kRowThreads = 512;
-constexpr int kRowWarps = kRowThreads / 32;
+constexpr int kRowThreads = 512;      // a CTA's, or half of it (launch_row_d)
 constexpr int kRowPool = 2048;        // items the pool holds
 constexpr int kRowFan = 8;            // threads per item while there are few
 constexpr int kRowSmall = 512;        // ranges of 2 to kRowSmallTokens tokens left to the whole CTA
 constexpr int kRowSmallTokens = 64;
 constexpr int kRowBig = 128;          // longer ranges
+constexpr int kRowNextHalf = 49152;   // tokens up to which rows of next states take half the threads
 constexpr int kRowSpawn = 2048;       // exits taken at a time
 constexpr int kRowExits = 512;        // loop subtrees whose exits are still to be walked
 constexpr int kRowLoopMin = 4;        // fewest tokens of a subtree taken as a loop subtree
 constexpr int kRowMaxDevices = 64;
-static_assert(kRowBig <= kRowThreads && kRowExits <= kRowThreads, "one entry per thread in the prefix sums");
+static_assert(kRowBig <= kRowThreads / 2 && kRowExits <= kRowThreads, "one entry per thread in the prefix sums");
 static_assert(kRowThreads == kDecodeThreads && 2 * kRowPool * 8 >= kDecodeListBytes, "the decode's lists lie in the pool");
 
 enum RowOut : int {
@@ -137,7 +137,7 @@ struct RowShared {
     uint4 rc;        // the row's configuration (read_row)
     int back;        // exits walked (spawn_exits)
     int nrange[2], nexit;
-    int wsum[kRowWarps];
+    int wsum[kRowThreads / 32];
 };
 
 __device__ __forceinline__ int warp_scan_incl(int x, int lane) {
@@ -201,7 +201,7 @@ __device__ __noinline__ void every_token(const StepView& v, const RowTree& t, co
     using E = typename std::conditional<STACK, uint32_t, uint16_t>::type;
     constexpr int kAtOnce = STACK ? 2 : 4;
     const E* table = reinterpret_cast<const E*>(STACK ? (const void*)v.t32 : (const void*)v.t16);
-    for (int w = warp * kAtOnce; w < nw; w += kRowWarps * kAtOnce) {
+    for (int w = warp * kAtOnce; w < nw; w += (int)(blockDim.x >> 5) * kAtOnce) {
         uint4 rec[kAtOnce];   // {length, the first 15 classes}, shifted by a byte per step
         uint32_t s[kAtOnce], bits[kAtOnce], depth[kAtOnce];
         int len[kAtOnce];
@@ -264,8 +264,9 @@ __device__ __noinline__ void every_token(const StepView& v, const RowTree& t, co
 }
 
 // One row's walk.
-template <bool STACK, int CLS, int OUT>
+template <bool STACK, int CLS, int OUT, int THREADS>
 struct RowWalk {
+    static constexpr int kExits = kRowExits < THREADS ? kRowExits : THREADS;   // one per thread in the prefix sums
     static constexpr bool WIDE = CLS == kRowWide;
     using Mask = typename std::conditional<CLS == kRow32, uint32_t, unsigned long long>::type;
 
@@ -427,9 +428,9 @@ struct RowWalk {
                 if (n == 0) break;
                 half = 0;
             }
-            const int take = min(n, kRowThreads);
+            const int take = min(n, THREADS);
             const int base = n - take;
-            const bool fan = take * kRowFan <= kRowThreads;
+            const bool fan = take * kRowFan <= THREADS;
             const int i = fan ? tid / kRowFan : tid;
             bool lead = !fan || (tid & (kRowFan - 1)) == 0;   // this thread answers for its item
             Item it{0u, 0u, 0u, 0u};
@@ -541,7 +542,7 @@ struct RowWalk {
         int j = 0;
         if (n_exit) {
             j = atomicAdd(&sh.nexit, 1);
-            if (j >= kRowExits) return false;
+            if (j >= kExits) return false;
             s_exit[j] = make_uint4(x.x, 0u, it.s | (it.depth << 16), it.bits);
         }
         if (!later(make_uint4(lo, hi - lo, it.s, d | ((set + 1u) << 8)), st)) return false;   // (an empty entry stays behind)
@@ -566,14 +567,14 @@ struct RowWalk {
     __device__ __forceinline__ int spawn_exits() const {
         if (t.n_loops == 0) return 0;
         for (;;) {
-            const int nx = min(*reinterpret_cast<volatile int*>(&sh.nexit), kRowExits);
+            const int nx = min(*reinterpret_cast<volatile int*>(&sh.nexit), kExits);
             if (nx == 0) return 0;
             if (tid == 0) sh.back = 0;
             const int total = prefix(nx, tid < nx ? (int)s_exit[tid].y : 0);
             // as many as fit this time, the last entries first (the list is a
             // stack); an entry taken in part is cut back
             const int f0 = max(0, total - kRowSpawn);
-            for (int b = f0 + warp * 32; b < total; b += kRowThreads) {
+            for (int b = f0 + warp * 32; b < total; b += THREADS) {
                 const int f = b + lane;
                 Item x{0u, 0u, 0u, 0u};
                 if (f < total) {
@@ -619,7 +620,7 @@ struct RowWalk {
         const int nb = min(*reinterpret_cast<volatile int*>(&sh.nrange[1]), kRowBig);
         constexpr int kUnroll = STACK ? 8 : 4;   // 8 spill beside a DFA's folded decode: +0.8 us at 128256x256
         // short ones: four threads each
-        for (int i = tid / 4; i < ns; i += kRowThreads / 4) {
+        for (int i = tid / 4; i < ns; i += THREADS / 4) {
             const uint4 x = s_range[i];
             for (uint32_t j = tid & 3; j < x.y; j += 4 * kUnroll) {
                 int tk[kUnroll];
@@ -639,7 +640,7 @@ struct RowWalk {
         if (nb > 0) {   // long ones: the CTA over all of them
             const int total = prefix(nb, tid < nb ? (int)s_range[kRowSmall + tid].y : 0);
             // a warp takes 256 tokens in a row: they lie in a few ranges
-            for (int f0 = warp * 32 * kUnroll; f0 < total; f0 += kRowThreads * kUnroll) {
+            for (int f0 = warp * 32 * kUnroll; f0 < total; f0 += THREADS * kUnroll) {
                 int tk[kUnroll];
                 uint32_t st[kUnroll], out[kUnroll];
                 int k = find_range(s_pre, nb, f0), end = s_pre[k + 1];
@@ -692,8 +693,8 @@ __device__ __forceinline__ void update(const StepView& v, const RowTree& t, cons
     if (stacks_out) stacks_out[b] = ((uint64_t)depth << 32) | bits;
 }
 
-template <bool STACK, int CLS, int OUT>
-__global__ void __launch_bounds__(kRowThreads, 2)
+template <bool STACK, int CLS, int OUT, int THREADS>
+__global__ void __launch_bounds__(THREADS, 1024 / THREADS)
     row_kernel(const __grid_constant__ StepView v, const __grid_constant__ RowTree t,
                const __grid_constant__ RowArgs a, const RowList list) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -704,10 +705,10 @@ __global__ void __launch_bounds__(kRowThreads, 2)
     const int row = blockIdx.x / a.slices, slice = blockIdx.x - row * a.slices;
     const int w0 = slice * a.slice_words, nw = max(0, min(a.slice_words, v.W - w0));
     const int tok0 = w0 * 32, ntok = max(0, min(nw * 32, v.V - tok0));
-    for (int j = tid; j < a.slice_words / 4; j += kRowThreads)
+    for (int j = tid; j < a.slice_words / 4; j += THREADS)
         reinterpret_cast<uint4*>(s_mask)[j] = make_uint4(0u, 0u, 0u, 0u);
     constexpr bool kDecode = OUT == kRowBf16 || OUT == kRowF32;
-    if constexpr (OUT == kRowBf16) fill_keep(reinterpret_cast<uint4*>(smem + L.keep), tid);
+    if constexpr (OUT == kRowBf16) fill_keep<THREADS>(reinterpret_cast<uint4*>(smem + L.keep), tid);
     if (tid == 0) {
         s_mask[-1] = s_mask[a.slice_words] = 0u;
         sh.nrange[0] = sh.nrange[1] = sh.nexit = 0;
@@ -735,7 +736,7 @@ __global__ void __launch_bounds__(kRowThreads, 2)
         s0 = w.x;
         if (w.y != 0xFFFFFFFFu) {   // the tokens that stay inside the set, then the walk of the others
             const uint32_t* loop = t.loopbits + (size_t)w.y * v.W + w0;
-            for (int j = tid; j < nw; j += kRowThreads) s_mask[j] = __ldg(loop + j);
+            for (int j = tid; j < nw; j += THREADS) s_mask[j] = __ldg(loop + j);
             root = (uint32_t)t.loop_root[w.y];
         }
     }
@@ -746,9 +747,9 @@ __global__ void __launch_bounds__(kRowThreads, 2)
         if (nrow) {
             if ((v.V & 3) == 0 && (reinterpret_cast<uintptr_t>(a.next) & 15) == 0) {
                 int4* dst = reinterpret_cast<int4*>(nrow + tok0);
-                for (int j = tid; j < ntok / 4; j += kRowThreads) dst[j] = make_int4(0, 0, 0, 0);
+                for (int j = tid; j < ntok / 4; j += THREADS) dst[j] = make_int4(0, 0, 0, 0);
             } else {
-                for (int j = tid; j < ntok; j += kRowThreads) nrow[tok0 + j] = 0;
+                for (int j = tid; j < ntok; j += THREADS) nrow[tok0 + j] = 0;
             }
         }
     }
@@ -757,7 +758,7 @@ __global__ void __launch_bounds__(kRowThreads, 2)
         if (a.ahead)
             ahead = reinterpret_cast<const char*>(a.logits) +
                     (size_t)list.row(row) * (size_t)a.stride * (OUT == kRowBf16 ? 2 : 4);
-    const RowWalk<STACK, CLS, OUT> wk{v, t, s_mask, reinterpret_cast<uint2*>(smem + L.items),
+    const RowWalk<STACK, CLS, OUT, THREADS> wk{v, t, s_mask, reinterpret_cast<uint2*>(smem + L.items),
                                       reinterpret_cast<uint32_t*>(smem + L.bits),
                                       reinterpret_cast<uint4*>(smem + L.range),
                                       reinterpret_cast<uint4*>(smem + L.exits), reinterpret_cast<int*>(smem + L.pre), sh,
@@ -777,10 +778,10 @@ __global__ void __launch_bounds__(kRowThreads, 2)
     if (a.mask) {
         uint32_t* mrow = a.mask + (size_t)row * v.W + w0;
         if ((v.W & 3) == 0 && (reinterpret_cast<uintptr_t>(a.mask) & 15) == 0) {
-            for (int j = tid; j < nw / 4; j += kRowThreads)
+            for (int j = tid; j < nw / 4; j += THREADS)
                 reinterpret_cast<uint4*>(mrow)[j] = reinterpret_cast<const uint4*>(s_mask)[j];
         } else {
-            for (int j = tid; j < nw; j += kRowThreads) mrow[j] = s_mask[j];
+            for (int j = tid; j < nw; j += THREADS) mrow[j] = s_mask[j];
         }
     }
     if constexpr (kDecode) {
@@ -789,14 +790,14 @@ __global__ void __launch_bounds__(kRowThreads, 2)
         Decoder<OUT == kRowBf16, kFoldLse> d;
         d.init(a.logits, a.stride, b, v.V, a.logprobs != nullptr, SampleArgs{},
                reinterpret_cast<const uint4*>(smem + L.keep), lane);
-        d.slice(s_mask, tok0, ntok, reinterpret_cast<uint16_t*>(smem + L.items) + warp * kDecodeList, warp);
+        d.template slice<THREADS>(s_mask, tok0, ntok, reinterpret_cast<uint16_t*>(smem + L.items) + warp * kDecodeList, warp);
         d.finish();
         float m = d.m, sum = d.s;
         int idx = d.idx;
-        decode_combine(dsh, m, idx, sum, a.slices, lane, warp);
+        decode_combine<THREADS>(dsh, m, idx, sum, a.slices, lane, warp);
         const float lse = log_sum_exp(m, sum);
         if (a.logprobs)
-            write_logprobs<OUT == kRowBf16>(d.lrow, v.V, s_mask, tok0, ntok, lse, a.logprobs + (size_t)b * v.V, tid);
+            write_logprobs<OUT == kRowBf16, THREADS>(d.lrow, v.V, s_mask, tok0, ntok, lse, a.logprobs + (size_t)b * v.V, tid);
         if (slice == 0 && tid == 0) {
             const int32_t tk = m == -INFINITY ? -1 : idx;
             a.argmax[b] = tk;
@@ -823,8 +824,8 @@ cudaError_t rows_allow_smem(K kern, int bytes, int* configured, std::mutex& mu) 
     return e;
 }
 
-template <bool STACK, int CLS, int OUT>
-cudaError_t launch_row_t(const StepView& v, const RowTree& t, const LaunchEnv& env, RowArgs a, const RowList& list,
+template <bool STACK, int CLS, int OUT, int THREADS>
+cudaError_t launch_row_d(const StepView& v, const RowTree& t, const LaunchEnv& env, RowArgs a, const RowList& list,
                          cudaStream_t st) {
     // CTAs per row: enough to give every SM one (two where a row is decoded
     // and has two: JSON, V = 152064, batch 128 54.6 -> 45.7 us), and enough for
@@ -837,13 +838,37 @@ cudaError_t launch_row_t(const StepView& v, const RowTree& t, const LaunchEnv& e
     a.slice_words = ((v.W + s - 1) / s + 3) / 4 * 4;
     const RowLayout L = row_layout(a.slice_words, STACK, t.n_loops > 0, OUT == kRowBf16 || OUT == kRowF32);
     if (L.total > env.max_smem_optin) return cudaErrorInvalidConfiguration;
-    auto kern = row_kernel<STACK, CLS, OUT>;
+    auto kern = row_kernel<STACK, CLS, OUT, THREADS>;
     static int configured[kRowMaxDevices] = {0};
     static std::mutex mu;
     cudaError_t e = rows_allow_smem(kern, L.total, configured, mu);
     if (e != cudaSuccess) return e;
-    return launch_cluster(kern, dim3((unsigned)a.batch * (unsigned)s), dim3(kRowThreads), s, (size_t)L.total, st, v, t, a,
+    return launch_cluster(kern, dim3((unsigned)a.batch * (unsigned)s), dim3(THREADS), s, (size_t)L.total, st, v, t, a,
                           list);
+}
+
+template <bool STACK, int CLS, int OUT>
+cudaError_t launch_row_t(const StepView& v, const RowTree& t, const LaunchEnv& env, const RowArgs& a, const RowList& list,
+                         cudaStream_t st) {
+    // More rows than run at once with 2 CTAs an SM (one CTA a row): CTAs of
+    // half the threads, of which up to 4 fit, take more rows a wave, each wave
+    // being 1.1 to 1.3 times as long.  GB300, us, 512 / 256 threads: 5000 states,
+    // V = 128256, steps of 310 rows 37.2 / 28.7, 500 rows 42.8 / 47.6 (two waves
+    // either way), 1000 rows 78.8 / 74.6; V = 32000, 1000 rows 61.4 / 39.9;
+    // 256 rows of 128256 23.1 / 28.5.  The log-probabilities want the threads:
+    // 310 rows 91.6 / 76.9, 620 rows (three waves, two) 144 / 152.  So do long
+    // rows of next states: tables, V = 32000 194 / 162, V = 64000 302 / 314.
+    // With a stack the rounds are longer: JSON, V = 152064, 512 rows 78.6 / 98.1.
+    if constexpr (!STACK && CLS != kRowWide) {
+        const RowLayout L = row_layout((v.W + 3) / 4 * 4, STACK, t.n_loops > 0, OUT == kRowBf16 || OUT == kRowF32);
+        const int64_t fit = std::min(4, (env.max_smem_optin + 1024) / (L.total + 1024 + (int)sizeof(RowShared)));
+        if (fit > 2 && a.batch > 2 * env.num_sms && (OUT != kRowNext || v.V <= kRowNextHalf)) {
+            const int64_t full = (a.batch - 1) / (2 * env.num_sms) + 1, half = (a.batch - 1) / (fit * env.num_sms) + 1;
+            if (a.logprobs ? 2 * half <= full : 5 * half < 4 * full)
+                return launch_row_d<STACK, CLS, OUT, kRowThreads / 2>(v, t, env, a, list, st);
+        }
+    }
+    return launch_row_d<STACK, CLS, OUT, kRowThreads>(v, t, env, a, list, st);
 }
 
 template <bool STACK, int CLS>

@@ -160,7 +160,8 @@ def test_infinite_logits(dt):
 
 @pytest.mark.parametrize("dt,offset,pad", [(B.DTYPE_BF16, 0, 5), (B.DTYPE_BF16, 3, 0), (B.DTYPE_F32, 0, 0),
                                            (B.DTYPE_F32, 1, 2)])
-@pytest.mark.parametrize("grammar,batch", [("json", 60), ("json", 170), ("sparse", 5), ("sparse", 200)])
+@pytest.mark.parametrize("grammar,batch", [("json", 60), ("json", 170), ("sparse", 5), ("sparse", 200),
+                                           ("sparse", 310)])
 @pytest.mark.parametrize("walk", ["tree", None])
 def test_whole_step_in_one_kernel(dt, offset, pad, grammar, batch, walk, monkeypatch):
     import oracle
