@@ -238,7 +238,9 @@ int domino_advance(domino_t h, const int32_t* states_dev, const uint64_t* stacks
  * batch allocates scratch and synchronises `stream`; if `stream` is being
  * captured into a CUDA graph at that point, the call returns
  * DOMINO_E_INVALID_ARG and launches nothing (make one uncaptured call at the
- * largest batch first). */
+ * largest batch first); where no state loops and the logits are in device
+ * memory, the one kernel is captured instead.  Scratch named by a recorded
+ * graph stays valid until the handle is destroyed. */
 int domino_step_decode(domino_t h, const int32_t* states_dev, const uint64_t* stacks_dev, int32_t batch,
                        const void* logits_dev, int32_t dtype, int64_t row_stride_elems, uint32_t* mask_dev,
                        int32_t* argmax_dev, float* lse_dev, float* logprobs_dev, int32_t* states_out,

@@ -58,6 +58,7 @@ struct domino_ctx {
     DevBuf d_head, d_info, d_tail_off, d_tail, d_pos_of, d_cls_start, d_eos_slot;
     DevBuf d_dense, d_sparse, d_accept, d_self, d_tok_cls;
     DevBuf d_err, d_fpart;
+    std::vector<DevBuf> fpart_old;   // outgrown ones: recorded graphs may still name them
     bool arena_ready = false;
     // prefix tree of the class strings (domino_get_prefix_tree)
     std::vector<uint4> t_node;
@@ -137,9 +138,12 @@ void dev_free(DevBuf& b) {
 int64_t dev_bytes(const domino_ctx* h) {
     const DevBuf* all[] = {&h->d_head, &h->d_info, &h->d_tail_off, &h->d_tail, &h->d_pos_of, &h->d_cls_start,
                            &h->d_eos_slot, &h->d_dense, &h->d_sparse, &h->d_accept, &h->d_self, &h->d_tok_cls, &h->d_err, &h->d_fpart, &h->s_logits, &h->s_mask, &h->s_io,
-                           &h->o_prop, &h->o_rows, &h->o_count};
+                           &h->o_prop, &h->o_rows, &h->o_count, &h->d_rnode, &h->d_rncls, &h->d_rdtok, &h->d_srec,
+                           &h->d_srec_next, &h->d_rret, &h->d_rstart, &h->d_loop_of, &h->d_loopbits, &h->d_keeps,
+                           &h->d_xrange, &h->d_exits, &h->d_trec};
     int64_t n = 0;
     for (auto* b : all) n += (int64_t)b->n;
+    for (const DevBuf& b : h->fpart_old) n += (int64_t)b.n;
     return n;
 }
 
@@ -163,6 +167,19 @@ int dev_upload(DevBuf& b, const void* src, size_t n) {
 }
 
 int dev_reserve(DevBuf& b, size_t n) { return dev_upload(b, nullptr, n); }
+
+// The fused decode's partials, n bytes or more.  An outgrown buffer is kept
+// until the handle is destroyed: a graph that a caller recorded at a smaller
+// batch goes on using it.  Sizes at least double, so the outgrown ones take
+// no more than the buffer itself.
+int grow_fpart(domino_ctx* h, size_t n) {
+    if (h->d_fpart.n >= n) return DOMINO_OK;
+    DevBuf b;
+    if (int rc = dev_reserve(b, std::max(n, 2 * h->d_fpart.n))) return rc;
+    if (h->d_fpart.p) h->fpart_old.push_back(h->d_fpart);
+    h->d_fpart = b;
+    return DOMINO_OK;
+}
 
 bool is_host_only(const domino_ctx* h) { return h->device < 0; }
 
@@ -999,6 +1016,7 @@ int domino_destroy(domino_t h) {
                          &h->d_rstart, &h->d_loop_of, &h->d_loopbits, &h->d_keeps, &h->d_xrange, &h->d_exits,
                          &h->d_trec};
         for (auto* b : all) dev_free(*b);
+        for (DevBuf& b : h->fpart_old) dev_free(b);
         for (cudaEvent_t& e : h->ev_chunk)
             if (e) cudaEventDestroy(e);
         for (cudaEvent_t& e : h->ev_t)
@@ -1445,7 +1463,7 @@ int domino_step_decode(domino_t h, const int32_t* states_dev, const uint64_t* st
         if (cs != cudaStreamCaptureStatusNone) return DOMINO_E_INVALID_ARG;
         if (cudaStreamSynchronize(st) != cudaSuccess) return cuda_status(cudaGetLastError());
         clear_host_graphs(h);   // recorded host-buffer steps name this buffer
-        if ((rc = dev_reserve(h->d_fpart, part_bytes))) return rc;
+        if ((rc = grow_fpart(h, part_bytes))) return rc;
     }
     const int mode = choose_mode(h, v, false);
     cudaError_t e = launch_step_mask(v, h->env, h->stack, mode, states_dev, stacks_dev, batch, false, mask_dev, nullptr,
@@ -1749,7 +1767,7 @@ int domino_decode_step_host(domino_t h, const void* logits_host, int32_t dtype, 
         clear_host_graphs(h);
     }
     if (!mapped && (rc = dev_reserve(h->s_logits, logit_bytes))) return rc;
-    if (mapped && (rc = dev_reserve(h->d_fpart, fpart_bytes))) return rc;
+    if (mapped && (rc = grow_fpart(h, fpart_bytes))) return rc;
     if ((rc = dev_reserve(h->s_mask, (size_t)batch * (size_t)h->W * 4))) return rc;
     if ((rc = dev_reserve(h->s_io, L.in_end))) return rc;
     if (h->h_io_n < L.in_end) {

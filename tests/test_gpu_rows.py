@@ -242,3 +242,36 @@ def test_rows_of_half_the_threads(batch):
     check(a, v, rng.integers(0, 400, batch).astype(np.int32), want_next=True)
     a, _ = synth.kv200_dfa(rng)
     check(a, v, rng.integers(0, 200, batch).astype(np.int32))
+
+
+def test_recorded_step_outlives_larger_batches():
+    """A graph recorded at a small batch is replayed after larger batches have grown the scratch."""
+    from paper_2403_06988_gb300 import _binding as B
+    rng = np.random.default_rng(14)
+    a = synth.random_sparse_dfa(rng, 300)
+    V = 8000
+    v = synth.random_vocab(rng, V, bytes(range(256)), synth.geometric_lengths(4.0, 16), synth._mixed_bytes)
+    d = Domino.from_parts(a, v, device=0)
+    states = torch.from_numpy(rng.integers(1, 300, 300).astype(np.int32)).cuda()
+    lg = torch.randn((300, V), device="cuda", generator=torch.Generator("cuda").manual_seed(2)).to(torch.bfloat16)
+    mask = poison.empty((300, d.info()["n_words"]), torch.int32)
+    arg, out = poison.empty(300, torch.int32), poison.empty(300, torch.int32)
+
+    def run(n):
+        B.domino_step_decode(d.h, states, None, n, lg.data_ptr(), B.DTYPE_BF16, V, mask, arg, None, None, out, None,
+                             torch.cuda.current_stream().cuda_stream)
+    run(4)
+    want = arg[:4].cpu().numpy().copy()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        run(4)
+    for n in (20, 90, 300):
+        run(n)
+    full = arg.cpu().numpy().copy()
+    arg.fill_(-7)
+    g.replay()
+    torch.cuda.synchronize()
+    assert_exact(arg[:4], want, "recorded")
+    assert_exact(full[:4], want, "largest batch")
+    assert d.device_error() == 0
+    d.close()
