@@ -52,13 +52,12 @@ __device__ __forceinline__ uint32_t nonzero_bytes(uint32_t x) {
     return ((x & 0x01010101u) * 0x10204080u) >> 28;
 }
 
-// (a, b) * (c, c) + (d, d), both lanes rounded once
-__device__ __forceinline__ float2 fma2(float2 a, float c, float d) {
-    unsigned long long x, y, z, r;
+// (a, b) * (c, c)
+__device__ __forceinline__ float2 mul2(float2 a, float c) {
+    unsigned long long x, y, r;
     asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(a.x), "f"(a.y));
     asm("mov.b64 %0, {%1, %1};" : "=l"(y) : "f"(c));
-    asm("mov.b64 %0, {%1, %1};" : "=l"(z) : "f"(d));
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(x), "l"(y), "l"(z));
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(x), "l"(y));
     float2 o;
     asm("mov.b64 {%0, %1}, %2;" : "=f"(o.x), "=f"(o.y) : "l"(r));
     return o;
@@ -157,7 +156,7 @@ constexpr float kGumbelMax = 17.0f;
 // A lane's fold over a row's tokens.  The sum of exponentials is kept against
 // a reference that follows the maximum only when it falls more than kLag
 // behind, and the maximum's vector is kept instead of its token, so that a
-// vector costs no branch in the common case: the bf16 vector takes about 55
+// vector costs no branch in the common case: the bf16 vector takes about 60
 // instructions for 8 tokens (208 with the maximum's token found and the sum
 // rescaled whenever some lane's maximum rose), 8 of them ex2, whose unit
 // (16 a clock and SM) then bounds dense rows.
@@ -182,7 +181,7 @@ struct Decoder {
     int lane;
     const uint4* keep;       // fill_keep's table
     float m;                 // maximum (sampling: the best score)
-    float ref, s;            // the sum's reference (times log2(e)) and the sum of 2^(x log2(e) - ref)
+    float ref, s;            // the sum's reference and the sum of e^(x - ref)
     int idx;                 // sampling: its token; else the token of element 0 of the maximum's vector
     uint32_t top[kWords];    // the maximum's vector, -inf where not allowed
     float seen;              // sampling: a score some lane of the warp has seen
@@ -260,14 +259,13 @@ struct Decoder {
                 }
             }
             if constexpr (FOLD == kFoldLse) {
-                constexpr float kLag = 16.0f;   // terms of 2^16 at most: no overflow, and nothing lost in relative terms
+                constexpr float kLag = 11.0f;   // terms of e^16 at most (ref + kLag rounds): no overflow, and nothing lost in relative terms
                 float most = vm[0];
 #pragma unroll
                 for (int k = 1; k < N; ++k) most = fmaxf(most, vm[k]);
-                const float vL = most * kLog2e;
-                if ((vL > ref + kLag || m == -INFINITY) && most != -INFINITY) {   // rare after the first vectors
-                    s *= s == 0.0f ? 0.0f : ex2(ref - vL);
-                    ref = vL;
+                if ((most > ref + kLag || m == -INFINITY) && most != -INFINITY) {   // rare after the first vectors
+                    s *= s == 0.0f ? 0.0f : exp_diff(ref, most);
+                    ref = most;
                 }
             }
 #pragma unroll
@@ -287,7 +285,7 @@ struct Decoder {
                     for (int e = 0; e < 4; ++e) {
                         const float2 z = BF16 ? make_float2(bf16_lo(w[k][e]), bf16_hi(w[k][e]))
                                               : make_float2(__uint_as_float(w[k][BF16 ? 0 : 2 * e]), __uint_as_float(w[k][BF16 ? 0 : 2 * e + 1]));
-                        const float2 y = fma2(z, kLog2e, -ref);
+                        const float2 y = mul2(add2(z, make_float2(-ref, -ref)), kLog2e);   // as exp_diff
                         acc[k] = add2(acc[k], make_float2(ex2(y.x), ex2(y.y)));   // not allowed: 2^-inf = 0
                     }
                 }
@@ -313,7 +311,7 @@ struct Decoder {
                 if (v == m) e = k;
             }
             idx += e;
-            if constexpr (FOLD == kFoldLse) s *= ex2(ref - m * kLog2e);
+            if constexpr (FOLD == kFoldLse) s *= exp_diff(ref, m);
         }
     }
 
@@ -588,10 +586,6 @@ __device__ __forceinline__ void decode_combine(DecodeShared& sh, float& m, int& 
         idx = __float_as_int(p.y);
         s = p.z;
     }
-}
-
-__device__ __forceinline__ float log_sum_exp(float m, float s) {
-    return isinf(m) ? m : m + logf(s);   // nothing allowed: -inf
 }
 
 // Log-probabilities of a slice's tokens (tok0 a multiple of 128): logit - lse

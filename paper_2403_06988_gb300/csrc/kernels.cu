@@ -69,7 +69,7 @@ __device__ __forceinline__ void fold_listed(float4* out, unsigned short raw, int
             idx = i2;
         }
     }
-    float e = t != INT_MAX ? ex2(fmaf(x, kLog2e, -m * kLog2e)) : 0.0f;
+    float e = t != INT_MAX ? exp_diff(x, sum_ref(m)) : 0.0f;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) e += __shfl_xor_sync(0xffffffffu, e, off);
     if (lane == 0) *out = make_float4(m, __int_as_float(idx), e, 0.f);
@@ -164,17 +164,17 @@ __device__ __forceinline__ void fold_window(uint32_t* mrow, const char* lrow, in
                 idx = i2;
             }
         }
-        const float mL = m * kLog2e;
+        const float ref = sum_ref(m);
         float sum = 0.0f;
 #pragma unroll
         for (int q = 0; q < 4; ++q)
-            if (tk[q] != INT_MAX) sum += ex2(fmaf(__uint_as_float((uint32_t)raw[q] << 16), kLog2e, -mL));
+            if (tk[q] != INT_MAX) sum += exp_diff(__uint_as_float((uint32_t)raw[q] << 16), ref);
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
         if (lane == 0)
             *out = make_float4(m, __int_as_float(idx), sum, 0.f);
     } else {
-        float m = -INFINITY, mL = -INFINITY, sum = 0.0f;
+        float m = -INFINITY, ref = sum_ref(m), sum = 0.0f;
         int idx = INT_MAX;
         uint32_t wd = word;
         const int t0 = j * 32;
@@ -206,7 +206,7 @@ __device__ __forceinline__ void fold_window(uint32_t* mrow, const char* lrow, in
                     }
                 }
             }
-            mL = m * kLog2e;
+            ref = sum_ref(m);
             idx = t0 + wi;
 #pragma unroll 1
             for (int k = 0; k < 4; ++k) {
@@ -217,7 +217,7 @@ __device__ __forceinline__ void fold_window(uint32_t* mrow, const char* lrow, in
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {
                     const float x = (e & 1) ? bf16_hi(qs[e >> 1]) : bf16_lo(qs[e >> 1]);
-                    acc += ((bits >> e) & 1u) ? ex2(fmaf(x, kLog2e, -mL)) : 0.0f;
+                    acc += ((bits >> e) & 1u) ? exp_diff(x, ref) : 0.0f;
                 }
                 sum += acc;
             }
@@ -226,7 +226,7 @@ __device__ __forceinline__ void fold_window(uint32_t* mrow, const char* lrow, in
                 const int e = __ffs(wd) - 1;
                 wd &= wd - 1;
                 if (t0 + e < V)
-                    acc_add(m, mL, idx, sum, __uint_as_float((uint32_t)__ldcs(u + t0 + e) << 16), t0 + e);
+                    acc_add(m, ref, idx, sum, __uint_as_float((uint32_t)__ldcs(u + t0 + e) << 16), t0 + e);
             }
         }
         warp_merge(m, idx, sum);
@@ -980,7 +980,7 @@ __global__ void __launch_bounds__(kLogitThreads)
     if (lane == 0) {
         const int32_t t = m == -INFINITY ? -1 : idx;
         argmax[r] = t;
-        if (lse) lse[r] = m == -INFINITY ? -INFINITY : m + logf(s);
+        if (lse) lse[r] = log_sum_exp(m, s);
         if constexpr (ADV) advance_row<STACK, MODE>(v, adv.states, adv.stacks, r, t, adv.states_out, adv.stacks_out);
     }
 }

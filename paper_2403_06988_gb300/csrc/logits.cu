@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(kGatherMaxWarps * 32, 2)
     const uint32_t* mrow = mask.row(r, W, threadIdx.x == 0);
     const int orow = list.row(r);
     const char* lrow = reinterpret_cast<const char*>(logits) + (size_t)orow * stride * 2;
-    float m = -INFINITY, mL = -INFINITY, s = 0.0f;
+    float m = -INFINITY, ref = sum_ref(m), s = 0.0f;
     int idx = INT_MAX;
     int blk = -1;   // Philox block cached by gumbel()
     uint4 rnd = make_uint4(0u, 0u, 0u, 0u);
@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(kGatherMaxWarps * 32, 2)
                 idx = t;
             }
         } else {
-            acc_add(m, mL, idx, s, x, t);
+            acc_add(m, ref, idx, s, x, t);
         }
     };
     for (int js = j0; js < j1; js += kSpanWords) {
@@ -332,15 +332,13 @@ __global__ void __launch_bounds__(kGatherMaxWarps * 32, 2)
                         }
                     } else {
                         if (vm > m) {
-                            const float vL = vm * kLog2e;
-                            s = s == 0.0f ? 0.0f : s * ex2(mL - vL);
-                            m = vm;
-                            mL = vL;
+                            s = s == 0.0f ? 0.0f : s * exp_diff(ref, vm);
+                            m = ref = vm;
                             idx = t0 + ve;
                         }
                         float acc = 0.0f;
 #pragma unroll
-                        for (int e = 0; e < 8; ++e) acc += ((bm >> e) & 1u) ? ex2(fmaf(xs[e], kLog2e, -mL)) : 0.0f;
+                        for (int e = 0; e < 8; ++e) acc += ((bm >> e) & 1u) ? exp_diff(xs[e], ref) : 0.0f;
                         s += acc;
                     }
                 } else {
@@ -377,7 +375,7 @@ __global__ void __launch_bounds__(kGatherMaxWarps * 32, 2)
         warp_merge(m, idx, s);
         if (lane == 0) {
             argmax[orow] = m == -INFINITY ? -1 : idx;
-            if (lse) lse[orow] = m == -INFINITY ? -INFINITY : m + logf(s);
+            if (lse) lse[orow] = log_sum_exp(m, s);
         }
     }
 }

@@ -6,6 +6,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <cfloat>
 #include <climits>
 #include <cstdint>
 #include <type_traits>
@@ -86,6 +87,22 @@ __device__ __forceinline__ float ex2(float x) {
     return y;
 }
 
+// e^(x - ref).  The difference is taken before it is scaled: x log2(e) minus a
+// rounded ref log2(e) is off by half a unit in the last place of the latter,
+// which passes 2^7 (2^x out of range, so that the sum turns to infinity or
+// NaN) from |ref| = 2^31 on, and overflows itself from 2.4e38 on; logits that
+// ban a token, -1e10 or the lowest value of the type, lie there.
+__device__ __forceinline__ float exp_diff(float x, float ref) { return ex2((x - ref) * kLog2e); }
+
+// What a sum is kept against: its maximum, or the lowest number while that is
+// -inf (x - ref is never -inf minus -inf).
+__device__ __forceinline__ float sum_ref(float m) { return fmaxf(m, -FLT_MAX); }
+
+// m + ln(s), s the sum of exp against m
+__device__ __forceinline__ float log_sum_exp(float m, float s) {
+    return isinf(m) ? m : m + logf(s);   // nothing allowed: -inf
+}
+
 // (m, idx, s) <- (m, idx, s) (+) (m2, i2, s2): larger max wins, lower index on
 // equal maxima; the other sum is rescaled to the winner's max.
 __device__ __forceinline__ void acc_merge(float& m, int& idx, float& s, float m2, int i2, float s2) {
@@ -99,19 +116,17 @@ __device__ __forceinline__ void acc_merge(float& m, int& idx, float& s, float m2
         i2 = ti;
         s2 = ts;
     }
-    if (s2 != 0.0f) s += s2 * ex2((m2 - m) * kLog2e);
+    if (s2 != 0.0f) s += s2 * exp_diff(m2, m);
 }
 
-// one allowed logit x at index t; mL = m * log2(e) is kept with m
-__device__ __forceinline__ void acc_add(float& m, float& mL, int& idx, float& s, float x, int t) {
+// one allowed logit x at index t; ref = sum_ref(m) is kept with m
+__device__ __forceinline__ void acc_add(float& m, float& ref, int& idx, float& s, float x, int t) {
     if (x > m) {
-        const float xL = x * kLog2e;
-        s = s * ex2(mL - xL) + 1.0f;
-        m = x;
-        mL = xL;
+        s = s * exp_diff(ref, x) + 1.0f;
+        m = ref = x;
         idx = t;
     } else {
-        s += ex2(fmaf(x, kLog2e, -mL));
+        s += exp_diff(x, ref);
     }
 }
 

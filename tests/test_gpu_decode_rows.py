@@ -158,6 +158,92 @@ def test_infinite_logits(dt):
             assert abs(float(lse[b]) - np.logaddexp.reduce(v[np.isfinite(v)])) < TOL
 
 
+def extreme_logits(dt, batch, V, seed):
+    """float32 rows whose logits reach the type's ends: banned tokens at the lowest value and the like."""
+    rng = np.random.default_rng(seed)
+    top = float(torch.finfo(torch.bfloat16 if dt == B.DTYPE_BF16 else torch.float32).max)
+    x = (rng.standard_normal((batch, V)) * 3).astype(np.float32)
+    few = rng.random((batch, V)) < 0.02
+    for b in range(batch):
+        kind = b % 10
+        if kind == 0:
+            x[b] = -top                                                  # nothing but the lowest value
+        elif kind == 1:
+            x[b] = np.where(few[b], x[b], np.float32(-top))              # a few tokens left
+        elif kind == 2:
+            x[b] = np.where(few[b], np.float32(-top), x[b])              # a few tokens banned
+        elif kind == 3:
+            x[b] = top
+        elif kind == 4:
+            x[b] = np.where(few[b], np.float32(top), np.where(rng.random(V) < 0.5, np.float32(-top), x[b]))
+        elif kind == 5:
+            x[b] = rng.choice(np.array([-2.4e38, -2.3e38, -3e38], np.float32), V)
+        elif kind == 6:
+            x[b] = (rng.random(V) * 2 - 1).astype(np.float32) * np.float32(3.3e38)
+        elif kind == 7:                                                  # every magnitude, either sign
+            x[b] = np.where(rng.random(V) < 0.5, 1, -1) * np.exp(rng.random(V) * 88).astype(np.float32)
+        elif kind == 8:
+            x[b] = np.where(few[b], x[b], -np.exp(rng.random() * 88).astype(np.float32))
+        else:
+            x[b] = np.where(few[b], -np.float32(2.36e38), np.float32(-top))
+    return x
+
+
+def check_extreme(x, m, V, arg, lse):
+    """As check(); lse to TOL beside an fp32 rounding of the result."""
+    import oracle
+    a_o, l_o, _ = oracle.mask_logits(x, m, n_tokens=V, n_threads=NT)
+    assert_exact(arg, np.asarray(a_o, np.int32), "argmax")
+    g = lse.cpu().numpy().astype(np.float64)
+    fin = np.isfinite(l_o)
+    assert (np.isfinite(g) == fin).all() and not np.isnan(g).any()
+    assert (np.abs(g[fin] - l_o[fin]) <= TOL + 2.0 ** -23 * np.abs(l_o[fin])).all()
+
+
+@pytest.mark.parametrize("dt,batch", [(B.DTYPE_BF16, 24), (B.DTYPE_BF16, 200), (B.DTYPE_F32, 24), (B.DTYPE_F32, 200)])
+@pytest.mark.parametrize("share", [0.01, 0.6])
+def test_logits_at_the_ends_of_their_type(dt, batch, share):
+    """Given masks: the cluster kernel, and the gather (bf16, more rows than SMs)."""
+    V = 8000
+    f = extreme_logits(dt, batch, V, batch)
+    x = f if dt == B.DTYPE_F32 else synth.f32_to_bf16_bits(f)
+    t = torch.from_numpy(x.view(np.int16) if dt == B.DTYPE_BF16 else x).cuda()
+    m = masks(batch, V, share, 5)
+    arg, lse = poison.empty(batch, torch.int32), poison.empty(batch, torch.float32)
+    B.domino_mask_logits(handle(V).h, t.data_ptr(), dt, batch, V, torch.from_numpy(m.view(np.int32)).cuda(), arg, lse)
+    check_extreme(x, m, V, arg, lse)
+
+
+@pytest.mark.parametrize("dt", [B.DTYPE_BF16, B.DTYPE_F32])
+@pytest.mark.parametrize("walk", ["tree", "token"])
+@pytest.mark.parametrize("grammar", ["kv200", "sparse"])
+def test_folded_logits_at_the_ends_of_their_type(dt, walk, grammar, monkeypatch):
+    """The decode folded into either walk, over windows of few, some (the single bytes' window of the sparse grammar)
+    and many allowed tokens."""
+    import oracle
+    monkeypatch.setenv("DOMINO_WALK", walk)
+    rng = np.random.default_rng(31)
+    V, batch = 12000, 96
+    v = synth.random_vocab(rng, V, bytes(range(256)), synth.geometric_lengths(4.0, 32), synth._mixed_bytes)
+    a = synth.kv200_dfa(rng)[0] if grammar == "kv200" else synth.random_sparse_dfa(rng, 300)
+    states = rng.integers(1, a.n_states, batch)
+    wide = 1 + np.nonzero((a.delta[1:] == np.arange(1, a.n_states)[:, None]).sum(1) > 64)[0]   # inside strings
+    if grammar == "kv200":
+        states = np.where(rng.random(batch) < 0.5, rng.choice(wide, batch), states)
+    states = states.astype(np.int32)
+    d = Domino.from_parts(a, v, device=0)
+    m_o, _, _ = oracle.Problem.from_parts(a, v).step_mask(states, None, n_threads=NT)
+    f = extreme_logits(dt, batch, V, 7)
+    x = f if dt == B.DTYPE_F32 else synth.f32_to_bf16_bits(f)
+    t = torch.from_numpy(x.view(np.int16) if dt == B.DTYPE_BF16 else x).cuda()
+    mask = poison.empty((batch, d.info()["n_words"]), torch.int32)
+    arg, lse = poison.empty(batch, torch.int32), poison.empty(batch, torch.float32)
+    B.domino_step_decode(d.h, torch.from_numpy(states).cuda(), None, batch, t.data_ptr(), dt, V, mask, arg, lse)
+    assert_exact(mask, m_o, "mask")
+    check_extreme(x, m_o, V, arg, lse)
+    d.close()
+
+
 @pytest.mark.parametrize("dt,offset,pad", [(B.DTYPE_BF16, 0, 5), (B.DTYPE_BF16, 3, 0), (B.DTYPE_F32, 0, 0),
                                            (B.DTYPE_F32, 1, 2)])
 @pytest.mark.parametrize("grammar,batch", [("json", 60), ("json", 170), ("sparse", 5), ("sparse", 200),
