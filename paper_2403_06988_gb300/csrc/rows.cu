@@ -74,6 +74,7 @@ constexpr int kRowBig = 128;          // longer ranges
 constexpr int kRowNextHalf = 49152;   // tokens up to which rows of next states take half the threads
 constexpr int kRowSpawn = 2048;       // exits taken at a time
 constexpr int kRowExits = 512;        // loop subtrees whose exits are still to be walked
+constexpr int kWideAtOnce = 8;        // children of a wide node read together
 constexpr int kRowLoopMin = 4;        // fewest tokens of a subtree taken as a loop subtree
 constexpr int kRowMaxDevices = 64;
 static_assert(kRowBig <= kRowThreads / 2 && kRowExits <= kRowThreads, "one entry per thread in the prefix sums");
@@ -393,7 +394,7 @@ struct RowWalk {
         x.em.s = it.s;
         x.em.n = A.z >> 24;   // the tokens that end here
         if constexpr (WIDE) {
-            x.c = (int)A.x;   // refused children become dead items
+            x.c = (int)A.x;   // dead children too
             if (x.c == 0) x.em.n = B.y - B.x;
             else if (x.em.n == 255u) x.em.n = __ldg(&t.node[2 * (size_t)x.first_child + 1].x) - B.x;
         } else {
@@ -411,6 +412,59 @@ struct RowWalk {
             }
         }
         return x;
+    }
+
+    // Places in the pool for c items of every thread of the warp, behind the
+    // base items that stay: the slot of the thread's first, or -1 when the pool
+    // is full.  some: the threads with c > 0 (not 0).
+    __device__ __forceinline__ int places(int c, unsigned some, int base, int half, int4* st) const {
+        int at, tot;
+        if (!__any_sync(0xffffffffu, c > 1)) {
+            at = __popc(some & ((1u << lane) - 1u));
+            tot = __popc(some);
+        } else {
+            const int incl = warp_scan_incl(c, lane);
+            at = incl - c;
+            tot = __shfl_sync(0xffffffffu, incl, 31);
+        }
+        int first = 0;
+        if (lane == 0) first = base + atomicAdd(&st->x, tot);
+        first = __shfl_sync(0xffffffffu, first, 0);
+        if (first + tot > kRowPool) {
+            st->y = 1;
+            return -1;
+        }
+        return at + half + first;
+    }
+
+    // WIDE: adds the item's live children, kWideAtOnce of them at a time, whose
+    // classes and then entries are read together; kRowFan threads share an item
+    // when split.  A wide node has up to 256 children of which few live in any
+    // one state: with every child placed (and dropped a round later) rows of 1000
+    // live nodes filled the pool.  GB300, 500 states, V = 128256, batch 256, masks,
+    // us: 100 classes, 20 live 168 -> 27, 256 classes, 40 live 156 -> 26.
+    __device__ __forceinline__ void add_wide(const Item& it, const Node& x, bool split, int base, int half,
+                                             int4* st) const {
+        const int by = split ? kRowFan : 1;
+        for (int k0 = split ? tid & (kRowFan - 1) : 0; __any_sync(0xffffffffu, k0 < x.c); k0 += kWideAtOnce * by) {
+            uint32_t e[kWideAtOnce];
+#pragma unroll
+            for (int q = 0; q < kWideAtOnce; ++q)
+                e[q] = k0 + q * by < x.c ? (uint32_t)__ldg(t.ncls + x.first_child + (uint32_t)(k0 + q * by)) : 0u;
+            int c = 0;
+#pragma unroll
+            for (int q = 0; q < kWideAtOnce; ++q) {
+                e[q] = k0 + q * by < x.c ? dense(it.s, e[q]) : 0u;
+                c += e[q] != 0u;
+            }
+            const unsigned some = __ballot_sync(0xffffffffu, c > 0);
+            if (!some) continue;
+            int at = places(c, some, base, half, st);
+            if (at < 0) return;
+#pragma unroll
+            for (int q = 0; q < kWideAtOnce; ++q)
+                if (e[q]) put(at++, step(x.first_child + (uint32_t)(k0 + q * by), e[q], it.depth, it.bits));
+        }
     }
 
     // Expands the pool's n items until none are left.  In a round every
@@ -441,23 +495,18 @@ struct RowWalk {
             if ((fan ? (tid & ~31) / kRowFan : tid & ~31) < take) {   // warps with an item
               for (bool split = fan;;) {
                 Node x = read(it, lead, before, st);
-                // this thread's share of the children
-                int c;
-                Mask m = 0;
                 if constexpr (WIDE) {
-                    const int q = split ? tid & (kRowFan - 1) : 0, step = split ? kRowFan : 1;
-                    c = x.c > q ? (x.c - q + step - 1) / step : 0;
+                    add_wide(it, x, split, base, half, st);
                 } else {
-                    m = x.m;
+                    // this thread's share of the children
+                    Mask m = x.m;
                     if (split) {
                         if (t.n_loops > 0) m = shfl_lead(m);   // the lead may have taken the subtree whole
                         constexpr int kWidth = (int)sizeof(Mask) * 8 / kRowFan;   // classes per thread
                         m &= (((Mask)1 << kWidth) - 1) << (kWidth * (tid & (kRowFan - 1)));
                     }
-                    c = popc(m);
-                }
-                const unsigned some = __ballot_sync(0xffffffffu, c > 0);
-                if constexpr (!WIDE) {
+                    const int c = popc(m);
+                    const unsigned some = __ballot_sync(0xffffffffu, c > 0);
                     // thin tails: while no warp has left work in the pool and
                     // this one's items have at most one child each, its
                     // threads go on with the children themselves
@@ -477,31 +526,10 @@ struct RowWalk {
                         lead = true;
                         continue;
                     }
-                }
-                // places for the children, warp by warp
-                if (some) {
-                    int at, tot;
-                    if (!__any_sync(0xffffffffu, c > 1)) {
-                        at = __popc(some & ((1u << lane) - 1u));
-                        tot = __popc(some);
-                    } else {
-                        const int incl = warp_scan_incl(c, lane);
-                        at = incl - c;
-                        tot = __shfl_sync(0xffffffffu, incl, 31);
-                    }
-                    int first = 0;
-                    if (lane == 0) first = base + atomicAdd(&st->x, tot);
-                    first = __shfl_sync(0xffffffffu, first, 0);
-                    at += half + first;
-                    if (first + tot > kRowPool) {
-                        st->y = 1;
-                    } else if constexpr (WIDE) {
-                        for (int k = split ? tid & (kRowFan - 1) : 0; c > 0; k += split ? kRowFan : 1, --c) {
-                            const uint32_t child = x.first_child + (uint32_t)k;
-                            put(at++, step(child, dense(it.s, __ldg(t.ncls + child)), it.depth, it.bits));
-                        }
-                    } else {
-                        for (; m; m &= m - 1) {
+                    // places for the children, warp by warp
+                    if (some) {
+                        int at = places(c, some, base, half, st);
+                        for (m = at < 0 ? 0 : m; m; m &= m - 1) {
                             const Mask below = (m & (~m + 1)) - 1;
                             put(at++, step(x.first_child + (uint32_t)popc(x.kids & below),
                                            target(it.s, popc(x.live & below)), it.depth, it.bits));

@@ -1,0 +1,63 @@
+"""The walk that is chosen for a mask step is not much slower than the
+per-token walk, on random automata whose rows visit 1000 to 4000 nodes of the
+prefix tree: few of many byte classes live in a state.  A row whose live nodes
+do not fit row_kernel's pool is walked twice, which took 1.5 to 3.7 times the
+per-token walk's time here; the bound of 1.25 leaves room for the clock."""
+import functools
+
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+from paper_2403_06988_gb300 import Domino, synth  # noqa: E402
+from paper_2403_06988_gb300 import _binding as B  # noqa: E402
+
+V, Q = 128256, 500
+
+
+@functools.lru_cache(maxsize=1)
+def vocab():
+    return synth.random_vocab(np.random.default_rng(77), V, bytes(range(256)), synth.geometric_lengths(4.5, 32),
+                              synth._mixed_bytes)
+
+
+def mask_us(a, batch):
+    """(time of a mask step, the masks) on a new handle: the shortest of 8 replays of 10 steps."""
+    d = Domino.from_parts(a, vocab(), device=0)
+    st = torch.from_numpy(np.random.default_rng(3).integers(1, Q, batch).astype(np.int32)).cuda()
+    mask = torch.empty((batch, d.info()["n_words"]), dtype=torch.int32, device="cuda")
+    run = lambda: B.domino_step_mask(d.h, st, None, batch, mask)
+    for _ in range(3):
+        run()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        for _ in range(10):
+            run()
+    us = []
+    for _ in range(8):
+        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        e0.record()
+        g.replay()
+        e1.record()
+        torch.cuda.synchronize()
+        us.append(e0.elapsed_time(e1) * 100)
+    out = mask.cpu().numpy().copy()
+    d.close()
+    return min(us), out
+
+
+@pytest.mark.parametrize("classes,live", [(66, 16), (100, 20), (256, 40)])
+@pytest.mark.parametrize("batch", [32, 256])
+def test_chosen_walk_is_not_much_slower_than_the_per_token_walk(classes, live, batch, monkeypatch):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    a = synth.random_sparse_dfa(np.random.default_rng(5), Q, classes, live)
+    monkeypatch.delenv("DOMINO_WALK", raising=False)
+    chosen, m = mask_us(a, batch)
+    monkeypatch.setenv("DOMINO_WALK", "token")
+    token, want = mask_us(a, batch)
+    assert (m == want).all()
+    assert chosen < 1.25 * token, (chosen, token)
