@@ -66,7 +66,8 @@ namespace domino {
 namespace {
 
 constexpr int kRowThreads = 512;      // a CTA's, or half of it (launch_row_d)
-constexpr int kRowPool = 2048;        // items the pool holds
+constexpr int kRowPool = 2816;        // items the pool holds
+constexpr int kRowSlots = 4096;       // their slots (run)
 constexpr int kRowFan = 8;            // threads per item while there are few
 constexpr int kRowSmall = 512;        // ranges of 2 to kRowSmallTokens tokens left to the whole CTA
 constexpr int kRowSmallTokens = 64;
@@ -78,7 +79,8 @@ constexpr int kWideAtOnce = 8;        // children of a wide node read together
 constexpr int kRowLoopMin = 4;        // fewest tokens of a subtree taken as a loop subtree
 constexpr int kRowMaxDevices = 64;
 static_assert(kRowBig <= kRowThreads / 2 && kRowExits <= kRowThreads, "one entry per thread in the prefix sums");
-static_assert(kRowThreads == kDecodeThreads && 2 * kRowPool * 8 >= kDecodeListBytes, "the decode's lists lie in the pool");
+static_assert(kRowSlots - kRowPool >= kRowThreads && kRowSpawn <= kRowPool, "the next round's items fit");
+static_assert(kRowThreads == kDecodeThreads && kRowSlots * 8 >= kDecodeListBytes, "the decode's lists lie in the pool");
 
 enum RowOut : int {
     kRowMask = 0,    // the mask
@@ -122,8 +124,8 @@ __host__ __device__ inline RowLayout row_layout(int slice_words, bool stack, boo
     RowLayout L{};
     int o = 16;
     L.mask = o;   o += align16(slice_words * 4) + 16;
-    L.items = o;  o += align16(2 * kRowPool * 8);
-    L.bits = o;   o += stack ? align16(2 * kRowPool * 4) : 0;
+    L.items = o;  o += align16(kRowSlots * 8);
+    L.bits = o;   o += stack ? align16(kRowSlots * 4) : 0;
     L.range = o;  o += (kRowSmall + kRowBig) * 16;
     L.exits = o;  o += loops ? kRowExits * 16 : 0;
     L.pre = o;    o += align16((kRowThreads + 1) * 4);
@@ -414,10 +416,11 @@ struct RowWalk {
         return x;
     }
 
-    // Places in the pool for c items of every thread of the warp, behind the
-    // base items that stay: the slot of the thread's first, or -1 when the pool
-    // is full.  some: the threads with c > 0 (not 0).
-    __device__ __forceinline__ int places(int c, unsigned some, int base, int half, int4* st) const {
+    // Places in the pool for c items of every thread of the warp: the slot of
+    // the thread's first, or -1 when the pool is full.  `base` items stay in
+    // the pool and the next round's item j lies in slot lo + j.  some: the
+    // threads with c > 0 (not 0).
+    __device__ __forceinline__ int places(int c, unsigned some, int base, int lo, int4* st) const {
         int at, tot;
         if (!__any_sync(0xffffffffu, c > 1)) {
             at = __popc(some & ((1u << lane) - 1u));
@@ -434,7 +437,7 @@ struct RowWalk {
             st->y = 1;
             return -1;
         }
-        return at + half + first;
+        return lo + first + at;
     }
 
     // WIDE: adds the item's live children, kWideAtOnce of them at a time, whose
@@ -443,7 +446,7 @@ struct RowWalk {
     // one state: with every child placed (and dropped a round later) rows of 1000
     // live nodes filled the pool.  GB300, 500 states, V = 128256, batch 256, masks,
     // us: 100 classes, 20 live 168 -> 27, 256 classes, 40 live 156 -> 26.
-    __device__ __forceinline__ void add_wide(const Item& it, const Node& x, bool split, int base, int half,
+    __device__ __forceinline__ void add_wide(const Item& it, const Node& x, bool split, int base, int lo,
                                              int4* st) const {
         const int by = split ? kRowFan : 1;
         for (int k0 = split ? tid & (kRowFan - 1) : 0; __any_sync(0xffffffffu, k0 < x.c); k0 += kWideAtOnce * by) {
@@ -459,7 +462,7 @@ struct RowWalk {
             }
             const unsigned some = __ballot_sync(0xffffffffu, c > 0);
             if (!some) continue;
-            int at = places(c, some, base, half, st);
+            int at = places(c, some, base, lo, st);
             if (at < 0) return;
 #pragma unroll
             for (int q = 0; q < kWideAtOnce; ++q)
@@ -469,18 +472,24 @@ struct RowWalk {
 
     // Expands the pool's n items until none are left.  In a round every
     // thread takes one item from the pool's top (kRowFan threads share one
-    // while there are few) and adds its live children: to the pool's other
-    // half when the round takes all items, else in their place.  false: the
-    // pool was full (every_token() takes the row).
+    // while there are few) and adds its live children.  A round that takes all
+    // items puts them behind those, so that no warp waits for the others to have
+    // read theirs; only when the items lie past the spare slots, or some stay,
+    // do they take the place of those read.  In two halves of 2048 slots, taken
+    // in turn, rows with levels of 2000 live nodes were full and walked twice
+    // (GB300, 500 states, V = 128256, batch 256, masks, us: 48 classes, 16 live
+    // 192 -> 36, 64 classes, 20 live 189 -> 35, 32 classes, 14 live 225 -> 56;
+    // 5000 states 15.8 -> 15.9, JSON, V = 152064, batch 128 23.8 -> 23.9).
+    // false: the pool was full (every_token() takes the row).
     __device__ __forceinline__ bool run(int n) const {
-        int half = 0;   // where the items lie
+        int lo = 0;   // the items lie in slots lo to lo + n - 1
         Tokens before{0u, 0u, 0u, 0u};
         for (int r = 0;; r = r == 2 ? 0 : r + 1) {
             int4* st = &sh.st[r];
             if (n == 0) {
                 n = spawn_exits();   // the same for every thread of the CTA
                 if (n == 0) break;
-                half = 0;
+                lo = 0;
             }
             const int take = min(n, THREADS);
             const int base = n - take;
@@ -488,15 +497,19 @@ struct RowWalk {
             const int i = fan ? tid / kRowFan : tid;
             bool lead = !fan || (tid & (kRowFan - 1)) == 0;   // this thread answers for its item
             Item it{0u, 0u, 0u, 0u};
-            if (i < take) it = get(half + base + i);
+            if (i < take) it = get(lo + base + i);
             if (tid == 0) sh.st[r == 2 ? 0 : r + 1] = make_int4(0, 0, 0, 0);   // read by all two rounds ago
-            if (base > 0) __syncthreads();   // the items are read before others take their place
-            else half ^= kRowPool;
+            if (base > 0 || lo + take > kRowSlots - kRowPool) {
+                __syncthreads();   // the items are read before others take their place
+                if (base == 0) lo = 0;
+            } else {
+                lo += take;
+            }
             if ((fan ? (tid & ~31) / kRowFan : tid & ~31) < take) {   // warps with an item
               for (bool split = fan;;) {
                 Node x = read(it, lead, before, st);
                 if constexpr (WIDE) {
-                    add_wide(it, x, split, base, half, st);
+                    add_wide(it, x, split, base, lo, st);
                 } else {
                     // this thread's share of the children
                     Mask m = x.m;
@@ -528,7 +541,7 @@ struct RowWalk {
                     }
                     // places for the children, warp by warp
                     if (some) {
-                        int at = places(c, some, base, half, st);
+                        int at = places(c, some, base, lo, st);
                         for (m = at < 0 ? 0 : m; m; m &= m - 1) {
                             const Mask below = (m & (~m + 1)) - 1;
                             put(at++, step(x.first_child + (uint32_t)popc(x.kids & below),
@@ -590,7 +603,7 @@ struct RowWalk {
         return s_pre[n];
     }
 
-    // The loop subtrees' exits become the pool's items, in its first half
+    // The loop subtrees' exits become the pool's items, in its first slots
     // (the pool is empty before).  Returns their number, 0 when none are left.
     __device__ __forceinline__ int spawn_exits() const {
         if (t.n_loops == 0) return 0;
