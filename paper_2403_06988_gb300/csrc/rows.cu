@@ -899,8 +899,10 @@ cudaError_t launch_row_t(const StepView& v, const RowTree& t, const LaunchEnv& e
     // 256 rows of 128256 23.1 / 28.5.  The log-probabilities want the threads:
     // 310 rows 91.6 / 76.9, 620 rows (three waves, two) 144 / 152.  So do long
     // rows of next states: tables, V = 32000 194 / 162, V = 64000 302 / 314.
+    // 100 classes, 20 live, V = 32000, masks of 400 rows 29.7 / 22.5, 1000 rows
+    // 58.5 / 39.6.
     // With a stack the rounds are longer: JSON, V = 152064, 512 rows 78.6 / 98.1.
-    if constexpr (!STACK && CLS != kRowWide) {
+    if constexpr (!STACK) {
         const RowLayout L = row_layout((v.W + 3) / 4 * 4, STACK, t.n_loops > 0, OUT == kRowBf16 || OUT == kRowF32);
         const int64_t fit = std::min(4, (env.max_smem_optin + 1024) / (L.total + 1024 + (int)sizeof(RowShared)));
         if (fit > 2 && a.batch > 2 * env.num_sms && (OUT != kRowNext || v.V <= kRowNextHalf)) {

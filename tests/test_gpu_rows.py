@@ -235,13 +235,15 @@ def test_first_step_in_a_capture():
 
 @pytest.mark.parametrize("batch", [309, 701])
 def test_rows_of_half_the_threads(batch):
-    """More rows than run at once: CTAs of 256 threads, with and without loop sets."""
+    """More rows than run at once: CTAs of 256 threads, with and without loop sets, and with more than 64 classes."""
     rng = np.random.default_rng(13)
     v = synth.random_vocab(rng, 15987, bytes(range(256)), synth.geometric_lengths(4.0, 32), synth._mixed_bytes)
     a = synth.random_sparse_dfa(rng, 400)
     check(a, v, rng.integers(0, 400, batch).astype(np.int32), want_next=True)
     a, _ = synth.kv200_dfa(rng)
     check(a, v, rng.integers(0, 200, batch).astype(np.int32))
+    a = random_dfa(rng, 400, 100, 12)
+    check(a, v, rng.integers(0, 400, batch).astype(np.int32), want_next=True)
 
 
 def test_recorded_step_outlives_larger_batches():
