@@ -573,11 +573,23 @@ bool rows_dense(const domino_ctx* h, const RowBuild& rb, const RowEntries& merge
     return 8 * over > n;
 }
 
-// The trees, state records and loop sets of RowTree.  rows_ready stays false
-// (the per-token walk is used) when the vocabulary or its tree is too large.
-int build_rows(domino_ctx* h) {
-    h->rows_ready = false;
-    if (!h->trie_built || h->W > kRowMaxSlices * kRowSliceWords) return DOMINO_OK;
+// RowTree's arrays on the host.
+struct RowImage {
+    RowBuild rb;                     // the trees
+    std::vector<int64_t> roots;      // per loop set its tree
+    std::vector<uint32_t> loopbits;
+    std::vector<uint8_t> keeps, srec, srec_next, trec;
+    std::vector<uint2> xrange, exits, start;
+    std::vector<uint32_t> loop_of;
+    std::vector<uint16_t> ret;       // the merged states' pop targets
+    int32_t stride = 0, stride_next = 0;
+    bool dense = false;
+};
+
+// The trees, state records and loop sets of RowTree; false when the vocabulary
+// or its tree is too large (the per-token walk is used).
+bool make_row_image(const domino_ctx* h, RowImage& im) {
+    if (!h->trie_built || h->W > kRowMaxSlices * kRowSliceWords) return false;
     const int smem = h->env.max_smem_optin > 0 ? h->env.max_smem_optin : 232448;
     const bool wide = h->K > 64;
     const int32_t Q = h->Q, K = h->K;
@@ -612,9 +624,9 @@ int build_rows(domino_ctx* h) {
         std::stable_sort(all.begin(), all.end(), [](const auto& a, const auto& b) { return a.second > b.second; });
         for (size_t i = 0; i < all.size() && i < (size_t)kRowLoopSets; i++) sets.push_back(all[i].first);
     }
-    RowBuild rb;
-    std::vector<int64_t> roots;
-    std::vector<uint32_t> loopbits;
+    RowBuild& rb = im.rb;
+    std::vector<int64_t>& roots = im.roots;
+    std::vector<uint32_t>& loopbits = im.loopbits;
     for (bool ok = false; !ok;) {   // once more without loop sets when they make the trees too large
         rb = RowBuild();
         rb.wide = wide;
@@ -643,62 +655,67 @@ int build_rows(domino_ctx* h) {
         for (auto& e : rb.exits) n_exits += e.size();
         ok = ok && n_exits < (size_t)(1u << 24) &&
              row_smem_bytes(h->W, h->stack, !sets.empty()) <= smem - 1024;
-        if (!ok && sets.empty()) return DOMINO_OK;
+        if (!ok && sets.empty()) return false;
         if (!ok) sets.clear();
     }
     const size_t n_sets = sets.size();
-    std::vector<uint8_t> keeps;
-    std::vector<uint2> xrange, exits;
     for (size_t i = 0; i < n_sets; i++) {
-        const uint32_t base = (uint32_t)exits.size();
-        keeps.insert(keeps.end(), rb.keeps[i].begin(), rb.keeps[i].end());
-        for (uint2 x : rb.xrange[i]) xrange.push_back(make_uint2(x.x + base, x.y + base));
-        exits.insert(exits.end(), rb.exits[i].begin(), rb.exits[i].end());
+        const uint32_t base = (uint32_t)im.exits.size();
+        im.keeps.insert(im.keeps.end(), rb.keeps[i].begin(), rb.keeps[i].end());
+        for (uint2 x : rb.xrange[i]) im.xrange.push_back(make_uint2(x.x + base, x.y + base));
+        im.exits.insert(im.exits.end(), rb.exits[i].begin(), rb.exits[i].end());
     }
-    std::vector<uint32_t> loop_of;   // per merged state its loop set
-    std::vector<uint2> start;        // per state {merged state, its loop set}
-    std::vector<uint8_t> srec, srec_next;
-    int32_t stride = 0, stride_next = 0;
     const bool same = wide || merged.Q == Q;   // nothing was merged: one set of records
     if (!wide) {
-        loop_of.assign((size_t)merged.Q, 0xFFFFFFFFu);
+        im.loop_of.assign((size_t)merged.Q, 0xFFFFFFFFu);   // per merged state its loop set
         for (int32_t q = 1; q < merged.Q; q++) {
             const auto it = std::find(sets.begin(), sets.end(), self[(size_t)q]);
-            if (it != sets.end()) loop_of[(size_t)q] = (uint32_t)(it - sets.begin());
+            if (it != sets.end()) im.loop_of[(size_t)q] = (uint32_t)(it - sets.begin());
         }
-        srec = state_records(merged, K, h->stack, loop_of, &stride);
+        im.srec = state_records(merged, K, h->stack, im.loop_of, &im.stride);
         if (!same || n_sets) {
-            for (int32_t q = 0; q < Q; q++)
-                start.push_back(make_uint2((uint32_t)id[(size_t)q], loop_of[(size_t)id[(size_t)q]]));
+            for (int32_t q = 0; q < Q; q++)   // per state {merged state, its loop set}
+                im.start.push_back(make_uint2((uint32_t)id[(size_t)q], im.loop_of[(size_t)id[(size_t)q]]));
             // next states: the automaton's own, without loop sets
             RowEntries own;
             own.Q = Q;
             own.e.resize((size_t)Q * (size_t)K);
             for (size_t i = 0; i < own.e.size(); i++) own.e[i] = h->stack ? h->t32[i] : h->t16[i];
-            srec_next = state_records(own, K, h->stack, {}, &stride_next);
+            im.srec_next = state_records(own, K, h->stack, {}, &im.stride_next);
         }
     }
-    int rc;
-    auto up = [&](DevBuf& b, const void* p, size_t n) { return dev_upload(b, n ? p : nullptr, std::max<size_t>(16, n)); };
-    if ((rc = up(h->d_rnode, rb.node.data(), rb.node.size() * sizeof(uint4)))) return rc;
-    if ((rc = up(h->d_rncls, rb.ncls.data(), rb.ncls.size()))) return rc;
-    if ((rc = up(h->d_rdtok, rb.dtok.data(), rb.dtok.size() * 4))) return rc;
-    if ((rc = up(h->d_srec, srec.data(), srec.size()))) return rc;
-    if ((rc = up(h->d_srec_next, srec_next.data(), srec_next.size()))) return rc;
-    if ((rc = up(h->d_rret, merged.ret.data(), merged.ret.size() * 2))) return rc;
-    if ((rc = up(h->d_rstart, start.data(), start.size() * sizeof(uint2)))) return rc;
-    if ((rc = up(h->d_loop_of, loop_of.data(), loop_of.size() * 4))) return rc;
-    if ((rc = up(h->d_loopbits, loopbits.data(), loopbits.size() * 4))) return rc;
-    if ((rc = up(h->d_keeps, keeps.data(), keeps.size()))) return rc;
-    if ((rc = up(h->d_xrange, xrange.data(), xrange.size() * sizeof(uint2)))) return rc;
-    if ((rc = up(h->d_exits, exits.data(), exits.size() * sizeof(uint2)))) return rc;
-    std::vector<uint8_t> trec((size_t)h->V * 32, 0);
+    im.trec.assign((size_t)h->V * 32, 0);
     for (int32_t t = 0; t < h->V; t++) {
         const int64_t len = t == h->eos_id ? 0 : h->tok_off[t + 1] - h->tok_off[t];
-        trec[(size_t)t * 32] = (uint8_t)std::min<int64_t>(len, 255);
-        if (len > 0) std::memcpy(&trec[(size_t)t * 32 + 1], cls.data() + h->tok_off[t], (size_t)std::min<int64_t>(len, 31));
+        im.trec[(size_t)t * 32] = (uint8_t)std::min<int64_t>(len, 255);
+        if (len > 0)
+            std::memcpy(&im.trec[(size_t)t * 32 + 1], cls.data() + h->tok_off[t], (size_t)std::min<int64_t>(len, 31));
     }
-    if ((rc = up(h->d_trec, trec.data(), trec.size()))) return rc;
+    im.dense = rows_dense(h, rb, merged, self);
+    im.ret = std::move(merged.ret);
+    return true;
+}
+
+// The row walk's arrays on the device.
+int build_rows(domino_ctx* h) {
+    h->rows_ready = false;
+    RowImage im;
+    if (!make_row_image(h, im)) return DOMINO_OK;
+    int rc;
+    auto up = [&](DevBuf& b, const void* p, size_t n) { return dev_upload(b, n ? p : nullptr, std::max<size_t>(16, n)); };
+    if ((rc = up(h->d_rnode, im.rb.node.data(), im.rb.node.size() * sizeof(uint4)))) return rc;
+    if ((rc = up(h->d_rncls, im.rb.ncls.data(), im.rb.ncls.size()))) return rc;
+    if ((rc = up(h->d_rdtok, im.rb.dtok.data(), im.rb.dtok.size() * 4))) return rc;
+    if ((rc = up(h->d_srec, im.srec.data(), im.srec.size()))) return rc;
+    if ((rc = up(h->d_srec_next, im.srec_next.data(), im.srec_next.size()))) return rc;
+    if ((rc = up(h->d_rret, im.ret.data(), im.ret.size() * 2))) return rc;
+    if ((rc = up(h->d_rstart, im.start.data(), im.start.size() * sizeof(uint2)))) return rc;
+    if ((rc = up(h->d_loop_of, im.loop_of.data(), im.loop_of.size() * 4))) return rc;
+    if ((rc = up(h->d_loopbits, im.loopbits.data(), im.loopbits.size() * 4))) return rc;
+    if ((rc = up(h->d_keeps, im.keeps.data(), im.keeps.size()))) return rc;
+    if ((rc = up(h->d_xrange, im.xrange.data(), im.xrange.size() * sizeof(uint2)))) return rc;
+    if ((rc = up(h->d_exits, im.exits.data(), im.exits.size() * sizeof(uint2)))) return rc;
+    if ((rc = up(h->d_trec, im.trec.data(), im.trec.size()))) return rc;
     const StepView v = make_view(h);
     RowTree t{};
     t.trec = (const uint8_t*)h->d_trec.p;
@@ -706,28 +723,28 @@ int build_rows(domino_ctx* h) {
     t.ncls = (const uint8_t*)h->d_rncls.p;
     t.dtok = (const int32_t*)h->d_rdtok.p;
     t.srec = (const uint4*)h->d_srec.p;
-    t.ret = wide ? v.ret : (const uint16_t*)h->d_rret.p;
-    t.start = start.empty() ? nullptr : (const uint2*)h->d_rstart.p;
+    t.ret = im.rb.wide ? v.ret : (const uint16_t*)h->d_rret.p;
+    t.start = im.start.empty() ? nullptr : (const uint2*)h->d_rstart.p;
     t.loop_of = (const uint32_t*)h->d_loop_of.p;
     t.loopbits = (const uint32_t*)h->d_loopbits.p;
     t.keeps = (const uint8_t*)h->d_keeps.p;
     t.xrange = (const uint2*)h->d_xrange.p;
     t.exits = (const uint2*)h->d_exits.p;
-    t.srec_stride = stride;
-    t.n_nodes = (int32_t)(rb.node.size() / 2);
-    t.n_dtok = (int32_t)rb.dtok.size();
-    t.n_loops = (int32_t)n_sets;
-    for (size_t i = 0; i < n_sets; i++) t.loop_root[i] = (int32_t)roots[i];
+    t.srec_stride = im.stride;
+    t.n_nodes = (int32_t)(im.rb.node.size() / 2);
+    t.n_dtok = (int32_t)im.rb.dtok.size();
+    t.n_loops = (int32_t)im.roots.size();
+    for (size_t i = 0; i < im.roots.size(); i++) t.loop_root[i] = (int32_t)im.roots[i];
     h->rows = t;
-    if (!start.empty()) {
+    if (!im.start.empty()) {
         t.srec = (const uint4*)h->d_srec_next.p;
-        t.srec_stride = stride_next;
+        t.srec_stride = im.stride_next;
         t.ret = v.ret;
         t.start = nullptr;
         t.n_loops = 0;
     }
     h->rows_next = t;
-    h->rows_dense = rows_dense(h, rb, merged, self);
+    h->rows_dense = im.dense;
     h->rows_ready = true;
     return DOMINO_OK;
 }
