@@ -131,6 +131,9 @@ struct RowTree {
 constexpr int kRowLoopSets = 4;           // loop sets with a tree of their own
 constexpr int kRowMaxSlices = 8;          // CTAs per row (one cluster)
 constexpr int kRowSliceWords = 16384;     // mask words a CTA can hold
+constexpr int kRowThreads = 512;          // a CTA's, or half of it (launch_row_d)
+constexpr int kRowPool = 2816;            // (node, state) items a row may have at a time; a row with more is walked
+                                          // token by token
 
 struct LaunchEnv {
     int num_sms;

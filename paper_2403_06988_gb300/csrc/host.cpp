@@ -73,7 +73,8 @@ struct domino_ctx {
         d_exits, d_trec;
     RowTree rows{}, rows_next{};     // for masks; for next states
     bool rows_ready = false;
-    bool rows_dense = false;         // most states' walks visit many nodes (rows_dense())
+    bool rows_dense = false;         // most rows' walks are too large for it (row_cost)
+    int64_t rows_visits = 0;         // nodes a row's walk visits
     // which walk the mask step takes: -1 chosen from the automaton (see
     // use_tree), 1 the prefix tree, 0 every token on its own (DOMINO_WALK=tree
     // or =token in the environment when the handle is created)
@@ -535,42 +536,62 @@ std::vector<uint8_t> state_records(const RowEntries& r, int K, bool stack, const
     return out;
 }
 
-// Whether the walks of more than an eighth of the states (an even sample)
-// visit more than kDenseNodes nodes of the tree.  Subtrees below a state that
-// loops on their classes are left out, and so are the classes of a wide loop:
-// those are not walked node by node.
+// What row_kernel's walk of a row costs, from an even sample of the states,
+// walked on the host as the kernel does: rounds of kRowThreads items from the
+// pool's top, their live children in their place.  visits: the nodes a row
+// visits (the median).  dense: more than an eighth of the rows visit more than
+// kDenseNodes or have more items at a time than the pool holds (those are walked
+// twice), so that the per-token walk is the better one.  Subtrees below a state
+// that loops on their classes are left out, and so are the classes of a wide
+// loop: those are not walked node by node.
 constexpr int64_t kDenseNodes = 8192;
 constexpr int kDenseSample = 256;
-bool rows_dense(const domino_ctx* h, const RowBuild& rb, const RowEntries& merged, const std::vector<uint64_t>& self) {
+struct RowCost {
+    int64_t visits = 0;
+    bool dense = false;
+};
+RowCost row_cost(const domino_ctx* h, const RowBuild& rb, const RowEntries& merged, const std::vector<uint64_t>& self) {
     const int64_t K = h->K, n_states = rb.wide ? h->Q : merged.Q;
     const int n = (int)std::min<int64_t>(kDenseSample, n_states - 1);
     int over = 0;
-    std::vector<std::pair<uint32_t, uint32_t>> work;   // (node, state)
+    std::vector<int64_t> visits((size_t)n, 0);
+    std::vector<std::pair<uint32_t, uint32_t>> pool, taken;   // (node, state)
     for (int i = 0; i < n; i++) {
-        int64_t visits = 0;
-        work.assign(1, {0u, (uint32_t)(1 + (n_states - 1) * i / n)});
-        while (!work.empty() && visits <= kDenseNodes) {
-            const auto [node, q] = work.back();
-            work.pop_back();
-            visits++;
-            const uint4 a = rb.node[2 * (size_t)node], b = rb.node[2 * (size_t)node + 1];
-            const uint64_t keep = rb.wide ? 0 : self[q], below = ((uint64_t)b.w << 32) | b.z;
-            if (!rb.wide && (below & ~keep) == 0) continue;
-            const bool loop = 4 * __builtin_popcountll(keep) >= K;
-            const uint32_t first = a.z & 0xFFFFFFu;
-            const int kids = rb.wide ? (int)a.x : __builtin_popcountll(((uint64_t)a.y << 32) | a.x);
-            for (int k = 0; k < kids; k++) {
-                const uint32_t c = rb.ncls[(size_t)first + (size_t)k];
-                if (loop && ((keep >> c) & 1ull)) continue;
-                const size_t at = (size_t)(q * K + c);
-                const uint32_t e = !rb.wide ? merged.e[at] : h->stack ? h->t32[at] : h->t16[at];
-                const uint32_t to = h->stack && ((e >> kKindShift) & 3u) == 2u ? 0u : e & 0xFFFFu;   // not past a pop
-                if (to) work.push_back({first + (uint32_t)k, to});
+        int64_t& v = visits[(size_t)i];
+        bool full = false;
+        pool.assign(1, {0u, (uint32_t)(1 + (n_states - 1) * i / n)});
+        while (!pool.empty() && !full && v <= kDenseNodes) {
+            const size_t stay = pool.size() - std::min<size_t>(pool.size(), kRowThreads);
+            taken.assign(pool.begin() + (ptrdiff_t)stay, pool.end());
+            pool.resize(stay);
+            for (const auto& [node, q] : taken) {
+                v++;
+                const uint4 a = rb.node[2 * (size_t)node], b = rb.node[2 * (size_t)node + 1];
+                const uint64_t keep = rb.wide ? 0 : self[q], below = ((uint64_t)b.w << 32) | b.z;
+                if (!rb.wide && (below & ~keep) == 0) continue;
+                const bool loop = 4 * __builtin_popcountll(keep) >= K;
+                const uint32_t first = a.z & 0xFFFFFFu;
+                const int kids = rb.wide ? (int)a.x : __builtin_popcountll(((uint64_t)a.y << 32) | a.x);
+                for (int k = 0; k < kids; k++) {
+                    const uint32_t c = rb.ncls[(size_t)first + (size_t)k];
+                    if (loop && ((keep >> c) & 1ull)) continue;
+                    const size_t at = (size_t)(q * K + c);
+                    const uint32_t e = !rb.wide ? merged.e[at] : h->stack ? h->t32[at] : h->t16[at];
+                    const uint32_t to = h->stack && ((e >> kKindShift) & 3u) == 2u ? 0u : e & 0xFFFFu;   // not past a pop
+                    if (to) pool.push_back({first + (uint32_t)k, to});
+                }
             }
+            full = pool.size() > (size_t)kRowPool;
         }
-        over += visits > kDenseNodes;
+        over += full || v > kDenseNodes;
     }
-    return 8 * over > n;
+    RowCost r;
+    r.dense = 8 * over > n;
+    if (n > 0) {
+        std::nth_element(visits.begin(), visits.begin() + n / 2, visits.end());
+        r.visits = visits[(size_t)(n / 2)];
+    }
+    return r;
 }
 
 // RowTree's arrays on the host.
@@ -583,7 +604,7 @@ struct RowImage {
     std::vector<uint32_t> loop_of;
     std::vector<uint16_t> ret;       // the merged states' pop targets
     int32_t stride = 0, stride_next = 0;
-    bool dense = false;
+    RowCost cost;
 };
 
 // The trees, state records and loop sets of RowTree; false when the vocabulary
@@ -691,7 +712,7 @@ bool make_row_image(const domino_ctx* h, RowImage& im) {
         if (len > 0)
             std::memcpy(&im.trec[(size_t)t * 32 + 1], cls.data() + h->tok_off[t], (size_t)std::min<int64_t>(len, 31));
     }
-    im.dense = rows_dense(h, rb, merged, self);
+    im.cost = row_cost(h, rb, merged, self);
     im.ret = std::move(merged.ret);
     return true;
 }
@@ -744,7 +765,8 @@ int build_rows(domino_ctx* h) {
         t.n_loops = 0;
     }
     h->rows_next = t;
-    h->rows_dense = im.dense;
+    h->rows_dense = im.cost.dense;
+    h->rows_visits = im.cost.visits;
     h->rows_ready = true;
     return DOMINO_OK;
 }
@@ -892,10 +914,21 @@ bool use_tree(const domino_ctx* h) {
 // The (row, token) pairs from which row_kernel is the faster walk.  Its time
 // is the latency of a row's rounds (8 to 40 us), once for every 2 * SMs rows;
 // the per-token walk's grows with the pairs.  In units of 2^19 pairs: `first`
-// for up to 2 * SMs rows, `more` for every further such wave.
+// for up to 2 * SMs rows, `more` for every further such wave.  Both hold for
+// rows that visit up to kVisits nodes, and grow by kVisitUnits for every 1000
+// more (us per token / row_kernel, masks, 500 states, V = 128256: 3770 visits
+// (12 of 32 classes live), batch 32 23 / 33, batch 96 28 / 32, batch 128 35 / 32,
+// batch 256 58 / 37; 7030 visits (14 live), batch 96 33 / 47, batch 192 49 / 53,
+// batch 256 66 / 56; V = 32000, 2560 visits, batch 800 60 / 74; 100 classes, 20
+// live, 1300 visits, V = 128256, batch 24 21 / 24, batch 64 26 / 23, batch 256 47
+// / 27; 256 classes, 40 live, 1030 visits, batch 256 102 / 26).
+constexpr int64_t kVisits = 1100;
+constexpr double kVisitUnits = 8.0;
 bool rows_pay(const domino_ctx* h, int64_t batch, int first, int more) {
     const int64_t at_once = 2 * std::max(1, h->env.num_sms);
-    return batch * h->V >= (first + (batch - 1) / at_once * more) * ((int64_t)1 << 19);
+    const double beyond = kVisitUnits * (double)std::max<int64_t>(0, h->rows_visits - kVisits) / 1000.0;
+    return (double)(batch * h->V) >=
+           (first + beyond + (double)((batch - 1) / at_once) * (more + beyond)) * (double)((int64_t)1 << 19);
 }
 
 // Whether row_kernel takes a mask step (GB300, us per-token / row_kernel).
@@ -910,9 +943,10 @@ bool rows_pay(const domino_ctx* h, int64_t batch, int first, int more) {
 // 9.2, V = 64000, batch 98 10.7 / 8.3; V = 16000, batch 400 26.2 / 8.3, V =
 // 8000, batch 1000 11.1 / 15.2; their next states are the per-token walk's
 // (loop sets hold masks only).
-// Automata most of whose rows visit much of the tree (rows_dense) are the
-// per-token walk's: 500 states with 16 of 32 classes live, V = 128256, batch
-// 256 76 / 235, 28 live 179 / 521 (12 live, 2.6 % of the tokens: 58 / 36, row_kernel's).
+// Automata most of whose rows are too large (row_cost) are the per-token
+// walk's: 500 states with 16 of 32 classes live, V = 128256, batch 256 76 / 247,
+// 18 live 86 / 274, 28 live 179 / 542 (14 live, 4.3 % of the tokens: 66 / 56,
+// row_kernel's).
 bool use_rows(const domino_ctx* h, int64_t batch, bool next) {
     if (!h->rows_ready || h->walk_pref == 0) return false;
     if (h->walk_pref == 1) return true;

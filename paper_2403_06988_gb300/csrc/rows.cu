@@ -65,9 +65,7 @@
 namespace domino {
 namespace {
 
-constexpr int kRowThreads = 512;      // a CTA's, or half of it (launch_row_d)
-constexpr int kRowPool = 2816;        // items the pool holds
-constexpr int kRowSlots = 4096;       // their slots (run)
+constexpr int kRowSlots = 4096;       // slots of the pool's items (run)
 constexpr int kRowFan = 8;            // threads per item while there are few
 constexpr int kRowSmall = 512;        // ranges of 2 to kRowSmallTokens tokens left to the whole CTA
 constexpr int kRowSmallTokens = 64;

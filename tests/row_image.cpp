@@ -30,7 +30,7 @@ void* row_image_make(domino_t h) {
 }
 void row_image_free(void* p) { delete static_cast<RowImage*>(p); }
 
-// Array `which` of an image, and {record strides, loop sets, wide, dense}.
+// Array `which` of an image, and {record strides, loop sets, wide, dense, visits}.
 int row_image_get(void* p, int which, const void** data, int64_t* bytes) {
     const RowImage& im = *static_cast<RowImage*>(p);
     const Array all[] = {array_of(im.rb.node),  array_of(im.rb.ncls), array_of(im.rb.dtok), array_of(im.roots),
@@ -48,7 +48,8 @@ void row_image_info(void* p, int64_t* out) {
     out[1] = im.stride_next;
     out[2] = (int64_t)im.roots.size();
     out[3] = im.rb.wide;
-    out[4] = im.dense;
+    out[4] = im.cost.dense;
+    out[5] = im.cost.visits;
 }
 
 // The automaton's own table and pop targets, as the wide form reads them.

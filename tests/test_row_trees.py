@@ -56,9 +56,9 @@ class Image:
         for i, name in enumerate(NAMES):
             setattr(self, name, take(lambda p, b: L.row_image_get(im, i, p, b), TYPES.get(name, np.uint32)))
         self.node = self.node.reshape(-1, 8)
-        info = (ctypes.c_int64 * 5)()
+        info = (ctypes.c_int64 * 6)()
         L.row_image_info(im, info)
-        self.stride, self.stride_next, self.n_loops, self.wide, self.dense = info[0], info[1], info[2], info[3], info[4]
+        self.stride, self.stride_next, self.n_loops, self.wide, self.dense, self.visits = info
         self.xrange, self.exits = self.xrange.reshape(self.n_loops or 1, -1, 2), self.exits.reshape(-1, 2)
         self.keeps = self.keeps.reshape(self.n_loops or 1, -1)
         self.loopbits = self.loopbits.reshape(self.n_loops or 1, -1)
@@ -274,6 +274,49 @@ def test_many_tokens_at_a_node(lib):
     live = np.array([0, 1, 1, 1], np.uint8)
     a = synth.Automaton(delta=delta, live=live, accepting=live.copy(), start=1, rules=None, max_depth=0, name="two")
     check(lib, a, random_tokens(rng, 6000, bytes(range(30, 128)), 3), range(4))
+
+
+def visited(a, v, q):
+    """The class-string prefixes that are alive from state q: the nodes its walk visits, by definition."""
+    seen = {b""}
+    cols, cls = np.unique(a.delta, axis=1, return_inverse=True)
+    for t in range(v.n_tokens):
+        s, key = q, b""
+        for c in v.data[v.offsets[t]:v.offsets[t + 1]] if t != v.eos_id else b"":
+            s = int(a.delta[s, c])
+            if not a.live[s]:
+                break
+            key += bytes([cls.reshape(-1)[c]])
+            seen.add(key)
+    return len(seen)
+
+
+@pytest.mark.parametrize("classes,live", [(32, 6), (64, 12), (100, 30), (256, 60)])
+def test_nodes_that_a_row_visits(lib, classes, live):
+    """The cost by which a walk is chosen counts live nodes, not the children looked at."""
+    rng = np.random.default_rng(classes)
+    a = synth.random_sparse_dfa(rng, 12, classes, live)
+    v = random_tokens(rng, 1200, bytes(range(256)), 3)
+    im = Image(lib, a, v)
+    want = sorted(visited(a, v, q) for q in range(1, 12))
+    assert im.visits == want[len(want) // 2] and not im.dense
+
+
+@pytest.mark.parametrize("live,dense", [(40, 0), (60, 1)])
+def test_levels_that_the_pool_does_not_hold(lib, live, dense):
+    """1600 and 3600 nodes alive two classes deep (below the 8192 in all that count as dense): the pool holds 2816."""
+    rng = np.random.default_rng(live)
+    delta = np.zeros((40, 256), np.int32)
+    for q in range(1, 40):
+        for c in rng.permutation(64)[:live]:
+            delta[q, 4 * c:4 * c + 4] = 1 + (q + int(rng.integers(0, 38))) % 39   # never q
+    alive = np.ones(40, np.uint8)
+    alive[0] = 0
+    a = synth.Automaton(delta=delta, live=alive, accepting=alive.copy(), start=1, rules=None, max_depth=0, name="wide levels")
+    pairs = [bytes([4 * i, 4 * j]) for i in range(64) for j in range(64)]
+    v = synth.Vocab.from_tokens(pairs + [b""], eos_id=len(pairs))
+    im = Image(lib, a, v)
+    assert im.dense == dense and (dense or im.visits == 1 + live + live * live)
 
 
 def test_token_records(lib):
