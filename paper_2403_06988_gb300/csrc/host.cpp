@@ -977,6 +977,16 @@ bool decode_rows(const domino_ctx* h, int64_t batch, bool fusable) {
     return h->self_mask.empty() ? rows_pay(h, batch, 6, 5) : rows_pay(h, batch, 16, 6);
 }
 
+// Whether the decode can ride on the per-token walk, whose partials then take
+// fpart_bytes().
+bool can_fuse(const domino_ctx* h, const void* logits, int32_t dtype, int32_t batch, int64_t stride) {
+    return dtype == DOMINO_DTYPE_BF16 && reinterpret_cast<uintptr_t>(logits) % 16 == 0 &&
+           ((size_t)stride * 2) % 16 == 0 && (int64_t)batch * h->n_windows < (int64_t)INT32_MAX;   // partial slots are int
+}
+size_t fpart_bytes(const domino_ctx* h, int32_t batch) {
+    return (size_t)batch * (size_t)h->n_windows * sizeof(float4);
+}
+
 int ready_for_compute(domino_ctx* h) {
     if (!h) return DOMINO_E_INVALID_ARG;
     if (is_host_only(h)) return DOMINO_E_NO_DEVICE;
@@ -1475,17 +1485,14 @@ int domino_step_decode(domino_t h, const int32_t* states_dev, const uint64_t* st
         return DOMINO_E_INVALID_ARG;
     DeviceGuard g(h->device);
     cudaStream_t st = (cudaStream_t)stream;
-    // the decode can ride on the per-token walk
-    const bool fusable = dtype == DOMINO_DTYPE_BF16 && reinterpret_cast<uintptr_t>(logits_dev) % 16 == 0 &&
-                         ((size_t)row_stride_elems * 2) % 16 == 0 &&
-                         (int64_t)batch * h->n_windows < (int64_t)INT32_MAX;   // partial slots are int
+    const bool fusable = can_fuse(h, logits_dev, dtype, batch, row_stride_elems);
     // logits in device memory are pulled into L2 ahead of their fold;
     // host-resident logits are read only where the mask allows a token
     cudaPointerAttributes pa{};
     const bool on_device = cudaPointerGetAttributes(&pa, logits_dev) == cudaSuccess && pa.type == cudaMemoryTypeDevice;
     if (!on_device) cudaGetLastError();
     bool rows = decode_rows(h, batch, fusable);
-    const size_t part_bytes = (size_t)batch * (size_t)h->n_windows * sizeof(float4);
+    const size_t part_bytes = fpart_bytes(h, batch);
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (!rows && fusable && h->d_fpart.n < part_bytes) {
         // growing the partials buffer synchronises the stream and reallocates,
@@ -1807,18 +1814,19 @@ int domino_decode_step_host(domino_t h, const void* logits_host, int32_t dtype, 
         else if (h->t_wall_ms[0] == 0.0) mapped = false;
         else mapped = (h->t_wall_ms[1] <= h->t_wall_ms[0]) != (h->host_calls % 64 == 63);
     }
-    // the in-place path runs the fused decode, whose per-window partials
-    // buffer is grown here too, before any recording
-    const size_t fpart_bytes = (size_t)batch * (size_t)h->n_windows * sizeof(float4);
+    // where the in-place path folds the decode into the per-token walk, its
+    // partials are grown here too, before any recording
+    const bool fuse = mapped && can_fuse(h, pa.devicePointer, dtype, batch, h->V);
+    const size_t part_bytes = fuse && !decode_rows(h, batch, fuse) ? fpart_bytes(h, batch) : 0;
     const bool grow = (!mapped && h->s_logits.n < logit_bytes) || h->s_io.n < L.in_end ||
                       h->s_mask.n < (size_t)batch * (size_t)h->W * 4 || h->h_io_n < L.in_end || !h->cp_stream ||
-                      (mapped && h->d_fpart.n < fpart_bytes);
+                      h->d_fpart.n < part_bytes;
     if (grow) {   // buffers may move: recorded steps that use them are dropped
         if (cudaStreamSynchronize(st) != cudaSuccess) return cuda_status(cudaGetLastError());
         clear_host_graphs(h);
     }
     if (!mapped && (rc = dev_reserve(h->s_logits, logit_bytes))) return rc;
-    if (mapped && (rc = grow_fpart(h, fpart_bytes))) return rc;
+    if ((rc = grow_fpart(h, part_bytes))) return rc;
     if ((rc = dev_reserve(h->s_mask, (size_t)batch * (size_t)h->W * 4))) return rc;
     if ((rc = dev_reserve(h->s_io, L.in_end))) return rc;
     if (h->h_io_n < L.in_end) {

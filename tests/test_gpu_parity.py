@@ -404,6 +404,30 @@ def test_decode_step_host_path_choice_keeps_results():
     d.close()
 
 
+@pytest.mark.parametrize("walk", ["tree", "token"])
+def test_decode_step_host_reserves_what_its_walk_needs(walk, monkeypatch):
+    """The per-window partials (float4 per row and 1024 tokens) are the per-token walk's: where row_kernel takes the
+    in-place step, none are reserved (and no recorded step is dropped for them)."""
+    monkeypatch.setenv("DOMINO_WALK", walk)
+    rng = np.random.default_rng(41)
+    V, b = 8000, 24
+    a = synth.random_sparse_dfa(rng, 100)
+    d = Domino.from_parts(a, synth.random_vocab(rng, V, bytes(range(256)), synth.geometric_lengths(4.0, 16),
+                                                synth._mixed_bytes), device=0)
+    before = d.info()["device_bytes"]
+    lg = torch.zeros((b, V), dtype=torch.bfloat16).pin_memory()
+    st = torch.ones(b, dtype=torch.int32).pin_memory()
+    tok, lse = torch.empty(b, dtype=torch.int32).pin_memory(), torch.empty(b, dtype=torch.float32).pin_memory()
+    B.domino_decode_step_host(d.h, lg.data_ptr(), B.DTYPE_BF16, b, st.data_ptr(), None, tok.data_ptr(), lse.data_ptr(),
+                              stream=0)
+    up = lambda n: (n + 15) // 16 * 16
+    io = up(up(4 * b) + up(4 * b) + 4 * b)              # tokens, lse, states
+    partials = b * ((V + 1023) // 1024) * 16
+    assert d.info()["device_bytes"] - before == up(b * (V // 32) * 4) + io + (partials if walk == "token" else 0)
+    assert d.device_error() == 0
+    d.close()
+
+
 def test_decode_step_host_batch_grows_on_a_recording_stream():
     """Pinned bf16 logits on a non-default stream, with batches growing from
     call to call.  On a fresh handle the first calls take the in-place path
