@@ -180,8 +180,8 @@ __device__ __forceinline__ float gumbel(const SampleArgs& a, int r, int t, int& 
 // still sees its tokens in increasing order) and folds them.  Zero words cost
 // a few instructions, every load of a span is independent, and a span costs
 // one memory latency whatever its density.  The warps' partials are merged in
-// shared memory.  Logit lines are not kept in L1, and in L2 only when a
-// log-prob pass reads them again (evict-last; otherwise evict-first).
+// shared memory.  Logit lines are not kept in L1 and go first in L2: no pass
+// after this one reads them.
 constexpr int kGatherMaxWarps = 16;   // warps per CTA (one row); two CTAs per SM
 constexpr int kGatherSpan = 8;     // mask words per lane per span (8192 tokens)
 constexpr int kGatherWarpSmem = 32 * kGatherSpan * (4 + 4 * 2);   // a span's words and its list
@@ -194,12 +194,12 @@ __device__ __forceinline__ float bf16_of(const uint4& q, int e) {
 }
 
 // chunk: words per warp, a multiple of kGatherSpan.  A sampling pass draws
-// row r with counter row row0 + (batch row of r).
+// row r with the counter of its batch row.
 template <int FOLD>
 __global__ void __launch_bounds__(kGatherMaxWarps * 32, 2)
     logits_gather_kernel(const void* __restrict__ logits, int64_t stride, const MaskRows mask, int V, int W, int B,
                          int chunk, int32_t* __restrict__ argmax, float* __restrict__ lse, const SampleArgs sa,
-                         int row0, int keep_l2, const RowList list) {
+                         const RowList list) {
     constexpr int kSpanWords = 32 * kGatherSpan;
     extern __shared__ __align__(16) unsigned char g_smem[];   // per warp: words, then list
     __shared__ float4 s_part[kGatherMaxWarps];
@@ -210,7 +210,7 @@ __global__ void __launch_bounds__(kGatherMaxWarps * 32, 2)
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     uint32_t* sw = reinterpret_cast<uint32_t*>(g_smem + wid * kGatherWarpSmem);   // a span's mask words
     uint16_t* lst = reinterpret_cast<uint16_t*>(sw + kSpanWords);                // its vectors, in token order
-    const uint64_t pol = l2_policy(keep_l2 != 0);
+    const uint64_t pol = l2_policy(false);
     const int full_vec = V / 8;   // vectors that lie wholly inside the row
     const int j0 = wid * chunk, j1 = min(W, j0 + chunk);
     const uint32_t* mrow = mask.row(r, W, threadIdx.x == 0);
@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(kGatherMaxWarps * 32, 2)
         if constexpr (FOLD == kFoldSample) {
             const float sx = __fmul_rn(x, sa.inv_t);
             if (__fadd_rn(sx, kGumbelMax) < m) return;
-            const float sc = __fadd_rn(sx, gumbel(sa, row0 + orow, t, blk, rnd));
+            const float sc = __fadd_rn(sx, gumbel(sa, orow, t, blk, rnd));
             if (sc > m) {
                 m = sc;
                 idx = t;
@@ -426,7 +426,7 @@ cudaError_t launch_gather(const LogitsArgs& a, const RowList& list, cudaStream_t
     if (cudaError_t e = gather_smem_ready<FOLD>(); e != cudaSuccess) return e;
     return launch_pdl(logits_gather_kernel<FOLD>, dim3((unsigned)a.batch), dim3(nwarps * 32),
                       (size_t)(nwarps * kGatherWarpSmem), st, a.logits, a.stride, a.mask, a.V, a.W, a.batch, chunk,
-                      a.argmax, a.lse, a.sample, 0, 0, list);
+                      a.argmax, a.lse, a.sample, list);
 }
 
 template <bool BF16, int FOLD>
@@ -460,7 +460,7 @@ cudaError_t launch_mask_logits(const LaunchEnv& env, const void* logits, int dty
     a.logprobs = logprobs;
     a.sample = sample ? *sample : SampleArgs{0u, 0u, 0u, 0u, 1.0f};
     cut_rows(a, env.num_sms);
-    const RowList list{row_ids, row_count, 0};
+    const RowList list{row_ids, row_count};
     // The gather wants one CTA per row to fill the SMs, aligned bf16 rows, and
     // no second pass: there it is the faster one where masks are sparse
     // (GB300, V = 128256, 1 % allowed, batch 256: 6.0 against 8.0 us, batch

@@ -95,7 +95,7 @@ enum RowClasses : int { kRow32 = 0, kRow64 = 1, kRowWide = 2 };
 struct RowArgs {
     const int32_t* states;
     const uint64_t* stacks;
-    int32_t batch;          // rows (the cap of a row list)
+    int32_t batch;
     int32_t row_is_state;
     int32_t slices;         // CTAs per row (a cluster)
     int32_t slice_words;    // mask words per CTA (a multiple of 4)
@@ -477,7 +477,7 @@ struct RowWalk {
     // in turn, rows with levels of 2000 live nodes were full and walked twice
     // (GB300, 500 states, V = 128256, batch 256, masks, us: 48 classes, 16 live
     // 192 -> 36, 64 classes, 20 live 189 -> 35, 32 classes, 14 live 225 -> 56;
-    // 5000 states 15.8 -> 15.9, JSON, V = 152064, batch 128 23.8 -> 23.9).
+    // 5000 states 15.8 -> 15.6, JSON, V = 152064, batch 128 23.9 -> 24.0).
     // false: the pool was full (every_token() takes the row).
     __device__ __forceinline__ bool run(int n) const {
         int lo = 0;   // the items lie in slots lo to lo + n - 1
@@ -735,7 +735,7 @@ __device__ __forceinline__ void update(const StepView& v, const RowTree& t, cons
 template <bool STACK, int CLS, int OUT, int THREADS>
 __global__ void __launch_bounds__(THREADS, 1024 / THREADS)
     row_kernel(const __grid_constant__ StepView v, const __grid_constant__ RowTree t,
-               const __grid_constant__ RowArgs a, const RowList list) {
+               const __grid_constant__ RowArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ RowShared sh;
     const RowLayout L = row_layout(a.slice_words, STACK, t.n_loops > 0, OUT == kRowBf16 || OUT == kRowF32);
@@ -755,7 +755,6 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS)
     }
     pdl_wait();
     pdl_trigger();
-    if (row >= list.rows(a.batch)) return;   // the whole cluster
     // The row's configuration (invalid ones set the error word, once per row),
     // in shared memory: one in pinned host memory crosses the host link once
     // per CTA, not once per warp (128256 tokens, batch 16, states read there:
@@ -764,7 +763,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS)
         const uint32_t q = (uint32_t)row;
         sh.rc = a.row_is_state
                     ? make_uint4(q, 0u, 0u, 1u | (((__ldg(v.accept_bits + (q >> 5)) >> (q & 31u)) & 1u) ? 2u : 0u))
-                    : read_row_rw(v, a.states, a.stacks, list.row(row), slice == 0);
+                    : read_row_rw(v, a.states, a.stacks, row, slice == 0);
     }
     __syncthreads();
     const uint4 rc = sh.rc;
@@ -796,7 +795,7 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS)
     if constexpr (kDecode)
         if (a.ahead)
             ahead = reinterpret_cast<const char*>(a.logits) +
-                    (size_t)list.row(row) * (size_t)a.stride * (OUT == kRowBf16 ? 2 : 4);
+                    (size_t)row * (size_t)a.stride * (OUT == kRowBf16 ? 2 : 4);
     const RowWalk<STACK, CLS, OUT, THREADS> wk{v, t, s_mask, reinterpret_cast<uint2*>(smem + L.items),
                                       reinterpret_cast<uint32_t*>(smem + L.bits),
                                       reinterpret_cast<uint4*>(smem + L.range),
@@ -825,9 +824,8 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS)
     }
     if constexpr (kDecode) {
         DecodeShared& dsh = *reinterpret_cast<DecodeShared*>(smem + L.dec);
-        const int b = list.row(row);
         Decoder<OUT == kRowBf16, kFoldLse> d;
-        d.init(a.logits, a.stride, b, v.V, a.logprobs != nullptr, SampleArgs{},
+        d.init(a.logits, a.stride, row, v.V, a.logprobs != nullptr, SampleArgs{},
                reinterpret_cast<const uint4*>(smem + L.keep), lane);
         d.template slice<THREADS>(s_mask, tok0, ntok, reinterpret_cast<uint16_t*>(smem + L.items) + warp * kDecodeList, warp);
         d.finish();
@@ -836,13 +834,13 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS)
         decode_combine<THREADS>(dsh, m, idx, sum, a.slices, lane, warp);
         const float lse = log_sum_exp(m, sum);
         if (a.logprobs)
-            write_logprobs<OUT == kRowBf16, THREADS>(d.lrow, v.V, s_mask, tok0, ntok, lse, a.logprobs + (size_t)b * v.V, tid);
+            write_logprobs<OUT == kRowBf16, THREADS>(d.lrow, v.V, s_mask, tok0, ntok, lse, a.logprobs + (size_t)row * v.V, tid);
         if (slice == 0 && tid == 0) {
             const int32_t tk = m == -INFINITY ? -1 : idx;
-            a.argmax[b] = tk;
-            if (a.lse) a.lse[b] = lse;
+            a.argmax[row] = tk;
+            if (a.lse) a.lse[row] = lse;
             // every CTA of the row has read its configuration (the outputs may alias it)
-            if (a.states_out) update<STACK>(v, t, sh.rc, tk, b, a.states_out, a.stacks_out);
+            if (a.states_out) update<STACK>(v, t, sh.rc, tk, row, a.states_out, a.stacks_out);
         }
         if (a.slices > 1) cluster_wait();
     }
@@ -864,8 +862,7 @@ cudaError_t rows_allow_smem(K kern, int bytes, int* configured, std::mutex& mu) 
 }
 
 template <bool STACK, int CLS, int OUT, int THREADS>
-cudaError_t launch_row_d(const StepView& v, const RowTree& t, const LaunchEnv& env, RowArgs a, const RowList& list,
-                         cudaStream_t st) {
+cudaError_t launch_row_d(const StepView& v, const RowTree& t, const LaunchEnv& env, RowArgs a, cudaStream_t st) {
     // CTAs per row: enough to give every SM one (two where a row is decoded
     // and has two: JSON, V = 152064, batch 128 54.6 -> 45.7 us), and enough for
     // the row's words to fit
@@ -882,13 +879,11 @@ cudaError_t launch_row_d(const StepView& v, const RowTree& t, const LaunchEnv& e
     static std::mutex mu;
     cudaError_t e = rows_allow_smem(kern, L.total, configured, mu);
     if (e != cudaSuccess) return e;
-    return launch_cluster(kern, dim3((unsigned)a.batch * (unsigned)s), dim3(THREADS), s, (size_t)L.total, st, v, t, a,
-                          list);
+    return launch_cluster(kern, dim3((unsigned)a.batch * (unsigned)s), dim3(THREADS), s, (size_t)L.total, st, v, t, a);
 }
 
 template <bool STACK, int CLS, int OUT>
-cudaError_t launch_row_t(const StepView& v, const RowTree& t, const LaunchEnv& env, const RowArgs& a, const RowList& list,
-                         cudaStream_t st) {
+cudaError_t launch_row_t(const StepView& v, const RowTree& t, const LaunchEnv& env, const RowArgs& a, cudaStream_t st) {
     // More rows than run at once with 2 CTAs an SM (one CTA a row): CTAs of
     // half the threads, of which up to 4 fit, take more rows a wave, each wave
     // being 1.1 to 1.3 times as long.  GB300, us, 512 / 256 threads: 5000 states,
@@ -906,33 +901,33 @@ cudaError_t launch_row_t(const StepView& v, const RowTree& t, const LaunchEnv& e
         if (fit > 2 && a.batch > 2 * env.num_sms && (OUT != kRowNext || v.V <= kRowNextHalf)) {
             const int64_t full = (a.batch - 1) / (2 * env.num_sms) + 1, half = (a.batch - 1) / (fit * env.num_sms) + 1;
             if (a.logprobs ? 2 * half <= full : 5 * half < 4 * full)
-                return launch_row_d<STACK, CLS, OUT, kRowThreads / 2>(v, t, env, a, list, st);
+                return launch_row_d<STACK, CLS, OUT, kRowThreads / 2>(v, t, env, a, st);
         }
     }
-    return launch_row_d<STACK, CLS, OUT, kRowThreads>(v, t, env, a, list, st);
+    return launch_row_d<STACK, CLS, OUT, kRowThreads>(v, t, env, a, st);
 }
 
 template <bool STACK, int CLS>
 cudaError_t launch_row_o(const StepView& v, const RowTree& t, const LaunchEnv& env, const RowArgs& a, int dtype,
-                         const RowList& list, cudaStream_t st) {
+                         cudaStream_t st) {
     if (a.logits)
-        return dtype == DOMINO_DTYPE_BF16 ? launch_row_t<STACK, CLS, kRowBf16>(v, t, env, a, list, st)
-                                          : launch_row_t<STACK, CLS, kRowF32>(v, t, env, a, list, st);
-    return a.next ? launch_row_t<STACK, CLS, kRowNext>(v, t, env, a, list, st)
-                  : launch_row_t<STACK, CLS, kRowMask>(v, t, env, a, list, st);
+        return dtype == DOMINO_DTYPE_BF16 ? launch_row_t<STACK, CLS, kRowBf16>(v, t, env, a, st)
+                                          : launch_row_t<STACK, CLS, kRowF32>(v, t, env, a, st);
+    return a.next ? launch_row_t<STACK, CLS, kRowNext>(v, t, env, a, st)
+                  : launch_row_t<STACK, CLS, kRowMask>(v, t, env, a, st);
 }
 
 cudaError_t launch_row(const StepView& v, const RowTree& t, const LaunchEnv& env, bool stack, const RowArgs& a,
-                       int dtype, const RowList& list, cudaStream_t st) {
+                       int dtype, cudaStream_t st) {
     if (a.batch <= 0) return cudaSuccess;
     if (v.K <= 32)
-        return stack ? launch_row_o<true, kRow32>(v, t, env, a, dtype, list, st)
-                     : launch_row_o<false, kRow32>(v, t, env, a, dtype, list, st);
+        return stack ? launch_row_o<true, kRow32>(v, t, env, a, dtype, st)
+                     : launch_row_o<false, kRow32>(v, t, env, a, dtype, st);
     if (v.K <= 64)
-        return stack ? launch_row_o<true, kRow64>(v, t, env, a, dtype, list, st)
-                     : launch_row_o<false, kRow64>(v, t, env, a, dtype, list, st);
-    return stack ? launch_row_o<true, kRowWide>(v, t, env, a, dtype, list, st)
-                 : launch_row_o<false, kRowWide>(v, t, env, a, dtype, list, st);
+        return stack ? launch_row_o<true, kRow64>(v, t, env, a, dtype, st)
+                     : launch_row_o<false, kRow64>(v, t, env, a, dtype, st);
+    return stack ? launch_row_o<true, kRowWide>(v, t, env, a, dtype, st)
+                 : launch_row_o<false, kRowWide>(v, t, env, a, dtype, st);
 }
 
 }  // namespace
@@ -947,7 +942,7 @@ cudaError_t launch_row_step(const StepView& v, const RowTree& t, const LaunchEnv
     a.row_is_state = row_is_state ? 1 : 0;
     a.mask = mask;
     a.next = next;
-    return launch_row(v, t, env, stack, a, 0, RowList{nullptr, nullptr, 0}, st);
+    return launch_row(v, t, env, stack, a, 0, st);
 }
 
 cudaError_t launch_row_decode(const StepView& v, const RowTree& t, const LaunchEnv& env, bool stack,
@@ -967,7 +962,7 @@ cudaError_t launch_row_decode(const StepView& v, const RowTree& t, const LaunchE
     a.logprobs = logprobs;
     a.states_out = states_out;
     a.stacks_out = stacks_out;
-    return launch_row(v, t, env, stack, a, dtype, RowList{nullptr, nullptr, 0}, st);
+    return launch_row(v, t, env, stack, a, dtype, st);
 }
 
 int row_smem_bytes(int32_t n_words, bool stack, bool loops) {
