@@ -1011,6 +1011,11 @@ struct ApiRange {
 };
 #define DOMINO_API_RANGE() const ApiRange api_range_(__func__)
 
+// The entry points below that allocate host memory are function-try-blocks: an
+// exception must not pass into the C caller.  A load that ends this way leaves
+// the handle refusing what needs the part that was being built (its flag is
+// cleared first and set last).
+
 }  // namespace
 
 extern "C" {
@@ -1093,7 +1098,7 @@ int domino_destroy(domino_t h) {
 }
 
 int domino_load_vocab(domino_t h, const uint8_t* bytes, const int64_t* offsets, int32_t n_tokens,
-                      int32_t eos_id) {
+                      int32_t eos_id) try {
     DOMINO_API_RANGE();
     if (h) clear_host_graphs(h);
     if (!h || !offsets || n_tokens < 1 || n_tokens > (1 << 24)) return DOMINO_E_INVALID_ARG;
@@ -1123,11 +1128,13 @@ int domino_load_vocab(domino_t h, const uint8_t* bytes, const int64_t* offsets, 
         return DOMINO_OK;
     }
     return build_arena(h);
+} catch (...) {   // std::bad_alloc
+    return DOMINO_E_OOM;
 }
 
 int domino_load_automaton(domino_t h, const int32_t* delta, int32_t n_states, const uint8_t* live,
                           const uint8_t* accepting, int32_t start_state, const domino_stack_rule* rules,
-                          int32_t n_rules, int32_t max_depth) {
+                          int32_t n_rules, int32_t max_depth) try {
     DOMINO_API_RANGE();
     if (!h || !delta || !live || n_states < 1 || n_states > DOMINO_MAX_STATES) return DOMINO_E_INVALID_ARG;
     if (start_state < 0 || start_state >= n_states || max_depth < 0 || max_depth > DOMINO_MAX_DEPTH)
@@ -1344,6 +1351,8 @@ int domino_load_automaton(domino_t h, const int32_t* delta, int32_t n_states, co
         dev_free(h->d_self);
     }
     return build_arena(h);
+} catch (...) {   // std::bad_alloc
+    return DOMINO_E_OOM;
 }
 
 int domino_get_info(domino_t h, domino_info* out) {
@@ -1473,7 +1482,7 @@ int domino_advance(domino_t h, const int32_t* states_dev, const uint64_t* stacks
 int domino_step_decode(domino_t h, const int32_t* states_dev, const uint64_t* stacks_dev, int32_t batch,
                        const void* logits_dev, int32_t dtype, int64_t row_stride_elems, uint32_t* mask_dev,
                        int32_t* argmax_dev, float* lse_dev, float* logprobs_dev, int32_t* states_out,
-                       uint64_t* stacks_out, void* stream) {
+                       uint64_t* stacks_out, void* stream) try {
     DOMINO_API_RANGE();
     int rc = ready_for_compute(h);
     if (rc) return rc;
@@ -1534,6 +1543,8 @@ int domino_step_decode(domino_t h, const int32_t* states_dev, const uint64_t* st
         e = launch_logprobs_bf16(h->env, logits_dev, batch, row_stride_elems, h->V, mask_dev, lse_dev, logprobs_dev,
                                  st);
     return cuda_status(e);
+} catch (...) {   // std::bad_alloc
+    return DOMINO_E_OOM;
 }
 
 int domino_mask_sample(domino_t h, const void* logits_dev, int32_t dtype, int32_t batch, int64_t row_stride_elems,
@@ -1721,11 +1732,11 @@ int copy_and_decode_chunks(domino_ctx* h, const void* logits_host, int32_t dtype
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(io + L.st, (char*)h->h_io + L.st, L.in_end - L.st, cudaMemcpyHostToDevice, h->cp_stream);
     if (e == cudaSuccess) e = cudaEventRecord(h->ev_cfg, h->cp_stream);
-    std::vector<int32_t> r0s((size_t)n_chunks + 1);
-    for (int k = 0; k <= n_chunks; ++k) r0s[(size_t)k] = (int32_t)(((int64_t)batch * k) / n_chunks);
+    int32_t r0s[9];   // at most 8 chunks
+    for (int k = 0; k <= n_chunks; ++k) r0s[k] = (int32_t)(((int64_t)batch * k) / n_chunks);
     if (e == cudaSuccess) e = cudaEventRecord(h->ev_t[2], h->cp_stream);
     for (int k = 0; k < n_chunks && e == cudaSuccess; ++k) {
-        const size_t off = (size_t)r0s[(size_t)k] * row_bytes, n = (size_t)(r0s[(size_t)k + 1] - r0s[(size_t)k]) * row_bytes;
+        const size_t off = (size_t)r0s[k] * row_bytes, n = (size_t)(r0s[k + 1] - r0s[k]) * row_bytes;
         e = cudaMemcpyAsync((char*)h->s_logits.p + off, (const char*)logits_host + off, n, cudaMemcpyHostToDevice,
                             h->cp_stream);
         if (e == cudaSuccess) e = cudaEventRecord(h->ev_chunk[k], h->cp_stream);
@@ -1735,7 +1746,7 @@ int copy_and_decode_chunks(domino_ctx* h, const void* logits_host, int32_t dtype
     if (e != cudaSuccess) return cuda_status(e);
     if ((rc = domino_step_mask(h, d_states, d_stacks, batch, d_mask, nullptr, stream))) return rc;
     for (int k = 0; k < n_chunks; ++k) {
-        const int32_t r0 = r0s[(size_t)k], rows = r0s[(size_t)k + 1] - r0;
+        const int32_t r0 = r0s[k], rows = r0s[k + 1] - r0;
         if ((e = cudaStreamWaitEvent(st, h->ev_chunk[k], 0)) != cudaSuccess) return cuda_status(e);
         if ((rc = domino_mask_logits(h, (const char*)h->s_logits.p + (size_t)r0 * row_bytes, dtype, rows, h->V,
                                      d_mask + (size_t)r0 * h->W, d_tok + r0, d_lse + r0, nullptr, stream)))
@@ -1779,7 +1790,7 @@ int enqueue_host_step(domino_ctx* h, const void* logits_host, void* logits_mappe
 
 int domino_decode_step_host(domino_t h, const void* logits_host, int32_t dtype, int32_t batch,
                             int32_t* states_host, uint64_t* stacks_host, int32_t* tokens_host, float* lse_host,
-                            void* stream) {
+                            void* stream) try {
     DOMINO_API_RANGE();
     int rc = ready_for_compute(h);
     if (rc) return rc;
@@ -1921,6 +1932,8 @@ int domino_decode_step_host(domino_t h, const void* logits_host, int32_t dtype, 
         avg = avg == 0.0 ? t : 0.75 * avg + 0.25 * t;
     }
     return DOMINO_OK;
+} catch (...) {   // std::bad_alloc
+    return DOMINO_E_OOM;
 }
 
 
