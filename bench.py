@@ -206,17 +206,39 @@ def csrc_digest() -> str:
     return hs.hexdigest()[:16]
 
 
-def takes_rows(info, dev_id, batch, V, decode=False, fusable=True):
-    """Whether the call is row_kernel's (use_rows and decode_rows in host.cpp, for the launch counts)."""
-    import torch
-    sms = torch.cuda.get_device_properties(dev_id).multi_processor_count
-    if not decode:
-        first, more = (4, 4) if info["has_stack"] else (6, 5) if info["walk_tree"] else (10, 2)
-    elif not fusable:
-        first, more = 1, 1
-    else:
-        first, more = (4, 4) if info["has_stack"] else (6, 5) if info["walk_tree"] else (16, 6)
-    return batch * V >= (first + (batch - 1) // (2 * sms) * more) << 19
+def recorded_kernels(call, stream):
+    """The names of the kernels that call(stream) launches: recorded into a CUDA graph that is not run."""
+    import ctypes
+    cu = ctypes.CDLL("libcuda.so.1")
+
+    def ok(rc):
+        if rc:
+            raise RuntimeError(f"CUDA driver error {rc}")
+
+    class Params(ctypes.Structure):   # CUDA_KERNEL_NODE_PARAMS_v2
+        _fields_ = [("func", ctypes.c_void_p)] + [(f"dim{k}", ctypes.c_uint) for k in range(7)] + \
+                   [(n, ctypes.c_void_p) for n in ("params", "extra", "kern", "ctx")]
+    st, graph, n = ctypes.c_void_p(stream), ctypes.c_void_p(), ctypes.c_size_t()
+    ok(cu.cuStreamBeginCapture_v2(st, 2))           # relaxed
+    call(stream)
+    ok(cu.cuStreamEndCapture(st, ctypes.byref(graph)))
+    ok(cu.cuGraphGetNodes(graph, None, ctypes.byref(n)))
+    nodes = (ctypes.c_void_p * n.value)()
+    ok(cu.cuGraphGetNodes(graph, nodes, ctypes.byref(n)))
+    names = []
+    for node in nodes:
+        kind, prm, name = ctypes.c_int(), Params(), ctypes.c_char_p()
+        ok(cu.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)))
+        if kind.value:                              # not a kernel node
+            continue
+        ok(cu.cuGraphKernelNodeGetParams_v2(ctypes.c_void_p(node), ctypes.byref(prm)))
+        if prm.func:
+            ok(cu.cuFuncGetName(ctypes.byref(name), ctypes.c_void_p(prm.func)))
+        else:
+            ok(cu.cuKernelGetName(ctypes.byref(name), ctypes.c_void_p(prm.kern)))
+        names.append(name.value.decode())
+    ok(cu.cuGraphDestroy(graph))
+    return names
 
 
 def ncu_traffic(name: str) -> dict:
@@ -529,10 +551,6 @@ def run_domino(args, dist: Dist):
     # bf16 logits, the per-token walk with the greedy decode folded in, then the
     # per-row merge that also advances each row, plus the log-probs pass where
     # the workload asks for them; or (fp32) mask step, logits pass, update.
-    rows_decode = takes_rows(info, dev_id, Bsz, V, decode=True, fusable=w.logits_dtype == "bf16")
-    rows_mask = takes_rows(info, dev_id, Bsz, V)
-    fused = not rows_decode and w.logits_dtype == "bf16"
-    launches_per_step = 1 if rows_decode else 2 + (1 if w.want_logprobs else 0) if fused else 3
 
     def step(i, stream_ptr):
         rc = L.domino_step_decode(h, p_states, p_stacks, Bsz, p_logits[i % nbuf], dtype_code, V, p_mask, p_arg, p_lse,
@@ -548,6 +566,12 @@ def run_domino(args, dist: Dist):
         for i in range(Wm):
             step(i, sp)
     torch.cuda.synchronize()
+    step_kernels = recorded_kernels(lambda sp: step(0, sp), s.cuda_stream)
+    launches_per_step = len(step_kernels)
+    rows_decode = any("row_kernel" in k for k in step_kernels)
+    fused = any("fused_combine" in k for k in step_kernels)
+    rows_mask = any("row_kernel" in k for k in recorded_kernels(
+        lambda sp: L.domino_step_mask(h, p_states, p_stacks, Bsz, p_mask, None, sp), s.cuda_stream))
 
     def capture(n, body):
         """A CUDA graph of n calls of body(i, stream) on stream s (None: eager)."""
