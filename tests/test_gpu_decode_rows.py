@@ -1,15 +1,19 @@
 """The decode of one row by a CTA or a cluster of CTAs (decode.cuh) against
 the oracle: bf16 and fp32 rows at every alignment, vocabularies around the
 vector, word and segment sizes, 1 to 8 CTAs per row, sparse and dense masks,
-masks with bits past V, rows with nothing allowed, ties, infinite logits; the
-Gumbel-max draw over the same rows; and the mask step with the decode and the
-update folded in, over unaligned rows.  Tokens bit-exact.
+masks with bits past V, rows with nothing allowed, ties, infinite logits, the
+largest and lowest finite ones; masks that allow only the tokens around the
+edges of rows, slices and segments; the Gumbel-max draw over the same rows; and
+the mask step with the decode and the update folded in, over unaligned rows and
+over rows that row_kernel walks token by token.  Tokens bit-exact.
 
-Tolerance of lse and log-probabilities: a lane's sequential fp32 sum of at most
-1024 terms errs by at most 1024 * 2^-24 = 6.1e-5 relative, a term's exponent
-(below 64 in log2) by 64 * 2^-24 * ln 2 = 2.7e-6 and ex2 by 2^-22, so
-ln(sum) errs by less than 6.5e-5, and its rounding below 32 by 2^-19 = 2e-6:
-1e-4 in all.  Output buffers start as 0xAB bytes (tests/poison.py)."""
+Tolerance of lse and log-probabilities: a lane adds the sums of at most 36
+vectors (140000 tokens over 512 lanes) of 8 terms (5 additions deep), and lanes,
+warps and CTAs are merged in 12 steps: 53 roundings, 53 * 2^-24 = 3.2e-6
+relative.  A term e^-d errs by 2^-22 (ex2) and d * 2^-23 (its exponent's two
+roundings), 3e-7 of the sum at most.  So ln(sum) errs by less than 3.5e-6, and
+the roundings of logf, m + ln(sum) and x - lse (below 32) by 2^-20 each: 6.4e-6,
+1e-5 allowed.  Output buffers start as 0xAB bytes (tests/poison.py)."""
 import functools
 import os
 
@@ -26,7 +30,7 @@ import poison  # noqa: E402
 from poison import assert_exact, assert_no_poison  # noqa: E402
 
 NT = os.cpu_count() or 1
-TOL = 1e-4
+TOL = 1e-5
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -109,6 +113,132 @@ def test_rows_of_any_alignment(dt, V, batch, offset, pad, share):
     if V % 32:
         clean[:, -1] &= (1 << (V % 32)) - 1
     assert_exact(tok, np.asarray(oracle.mask_sample(x, clean, 0.7, 11, 5), np.int32), "drawn token")
+    del t
+
+
+def edge_tokens(V):
+    """The tokens within 9 of the ends of the row, of the slices of 1 to 8 CTAs and of segments of 4096 mask words."""
+    W = (V + 31) // 32
+    edges = {0, V}
+    for s in (1, 2, 4, 8):
+        words = ((W + s - 1) // s + 3) // 4 * 4
+        edges |= {32 * words * i for i in range(1, s)} | {131072 * i for i in range(1, V // 131072 + 1)}
+    return np.array(sorted({t for e in edges for t in range(e - 9, e + 9) if 0 <= t < V}))
+
+
+def edge_rows(dt, batch, V, seed):
+    """(logits, allowed tokens per row): tokens that are not allowed are the largest; a row allows every edge token,
+    with equal logits (lse = x + ln(n) then shows a token that is missing or taken twice), or one of them."""
+    rng = np.random.default_rng(seed)
+    edges = edge_tokens(V)
+    x = np.full((batch, V), 50.0, np.float32)
+    allowed = [edges if b % 3 == 0 else edges[[int(rng.integers(0, len(edges)))]] for b in range(batch)]
+    for b in range(batch):
+        x[b, allowed[b]] = 1.5
+    return (x if dt == B.DTYPE_F32 else synth.f32_to_bf16_bits(x)), allowed
+
+
+def check_edges(allowed, arg, lse, lp, V):
+    a, l = arg.cpu().numpy(), lse.cpu().numpy()
+    for b, t in enumerate(allowed):
+        assert a[b] == t[0], (b, a[b], t[0])
+        assert abs(float(l[b]) - (1.5 + np.log(len(t)))) < TOL, (b, len(t), l[b])
+    if lp is not None:
+        p = lp.cpu().numpy()
+        for b, t in enumerate(allowed):
+            assert (np.nonzero(np.isfinite(p[b]))[0] == t).all() and (p[b][~np.isfinite(p[b])] == -np.inf).all()
+            assert np.abs(p[b][t] + np.log(len(t))).max() < TOL
+
+
+def placed(x, dt, offset, pad):
+    """(the device buffer, address of row 0, row stride) of rows of V + pad elements, `offset` elements in."""
+    batch, V = x.shape
+    buf = np.zeros(offset + batch * (V + pad), x.dtype)
+    buf[offset:].reshape(batch, V + pad)[:, :V] = x
+    t = torch.from_numpy(buf.view(np.int16) if dt == B.DTYPE_BF16 else buf).cuda()
+    return t, t.data_ptr() + offset * x.dtype.itemsize, V + pad
+
+
+def bits_of(allowed, V):
+    m = np.zeros((len(allowed), (V + 31) // 32 * 32), np.uint8)
+    for b, t in enumerate(allowed):
+        m[b, t] = 1
+    return np.packbits(m, axis=1, bitorder="little").view(np.uint32)
+
+
+SHIFTS = [(B.DTYPE_BF16, k) for k in range(8)] + [(B.DTYPE_F32, k) for k in range(4)]
+
+
+@pytest.mark.parametrize("dt,shift,V,batch",
+                         [(dt, k, V, b) for dt, k in SHIFTS for V, b in ((1000, 9), (20001, 9), (20000, 40), (33000, 100),
+                                                                         (140000, 3))] +
+                         # more rows than SMs: one CTA a row, two segments (bf16 on 16-byte boundaries: the gather)
+                         [(B.DTYPE_BF16, 0, 140000, 160), (B.DTYPE_BF16, 3, 140000, 160), (B.DTYPE_F32, 1, 140000, 160)])
+def test_tokens_at_the_edges(dt, shift, V, batch):
+    """Every shift of the vectors against the mask: rows of V elements (odd V: every row at another shift) or padded to
+    whole 16 bytes (all rows at one)."""
+    x, allowed = edge_rows(dt, batch, V, V + batch + shift)
+    m = torch.from_numpy(bits_of(allowed, V).view(np.int32)).cuda()
+    for pad in {0, -V % 8}:
+        t, ptr, stride = placed(x, dt, shift, pad)
+        arg, lse, lp = (poison.empty(n, d) for n, d in ((batch, torch.int32), (batch, torch.float32),
+                                                        ((batch, V), torch.float32)))
+        B.domino_mask_logits(handle(V).h, ptr, dt, batch, stride, m, arg, lse, lp)
+        check_edges(allowed, arg, lse, lp, V)
+        arg, lse = poison.empty(batch, torch.int32), poison.empty(batch, torch.float32)
+        B.domino_mask_logits(handle(V).h, ptr, dt, batch, stride, m, arg, lse)
+        check_edges(allowed, arg, lse, None, V)
+        del t
+
+
+@functools.lru_cache(maxsize=2)
+def edge_grammar(V):
+    """An automaton and a vocabulary whose allowed tokens are the edge tokens (state 1) or one of them (the others)."""
+    edges = edge_tokens(V)
+    n = len(edges)
+    digits = lambda i: bytes([97 + i // 26 % 26, 97 + i % 26, 97 + i // 676])
+    toks = [b"#%d" % t for t in range(V)]
+    for i, t in enumerate(edges):
+        toks[t] = digits(i)
+    delta = np.zeros((4 + n, 256), np.int32)
+    delta[1, 97:123], delta[2, 97:123], delta[3, 97:123] = 2, 3, 1    # any three letters
+    live = np.ones(4 + n, np.uint8)
+    live[0] = 0
+    singles = []
+    for i in range(0, n, 7):                                          # one token's letters only, then nothing
+        q = len(singles) * 3 + 4
+        if q + 3 > 4 + n:
+            break
+        a, b, c = digits(i)
+        delta[q, a], delta[q + 1, b], delta[q + 2, c] = q + 1, q + 2, 1
+        singles.append((q, i))
+    a = synth.Automaton(delta=delta, live=live, accepting=np.zeros_like(live), start=1, rules=None, max_depth=0, name="edges")
+    return a, synth.Vocab.from_tokens(toks, eos_id=-1), edges, singles
+
+
+@pytest.mark.parametrize("dt,shift", SHIFTS)
+@pytest.mark.parametrize("V,batch", [(20001, 9), (20001, 40), (20001, 100), (20001, 200), (140001, 5)])
+def test_folded_tokens_at_the_edges(dt, shift, V, batch, monkeypatch):
+    """The same with the decode folded into row_kernel."""
+    monkeypatch.setenv("DOMINO_WALK", "tree")
+    a, v, edges, singles = edge_grammar(V)
+    rng = np.random.default_rng(batch + shift)
+    pick = [None if b % 3 == 0 else singles[int(rng.integers(0, len(singles)))] for b in range(batch)]
+    states = np.array([1 if p is None else p[0] for p in pick], np.int32)
+    allowed = [edges if p is None else edges[[p[1]]] for p in pick]
+    x = np.full((batch, V), 50.0, np.float32)
+    for b in range(batch):
+        x[b, allowed[b]] = 1.5
+    t, ptr, stride = placed(x if dt == B.DTYPE_F32 else synth.f32_to_bf16_bits(x), dt, shift, 0)
+    d = Domino.from_parts(a, v, device=0)
+    mask = poison.empty((batch, (V + 31) // 32), torch.int32)
+    arg, lse, lp = (poison.empty(n, k) for n, k in ((batch, torch.int32), (batch, torch.float32),
+                                                    ((batch, V), torch.float32)))
+    B.domino_step_decode(d.h, torch.from_numpy(states).cuda(), None, batch, ptr, dt, stride, mask, arg, lse, lp)
+    assert_exact(mask, bits_of(allowed, V), "mask")
+    check_edges(allowed, arg, lse, lp, V)
+    assert d.device_error() == 0
+    d.close()
     del t
 
 
