@@ -26,6 +26,7 @@ torch = pytest.importorskip("torch")
 
 from paper_2403_06988_gb300 import Domino, synth  # noqa: E402
 from paper_2403_06988_gb300 import _binding as B  # noqa: E402
+import full_pools  # noqa: E402
 import poison  # noqa: E402
 from poison import assert_exact, assert_no_poison  # noqa: E402
 
@@ -377,7 +378,7 @@ def test_folded_logits_at_the_ends_of_their_type(dt, walk, grammar, monkeypatch)
 @pytest.mark.parametrize("dt,offset,pad", [(B.DTYPE_BF16, 0, 5), (B.DTYPE_BF16, 3, 0), (B.DTYPE_F32, 0, 0),
                                            (B.DTYPE_F32, 1, 2)])
 @pytest.mark.parametrize("grammar,batch", [("json", 60), ("json", 170), ("sparse", 5), ("sparse", 200),
-                                           ("sparse", 310)])
+                                           ("sparse", 310), ("wide", 20), ("wide", 320)])
 @pytest.mark.parametrize("walk", ["tree", None])
 def test_whole_step_in_one_kernel(dt, offset, pad, grammar, batch, walk, monkeypatch):
     import oracle
@@ -393,7 +394,7 @@ def test_whole_step_in_one_kernel(dt, offset, pad, grammar, batch, walk, monkeyp
         states = np.array([cfg[i][0] for i in pick], np.int32)
         stacks = np.array([synth.pack_stack(cfg[i][1]) for i in pick], np.uint64)
     else:
-        a = synth.random_sparse_dfa(rng, 300)
+        a = synth.random_sparse_dfa(rng, 300, *((100, 12) if grammar == "wide" else ()))
         states, stacks = rng.integers(0, 300, batch).astype(np.int32), None
     d = Domino.from_parts(a, v, device=0)
     P = oracle.Problem.from_parts(a, v)
@@ -409,6 +410,51 @@ def test_whole_step_in_one_kernel(dt, offset, pad, grammar, batch, walk, monkeyp
     assert_exact(mask, m_o, "mask")
     check(x, m_o, V, arg, lse, lp)
     a_o, _, _ = oracle.mask_logits(x, m_o, n_tokens=V, n_threads=NT)
+    s_o, k_o, _ = P.advance(states, stacks, a_o, a.start)
+    assert_exact(st, s_o, "states")
+    if sk is not None:
+        assert_exact(sk, k_o, "stacks")
+    assert d.device_error() == 0
+    d.close()
+    del t
+
+
+@pytest.mark.parametrize("dt,offset,pad", [(B.DTYPE_BF16, 0, 0), (B.DTYPE_BF16, 3, 1), (B.DTYPE_F32, 0, 0),
+                                           (B.DTYPE_F32, 1, 2)])
+@pytest.mark.parametrize("kind", ["plain", "stack", "wide"])
+@pytest.mark.parametrize("batch", [3, 60, 200, 400])
+def test_whole_step_of_rows_that_fill_the_pool(dt, offset, pad, kind, batch, monkeypatch):
+    """1 to 8 CTAs per row; the winner of most rows is a token of 14 to 60 classes, which the update walks."""
+    import oracle
+    monkeypatch.setenv("DOMINO_WALK", "tree")
+    a, v = full_pools.problem(kind)
+    V = v.n_tokens
+    assert min(full_pools.widest_level(kind, q) for q in (1, 2)) > full_pools.POOL
+    rng = np.random.default_rng(batch)
+    states, stacks = full_pools.configurations(kind, batch, batch)
+    P = oracle.Problem.from_parts(a, v)
+    m_o, _, bad = P.step_mask(states, stacks, n_threads=NT)
+    assert bad == 0
+    f = (rng.standard_normal((batch, V)) * 2).astype(np.float32)
+    lens = np.diff(v.offsets)
+    bits = np.unpackbits(np.ascontiguousarray(m_o).view(np.uint8).reshape(batch, -1), axis=1, bitorder="little")[:, :V]
+    for b in range(1, batch):
+        far = np.nonzero(bits[b] & (lens >= 14))[0]
+        if len(far) and b % 5:
+            f[b, far[int(rng.integers(0, len(far)))]] = 20.0
+    x = f if dt == B.DTYPE_F32 else synth.f32_to_bf16_bits(f)
+    t, ptr, stride = placed(x, dt, offset, pad)
+    d = Domino.from_parts(a, v, device=0)
+    st = torch.from_numpy(states).cuda()
+    sk = None if stacks is None else torch.from_numpy(stacks.view(np.int64)).cuda()
+    mask = poison.empty((batch, d.info()["n_words"]), torch.int32)
+    arg, lse = poison.empty(batch, torch.int32), poison.empty(batch, torch.float32)
+    lp = poison.empty((batch, V), torch.float32)
+    B.domino_step_decode(d.h, st, sk, batch, ptr, dt, stride, mask, arg, lse, lp, st, sk)
+    assert_exact(mask, m_o, "mask")
+    check(x, m_o, V, arg, lse, lp)
+    a_o, _, _ = oracle.mask_logits(x, m_o, n_tokens=V, n_threads=NT)
+    assert (lens[np.asarray(a_o)[1:]] >= 14).mean() > 0.4
     s_o, k_o, _ = P.advance(states, stacks, a_o, a.start)
     assert_exact(st, s_o, "states")
     if sk is not None:

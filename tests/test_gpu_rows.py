@@ -17,6 +17,7 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 from paper_2403_06988_gb300 import Domino, synth  # noqa: E402
+import full_pools  # noqa: E402
 import poison  # noqa: E402
 from poison import assert_exact  # noqa: E402
 
@@ -55,6 +56,10 @@ def check(a, v, states, stacks=None, want_next=False):
     assert_exact(mask, m_o, "mask")
     if want_next:
         assert_exact(nxt, n_o, "next")
+        # the mask alone is another kernel, over merged states
+        alone = poison.empty((B, d.info()["n_words"]), torch.int32)
+        d.step_mask(dev(states), None if stacks is None else dev(stacks.view(np.int64)), out_mask=alone)
+        assert_exact(alone, m_o, "mask alone")
     assert d.device_error() == 0
     d.close()
 
@@ -164,41 +169,13 @@ def test_rows_many_tokens_per_node():
     check(a, v, np.tile(np.arange(4, dtype=np.int32), 14)[:53])
 
 
-@pytest.mark.parametrize("stack", [False, True])
+@pytest.mark.parametrize("kind", ["plain", "stack", "wide"])
 @pytest.mark.parametrize("batch", [3, 90, 400])
-def test_rows_full_pools_with_long_tokens(stack, batch):
-    """Two states that lead to one another on all but one of 40 letters, with
-    brackets between them: a row's live nodes pass any pool.  Tokens around the
-    lengths of the token records' parts (15, 31, 32 classes) and beyond."""
-    rng = np.random.default_rng(11)
-    b = synth._Builder()
-    A, C = b.state("a", accepting=True), b.state("c", accepting=True)
-    letters = bytes(range(64, 104))
-    b.edge(A, letters[1:], C)
-    b.edge(C, letters[:-1], A)
-    if stack:
-        b.push(A, b"(", 0, C)
-        b.push(C, b"(", 1, A)
-        b.pop(A, b")", 1, (C, A, C))
-        b.pop(C, b")", 0, (A, C, A))
-    a = b.build(A, 5 if stack else 0, "toggle")
-    al = np.frombuffer(letters + (b"()" if stack else b""), np.uint8)
-    toks = set()
-    for L in (14, 15, 16, 30, 31, 32, 33, 60):
-        for _ in range(20):
-            toks.add(rng.choice(al, L).tobytes())
-    while len(toks) < 9000:
-        toks.add(rng.choice(al, int(rng.integers(1, 6))).tobytes())
-    toks = sorted(toks)
-    rng.shuffle(toks)
-    toks = [bytes(t) for t in toks]
-    v = synth.Vocab.from_tokens(toks[:700] + [b""] + toks[700:], eos_id=700)
-    states = rng.integers(0, 3, batch).astype(np.int32)
-    stacks = None
-    if stack:
-        stacks = np.array([synth.pack_stack(list(rng.integers(0, 2, int(rng.integers(0, 6))))) for _ in range(batch)],
-                          np.uint64)
-        stacks[states == 0] = 0
+def test_rows_full_pools_with_long_tokens(kind, batch):
+    """Rows with more live nodes than the pool holds (tests/full_pools.py)."""
+    a, v = full_pools.problem(kind)
+    assert min(full_pools.widest_level(kind, q) for q in (1, 2)) > full_pools.POOL
+    states, stacks = full_pools.configurations(kind, batch, 11)
     check(a, v, states, stacks, want_next=True)
 
 
