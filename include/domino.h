@@ -145,10 +145,11 @@ int domino_get_info(domino_t h, domino_info* out);
 /* Byte -> class id map of the loaded automaton (256 bytes, host). */
 int domino_get_byte_classes(domino_t h, uint8_t* classes_out);
 
-/* The prefix tree that the mask step walks (host copies, for inspection):
- * Alg. 2's subterminal tree (Sec. 3.3) over the byte-class strings of every
- * token except EOS and empty tokens.  Nodes are numbered in preorder, children
- * by class; node n is 8 uint32 words:
+/* The prefix tree of the vocabulary (host copies, for inspection): Alg. 2's
+ * subterminal tree (Sec. 3.3) over the byte-class strings of every token except
+ * EOS and empty tokens.  The mask step walks the same tree, numbered breadth
+ * first.  Here nodes are numbered in preorder, children by class; node n is 8
+ * uint32 words:
  *   [0] skip | cls << 24  (n's subtree is nodes [n, skip); cls: the class on
  *                          the edge into n, 0 for the root, node 0)
  *   [1] tok_lo  [2] n_end [3] tok_hi   (tokens_out[tok_lo, tok_lo + n_end) end
@@ -158,10 +159,11 @@ int domino_get_byte_classes(domino_t h, uint8_t* classes_out);
  * tokens_out: original token ids in preorder.
  * upper_out [n_upper][2] = {node, depth}: the root and every node whose
  *   subtree has more than 64 nodes or more than 8 branching levels, in
- *   preorder; a row's configuration at each of them is computed first.
+ *   preorder.
  * units_out [n_units][2] = {root node, index of its parent in upper_out}: the
- *   subtrees hanging off upper nodes, in preorder; each live (row, unit) pair
- *   is walked on its own.
+ *   subtrees hanging off upper nodes, in preorder.  Upper nodes and units cut
+ *   the tree into parts that can be walked on their own; the mask step does not
+ *   use the cut.
  * sizes_out[4] (required) = {nodes, tokens, upper nodes, units}.  Each array
  * is copied up to its capacity (in entries) and may be NULL.  Available on
  * host-only handles too.  DOMINO_E_UNSUPPORTED: the tree exceeds 2^24 - 1

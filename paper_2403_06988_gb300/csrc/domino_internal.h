@@ -71,7 +71,8 @@ struct StepView {
 };
 
 // Prefix tree of the vocabulary's byte-class strings (the subterminal tree of
-// Sec. 3.3, Alg. 2, over byte classes) as domino_get_prefix_tree exports it.
+// Sec. 3.3, Alg. 2, over byte classes) as domino_get_prefix_tree exports it
+// (RowTree below is what the kernel reads).
 // Nodes are numbered in preorder (children by class), so a subtree is the
 // contiguous range [n, skip) and the tokens of a subtree are a contiguous
 // range of the token list: the tokens that end at n first, then those of its

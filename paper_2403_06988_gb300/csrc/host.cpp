@@ -195,8 +195,8 @@ void clear_host_graphs(domino_ctx* h) {
 // nodes of their longest common prefix and opens new nodes for the rest, so
 // nodes come out in preorder.  EOS and empty tokens are not in the tree (the
 // kernel sets EOS from the row's acceptance; other empty tokens are never
-// allowed).  Host arrays only (domino_get_prefix_tree; build_rows lays out
-// the trees the kernel walks).
+// allowed).  Host arrays only: domino_get_prefix_tree copies them, and
+// make_row_image takes the tokens' order for the trees the kernel walks.
 void build_trie_host(domino_ctx* h) {
     h->trie_built = false;
     h->t_node.clear();

@@ -464,8 +464,10 @@ cudaError_t launch_mask_logits(const LaunchEnv& env, const void* logits, int dty
     // The gather wants one CTA per row to fill the SMs, aligned bf16 rows, and
     // no second pass: there it is the faster one where masks are sparse
     // (GB300, V = 128256, 1 % allowed, batch 256: 6.0 against 8.0 us, batch
-    // 1000: 22 against 29 us; JSON, V = 152064, batch 512, mostly dense: 45
-    // against 38 us).  With fewer rows, or rows off 16-byte boundaries, fp32 or
+    // 1000: 22 against 29 us) and the slower one where they are dense (JSON, V =
+    // 152064, batch 512: 45 against 38 us).  The host does not see the masks
+    // and takes the gather for all of these batches, the unmasked argmax and
+    // draws among them.  With fewer rows, or rows off 16-byte boundaries, fp32 or
     // log-probabilities, the cluster kernel: V = 152064, batch 128, 80 %
     // allowed: 12.9 us (24.6 us for the flat split over one-warp CTAs that it
     // replaced), with log-probabilities 27.7 us (40.0); batch 24, V = 50001:

@@ -26,11 +26,13 @@
 // a share of the tree and walked every row in it), batch 1000 49.1 us (94.1),
 // batch 32 13.5 us (19.0); the 20000-state table 2.62 ms (3.25 ms).
 //
-// A row with more live nodes than the pool holds is walked token by token
-// instead (every_token), which bounds what a dense state costs: 500 states
-// with 16 of 32 classes live, V = 128256, one row 26 us, 28 classes live 51
-// us.  Small batches and automata most of whose states are like that are the
-// per-token walk's from the start (use_rows, decode_rows in host.cpp).
+// A row with more live nodes at a time than the pool holds is walked token by
+// token instead (every_token), which bounds what a dense state costs: 500
+// states with 16 of 32 classes live, V = 128256, one row 26 us, 28 classes live
+// 51 us.  Small batches and automata most of whose rows are like that are the
+// per-token walk's from the start (row_cost, use_rows, decode_rows in host.cpp).
+// With more than 64 classes the children's entries are read instead of masks
+// (add_wide).
 //
 // States that loop on most classes (string bodies) allow nearly every token.
 // For the widest such loop sets the host keeps the tokens that stay inside

@@ -1,15 +1,16 @@
-"""The prefix tree the mask step walks (Alg. 2's subterminal tree over byte
-classes, Sec. 3.3), checked on the CPU through a host-only handle:
+"""The prefix tree of the vocabulary (Alg. 2's subterminal tree over byte
+classes, Sec. 3.3) as domino_get_prefix_tree exports it, checked on the CPU
+through a host-only handle (the arrays that the row walk itself reads:
+tests/test_row_trees.py):
 
 - structure: preorder numbering, nested token ranges, every token of the
   vocabulary except EOS and empty tokens exactly once, at the node whose path
   spells its class string; children in class order; the classes-below sets;
   the upper nodes (large subtrees) and the units (the subtrees hanging off
   them) cover every node once;
-- a model of the two kernels over the exported arrays (each row's
-  configuration at the upper nodes, then one walk per live (row, unit) pair
-  with a stack of at most kTrieBranch entries) gives the oracle's masks and
-  next states on workload rows.
+- a walk over the exported arrays (each row's configuration at the upper nodes,
+  then one walk per live (row, unit) pair with a stack of at most kTrieBranch
+  entries) gives the oracle's masks and next states on workload rows.
 """
 import numpy as np
 import pytest
@@ -183,7 +184,7 @@ class Model:
         cfg0 = (int(s0), int(stack_word) & 0xFFFFFFFF, int(stack_word) >> 32)
         if self.v.eos_id >= 0 and cfg0[2] == 0 and self.a.accepting[cfg0[0]]:
             allowed[self.v.eos_id] = cfg0[0]
-        # the upper kernel: the row's configuration at every upper node
+        # the row's configuration at every upper node
         ucfg = []
         for (u, _), p in zip(self.upper.tolist(), self.upaths):
             cfg = cfg0
@@ -194,7 +195,7 @@ class Model:
                 lo, ne = int(nodes[u, 1]), int(nodes[u, 2])
                 for t in toks[lo:lo + ne].tolist():
                     allowed[t] = cfg[0]
-        # the tile kernel: one walk per live (unit, row) pair
+        # one walk per live (unit, row) pair
         for root, pu in self.units.tolist():
             if ucfg[pu] is not None:
                 self.walk(root, ucfg[pu], allowed)
