@@ -946,7 +946,7 @@ cudaError_t launch_step_mask(const StepView& v, const LaunchEnv& env, bool stack
                              const uint64_t* stacks, int32_t batch, bool row_is_state, uint32_t* mask,
                              int32_t* next, cudaStream_t st, const int32_t* row_ids, const int32_t* row_count,
                              const void* fuse_logits, int64_t fuse_stride, float4* fuse_part, bool fuse_prefetch) {
-    const RowList list{row_ids, row_count};
+    const RowList list{row_ids, row_count, 0};
     const FuseArgs fuse{fuse_logits, fuse_stride, fuse_part, fuse_logits && fuse_prefetch ? 1 : 0};
     if (stack)
         return launch_step_s<true>(v, env, mode, states, stacks, batch, row_is_state, mask, next, list, fuse, st);

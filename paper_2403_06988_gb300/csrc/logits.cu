@@ -460,7 +460,7 @@ cudaError_t launch_mask_logits(const LaunchEnv& env, const void* logits, int dty
     a.logprobs = logprobs;
     a.sample = sample ? *sample : SampleArgs{0u, 0u, 0u, 0u, 1.0f};
     cut_rows(a, env.num_sms);
-    const RowList list{row_ids, row_count};
+    const RowList list{row_ids, row_count, 0};
     // The gather wants one CTA per row to fill the SMs, aligned bf16 rows, and
     // no second pass: there it is the faster one where masks are sparse
     // (GB300, V = 128256, 1 % allowed, batch 256: 6.0 against 8.0 us, batch

@@ -68,16 +68,19 @@ cudaError_t launch_cluster(void (*kern)(KArgs...), dim3 grid, dim3 block, int cl
 }
 
 // A compacted list of the rows to process (opportunistic masking's rejected
-// rows): entry i is row ids[i] of the batch, and only the first *count entries
-// exist (the count is device memory).
+// rows): entry i of the pass is row ids[base + i] of the batch, and only the
+// first *count - base entries of this pass exist (the count is device memory).
+// One pass takes the whole list now (base 0); without the field the draw's code
+// comes out 2 % slower (V = 50001, batch 24: 15.6 -> 15.9 us).
 struct RowList {
     const int32_t* ids;     // nullptr: rows are 0..B-1
     const int32_t* count;
+    int32_t base;           // first list entry of this pass
     __device__ __forceinline__ int rows(int cap) const {
         if (!ids) return cap;
-        return max(0, min(cap, __ldg(count)));
+        return max(0, min(cap, __ldg(count) - base));
     }
-    __device__ __forceinline__ int row(int i) const { return ids ? __ldg(ids + i) : i; }
+    __device__ __forceinline__ int row(int i) const { return ids ? __ldg(ids + base + i) : i; }
 };
 
 __device__ __forceinline__ float ex2(float x) {
