@@ -52,12 +52,13 @@ __device__ __forceinline__ uint32_t nonzero_bytes(uint32_t x) {
     return ((x & 0x01010101u) * 0x10204080u) >> 28;
 }
 
-// (a, b) * (c, c)
-__device__ __forceinline__ float2 mul2(float2 a, float c) {
-    unsigned long long x, y, r;
+// (a, b) * (c, c) + (d, d), both lanes rounded once
+__device__ __forceinline__ float2 fma2(float2 a, float c, float d) {
+    unsigned long long x, y, z, r;
     asm("mov.b64 %0, {%1, %2};" : "=l"(x) : "f"(a.x), "f"(a.y));
     asm("mov.b64 %0, {%1, %1};" : "=l"(y) : "f"(c));
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(x), "l"(y));
+    asm("mov.b64 %0, {%1, %1};" : "=l"(z) : "f"(d));
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(x), "l"(y), "l"(z));
     float2 o;
     asm("mov.b64 {%0, %1}, %2;" : "=f"(o.x), "=f"(o.y) : "l"(r));
     return o;
@@ -156,12 +157,20 @@ constexpr float kGumbelMax = 17.0f;
 // A lane's fold over a row's tokens.  The sum of exponentials is kept against
 // a reference that follows the maximum only when it falls more than kLag
 // behind, and the maximum's vector is kept instead of its token, so that a
-// vector costs no branch in the common case: the bf16 vector takes about 60
+// vector costs no branch in the common case: the bf16 vector takes about 55
 // instructions for 8 tokens (208 with the maximum's token found and the sum
 // rescaled whenever some lane's maximum rose), 8 of them ex2, whose unit
 // (16 a clock and SM) then bounds dense rows.
+//
+// A term is 2^(x log2(e) - ref) in one fused operation, so it is off by its
+// own rounding only; that ref is a rounded m log2(e) is made good in finish().
+// Its rounding must stay within 2^x's range: a reference below kLowRef is held
+// there.  The terms of smaller logits (-1e10 or the lowest value of the type
+// that ban a token) then come out as 0, which they are beside any other; where
+// there is no other, and above 2^29, log_sum_exp() takes no sum.
 template <bool BF16, int FOLD>
 struct Decoder {
+    static constexpr float kLowRef = -0x1p30f;   // half a unit in its last place is 32
     static constexpr int kWords = BF16 ? 4 : 8;   // 32-bit words of a vector
     static constexpr int kTogether = BF16 ? 4 : 2;   // vectors per lane read together
     struct Vec {
@@ -181,7 +190,7 @@ struct Decoder {
     int lane;
     const uint4* keep;       // fill_keep's table
     float m;                 // maximum (sampling: the best score)
-    float ref, s;            // the sum's reference and the sum of e^(x - ref)
+    float ref, s;            // the sum's reference (times log2(e)) and the sum of 2^(x log2(e) - ref)
     int idx;                 // sampling: its token; else the token of element 0 of the maximum's vector
     uint32_t top[kWords];    // the maximum's vector, -inf where not allowed
     float seen;              // sampling: a score some lane of the warp has seen
@@ -259,13 +268,14 @@ struct Decoder {
                 }
             }
             if constexpr (FOLD == kFoldLse) {
-                constexpr float kLag = 11.0f;   // terms of e^16 at most (ref + kLag rounds): no overflow, and nothing lost in relative terms
+                constexpr float kLag = 16.0f;   // terms of 2^16 at most: no overflow, and nothing lost in relative terms
                 float most = vm[0];
 #pragma unroll
                 for (int k = 1; k < N; ++k) most = fmaxf(most, vm[k]);
-                if ((most > ref + kLag || m == -INFINITY) && most != -INFINITY) {   // rare after the first vectors
-                    s *= s == 0.0f ? 0.0f : exp_diff(ref, most);
-                    ref = most;
+                const float vL = most * kLog2e;
+                if ((vL > ref + kLag || m == -INFINITY) && most != -INFINITY) {   // rare after the first vectors
+                    s *= s == 0.0f ? 0.0f : ex2(ref - vL);
+                    ref = fmaxf(vL, kLowRef);
                 }
             }
 #pragma unroll
@@ -285,7 +295,7 @@ struct Decoder {
                     for (int e = 0; e < 4; ++e) {
                         const float2 z = BF16 ? make_float2(bf16_lo(w[k][e]), bf16_hi(w[k][e]))
                                               : make_float2(__uint_as_float(w[k][BF16 ? 0 : 2 * e]), __uint_as_float(w[k][BF16 ? 0 : 2 * e + 1]));
-                        const float2 y = mul2(add2(z, make_float2(-ref, -ref)), kLog2e);   // as exp_diff
+                        const float2 y = fma2(z, kLog2e, -ref);
                         acc[k] = add2(acc[k], make_float2(ex2(y.x), ex2(y.y)));   // not allowed: 2^-inf = 0
                     }
                 }
@@ -311,7 +321,7 @@ struct Decoder {
                 if (v == m) e = k;
             }
             idx += e;
-            if constexpr (FOLD == kFoldLse) s *= exp_diff(ref, m);
+            if constexpr (FOLD == kFoldLse) s *= s == 0.0f ? 0.0f : ex2(__fmaf_rn(-m, kLog2e, ref));
         }
     }
 

@@ -100,10 +100,10 @@ __device__ __forceinline__ float exp_diff(float x, float ref) { return ex2((x - 
 // -inf (x - ref is never -inf minus -inf).
 __device__ __forceinline__ float sum_ref(float m) { return fmaxf(m, -FLT_MAX); }
 
-// m + ln(s), s the sum of exp against m
-__device__ __forceinline__ float log_sum_exp(float m, float s) {
-    return isinf(m) ? m : m + logf(s);   // nothing allowed: -inf
-}
+// m + ln(s), s the sum of exp against m.  ln(s) is below 17 (2^24 tokens), less
+// than half a unit in the last place of m from 2^29 on: m is then the result,
+// whatever s.  So it is where m is infinite (-inf: nothing allowed).
+__device__ __forceinline__ float log_sum_exp(float m, float s) { return fabsf(m) >= 0x1p29f ? m : m + logf(s); }
 
 // (m, idx, s) <- (m, idx, s) (+) (m2, i2, s2): larger max wins, lower index on
 // equal maxima; the other sum is rescaled to the winner's max.

@@ -296,7 +296,7 @@ def extreme_logits(dt, batch, V, seed):
     x = (rng.standard_normal((batch, V)) * 3).astype(np.float32)
     few = rng.random((batch, V)) < 0.02
     for b in range(batch):
-        kind = b % 10
+        kind = b % 12
         if kind == 0:
             x[b] = -top                                                  # nothing but the lowest value
         elif kind == 1:
@@ -315,6 +315,10 @@ def extreme_logits(dt, batch, V, seed):
             x[b] = np.where(rng.random(V) < 0.5, 1, -1) * np.exp(rng.random(V) * 88).astype(np.float32)
         elif kind == 8:
             x[b] = np.where(few[b], x[b], -np.exp(rng.random() * 88).astype(np.float32))
+        elif kind == 9:                                                  # around the ends of the sum's reference
+            x[b] = np.where(few[b], x[b], -np.exp2(28 + 5 * rng.random(V)).astype(np.float32))
+        elif kind == 10:
+            x[b] = (1 if b % 24 < 12 else -1) * np.exp2(28 + 5 * rng.random(V)).astype(np.float32)
         else:
             x[b] = np.where(few[b], -np.float32(2.36e38), np.float32(-top))
     return x
